@@ -116,7 +116,7 @@ static int device_info(const DeviceInfo** out) {
     prepare(k_finalize<NSML_BF16, kFinLargeThreads, kFinLargeCache>, kFinLargeThreads, kFinLargeCache, &d.finalize_large);
     prepare(k_finalize_dense<NSML_F32, kFinLargeThreads, kFinDenseLargeCache>, kFinLargeThreads, kFinDenseLargeCache, &d.finalize_large);
     prepare(k_finalize_dense<NSML_BF16, kFinLargeThreads, kFinDenseLargeCache>, kFinLargeThreads, kFinDenseLargeCache, &d.finalize_large);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.merge, k_merge, kCta, 0);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.merge, k_merge<kDenseTileLarge>, kMergeThreads, 0);
     // The streaming kernels run as one wave of resident blocks (a second, partial wave would read
     // with a fraction of the SMs' loads in flight).
     auto resident = [&](auto kernel, int* out) {
@@ -199,6 +199,23 @@ static cudaError_t launch_prio(void (*kernel)(KArgs...), dim3 grid, dim3 block, 
   }
   cfg.attrs = attr;
   cfg.numAttrs = na;
+  return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+
+// Launches a kernel that may start while its predecessor in the stream still runs (programmatic dependent launch):
+// it calls pdl_wait before it touches anything the predecessor writes.
+template <class... KArgs, class... Args>
+static cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
 }
 
@@ -420,24 +437,18 @@ static int accumulate_impl(const void* const* payloads, const size_t* payload_by
   unsigned char* ws = static_cast<unsigned char*>(workspace);
   int* status = reinterpret_cast<int*>(ws);
   unsigned int* offsets = reinterpret_cast<unsigned int*>(ws + L.offsets);
-  const unsigned int tiles = (unsigned int)((n + kDenseTile - 1) / kDenseTile);
+  const unsigned int tile = (unsigned int)dense_tile(n);
+  const unsigned int tiles = (unsigned int)((n + tile - 1) / tile);
   {
     LaunchScope scope(K_PARTITION, st, timed);  // also clears the status word
-    const unsigned long long offsets_needed = (unsigned long long)W * (tiles + 1ull);
-    if (offsets_needed <= 4096) {  // few offsets: a warp each, few round trips (from about ten thousand offsets on the
-                                   // thread-per-offset form takes as long alone, 12.8 us, and leaves the SMs to other streams:
-                                   // eight-stream step of the default workload 0.645 -> 0.626 ms)
-      unsigned int grid = (unsigned int)((offsets_needed * 32 + kCta - 1) / kCta);
-      launch_prio(k_partition, dim3(grid), dim3(kCta), 0, st, false, 0, true, table, W, (unsigned long long)n, tiles, offsets, status);
-    } else {  // many offsets: a thread each
-      unsigned int grid = (unsigned int)((offsets_needed + kCta - 1) / kCta);
-      launch_prio(k_partition_wide, dim3(grid), dim3(kCta), 0, st, false, 0, true, table, W, (unsigned long long)n, tiles, offsets, status);
-    }
+    launch_prio(k_partition, dim3(tiles / kPartBounds + 1, W), dim3(kPartBounds), 0, st, false, 0, true, table, W, (unsigned long long)n,
+                tiles, tile, offsets, status);
   }
   {
     LaunchScope scope(K_MERGE, st, timed);
-    unsigned int grid = grid_for(tiles, 1, dev->sms * dev->merge);
-    k_merge<<<grid, kCta, 0, st>>>(table, W, dense, (unsigned long long)n, zero_first, tiles, offsets, status);
+    const unsigned int grid = grid_for(tiles, 1, dev->sms * dev->merge);
+    auto kernel = tile == kDenseTileLarge ? k_merge<kDenseTileLarge> : k_merge<kDenseTileSmall>;
+    launch_dependent(kernel, dim3(grid), dim3(kMergeThreads), 0, st, table, W, dense, (unsigned long long)n, zero_first, tiles, offsets, status);
   }
   if (cudaGetLastError() != cudaSuccess) return NSML_ERR_CUDA;
   return NSML_OK;

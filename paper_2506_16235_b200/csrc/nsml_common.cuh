@@ -96,6 +96,21 @@ inline PayloadLayout payload_layout(int64_t k, int bits) {
 
 __device__ __forceinline__ void set_status(int* status, int code) { atomicCAS(status, 0, code); }
 
+// ---- programmatic dependent launch: a kernel launched with the attribute may start while its predecessor in the
+// stream still runs; pdl_wait returns when the predecessor has completed and its writes are visible.
+__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// ---- bulk copy shared -> global by one thread (16-byte aligned addresses and size) ----
+// Writers of the shared memory call fence_async_shared, then the block synchronises, then one thread stores.
+__device__ __forceinline__ void fence_async_shared() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+__device__ __forceinline__ void bulk_store(void* gdst, const void* smem_src, unsigned int bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(gdst),
+               "r"((uint32_t)__cvta_generic_to_shared(smem_src)), "r"(bytes) : "memory");
+  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+__device__ __forceinline__ void bulk_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+
 // ------------------------------------------------------------------------
 // Element sources.  load_vals4 returns the float32 bit patterns of elements
 // i0..i0+3 (i0 a multiple of 4) and how many of them exist (0..4); missing
