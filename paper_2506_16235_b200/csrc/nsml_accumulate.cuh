@@ -260,7 +260,7 @@ k_merge(PayloadTable table, int W, float* __restrict__ dense, unsigned long long
   }
   pdl_wait();  // the offsets are complete
   const unsigned int* my_offsets = offsets + threadIdx.x * per;  // thread w looks after worker w's ranges
-  if (threadIdx.x < W && blockIdx.x < tiles) s_range[0][threadIdx.x] = make_uint2(my_offsets[blockIdx.x], my_offsets[blockIdx.x + 1]);
+  if (threadIdx.x < W && blockIdx.x < tiles) s_range[0][threadIdx.x] = make_uint2(__ldcg(my_offsets + blockIdx.x), __ldcg(my_offsets + blockIdx.x + 1));
   int buf = 0;
   for (unsigned int tile = blockIdx.x; tile < tiles; tile += gridDim.x, buf ^= 1) {
     const unsigned long long lo = (unsigned long long)tile * TILE;
@@ -272,7 +272,7 @@ k_merge(PayloadTable table, int W, float* __restrict__ dense, unsigned long long
     // the next tile's ranges are fetched while this tile is summed
     uint2 ahead = make_uint2(0u, 0u);
     const bool fetch = threadIdx.x < W && (unsigned long long)tile + gridDim.x < tiles;
-    if (fetch) ahead = make_uint2(my_offsets[tile + gridDim.x], my_offsets[tile + gridDim.x + 1]);
+    if (fetch) ahead = make_uint2(__ldcg(my_offsets + tile + gridDim.x), __ldcg(my_offsets + tile + gridDim.x + 1));
 
     bool staged = zero_first;
     if (!zero_first) {

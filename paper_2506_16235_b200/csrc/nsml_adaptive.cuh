@@ -244,7 +244,7 @@ k_prune_hist(BucketSrc<NSML_F32> src, unsigned long long n, unsigned int m, Prun
              uint2* __restrict__ tie_list) {
   constexpr int NB = (LEVEL == 2) ? 128 : kMaxBins;
   __shared__ unsigned int s_hist[NB];
-  __shared__ unsigned int s_tot[kCta / 32], s_out[2];
+  __shared__ unsigned int s_tot[kCta / 32], s_out[3];
   if (ctl->fast_ok != 0) return;  // the two-pass path has built the mask
   unsigned int prefix = 0;
   bool collect = false;
@@ -339,7 +339,7 @@ k_prune_hist(BucketSrc<NSML_F32> src, unsigned long long n, unsigned int m, Prun
 __global__ void __launch_bounds__(kCta)
 k_prune_ties(BucketSrc<NSML_F32> src, unsigned long long n, PruneCtl* ctl, const unsigned int* __restrict__ hist,
              const uint2* __restrict__ tie_list, unsigned int* __restrict__ tile_ties) {
-  __shared__ unsigned int s_tot[kCta / 32], s_out[2];
+  __shared__ unsigned int s_tot[kCta / 32], s_out[3];
   __shared__ unsigned int s_cnt[kCta / 32];
   __shared__ uint32_t s_tied[kTieCap];
   __shared__ unsigned int s_ntied;
@@ -573,7 +573,7 @@ k_prune_sample(BucketSrc<NSML_F32> src, unsigned long long n, unsigned int rank_
   constexpr int THREADS = 1024, PER_THREAD = kPruneSamples / THREADS;  // 8 scattered loads in flight per thread
   __shared__ __align__(16) unsigned int s_hist_lo[kMaxBins];
   __shared__ __align__(16) unsigned int s_hist_hi[kMaxBins];
-  __shared__ unsigned int s_tot[THREADS / 32], s_out[2];
+  __shared__ unsigned int s_tot[THREADS / 32], s_out[3];
   const int t = threadIdx.x;
   const unsigned long long width = n / kPruneSamples;  // >= 2
   uint32_t keys[PER_THREAD];
@@ -680,7 +680,7 @@ k_prune_count(BucketSrc<NSML_F32> src, unsigned long long n, PruneCtl* ctl, unsi
 // One block: the window's bin that holds the m-th largest key, if the window holds it at all.
 __global__ void __launch_bounds__(kCta)
 k_prune_settle(unsigned int m, PruneCtl* ctl, const unsigned int* __restrict__ fine) {
-  __shared__ unsigned int s_tot[kCta / 32], s_out[2];
+  __shared__ unsigned int s_tot[kCta / 32], s_out[3];
   __shared__ unsigned long long s_sum[kCta / 32];
   constexpr int PER = kPruneFineBins / kCta;
   unsigned int own[PER];

@@ -13,19 +13,20 @@
 #include "nsml_compact.cuh"
 #include "nsml_finalize.cuh"
 #include "nsml_dense.cuh"
+#include "nsml_list.cuh"
 #include "nsml_select.cuh"
 
 namespace nsml {
 
 enum KernelId {
   K_SAMPLE = 0, K_COMPACT_BUCKET, K_FINALIZE, K_PARTITION, K_MERGE, K_CLEAR, K_FINALIZE_DENSE,
-  K_SUMSQ, K_FEEDBACK_ADD, K_FEEDBACK_SUBTRACT, K_PRUNE_HIST, K_PRUNE_TIES, K_PRUNE_WRITE, K_PRUNE_WRITE_RANKED, K_GATHER, K_PRUNE_SAMPLE, K_PRUNE_COUNT, K_PRUNE_SETTLE, K_PRUNE_MARK, K_PRUNE_FIX, K_COUNT
+  K_SUMSQ, K_FEEDBACK_ADD, K_FEEDBACK_SUBTRACT, K_PRUNE_HIST, K_PRUNE_TIES, K_PRUNE_WRITE, K_PRUNE_WRITE_RANKED, K_PRUNE_SAMPLE, K_PRUNE_COUNT, K_PRUNE_SETTLE, K_PRUNE_MARK, K_PRUNE_FIX, K_COUNT
 };
 
 static const char* const kKernelNames[K_COUNT] = {"k_sample", "k_compact_bucket", "k_finalize", "k_partition", "k_merge",
                                                   "k_clear", "k_finalize_dense", "k_sumsq", "k_feedback_add",
                                                   "k_feedback_subtract", "k_prune_hist", "k_prune_ties", "k_prune_write",
-                                                  "k_prune_write_ranked", "k_gather", "k_prune_sample", "k_prune_count",
+                                                  "k_prune_write_ranked", "k_prune_sample", "k_prune_count",
                                                   "k_prune_settle", "k_prune_mark", "k_prune_fix"};
 
 static std::atomic<int64_t> g_launches{0};
@@ -80,9 +81,8 @@ struct LaunchScope {  // brackets one kernel launch
 struct DeviceInfo {
   bool ready = false;
   int sms = 0;
-  int compact_feedback = 0, finalize_small = 0, finalize_large = 0, merge = 0;  // resident blocks per SM
+  int dense_small = 0, dense_large = 0, merge = 0;  // resident blocks per SM
   int sumsq = 0, feedback_add = 0, prune_hist = 0, prune_write = 0, prune_write_ranked = 0;  // the same, streaming kernels
-  bool finalize_cluster = false;  // the one-cluster shape of the list stage fits an SM
 };
 static DeviceInfo g_dev[64];
 static std::mutex g_dev_mutex;
@@ -95,27 +95,25 @@ static int device_info(const DeviceInfo** out) {
   if (!d.ready) {
     if (cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return NSML_ERR_CUDA;
     cudaError_t e = cudaSuccess;
-    e = cudaFuncSetAttribute(k_compact_bucket<NSML_F32, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCompactFeedbackSmem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_compact_bucket<NSML_BF16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCompactFeedbackSmem);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.compact_feedback, k_compact_bucket<NSML_F32, true>, kCta, kCompactFeedbackSmem);
-    auto prepare = [&](auto kernel, int threads, int cache, int* resident) {
-      if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)finalize_dyn_smem(cache));
+    auto prepare = [&](auto kernel, int threads, size_t smem, int* resident) {
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       int r = 0;
-      if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, kernel, threads, finalize_dyn_smem(cache));
+      if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, kernel, threads, smem);
       if (*resident == 0 || r < *resident) *resident = r;
     };
-    prepare(k_finalize<NSML_F32, kFinSmallThreads, kFinSmallCache>, kFinSmallThreads, kFinSmallCache, &d.finalize_small);
-    prepare(k_finalize<NSML_BF16, kFinSmallThreads, kFinSmallCache>, kFinSmallThreads, kFinSmallCache, &d.finalize_small);
-    prepare(k_finalize_dense<NSML_F32, kFinSmallThreads, kFinSmallCache>, kFinSmallThreads, kFinSmallCache, &d.finalize_small);
-    prepare(k_finalize_dense<NSML_BF16, kFinSmallThreads, kFinSmallCache>, kFinSmallThreads, kFinSmallCache, &d.finalize_small);
-    int cluster_shape = 0;
-    prepare(k_finalize<NSML_F32, kFinClusterThreads, kFinClusterCache, true>, kFinClusterThreads, kFinClusterCache, &cluster_shape);
-    prepare(k_finalize<NSML_BF16, kFinClusterThreads, kFinClusterCache, true>, kFinClusterThreads, kFinClusterCache, &cluster_shape);
-    d.finalize_cluster = cluster_shape >= 1;
-    prepare(k_finalize<NSML_F32, kFinLargeThreads, kFinLargeCache>, kFinLargeThreads, kFinLargeCache, &d.finalize_large);
-    prepare(k_finalize<NSML_BF16, kFinLargeThreads, kFinLargeCache>, kFinLargeThreads, kFinLargeCache, &d.finalize_large);
-    prepare(k_finalize_dense<NSML_F32, kFinLargeThreads, kFinDenseLargeCache>, kFinLargeThreads, kFinDenseLargeCache, &d.finalize_large);
-    prepare(k_finalize_dense<NSML_BF16, kFinLargeThreads, kFinDenseLargeCache>, kFinLargeThreads, kFinDenseLargeCache, &d.finalize_large);
+    prepare(k_finalize_dense<NSML_F32, kFinSmallThreads, kFinSmallCache>, kFinSmallThreads, finalize_dyn_smem(kFinSmallCache), &d.dense_small);
+    prepare(k_finalize_dense<NSML_BF16, kFinSmallThreads, kFinSmallCache>, kFinSmallThreads, finalize_dyn_smem(kFinSmallCache), &d.dense_small);
+    prepare(k_finalize_dense<NSML_F32, kFinLargeThreads, kFinDenseLargeCache>, kFinLargeThreads, finalize_dyn_smem(kFinDenseLargeCache), &d.dense_large);
+    prepare(k_finalize_dense<NSML_BF16, kFinLargeThreads, kFinDenseLargeCache>, kFinLargeThreads, finalize_dyn_smem(kFinDenseLargeCache), &d.dense_large);
+    int list_fits = 0;  // every shape of the list stage is resident at least once per SM
+    prepare(k_finalize<NSML_F32, kListSmallCache, true>, kListThreads, list_dyn_smem(kListSmallCache), &list_fits);
+    prepare(k_finalize<NSML_BF16, kListSmallCache, true>, kListThreads, list_dyn_smem(kListSmallCache), &list_fits);
+    prepare(k_finalize<NSML_F32, kListSmallCache, false>, kListThreads, list_dyn_smem(kListSmallCache), &list_fits);
+    prepare(k_finalize<NSML_BF16, kListSmallCache, false>, kListThreads, list_dyn_smem(kListSmallCache), &list_fits);
+    prepare(k_finalize<NSML_F32, kListLargeCache, false>, kListThreads, list_dyn_smem(kListLargeCache), &list_fits);
+    prepare(k_finalize<NSML_BF16, kListLargeCache, false>, kListThreads, list_dyn_smem(kListLargeCache), &list_fits);
+    prepare(k_sample<NSML_F32>, kSampleThreads, kSampleSmem, &list_fits);
+    prepare(k_sample<NSML_BF16>, kSampleThreads, kSampleSmem, &list_fits);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.merge, k_merge<kDenseTileLarge>, kMergeThreads, 0);
     // The streaming kernels run as one wave of resident blocks (a second, partial wave would read
     // with a fraction of the SMs' loads in flight).
@@ -137,7 +135,7 @@ static int device_info(const DeviceInfo** out) {
     if (e == cudaSuccess && (d.sumsq < 1 || d.feedback_add < 1 || d.prune_hist < 1 || d.prune_write < 1 || d.prune_write_ranked < 1)) e = cudaErrorUnknown;
     int coop = 0;
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-    if (e != cudaSuccess || d.compact_feedback < 1 || d.finalize_small < 1 || d.finalize_large < 1 || d.merge < 1 || !coop) {
+    if (e != cudaSuccess || d.dense_small < 1 || d.dense_large < 1 || list_fits < 1 || d.merge < 1 || !coop) {
       cudaGetLastError();
       return NSML_ERR_CUDA;
     }
@@ -174,13 +172,13 @@ static int high_priority() {
 
 template <class... KArgs, class... Args>
 static cudaError_t launch_prio(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool cooperative,
-                               unsigned int cluster_x, bool high, Args... args) {
+                               unsigned int cluster_x, bool high, bool dependent, Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[3];
+  cudaLaunchAttribute attr[4];
   unsigned int na = 0;
   attr[na].id = cudaLaunchAttributePriority;
   attr[na].val.priority = high ? high_priority() : 0;
@@ -197,25 +195,14 @@ static cudaError_t launch_prio(void (*kernel)(KArgs...), dim3 grid, dim3 block, 
     attr[na].val.clusterDim.z = 1;
     ++na;
   }
+  if (dependent) {  // may start while its predecessor in the stream still runs (programmatic dependent launch); the
+                    // kernel calls pdl_wait before it touches anything the predecessor writes
+    attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[na].val.programmaticStreamSerializationAllowed = 1;
+    ++na;
+  }
   cfg.attrs = attr;
   cfg.numAttrs = na;
-  return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
-}
-
-// Launches a kernel that may start while its predecessor in the stream still runs (programmatic dependent launch):
-// it calls pdl_wait before it touches anything the predecessor writes.
-template <class... KArgs, class... Args>
-static cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
 }
 
@@ -228,34 +215,35 @@ static int64_t k_of(int64_t n, double ratio) {
   return k;
 }
 
-// Rank (from the top, 1-based) of the sample key that becomes the bracket's
-// lower bound: the expected rank of the k-th largest among kSamples draws plus
-// six standard deviations.  0 = do not sample (small bucket, or nearly
-// everything is kept): the bracket then starts at key 0.
-static unsigned int sample_rank(int64_t n, int64_t k) {
-  if (n < 2 * (int64_t)kSamples) return 0;
-  const double p = (double)k / (double)n;
-  const double j = std::ceil(kSamples * p + 6.0 * std::sqrt(kSamples * p * (1.0 - p))) + 1.0;
-  if (j >= (double)kSamples) return 0;
-  return (unsigned int)j;
+// What the sample of a call is asked for: the ranks (from the top, 1-based) of the two sample keys six standard
+// deviations either side of the expected rank of the k-th largest, and the number of candidates to expect above
+// the lower one.  rank_lo = 0: do not sample (small bucket, or nearly everything is kept).
+struct SamplePlan {
+  unsigned int rank_lo = 0, rank_hi = 0;
+  double expected = 0.0;
+};
+
+static SamplePlan sample_plan(int64_t n, int64_t k, int grad_dtype) {
+  SamplePlan s;
+  if (n < 2 * (int64_t)kSamples) return s;
+  const double keys = (double)kSamples * (grad_dtype == NSML_F32 ? sample_keys<NSML_F32>() : sample_keys<NSML_BF16>());
+  const double p = (double)k / (double)n, mean = keys * p, six = 6.0 * std::sqrt(keys * p * (1.0 - p));
+  const double lo = std::ceil(mean + six) + 1.0, hi = std::floor(mean - six);
+  if (lo >= keys) return s;
+  s.rank_lo = (unsigned int)lo;
+  s.rank_hi = hi < 1.0 ? 1u : (unsigned int)hi;
+  s.expected = (double)n * (mean + six) / keys * 1.04 + 64.0;  // (the bound is rounded down to 15 key bits: a few per cent more)
+  return s;
 }
 
 // Candidates per block of the list stage's small shape (nsml_set_list_block_candidates).
 static std::atomic<int> g_list_block_candidates{4096};
 
-// Kept fraction from which the select runs over the bucket itself.
-constexpr double kDenseRatioAny = 0.25;
-
-static unsigned long long finalize_large_blocks(const DeviceInfo& dev) {
-  return (unsigned long long)dev.sms * (dev.finalize_large < 2 ? dev.finalize_large : 2);
-}
-
-// Dense mode: the finalize kernel selects over the bucket itself, with no sample and no bucket pass.
-// Taken when the bucket cannot be sampled and when the candidate list (8 bytes per entry) would be about
-// as large as the bucket.
-static bool use_dense(int64_t n, int64_t k, const DeviceInfo&) {
+// Dense mode: the select runs over the bucket itself, with no sample and no bucket pass.
+// Taken when the bucket cannot be sampled and when the candidate list would be about as large as the bucket.
+static bool use_dense(int64_t n, int64_t k) {
   const double p_keep = (double)k / (double)n;
-  return sample_rank(n, k) == 0 || p_keep >= kDenseRatioAny;
+  return p_keep >= kDenseRatioAny || sample_plan(n, k, NSML_F32).rank_lo == 0;
 }
 
 // DTYPE: element type of `grad` (what the sample and the bucket pass read).  FDTYPE: element type of the
@@ -266,124 +254,83 @@ static int launch_compress(const void* grad, float* residual, const uint32_t* ma
                            unsigned char* ws, unsigned char* payload, const CompressLayout& L, const PayloadLayout& P,
                            const DeviceInfo& dev, cudaStream_t st, bool keep_status = false) {
   Ctl* ctl = reinterpret_cast<Ctl*>(ws);
-  unsigned short* seg_off = reinterpret_cast<unsigned short*>(ws + L.seg_off);
-  uint32_t* seg_val = reinterpret_cast<uint32_t*>(ws + L.seg_val);
-  unsigned short* seg_count = reinterpret_cast<unsigned short*>(ws + L.seg_count);
-  const unsigned long long nseg = ((unsigned long long)n + kSegElems - 1) / kSegElems;
   BucketSrc<DTYPE> src{grad, mask};
   BucketSrc<FDTYPE> fsrc{residual != nullptr ? static_cast<const void*>(residual) : grad, mask};
-  const double p_keep = (double)k / (double)n;
-  const unsigned long long large_cap_blocks = finalize_large_blocks(dev);
-  const bool dense = use_dense(n, k, dev);
-  unsigned int fgrid;
-  bool small_shape;
-  bool cluster_shape = false;
-  if (dense) {
-    small_shape = (unsigned long long)n <= (unsigned long long)dev.sms * kFinSmallCache;
-    unsigned long long cap = small_shape ? (unsigned long long)dev.sms : large_cap_blocks;
-    if (cap > (unsigned long long)kMaxFinalizeBlocks) cap = kMaxFinalizeBlocks;
-    unsigned long long want = (unsigned long long)n / 4096 + 1;  // at least about 4096 elements per block
-    if (want > nseg) want = nseg;
-    fgrid = (unsigned int)(want < cap ? want : cap);
-    LaunchScope scope(K_CLEAR, st);
-    k_clear<<<4, kCta, 0, st>>>(reinterpret_cast<uint4*>(ws), (unsigned int)(L.group_count / 16), keep_status ? 1 : 0);
-  } else {
-    {
-      LaunchScope scope(K_SAMPLE, st);  // one cluster of kSampleBlocks blocks
-      // (the cluster shape is part of the kernel's definition)
-      launch_prio(k_sample<DTYPE>, dim3(kSampleBlocks), dim3(kSampleThreads), 0, st, false, 0, true, src, residual, (unsigned long long)n,
-                  sample_rank(n, k), ctl, reinterpret_cast<uint4*>(ws), (unsigned int)(L.zero_bytes / 16), keep_status ? 1 : 0);
-    }
-    {
-      // bucket pass.  With a residual: persistent blocks, a block takes 8 segments per step, at most 4
-      // resident blocks per SM.  Without: a warp per 2 KB of the bucket, eight warps per block.
-      LaunchScope scope(K_COMPACT_BUCKET, st);
-      const int resident = dev.compact_feedback;
-      const int per_sm = resident < 4 ? resident : 4;
-      constexpr unsigned long long kPlainSegs = (kCta / 32) * compact_segs_per_warp<DTYPE>();  // segments per block
-      const unsigned int grid = residual != nullptr ? grid_for(nseg, kCta / 32, dev.sms * per_sm)
-                                                    : (unsigned int)((nseg + kPlainSegs - 1) / kPlainSegs);
-      unsigned int* group_count = reinterpret_cast<unsigned int*>(ws + L.group_count);
-      if (residual != nullptr)
-        k_compact_bucket<DTYPE, true><<<grid, kCta, kCompactFeedbackSmem, st>>>(src, residual, (unsigned long long)n, ctl, seg_off,
-                                                                                seg_val, seg_count, group_count);
-      else if (mask != nullptr)
-        k_compact_bucket<DTYPE, false, true><<<grid, kCta, 0, st>>>(src, nullptr, (unsigned long long)n, ctl, seg_off, seg_val,
-                                                                    seg_count, group_count);
-      else
-        k_compact_bucket<DTYPE, false, false><<<grid, kCta, 0, st>>>(src, nullptr, (unsigned long long)n, ctl, seg_off, seg_val,
-                                                                     seg_count, group_count);
-    }
-    // list stage: cooperative, every block co-resident.  The small shape when a block's share of the
-    // expected candidates (k plus the sampling margin) fits its shared-memory cache.
-    fgrid = (unsigned int)dev.sms;
-    if ((unsigned long long)fgrid > nseg) fgrid = (unsigned int)nseg;
-    if (fgrid > (unsigned int)kMaxFinalizeBlocks) fgrid = kMaxFinalizeBlocks;
-    const double expected = (double)n * (p_keep + 6.0 * std::sqrt(p_keep * (1.0 - p_keep) / kSamples)) + 64.0;
-    small_shape = expected / fgrid <= (double)kFinSmallCache;
-    cluster_shape = dev.finalize_cluster && expected <= kFinClusterMaxCandidates && nseg >= (unsigned long long)kFinClusterBlocks;
-    if (cluster_shape) {
-      fgrid = kFinClusterBlocks;
-    } else if (small_shape) {  // short lists: no more blocks than about 4096 candidates each (cheaper barriers, one block = none)
-      unsigned int want = (unsigned int)(expected / (double)g_list_block_candidates.load(std::memory_order_relaxed)) + 1;
-      if (want < fgrid) fgrid = want;
-    } else {  // long lists: as many blocks as stay co-resident (two per SM)
-      unsigned long long cap = large_cap_blocks;
-      // (a caller that asked for few, long list-stage blocks gets one per SM while a block's share still fits its cache)
-      if (g_list_block_candidates.load(std::memory_order_relaxed) > 4096 && expected / dev.sms <= (double)kFinLargeCache)
-        cap = (unsigned long long)dev.sms;
-      if (cap > nseg) cap = nseg;
-      if (cap > (unsigned long long)kMaxFinalizeBlocks) cap = kMaxFinalizeBlocks;
-      if (cap > fgrid) fgrid = (unsigned int)cap;
-    }
-  }
+  const unsigned long long tile = tile_elems<FDTYPE>();
   FinalizeParams fp;
   fp.n = (unsigned long long)n;
   fp.k = (unsigned long long)k;
   fp.bits = bits;
-  fp.nseg = nseg;
+  fp.nseg = ((unsigned long long)n + kSegElems - 1) / kSegElems;
   fp.ctl = ctl;
   fp.hist = reinterpret_cast<unsigned int*>(ws + L.hist);
   fp.block_counts = reinterpret_cast<unsigned long long*>(ws + L.block_counts);
-  fp.seg_count = seg_count;
-  fp.group_count = reinterpret_cast<const unsigned int*>(ws + L.group_count);
-  fp.seg_off = seg_off;
-  fp.seg_val = seg_val;
-  fp.list_idx = reinterpret_cast<uint32_t*>(ws + L.list_idx);
-  fp.list_val = reinterpret_cast<uint32_t*>(ws + L.list_val);
+  fp.bin_list = reinterpret_cast<uint2*>(ws + L.bin_list);
+  fp.tiles = (unsigned int)(((unsigned long long)n + tile - 1) / tile);
+  fp.list.off = reinterpret_cast<unsigned short*>(ws + L.cand_off);
+  fp.list.val = reinterpret_cast<uint32_t*>(ws + L.cand_val);
+  fp.list.tile_count = reinterpret_cast<unsigned int*>(ws + L.tile_count);
+  fp.list.group_count = reinterpret_cast<unsigned int*>(ws + L.group_count);
+  fp.list.window_hist = fp.hist + 3 * kMaxBins;
+  fp.list.group_shift = group_shift_of(fp.tiles);
   fp.raw_val = reinterpret_cast<float*>(ws + L.raw_val);
   fp.payload = payload;
   fp.P = P;
-  if (!dense) {
-    LaunchScope scope(K_GATHER, st);  // segmented list -> contiguous list and the histogram of the first digit
-    // blocks per group: about 1024 expected candidates (one step of the copy loop) per block, at least two
-    // (candidates crowd into parts of a bucket), at most eight
-    const unsigned long long ngroups = (nseg + kGatherSegs - 1) / kGatherSegs;
-    const double per_group = (double)n * (p_keep + 6.0 * std::sqrt(p_keep * (1.0 - p_keep) / kSamples)) / (double)ngroups;
-    unsigned int split = (unsigned int)(per_group / 1024.0) + 1;
-    // (with more than the default candidates per list-stage block the caller has asked for few, long blocks: one
-    // gather block per group then, 21 instead of 16 us alone, 2-3 % more throughput with eight streams)
-    const unsigned int min_split = g_list_block_candidates.load(std::memory_order_relaxed) > 4096 ? 1u : 2u;
-    split = split < min_split ? min_split : (split > 8 ? 8 : split);
-    launch_prio(k_gather, dim3((unsigned int)(ngroups * split)), dim3(kGatherThreads), 0, st, false, 0, true, fp, split);
+  cudaError_t le;
+  if (use_dense(n, k)) {
+    fp.raw_val = reinterpret_cast<float*>(ws + dense_raw_val(L));
+    const bool small_shape = (unsigned long long)n <= (unsigned long long)dev.sms * kFinSmallCache;
+    unsigned long long cap = (unsigned long long)dev.sms * (small_shape || dev.dense_large < 2 ? 1 : 2);
+    if (cap > (unsigned long long)kMaxFinalizeBlocks) cap = kMaxFinalizeBlocks;
+    unsigned long long want = (unsigned long long)n / 4096 + 1;  // at least about 4096 elements per block
+    if (want > fp.nseg) want = fp.nseg;
+    const unsigned int grid = (unsigned int)(want < cap ? want : cap);
+    {
+      LaunchScope scope(K_CLEAR, st);
+      k_clear<<<4, kCta, 0, st>>>(reinterpret_cast<uint4*>(ws), (unsigned int)(L.group_count / 16), keep_status ? 1 : 0);
+    }
+    LaunchScope scope(K_FINALIZE_DENSE, st);
+    // cooperative: every block co-resident; normal priority, it streams the whole bucket
+    if (small_shape)
+      le = launch_prio(k_finalize_dense<FDTYPE, kFinSmallThreads, kFinSmallCache>, dim3(grid), dim3(kFinSmallThreads),
+                       finalize_dyn_smem(kFinSmallCache), st, true, 0, false, false, fsrc, fp);
+    else
+      le = launch_prio(k_finalize_dense<FDTYPE, kFinLargeThreads, kFinDenseLargeCache>, dim3(grid), dim3(kFinLargeThreads),
+                       finalize_dyn_smem(kFinDenseLargeCache), st, true, 0, false, false, fsrc, fp);
+    return le == cudaSuccess ? NSML_OK : NSML_ERR_CUDA;
   }
+  const SamplePlan plan = sample_plan(n, k, DTYPE);
   {
-    LaunchScope scope(dense ? K_FINALIZE_DENSE : K_FINALIZE, st);
-    cudaError_t le;
-    auto launch = [&](auto kernel, int threads, int cache) {  // cooperative: every block co-resident
-      return launch_prio(kernel, dim3(fgrid), dim3(threads), finalize_dyn_smem(cache), st, true, 0, !dense, fsrc, fp);  // (the dense select streams the whole bucket: normal priority)
-    };
-    if (cluster_shape) {
-      // one cluster; the blocks of a cluster are co-scheduled by the hardware, so no cooperative launch is needed
-      le = launch_prio(k_finalize<FDTYPE, kFinClusterThreads, kFinClusterCache, true>, dim3(kFinClusterBlocks), dim3(kFinClusterThreads),
-                       finalize_dyn_smem(kFinClusterCache), st, false, kFinClusterBlocks, true, fsrc, fp);
-    } else if (small_shape && dense) le = launch(k_finalize_dense<FDTYPE, kFinSmallThreads, kFinSmallCache>, kFinSmallThreads, kFinSmallCache);
-    else if (small_shape) le = launch(k_finalize<FDTYPE, kFinSmallThreads, kFinSmallCache>, kFinSmallThreads, kFinSmallCache);
-    else if (dense) le = launch(k_finalize_dense<FDTYPE, kFinLargeThreads, kFinDenseLargeCache>, kFinLargeThreads, kFinDenseLargeCache);
-    else le = launch(k_finalize<FDTYPE, kFinLargeThreads, kFinLargeCache>, kFinLargeThreads, kFinLargeCache);
+    LaunchScope scope(K_SAMPLE, st);  // one cluster of kSampleBlocks blocks (the cluster shape is part of the kernel's definition)
+    le = launch_prio(k_sample<DTYPE>, dim3(kSampleBlocks), dim3(kSampleThreads), kSampleSmem, st, false, 0, true, true, src, residual,
+                     (unsigned long long)n, plan.rank_lo, plan.rank_hi, ctl, reinterpret_cast<uint4*>(ws),
+                     (unsigned int)(L.zero_bytes / 16), keep_status ? 1 : 0);
     if (le != cudaSuccess) return NSML_ERR_CUDA;
   }
-  return NSML_OK;
+  {
+    LaunchScope scope(K_COMPACT_BUCKET, st);  // a block per tile
+    const bool fb = residual != nullptr, masked = mask != nullptr;
+    le = launch_prio(fb ? (masked ? k_compact_bucket<DTYPE, true, true> : k_compact_bucket<DTYPE, true, false>)
+                        : (masked ? k_compact_bucket<DTYPE, false, true> : k_compact_bucket<DTYPE, false, false>),
+                     dim3(fp.tiles), dim3(kCta), 0, st, false, 0, false, true, src, residual, (unsigned long long)n, ctl, fp.list);
+    if (le != cudaSuccess) return NSML_ERR_CUDA;
+  }
+  LaunchScope scope(K_FINALIZE, st);
+  if (plan.expected <= kListClusterMaxCandidates && fp.tiles >= kListClusterBlocks) {
+    // the blocks of a cluster are co-scheduled by the hardware, so no cooperative launch is needed
+    le = launch_prio(k_finalize<FDTYPE, kListSmallCache, true>, dim3(kListClusterBlocks), dim3(kListThreads), list_dyn_smem(kListSmallCache),
+                     st, false, kListClusterBlocks, true, true, fsrc, fp);
+  } else if (plan.expected / dev.sms <= (double)kListSmallCache) {
+    // short lists: no more blocks than about 4096 candidates each (cheaper barriers)
+    unsigned int grid = (unsigned int)(plan.expected / (double)g_list_block_candidates.load(std::memory_order_relaxed)) + 1;
+    if (grid > (unsigned int)dev.sms) grid = (unsigned int)dev.sms;
+    le = launch_prio(k_finalize<FDTYPE, kListSmallCache, false>, dim3(grid), dim3(kListThreads), list_dyn_smem(kListSmallCache), st, true, 0,
+                     true, true, fsrc, fp);
+  } else {
+    le = launch_prio(k_finalize<FDTYPE, kListLargeCache, false>, dim3(dev.sms), dim3(kListThreads), list_dyn_smem(kListLargeCache), st, true, 0,
+                     true, true, fsrc, fp);
+  }
+  return le == cudaSuccess ? NSML_OK : NSML_ERR_CUDA;
 }
 
 static int compress_impl(const void* grad, int64_t n, int grad_dtype, double ratio, int bits,
@@ -441,14 +388,14 @@ static int accumulate_impl(const void* const* payloads, const size_t* payload_by
   const unsigned int tiles = (unsigned int)((n + tile - 1) / tile);
   {
     LaunchScope scope(K_PARTITION, st, timed);  // also clears the status word
-    launch_prio(k_partition, dim3(tiles / kPartBounds + 1, W), dim3(kPartBounds), 0, st, false, 0, true, table, W, (unsigned long long)n,
+    launch_prio(k_partition, dim3(tiles / kPartBounds + 1, W), dim3(kPartBounds), 0, st, false, 0, true, false, table, W, (unsigned long long)n,
                 tiles, tile, offsets, status);
   }
   {
     LaunchScope scope(K_MERGE, st, timed);
     const unsigned int grid = grid_for(tiles, 1, dev->sms * dev->merge);
     auto kernel = tile == kDenseTileLarge ? k_merge<kDenseTileLarge> : k_merge<kDenseTileSmall>;
-    launch_dependent(kernel, dim3(grid), dim3(kMergeThreads), 0, st, table, W, dense, (unsigned long long)n, zero_first, tiles, offsets, status);
+    launch_prio(kernel, dim3(grid), dim3(kMergeThreads), 0, st, false, 0, false, true, table, W, dense, (unsigned long long)n, zero_first, tiles, offsets, status);
   }
   if (cudaGetLastError() != cudaSuccess) return NSML_ERR_CUDA;
   return NSML_OK;
@@ -557,7 +504,7 @@ static int prune_impl(const float* weights, int64_t n, double ratio, uint32_t* m
       unsigned int* fine = reinterpret_cast<unsigned int*>(ws + L.fine);
       {
         LaunchScope scope(K_PRUNE_SAMPLE, st);
-        launch_prio(k_prune_sample, dim3(1), dim3(1024), 0, st, false, 0, true, src, un, (unsigned int)r_lo, (unsigned int)r_hi, ctl);
+        launch_prio(k_prune_sample, dim3(1), dim3(1024), 0, st, false, 0, true, false, src, un, (unsigned int)r_lo, (unsigned int)r_hi, ctl);
       }
       {
         LaunchScope scope(K_PRUNE_COUNT, st);
@@ -565,7 +512,7 @@ static int prune_impl(const float* weights, int64_t n, double ratio, uint32_t* m
       }
       {
         LaunchScope scope(K_PRUNE_SETTLE, st);
-        launch_prio(k_prune_settle, dim3(1), dim3(kCta), 0, st, false, 0, true, (unsigned int)m, ctl, fine);
+        launch_prio(k_prune_settle, dim3(1), dim3(kCta), 0, st, false, 0, true, false, (unsigned int)m, ctl, fine);
       }
       {
         LaunchScope scope(K_PRUNE_MARK, st);
@@ -575,7 +522,7 @@ static int prune_impl(const float* weights, int64_t n, double ratio, uint32_t* m
       }
       {
         LaunchScope scope(K_PRUNE_FIX, st);
-        launch_prio(k_prune_fix, dim3(kPruneFixBlocks), dim3(kCta), 0, st, false, 0, true, ctl, tie_list, mask);
+        launch_prio(k_prune_fix, dim3(kPruneFixBlocks), dim3(kCta), 0, st, false, 0, true, false, ctl, tie_list, mask);
       }
     }
   }
@@ -588,29 +535,29 @@ static int prune_impl(const float* weights, int64_t n, double ratio, uint32_t* m
   const unsigned int fwgrid = two_pass && wgrid > small ? small : wgrid;
   {
     LaunchScope scope(K_PRUNE_HIST, st);
-    launch_prio(k_prune_hist<0>, dim3(fgrid), dim3(kCta), 0, st, false, 0, two_pass, src, un, (unsigned int)m, ctl, hist, tie_list);
+    launch_prio(k_prune_hist<0>, dim3(fgrid), dim3(kCta), 0, st, false, 0, two_pass, false, src, un, (unsigned int)m, ctl, hist, tie_list);
   }
   {
     LaunchScope scope(K_PRUNE_HIST, st);
-    launch_prio(k_prune_hist<1>, dim3(fgrid), dim3(kCta), 0, st, false, 0, two_pass, src, un, (unsigned int)m, ctl, hist, tie_list);
+    launch_prio(k_prune_hist<1>, dim3(fgrid), dim3(kCta), 0, st, false, 0, two_pass, false, src, un, (unsigned int)m, ctl, hist, tie_list);
   }
   {
     LaunchScope scope(K_PRUNE_HIST, st);
-    launch_prio(k_prune_hist<2>, dim3(fgrid), dim3(kCta), 0, st, false, 0, two_pass, src, un, (unsigned int)m, ctl, hist, tie_list);
+    launch_prio(k_prune_hist<2>, dim3(fgrid), dim3(kCta), 0, st, false, 0, two_pass, false, src, un, (unsigned int)m, ctl, hist, tie_list);
   }
   {
     LaunchScope scope(K_PRUNE_TIES, st);
-    launch_prio(k_prune_ties, dim3(fgrid), dim3(kCta), 0, st, false, 0, two_pass, src, un, ctl, hist, tie_list, tile_ties);
+    launch_prio(k_prune_ties, dim3(fgrid), dim3(kCta), 0, st, false, 0, two_pass, false, src, un, ctl, hist, tie_list, tile_ties);
   }
   {
     LaunchScope scope(K_PRUNE_WRITE, st);
-    launch_prio(k_prune_write, dim3(fwgrid), dim3(kCta), 0, st, false, 0, two_pass, src, un, ctl, tile_ties, mask);
+    launch_prio(k_prune_write, dim3(fwgrid), dim3(kCta), 0, st, false, 0, two_pass, false, src, un, ctl, tile_ties, mask);
   }
   {
     LaunchScope scope(K_PRUNE_WRITE_RANKED, st);  // returns at once unless ties have to be ranked
     unsigned int rgrid = stream_grid(n, *dev, dev->prune_write_ranked < 8 ? dev->prune_write_ranked : 8, 1u << 16);
     if (two_pass && rgrid > small) rgrid = small;
-    launch_prio(k_prune_write_ranked, dim3(rgrid), dim3(kCta), 0, st, false, 0, two_pass, src, un, ctl, tile_ties, mask);
+    launch_prio(k_prune_write_ranked, dim3(rgrid), dim3(kCta), 0, st, false, 0, two_pass, false, src, un, ctl, tile_ties, mask);
   }
   if (cudaGetLastError() != cudaSuccess) return NSML_ERR_CUDA;
   return NSML_OK;
@@ -631,7 +578,7 @@ static int feedback_impl(const void* grad, float* residual, int64_t n, int grad_
   const DeviceInfo* dev = nullptr;
   int rc = device_info(&dev);
   if (rc != NSML_OK) return rc;
-  if (use_dense(n, k, *dev)) {
+  if (use_dense(n, k)) {
     // dense strategy (no bucket pass to fuse the add into): residual <- grad + residual first, then the select
     // over the residual buffer
     const unsigned int grid = stream_grid(n, *dev, dev->feedback_add < 8 ? dev->feedback_add : 8, 1u << 16);
@@ -706,11 +653,11 @@ int nsml_compress_strategy(int64_t n, double ratio) {
   const DeviceInfo* dev = nullptr;
   const int rc = device_info(&dev);
   if (rc != NSML_OK) return rc;
-  return use_dense(n, k, *dev) ? NSML_STRATEGY_DENSE : NSML_STRATEGY_LIST;
+  return use_dense(n, k) ? NSML_STRATEGY_DENSE : NSML_STRATEGY_LIST;
 }
 
 int nsml_set_list_block_candidates(int candidates) {
-  if (candidates < 1024 || candidates > kFinSmallCache) return NSML_ERR_ARG;
+  if (candidates < 1024 || candidates > kListSmallCache) return NSML_ERR_ARG;
   g_list_block_candidates.store(candidates, std::memory_order_relaxed);
   return NSML_OK;
 }

@@ -26,51 +26,89 @@ constexpr int kMaxPolls = 1 << 22;
 // the histograms that follow it) at the start of every call.
 struct Ctl {
   int status;                 // first device-detected error (NSML_ERR_*), 0 = ok
-  unsigned int lo;            // sampled lower bound of the threshold key
+  unsigned int lo, hi;        // sampled bounds of the threshold key: probably lo <= T < hi
   unsigned int barrier;       // arrivals at the finalize kernel's grid barriers
-  unsigned int pad;
+  unsigned int coarse;        // most sampled keys have zeros in their low 16 bits
+  unsigned int listed;        // entries of the threshold's bin appended to the bin list
 };
 static_assert(sizeof(Ctl) <= 256, "control block must fit its 256-byte slot");
 
-constexpr int kSegElems = 512;            // bucket elements per candidate-list segment (4 rounds of 128)
-constexpr int kGroupSegs = 64;            // segments per group; the bucket pass keeps a candidate count per group
-constexpr int kMaxFinalizeBlocks = 1024;  // upper bound on blocks of the finalize kernel
+// The window of keys the sample leaves open, cut into at most kMaxBins bins of 1 << shift keys.
+struct Window {
+  unsigned int lo, hi, shift;  // keys lo .. hi-1; bin (key - lo) >> shift
+  bool few;                    // there are at most kFewBins bins
+};
+constexpr unsigned int kFewBins = 64;
+// TYPE: element type of the keys; the low 16 bits of a bfloat16 key are zero, so a bin need not be narrower than that
+// (and holds one key then).  The same goes for a float32 bucket that was widened from bfloat16, which the sample tells
+// (`coarse`); there a narrower bin only costs a refinement later.
+template <int TYPE>
+__host__ __device__ constexpr unsigned int min_bin_shift() { return TYPE == NSML_F32 ? 0 : 16; }
+template <int TYPE>
+__device__ __forceinline__ Window make_window(const Ctl* ctl) {
+  Window w;
+  const unsigned int hi = ctl->hi;
+  w.lo = max(ctl->lo, 1u);  // zeros are never candidates of the list strategy
+  w.hi = hi > w.lo ? hi : 0x80000000u;
+  const unsigned int span = (w.hi - w.lo - 1) / kMaxBins;
+  w.shift = max(TYPE == NSML_BF16 || ctl->coarse ? 16u : 0u, span == 0 ? 0u : 32u - __clz(span));
+  w.few = (w.hi - w.lo - 1) >> w.shift < kFewBins;
+  return w;
+}
+
+constexpr int kSegElems = 512;            // granule of the index ranges that the dense select's blocks own
+constexpr int kTileBytes = 16384;         // bucket bytes per tile of the candidate list: what a block of the bucket pass takes
+constexpr int kMaxGroups = 1024;          // the bucket pass keeps a candidate count per group of tiles
+constexpr int kMaxFinalizeBlocks = 1024;  // upper bound on blocks of the finalize kernels
+constexpr unsigned int kBinCap = 1024;    // entries of the threshold's bin that can be settled one by one
+
+// elements per tile; TYPE: element type of the stream the tiles cut (a tile of a bucket with a residual holds
+// float32 sums)
+template <int TYPE>
+__host__ __device__ constexpr int tile_elems() { return kTileBytes / (TYPE == NSML_F32 ? 4 : 2); }
+// tiles per group, as a shift: 64, or more where the groups would be too many
+inline unsigned int group_shift_of(unsigned long long tiles) {
+  unsigned int s = 6;
+  while (((tiles + (1ull << s) - 1) >> s) > (unsigned long long)kMaxGroups) ++s;
+  return s;
+}
 
 struct CompressLayout {  // byte offsets inside a compress workspace
-  size_t hist;          // u32[4][kMaxBins]: digit histograms (levels 0..2, level 0 again after a rebuild)
-  size_t group_count;   // u32[ceil(segments / kGroupSegs)]: candidates per group of segments
-  size_t zero_bytes;    // everything before this offset is cleared per call 
-  size_t block_counts;  // u64[4][kMaxFinalizeBlocks]: per-block counts exchanged at barriers
-  size_t seg_count;     // u16[ceil(n / kSegElems)]: entries per segment
-  size_t seg_off;       // u16[n]: segmented candidate list (bucket pass output), a candidate's offset inside its segment; segment s starts at s * kSegElems
-  size_t seg_val;       // u32[n] (float32 bit patterns)
-  size_t list_idx;      // u32[n]: the same candidates, contiguous per finalize block
-  size_t list_val;      // u32[n]
-  size_t raw_val;       // f32[n]: survivor values before quantisation (the same memory as seg_val)
+  size_t hist;          // u32[4][kMaxBins]: digit histograms; the last one counts the candidates inside the sampled window
+  size_t group_count;   // u32[kMaxGroups]: candidates per group of tiles
+  size_t zero_bytes;    // everything before this offset is cleared per call
+  size_t block_counts;  // u64[kMaxFinalizeBlocks]: per-block counts exchanged at barriers
+  size_t bin_list;      // uint2[kBinCap]: (key, index) of the candidates in the threshold's bin
+  size_t tile_count;    // u32[tiles]: candidates per tile
+  size_t cand_off;      // u16[n]: a candidate's offset inside its tile; tile t's candidates start at t * tile_elems
+  size_t cand_val;      // u32[n]: float32 bit patterns (bfloat16 bucket: offset << 16 | bfloat16 bits, and no cand_off)
+  size_t raw_val;       // f32[k]: survivor values before int8 quantisation
   size_t total;
 };
 
 __host__ __device__ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
+// Kept fraction from which the select runs over the bucket itself.
+constexpr double kDenseRatioAny = 0.25;
+
 inline CompressLayout compress_layout(int64_t n) {
   CompressLayout L;
-  const size_t npad = align_up((size_t)n, kSegElems);
-  const size_t segs = npad / kSegElems;
+  const size_t npad = align_up((size_t)n, tile_elems<NSML_BF16>());
   L.hist = 256;
   L.group_count = L.hist + 4 * kMaxBins * sizeof(unsigned int);
-  L.zero_bytes = L.group_count + align_up(((segs + kGroupSegs - 1) / kGroupSegs) * 4, 256);
+  L.zero_bytes = L.group_count + kMaxGroups * sizeof(unsigned int);
   L.block_counts = L.zero_bytes;
-  L.seg_count = L.block_counts + 4 * kMaxFinalizeBlocks * 8;
-  L.seg_off = L.seg_count + align_up(segs * 2, 256);
-  L.seg_val = L.seg_off + npad * 2;
-  L.list_idx = L.seg_val + npad * 4;
-  L.list_val = L.list_idx + npad * 4;
-  // raw_val shares the memory of seg_val: the segmented list is dead once k_gather has copied it, the
-  // survivors' raw values are written after that (list strategy), and the dense strategy has no list at all
-  L.raw_val = L.seg_val;
-  L.total = L.list_val + npad * 4;
+  L.bin_list = L.block_counts + kMaxFinalizeBlocks * 8;
+  L.tile_count = L.bin_list + kBinCap * 8;
+  L.cand_off = L.tile_count + align_up(npad / tile_elems<NSML_F32>() * 4, 256);
+  L.cand_val = L.cand_off + npad * 2;
+  // The list strategy keeps less than kDenseRatioAny of the bucket; the dense strategy, which may keep all of it,
+  // has no candidate list, so its survivors' values start where the list would.
+  L.raw_val = L.cand_val + npad * 4;
+  L.total = L.raw_val + align_up((size_t)((double)n * kDenseRatioAny) * 4 + 4, 256);
   return L;
 }
+inline size_t dense_raw_val(const CompressLayout& L) { return L.cand_off; }  // npad * 6 bytes: room for n values
 
 struct PayloadLayout {
   int64_t k;

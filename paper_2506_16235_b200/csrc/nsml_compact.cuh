@@ -1,81 +1,19 @@
-// Bucket -> segmented candidate list: the one full pass over the bucket
-// (Alg. 2 Steps 2-3: pruned gradients read as zero; everything whose magnitude
-// is below the sampled lower bound is dropped here, in one streaming read).
+// Bucket -> candidate list: the one full pass over the bucket (Alg. 2 Steps 2-3:
+// pruned gradients read as zero; everything whose magnitude is below the sampled
+// lower bound is dropped here, in one streaming read).
 //
-// The bucket is cut into segments of kSegElems elements.  A warp takes one
-// segment at a time and appends what it keeps (every key >= lo, lo >= 1) to
-// the segment's own slots of the list, [s * kSegElems, s * kSegElems + count),
-// so nothing can overflow, nothing is allocated and no warp ever waits for
-// another: there is no block or grid synchronisation in this kernel.
-// Segments in increasing order are in index order.
-//
-// Blocks walk the bucket block-cyclically (block b takes segments 8b..8b+7,
-// then 8(b+G).., ...), so at any moment the whole grid reads one compact
-// window of the bucket, which is what DRAM row buffers like.  Every lane
-// keeps its part of the warp's next segment in flight: in registers (16-byte
-// loads issued a segment or two ahead), or, when a residual is streamed
-// beside the gradient, with asynchronous copies into a private
-// shared-memory slot, which a lane reads back only itself, so neither
-// buffer needs any synchronisation.
+// The bucket is cut into tiles of kTileBytes.  A block takes a tile and appends
+// what it keeps (every key >= lo, lo >= 1) to the tile's own slots of the list,
+// [t * tile, t * tile + count), in index order, so nothing can overflow, nothing
+// is allocated and no block ever waits for another; tiles in increasing order
+// are in index order.  Keys inside the sampled window are counted in 4096 bins
+// on the way (fire-and-forget reductions), so that the list stage knows the
+// threshold's bin without a pass over the list.
 #pragma once
 
 #include "nsml_common.cuh"
 
 namespace nsml {
-
-// dynamic shared memory of the bucket pass with local accumulation: the residual's double buffers
-// (a warp's segment of the residual: kSegElems float32, two of them per warp)
-constexpr size_t kCompactFeedbackSmem = (size_t)(kCta / 32) * 2 * kSegElems * 4;
-
-// Appends the kept elements of one round of 32 * EPL elements.  `f` holds this lane's keep flags (bit e =
-// element lane*EPL+e of the round).  Returns the round's total.
-template <int EPL>
-__device__ __forceinline__ unsigned int append_round(unsigned int f, const uint32_t (&bits)[EPL], unsigned int first_offset,
-                                                     unsigned long long out_base, unsigned short* __restrict__ seg_off,
-                                                     uint32_t* __restrict__ seg_val) {
-  const int lane = threadIdx.x & 31;
-  const unsigned int lt = (1u << lane) - 1u;
-  const unsigned int any = __ballot_sync(0xFFFFFFFFu, f != 0);
-  const unsigned int multi = __ballot_sync(0xFFFFFFFFu, (f & (f - 1)) != 0);
-  unsigned int before, total;
-  if (multi == 0) {  // usual case: no lane keeps more than one element
-    before = __popc(any & lt);
-    total = __popc(any);
-  } else {
-    const unsigned int mine = __popc(f);
-    unsigned int incl = mine;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned int up = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-      if (lane >= o) incl += up;
-    }
-    before = incl - mine;
-    total = __shfl_sync(0xFFFFFFFFu, incl, 31);
-  }
-  if (f != 0) {
-    unsigned long long pos = out_base + before;
-#pragma unroll
-    for (int e = 0; e < EPL; ++e) {
-      if (f & (1u << e)) {
-        seg_off[pos] = (unsigned short)(first_offset + lane * EPL + e);
-        seg_val[pos] = bits[e];
-        ++pos;
-      }
-    }
-  }
-  return total;
-}
-
-// ---- per-lane asynchronous copies (global -> shared) ----
-template <int BYTES>
-__device__ __forceinline__ void cp_async_lane(void* smem_dst, const void* gsrc) {
-  const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem_dst);
-  if (BYTES == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gsrc) : "memory");
-  else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(gsrc) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int PENDING>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory"); }
 
 // |v| >= t on floats equals key >= lo for finite v; written as !(|v| < t) so
 // that NaN is kept too (the finalize kernel reports non-finite candidates).
@@ -87,7 +25,7 @@ __device__ __forceinline__ unsigned int keep_flags(const uint32_t (&bits)[EPL], 
   return f;
 }
 
-// One segment's worth of 16-byte loads of a lane, unpacked: float32 as is, bfloat16 widened to float32 bit patterns.
+// One 16-byte load of a lane, unpacked: float32 as is, bfloat16 widened to float32 bit patterns.
 template <int DTYPE, int EPL>
 __device__ __forceinline__ void unpack16(const uint4& v, uint32_t (&bits)[EPL]) {
   if (DTYPE == NSML_F32) {
@@ -100,213 +38,250 @@ __device__ __forceinline__ void unpack16(const uint4& v, uint32_t (&bits)[EPL]) 
   }
 }
 
-// The bucket pass without a residual: NOT a persistent kernel.  A warp takes 2 KB of the bucket (one float32
-// segment, two bfloat16 segments), issues all of its 16-byte loads at once and is done; a block is eight
-// warps on 16 consecutive KB, and the hardware's block scheduler, which hands out blocks in order, keeps the
-// grid on one compact, moving window of the bucket.  Measured on a 100 MB float32 bucket whose candidates
-// crowd into a few tensors: 19.0 us, against 19.9 us for persistent blocks that prefetch the next segment into
-// registers, 21.9 us for a shared-memory ring of asynchronous copies and 18.6 us for a plain read of the
-// bucket; blocks that own 2, 4, 8 consecutive 16 KB steps take 20.5, 23.4, 29.4 us (the wider the window of
-// addresses in flight, the slower).  Short-lived blocks also share the SMs gracefully with other streams'
-// kernels, where a grid of persistent blocks that does not fit at once runs a second wave.  MASKED: a pruning
-// mask is applied (a segment's 16 mask words are fetched by lanes 0-15 with the data and handed out by shuffle).
-template <int DTYPE>
-__host__ __device__ constexpr int compact_segs_per_warp() { return DTYPE == NSML_F32 ? 1 : 2; }
+struct TileList {  // where the bucket pass leaves what it keeps
+  unsigned short* off;        // see CompressLayout
+  uint32_t* val;
+  unsigned int* tile_count;
+  unsigned int* group_count;
+  unsigned int* window_hist;
+  unsigned int group_shift;
+};
 
-template <int DTYPE, bool MASKED>
-__device__ __forceinline__ void compact_plain(const BucketSrc<DTYPE>& src, unsigned long long n, const Ctl* ctl,
-                                              unsigned short* __restrict__ seg_off, uint32_t* __restrict__ seg_val,
-                                              unsigned short* __restrict__ seg_count, unsigned int* __restrict__ group_count) {
-  constexpr int ESIZE = (DTYPE == NSML_F32) ? 4 : 2;
-  constexpr int EPL = 16 / ESIZE;                 // elements a lane takes per round: 16 bytes' worth
-  constexpr int ROUND = 32 * EPL;                 // elements a warp handles per step
-  constexpr int ROUNDS = kSegElems / ROUND;       // steps per segment: 4 or 2
-  constexpr int SEGS = compact_segs_per_warp<DTYPE>();
-  constexpr int kSegMaskWords = kSegElems / 32;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const unsigned long long nseg = (n + kSegElems - 1) / kSegElems;
-  const unsigned long long nseg_full = n / kSegElems;  // segments that need no bounds checks
-  const unsigned long long first = ((unsigned long long)blockIdx.x * (kCta / 32) + w) * SEGS;
-  if (first >= nseg) return;
-  const uint4* g = reinterpret_cast<const uint4*>(src.grad) + lane;  // round r of segment s: g[(s * ROUNDS + r) * 32]
-  uint4 q[SEGS][ROUNDS];
-  uint32_t mw[SEGS];
+// Shared memory of a block of the bucket pass: what it keeps of its tile, in index order.
+template <bool PACKED>
+struct KeepShared {
+  static constexpr int TILE = PACKED ? tile_elems<NSML_BF16>() : tile_elems<NSML_F32>();
+  __align__(16) uint32_t val[TILE];
+  __align__(8) unsigned short off[PACKED ? 4 : TILE];
+  unsigned int cnt[kCta / 32];
+  unsigned int few[kFewBins];
+};
+
+// Keeps a tile's candidates.  A warp's share of the tile is 4 rounds of 32 lanes x EPL elements, `first` = its offset
+// in the tile, bits_of(r, bits) fetches a lane's EPL elements of round r.  PACKED: entries are offset << 16 | bfloat16
+// bits.  The candidates are put in order in shared memory and then written, four per thread, in whole sectors; the
+// window's histogram is counted on the way out, by full warps.  Reductions to one address run at about two per
+// nanosecond, so adds must not pile up on a few of them: a window of few bins (bfloat16 keys: a window is a handful of
+// key values) is counted in shared memory first, and in a tile that is full of candidates the lanes of a warp with
+// equal bins add once.
+template <int EPL, bool PACKED, class Bits>
+__device__ __forceinline__ void keep_tile(const TileList& out, unsigned long long tile, unsigned int first, const Window& win,
+                                          Ctl* ctl, KeepShared<PACKED>& sh, Bits&& bits_of) {
+  constexpr unsigned int FULL = 0xFFFFFFFFu;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned int lt = (1u << lane) - 1u;
+  const float t = __uint_as_float(win.lo);
+  unsigned int flags[4], mine = 0;
 #pragma unroll
-  for (int s = 0; s < SEGS; ++s) {
-    mw[s] = 0;
-    if (first + s < nseg_full) {
-#pragma unroll
-      for (int r = 0; r < ROUNDS; ++r) q[s][r] = __ldcs(g + ((first + s) * ROUNDS + r) * 32);
-      if (MASKED && lane < kSegMaskWords) mw[s] = __ldg(src.mask + (first + s) * kSegMaskWords + lane);
-    }
+  for (int r = 0; r < 4; ++r) {
+    uint32_t bits[EPL];
+    bits_of(r, bits);
+    flags[r] = keep_flags<EPL>(bits, t);
+    mine += __popc(flags[r]);
   }
-  // Zeros are never candidates here; if they are needed (fewer than k non-zero
-  // keys) the list comes out short and the finalize kernel's slow path adds them.
-  const float t = __uint_as_float(max(ctl->lo, 1u));
+  const unsigned int warp_total = __reduce_add_sync(FULL, mine);
+  if (lane == 0) sh.cnt[warp] = warp_total;
+  if (win.few && threadIdx.x < kFewBins) sh.few[threadIdx.x] = 0;
+  __syncthreads();
+  unsigned int before = 0, total = 0;
 #pragma unroll
-  for (int s = 0; s < SEGS; ++s) {
-    const unsigned long long seg = first + s;
-    if (seg >= nseg) break;
-    const unsigned long long seg_base = seg * kSegElems;
-    unsigned int kept = 0;
+  for (int w = 0; w < kCta / 32; ++w) {
+    const unsigned int c = sh.cnt[w];
+    if (w < warp) before += c;
+    total += c;
+  }
+  if (threadIdx.x == 0) {
+    out.tile_count[tile] = total;
+    if (total) atomicAdd(out.group_count + (tile >> out.group_shift), total);
+  }
+  if (total == 0) return;
+  if (warp_total != 0) {
 #pragma unroll
-    for (int r = 0; r < ROUNDS; ++r) {
-      uint32_t bits[EPL];
-      if (seg < nseg_full) {
-        unpack16<DTYPE, EPL>(q[s][r], bits);
-        if (MASKED) {
-          // this lane's EPL mask bits inside the round's ROUND / 32 words
-          const uint32_t word = __shfl_sync(0xFFFFFFFFu, mw[s], r * (ROUND / 32) + lane * EPL / 32);
-          const uint32_t m = (word >> (unsigned)((lane * EPL) & 31)) & ((1u << EPL) - 1u);
-#pragma unroll
-          for (int e = 0; e < EPL; ++e)
-            if (m & (1u << e)) bits[e] = 0;
-        }
+    for (int r = 0; r < 4; ++r) {
+      const unsigned int f = flags[r];
+      const unsigned int any = __ballot_sync(FULL, f != 0);
+      if (any == 0) continue;
+      unsigned int rank, round_total;
+      if (__ballot_sync(FULL, (f & (f - 1)) != 0) == 0) {  // usual case: no lane keeps more than one element
+        rank = __popc(any & lt);
+        round_total = __popc(any);
       } else {
-        // the bucket's ragged last segment: plain loads, missing elements read as 0 and are never kept
-        // (load_vals4 applies the mask)
+        const unsigned int cnt = __popc(f);
+        unsigned int incl = cnt;
 #pragma unroll
-        for (int qq = 0; qq < EPL / 4; ++qq) {
-          uint32_t four[4];
-          src.load_vals4(seg_base + r * ROUND + lane * EPL + qq * 4, n, four);
+        for (int o = 1; o < 32; o <<= 1) {
+          const unsigned int up = __shfl_up_sync(FULL, incl, o);
+          if (lane >= o) incl += up;
+        }
+        rank = incl - cnt;
+        round_total = __shfl_sync(FULL, incl, 31);
+      }
+      uint32_t bits[EPL];
+      bits_of(r, bits);
+      unsigned int pos = before + rank;
 #pragma unroll
-          for (int e = 0; e < 4; ++e) bits[qq * 4 + e] = four[e];
+      for (int e = 0; e < EPL; ++e) {
+        if (f & (1u << e)) {
+          const unsigned int off = first + r * 32 * EPL + lane * EPL + e;
+          if (PACKED) {
+            sh.val[pos] = off << 16 | bits[e] >> 16;
+          } else {
+            sh.val[pos] = bits[e];
+            sh.off[pos] = (unsigned short)off;
+          }
+          ++pos;
         }
       }
-      const unsigned int f = keep_flags<EPL>(bits, t);
-      if (!__any_sync(0xFFFFFFFFu, f != 0)) continue;
-      kept += append_round<EPL>(f, bits, (unsigned int)(r * ROUND), seg_base + kept, seg_off, seg_val);
+      before += round_total;
     }
-    if (lane == 0) {
-      seg_count[seg] = (unsigned short)kept;
-      if (kept) atomicAdd(group_count + seg / kGroupSegs, kept);  // result unused: a fire-and-forget reduction
+  }
+  __syncthreads();
+  const unsigned long long base = tile * (unsigned long long)KeepShared<PACKED>::TILE;
+  const bool crowded = total > kCta * 4;
+  for (unsigned int i0 = warp * 128; i0 < total; i0 += kCta * 4) {  // (uniform over the warp)
+    const unsigned int i = i0 + lane * 4;
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if (i < total) {  // (up to three entries past the last one are copied too; the tile's slots have room)
+      v = *reinterpret_cast<const uint4*>(sh.val + i);
+      *reinterpret_cast<uint4*>(out.val + base + i) = v;
+      if (!PACKED) *reinterpret_cast<uint2*>(out.off + base + i) = *reinterpret_cast<const uint2*>(sh.off + (PACKED ? 0 : i));
+    }
+    const uint32_t e4[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const uint32_t key = (PACKED ? e4[e] << 16 : e4[e]) & 0x7FFFFFFFu;
+      const bool live = i + e < total;
+      if (live && key >= kInfKey) set_status(&ctl->status, NSML_ERR_NONFINITE);
+      const bool inside = live && key < win.hi;  // (key >= lo)
+      const unsigned int bin = (key - win.lo) >> win.shift;
+      unsigned int add = inside ? 1u : 0u;
+      if (crowded) {
+        const unsigned int who = __ballot_sync(FULL, inside);
+        if (inside) {
+          const unsigned int same = __match_any_sync(who, bin);
+          add = (same & lt) == 0 ? (unsigned int)__popc(same) : 0u;
+        }
+      }
+      if (add) {
+        if (win.few) atomicAdd(&sh.few[bin], add);
+        else atomicAdd(out.window_hist + bin, add);
+      }
+    }
+  }
+  if (win.few) {
+    __syncthreads();
+    if (threadIdx.x < kFewBins) {
+      const unsigned int c = sh.few[threadIdx.x];
+      if (c) atomicAdd(out.window_hist + threadIdx.x, c);
     }
   }
 }
 
-// FEEDBACK: the bucket that is compressed is gradient + residual (Section 4.2 Step 3, local accumulation of
-// the filtered gradients).  The residual is streamed beside the gradient, the sum (one float32 add per
-// element) is written back over the residual and is what the candidates are taken from; the pruning mask
-// zeroes a key, not the stored sum.  Here every lane keeps its part of the warp's next segment (gradient and
-// residual) in flight with asynchronous copies into a private shared-memory slot: a lane reads back only what
-// it copied itself, so the double buffer needs no synchronisation.
-template <int DTYPE, bool FEEDBACK = false, bool MASKED = true>
-__global__ void __launch_bounds__(kCta)
-k_compact_bucket(BucketSrc<DTYPE> src, float* __restrict__ residual, unsigned long long n, Ctl* ctl,
-                 unsigned short* __restrict__ seg_off, uint32_t* __restrict__ seg_val, unsigned short* __restrict__ seg_count,
-                 unsigned int* __restrict__ group_count) {
-  if (!FEEDBACK) {
-    compact_plain<DTYPE, MASKED>(src, n, ctl, seg_off, seg_val, seg_count, group_count);
-    return;
-  }
+// The bucket pass is NOT a persistent kernel.  A block is eight warps on one tile (16 consecutive KB); a warp issues
+// all of its loads at once and is done.  The hardware's block scheduler, which hands out blocks in order, keeps the
+// grid on one compact, moving window of the bucket.  Measured on a 100 MB float32 bucket whose candidates crowd into
+// a few tensors: 19.0 us, against 19.9 us for persistent blocks that prefetch the next segment into registers, 21.9 us
+// for a shared-memory ring of asynchronous copies and 18.6 us for a plain read of the bucket; blocks that own 2, 4, 8
+// consecutive 16 KB steps take 20.5, 23.4, 29.4 us (the wider the window of addresses in flight, the slower).
+// Short-lived blocks also share the SMs gracefully with other streams' kernels.  The first wave's loads are issued
+// while the sample kernel still runs.
+//
+// FEEDBACK: the bucket that is compressed is gradient + residual (Section 4.2 Step 3, local accumulation of the
+// filtered gradients).  The residual is streamed beside the gradient, the sum (one float32 add per element) is
+// written back over the residual and is what the candidates are taken from; the pruning mask zeroes a key, not the
+// stored sum.  A tile is then 4096 sums whatever the gradient's type.
+// MASKED: a pruning mask is applied (a warp's mask words are fetched with the data and handed out by shuffle).
+template <int DTYPE, bool FEEDBACK, bool MASKED>
+__global__ void __launch_bounds__(kCta, FEEDBACK ? 4 : 5)
+k_compact_bucket(BucketSrc<DTYPE> src, float* __restrict__ residual, unsigned long long n, Ctl* ctl, TileList out) {
+  __shared__ KeepShared<!FEEDBACK && DTYPE == NSML_BF16> sh;
   constexpr int ESIZE = (DTYPE == NSML_F32) ? 4 : 2;
-  constexpr int EPL = 4;                          // beside the residual (float32, 16 bytes per 4 elements) a lane takes 4 elements
-  constexpr int ROUND = 32 * EPL;                 // elements a warp handles per step
-  constexpr int ROUNDS = kSegElems / ROUND;       // steps per segment
-  constexpr int LANE_BYTES = EPL * ESIZE;         // 16, or 8 (bfloat16)
-  constexpr int BUF_BYTES = kSegElems * ESIZE;    // one segment of one warp
-  constexpr int RBUF_BYTES = kSegElems * 4;       // the same segment of the residual
-  __shared__ __align__(16) unsigned char s_fifo[FEEDBACK ? (kCta / 32) * 2 * BUF_BYTES : 16];
-  extern __shared__ __align__(16) unsigned char s_rfifo[];  // (kCta / 32) * 2 * RBUF_BYTES bytes
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  unsigned char* fifo = s_fifo + (FEEDBACK ? (size_t)w * 2 * BUF_BYTES + lane * LANE_BYTES : 0);  // round r of buffer b at + (b*ROUNDS + r)*32*LANE_BYTES
-  unsigned char* rfifo = s_rfifo + (size_t)w * 2 * RBUF_BYTES + lane * 16;       // the same for the residual: + (b*ROUNDS + r)*32*16
-
-  const unsigned long long nseg = (n + kSegElems - 1) / kSegElems;
-  const unsigned long long nseg_full = n / kSegElems;  // segments that need no bounds checks
-  const unsigned long long step = (unsigned long long)gridDim.x * (kCta / 32);
-  const unsigned char* g = static_cast<const unsigned char*>(src.grad) + (size_t)lane * LANE_BYTES;
-
-  // asynchronous copies of one whole segment into buffer b (nothing for the ragged last segment, which is
-  // read with plain loads); one commit group per segment, empty or not
-  auto fetch = [&](unsigned long long s, int b) {
-    if (s < nseg_full) {
+  constexpr int EPL = FEEDBACK ? 4 : 16 / ESIZE;  // elements a lane takes per round
+  constexpr int ROUND = 32 * EPL;                 // elements a warp handles per round
+  constexpr int SHARE = 4 * ROUND;                // elements of a warp: 512 or 1024
+  constexpr unsigned long long TILE = FEEDBACK ? tile_elems<NSML_F32>() : tile_elems<DTYPE>();
+  static_assert(SHARE * (kCta / 32) == TILE, "a block is a tile");
+  pdl_launch_dependents();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned long long tile = blockIdx.x;
+  const unsigned int first = warp * SHARE;
+  const unsigned long long i0 = tile * TILE + first;  // the warp's first element
+  uint4 q[4];  // the lane's elements: as loaded, or (FEEDBACK) the sums
+  float4 res[FEEDBACK ? 4 : 1];
+  const bool whole = i0 + SHARE <= n;
+  if (whole) {
+    const unsigned char* g = static_cast<const unsigned char*>(src.grad) + (i0 + lane * EPL) * ESIZE;
 #pragma unroll
-      for (int r = 0; r < ROUNDS; ++r) {
-        cp_async_lane<LANE_BYTES>(fifo + (b * ROUNDS + r) * 32 * LANE_BYTES, g + (s * kSegElems + r * ROUND) * ESIZE);
-        cp_async_lane<16>(rfifo + (b * ROUNDS + r) * 32 * 16, residual + s * kSegElems + r * ROUND + lane * 4);
+    for (int r = 0; r < 4; ++r) {
+      if (EPL * ESIZE == 16) {
+        q[r] = __ldcs(reinterpret_cast<const uint4*>(g + r * ROUND * ESIZE));
+      } else {  // four bfloat16
+        const uint2 v = __ldcs(reinterpret_cast<const uint2*>(g + r * ROUND * ESIZE));
+        q[r] = make_uint4(v.x, v.y, 0u, 0u);
       }
     }
-    cp_async_commit();
-  };
-
-  unsigned long long seg = (unsigned long long)blockIdx.x * (kCta / 32) + w;
-  fetch(seg, 0);
-  // The segment's 16 words of the pruning mask (64 bytes) are fetched by lanes 0-15 one segment ahead, like
-  // the data, and handed to the lanes by shuffle.
-  constexpr int kSegMaskWords = kSegElems / 32;
-  uint32_t mask_words = 0, mask_words_next = 0;
-  if (src.mask != nullptr && seg < nseg_full && lane < kSegMaskWords) mask_words = __ldg(src.mask + seg * kSegMaskWords + lane);
-  // Zeros are never candidates here; if they are needed (fewer than k non-zero
-  // keys) the list comes out short and the finalize kernel's slow path adds them.
-  const float t = __uint_as_float(max(ctl->lo, 1u));
-  int buf = 0;
-
-  while (seg < nseg) {
-    const unsigned long long next = seg + step;
-    fetch(next, buf ^ 1);
-    if (src.mask != nullptr && next < nseg_full && lane < kSegMaskWords)
-      mask_words_next = __ldg(src.mask + next * kSegMaskWords + lane);
-    cp_async_wait<1>();  // this segment's copies have landed; the next segment's stay in flight
-
-    const unsigned long long seg_base = seg * kSegElems;
-    unsigned int kept = 0;
+    if (FEEDBACK) {
 #pragma unroll
-    for (int r = 0; r < ROUNDS; ++r) {
-      uint32_t bits[EPL];
-      if (seg < nseg_full) {
-        const unsigned char* slot = fifo + (buf * ROUNDS + r) * 32 * LANE_BYTES;
-        if (DTYPE == NSML_F32) {
-          const uint4 v = *reinterpret_cast<const uint4*>(slot);
-          bits[0] = v.x; bits[1] = v.y; bits[2] = v.z; bits[3] = v.w;
-        } else {
-          const uint2 v = *reinterpret_cast<const uint2*>(slot);
-          bits[0] = v.x << 16; bits[1] = v.x & 0xFFFF0000u;
-          bits[2] = v.y << 16; bits[3] = v.y & 0xFFFF0000u;
-        }
-        const float4 rv = *reinterpret_cast<const float4*>(rfifo + (buf * ROUNDS + r) * 32 * 16);
-        float4 acc;
-        acc.x = __fadd_rn(__uint_as_float(bits[0]), rv.x);
-        acc.y = __fadd_rn(__uint_as_float(bits[1]), rv.y);
-        acc.z = __fadd_rn(__uint_as_float(bits[2]), rv.z);
-        acc.w = __fadd_rn(__uint_as_float(bits[3]), rv.w);
-        *reinterpret_cast<float4*>(residual + seg_base + r * ROUND + lane * 4) = acc;
-        bits[0] = __float_as_uint(acc.x); bits[1] = __float_as_uint(acc.y);
-        bits[2] = __float_as_uint(acc.z); bits[3] = __float_as_uint(acc.w);
-        if (src.mask != nullptr) {
-          // this lane's EPL mask bits inside the round's ROUND / 32 words
-          const uint32_t word = __shfl_sync(0xFFFFFFFFu, mask_words, r * (ROUND / 32) + lane * EPL / 32);
-          const uint32_t m = (word >> (unsigned)((lane * EPL) & 31)) & ((1u << EPL) - 1u);
-#pragma unroll
-          for (int e = 0; e < EPL; ++e)
-            if (m & (1u << e)) bits[e] = 0;
-        }
-      } else {
-        // the bucket's ragged last segment: plain loads, missing elements read as 0 and are never kept
-#pragma unroll
-        for (int e = 0; e < EPL; ++e) {
-          const unsigned long long i = seg_base + r * ROUND + lane * EPL + e;
-          bits[e] = 0;
-          if (i < n) {
-            const float acc = __fadd_rn(__uint_as_float(src.raw1(i)), residual[i]);
-            residual[i] = acc;
-            bits[e] = src.pruned(i) ? 0u : __float_as_uint(acc);
-          }
-        }
-      }
-      const unsigned int f = keep_flags<EPL>(bits, t);
-      if (!__any_sync(0xFFFFFFFFu, f != 0)) continue;
-      kept += append_round<EPL>(f, bits, (unsigned int)(r * ROUND), seg_base + kept, seg_off, seg_val);
+      for (int r = 0; r < 4; ++r) res[FEEDBACK ? r : 0] = __ldcs(reinterpret_cast<const float4*>(residual + i0 + r * ROUND + lane * EPL));
     }
-    if (lane == 0) {
-      seg_count[seg] = (unsigned short)kept;
-      if (kept) atomicAdd(group_count + seg / kGroupSegs, kept);  // result unused: a fire-and-forget reduction
-    }
-    seg = next;
-    buf ^= 1;
-    mask_words = mask_words_next;
   }
-  cp_async_wait<0>();
+  uint32_t mw = 0;
+  if (MASKED && lane < SHARE / 32 && i0 + lane * 32ull < n) mw = __ldg(src.mask + i0 / 32 + lane);
+  if (FEEDBACK && whole) {
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      uint32_t b[4];
+      if (DTYPE == NSML_F32) {
+        b[0] = q[r].x; b[1] = q[r].y; b[2] = q[r].z; b[3] = q[r].w;
+      } else {
+        b[0] = q[r].x << 16; b[1] = q[r].x & 0xFFFF0000u;
+        b[2] = q[r].y << 16; b[3] = q[r].y & 0xFFFF0000u;
+      }
+      const float4 a = res[FEEDBACK ? r : 0];
+      const float4 sum = make_float4(__fadd_rn(__uint_as_float(b[0]), a.x), __fadd_rn(__uint_as_float(b[1]), a.y),
+                                     __fadd_rn(__uint_as_float(b[2]), a.z), __fadd_rn(__uint_as_float(b[3]), a.w));
+      q[r] = make_uint4(__float_as_uint(sum.x), __float_as_uint(sum.y), __float_as_uint(sum.z), __float_as_uint(sum.w));
+    }
+  }
+  pdl_wait();
+  if (FEEDBACK && whole) {
+#pragma unroll
+    for (int r = 0; r < 4; ++r) *reinterpret_cast<uint4*>(residual + i0 + r * ROUND + lane * EPL) = q[r];
+  }
+  if (!whole) {
+    // the bucket's ragged end: plain loads, missing elements read as 0 and are never kept
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      uint32_t w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+      for (int e = 0; e < EPL; ++e) {
+        const unsigned long long i = i0 + r * ROUND + lane * EPL + e;
+        if (i >= n) continue;
+        if (FEEDBACK) {
+          const float sum = __fadd_rn(__uint_as_float(src.raw1(i)), residual[i]);
+          residual[i] = sum;
+          w[e & 3] = __float_as_uint(sum);
+        } else if (DTYPE == NSML_F32) {
+          w[e & 3] = src.raw1(i);
+        } else {
+          w[(e >> 1) & 3] |= (src.raw1(i) >> 16) << (16 * (e & 1));
+        }
+      }
+      q[r] = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+  }
+  const Window win = make_window<FEEDBACK ? NSML_F32 : DTYPE>(ctl);
+  keep_tile<EPL, !FEEDBACK && DTYPE == NSML_BF16>(out, tile, first, win, ctl, sh, [&](int r, uint32_t (&bits)[EPL]) {
+    unpack16<FEEDBACK ? NSML_F32 : DTYPE, EPL>(q[r], bits);
+    if (MASKED) {
+      // this lane's EPL mask bits inside the round's ROUND / 32 words
+      const uint32_t word = __shfl_sync(0xFFFFFFFFu, mw, r * (ROUND / 32) + lane * EPL / 32);
+      const uint32_t m = (word >> (unsigned)((lane * EPL) & 31)) & ((1u << EPL) - 1u);
+#pragma unroll
+      for (int e = 0; e < EPL; ++e)
+        if (m & (1u << e)) bits[e] = 0;
+    }
+  });
 }
 
 }  // namespace nsml

@@ -30,12 +30,12 @@
 
 namespace nsml {
 
-template <int DTYPE, int THREADS, int CACHE>
-__global__ void __launch_bounds__(THREADS, 1024 / THREADS)  // at most 64 registers per thread
-k_finalize_dense(BucketSrc<DTYPE> src, FinalizeParams p) {
+// s_cache: CACHE values of shared memory; stage: 256 words per warp for the write phase (may be sh.hist);
+// `barriers`: grid barriers passed so far.
+template <int DTYPE, int THREADS, int CACHE, bool CLUSTER>
+__device__ __forceinline__ void dense_select(const BucketSrc<DTYPE>& src, const FinalizeParams& p, FinalizeShared<THREADS>& sh, uint32_t* s_cache,
+                                             uint32_t* stage, unsigned int barriers) {
   static_assert(CACHE % 128 == 0, "a warp step (32 words) is cached as a whole or not at all");
-  __shared__ FinalizeShared<THREADS, true> sh;
-  extern __shared__ __align__(16) uint32_t s_cache[];
   uint4* cache4 = reinterpret_cast<uint4*>(s_cache);
   constexpr int NW = THREADS / 32;
   constexpr unsigned int CW = CACHE / 4;  // cached words
@@ -46,7 +46,6 @@ k_finalize_dense(BucketSrc<DTYPE> src, FinalizeParams p) {
   const unsigned long long range_hi = min(((unsigned long long)(blk + 1) * p.nseg / G) * kSegElems, p.n);
   const unsigned int E = (unsigned int)(range_hi - range_lo);  // >= 1: the grid has at most nseg blocks
   const unsigned int W = (E + 3) / 4;
-  unsigned int barriers = 0;
 
   // This warp's slices, in words: q = 0 cached, q = 1 not cached.  Slice lengths are multiples of 32.
   const unsigned int cached_w = min(W, CW);
@@ -142,7 +141,7 @@ k_finalize_dense(BucketSrc<DTYPE> src, FinalizeParams p) {
     if (nonfinite) set_status(&p.ctl->status, NSML_ERR_NONFINITE);
   }
   flush_hist<kMaxBins>(sh, p.hist);
-  if (!grid_barrier(p.ctl, ++barriers * G, sh)) return;
+  if (!grid_barrier<CLUSTER>(p.ctl, ++barriers * G, sh)) return;
 
   // ---------------- phase 1: resolve digit 0, histogram of digit 1 ----------------
   // Digit 0 splits the entries into those above the threshold's bin (survivors whatever T turns out
@@ -158,7 +157,7 @@ k_finalize_dense(BucketSrc<DTYPE> src, FinalizeParams p) {
   unsigned int above[2] = {0, 0};           // this lane's keys above bin d0, per slice
   unsigned int und_len = 0, und_len0 = 0;   // listed so far (warp-uniform); of those, from slice 0
   bool und_ok = E <= 65536u;                // warp-uniform
-  unsigned short* und = sh.g.und[warp];
+  unsigned short* und = sh.und[warp];
   const unsigned int lt = (1u << lane) - 1u;
   {
     unsigned int zeros = 0;
@@ -211,7 +210,7 @@ k_finalize_dense(BucketSrc<DTYPE> src, FinalizeParams p) {
     if (threadIdx.x == 0 && block_zeros != 0) atomicAdd(&sh.hist[0], (unsigned int)block_zeros);
   }
   flush_hist<kMaxBins>(sh, p.hist + 1 * kMaxBins);
-  if (!grid_barrier(p.ctl, ++barriers * G, sh)) return;
+  if (!grid_barrier<CLUSTER>(p.ctl, ++barriers * G, sh)) return;
 
   // Calls f(q, key) for this lane's share of the warp's listed undecided entries.
   auto for_listed = [&](auto&& f) {
@@ -256,7 +255,7 @@ k_finalize_dense(BucketSrc<DTYPE> src, FinalizeParams p) {
     if (threadIdx.x == 0 && block_zeros != 0) atomicAdd(&sh.hist[0], (unsigned int)block_zeros);
   }
   flush_hist<128>(sh, p.hist + 2 * kMaxBins);
-  if (!grid_barrier(p.ctl, ++barriers * G, sh)) return;
+  if (!grid_barrier<CLUSTER>(p.ctl, ++barriers * G, sh)) return;
 
   // ---------------- phase 3: T and r; this warp's keys > T and == T, per slice ----------------
   resolve_digit<128>(p.hist + 2 * kMaxBins, rem, sh);
@@ -300,9 +299,9 @@ k_finalize_dense(BucketSrc<DTYPE> src, FinalizeParams p) {
     block_a += sh.run[w] >> 32;
     block_c += sh.run[w] & 0xFFFFFFFFull;
   }
-  unsigned long long* ac_counts = p.block_counts + 1 * kMaxFinalizeBlocks;
+  unsigned long long* ac_counts = p.block_counts;
   if (threadIdx.x == 0) ac_counts[blk] = (block_a << 32) | block_c;
-  if (!grid_barrier(p.ctl, ++barriers * G, sh)) return;
+  if (!grid_barrier<CLUSTER>(p.ctl, ++barriers * G, sh)) return;
 
   // ---------------- phase 4: write the survivors in index order ----------------
   unsigned long long a_before = 0, c_before = 0, a_all = 0, c_all = 0;
@@ -324,8 +323,7 @@ k_finalize_dense(BucketSrc<DTYPE> src, FinalizeParams p) {
     return;
   }
   uint32_t* out_idx = reinterpret_cast<uint32_t*>(p.payload + p.P.idx_off);
-  static_assert(kMaxBins * 4 >= NW * 128 * 8, "the staging areas of all warps fit the histogram");
-  uint32_t* stage_idx = sh.hist + warp * 256;  // 128 indices, then 128 values, per warp
+  uint32_t* stage_idx = stage + warp * 256;  // 128 indices, then 128 values, per warp
   uint32_t* stage_val = stage_idx + 128;
 #pragma unroll
   for (int q = 0; q < 2; ++q) {
@@ -367,7 +365,7 @@ k_finalize_dense(BucketSrc<DTYPE> src, FinalizeParams p) {
       const unsigned int total = __shfl_sync(FULL, incl, 31);
       const unsigned int a_lane = (incl - mine) & 0xFFFFu, c_lane = (incl - mine) >> 16;  // of this step, in lower lanes
       // Survivors of this step go to consecutive payload positions.  They are first put in order into the
-      // warp's staging area (the histogram's shared memory, free in this phase), then written 32 at a time.
+      // warp's staging area (usually the histogram's shared memory, free in this phase), then written 32 at a time.
       const unsigned int c_room = r > c_here ? r - c_here : 0u;           // ties still to keep from here on
       const unsigned int ta = total & 0xFFFFu, tc = min(total >> 16, c_room);
       const unsigned int step_base = a_here + min(c_here, r);              // payload position of the step's first survivor
@@ -401,8 +399,17 @@ k_finalize_dense(BucketSrc<DTYPE> src, FinalizeParams p) {
   // ---------------- phase 5: the header; int8: quantise ----------------
   if (blk == 0 && threadIdx.x == 0) write_header(p);
   if (p.bits != NSML_BITS_INT8) return;  // float32 and fp16 values are in the payload already
-  if (!grid_barrier(p.ctl, ++barriers * G, sh)) return;
+  if (!grid_barrier<CLUSTER>(p.ctl, ++barriers * G, sh)) return;
   quantize_all(p, sh);
+}
+
+template <int DTYPE, int THREADS, int CACHE>
+__global__ void __launch_bounds__(THREADS, 1024 / THREADS)  // at most 64 registers per thread
+k_finalize_dense(BucketSrc<DTYPE> src, FinalizeParams p) {
+  __shared__ FinalizeShared<THREADS> sh;
+  extern __shared__ __align__(16) uint32_t s_cache[];
+  static_assert(kMaxBins >= THREADS / 32 * 256, "the staging areas of all warps fit the histogram");
+  dense_select<DTYPE, THREADS, CACHE, false>(src, p, sh, s_cache, sh.hist, 0);
 }
 
 }  // namespace nsml

@@ -1,19 +1,22 @@
-// Sampled lower bound for the top-k threshold (Alg. 2 Step 3: which
-// k = ceil(ratio*n) gradients have the largest absolute value).
+// Sampled bounds of the top-k threshold (Alg. 2 Step 3: which k = ceil(ratio*n)
+// gradients have the largest absolute value).
 //
 // The bucket is streamed exactly once, by the compaction pass, which needs a
-// key `lo` such that a little more than k keys are >= lo.  k_sample draws one
-// element from each of 8192 equal strata of the bucket and radix-selects the
-// sample key whose rank leaves a six-sigma margin above the expected rank of
-// the k-th largest; lo is that key rounded down to its top 24 bits.  The exact
-// threshold is found afterwards on the short candidate list
-// (nsml_finalize.cuh), which also repairs the rare case of a misleading
+// key `lo` such that a little more than k keys are >= lo, and counts the keys
+// between lo and a second bound `hi` that a little fewer than k keys exceed.
+// k_sample reads one 32-byte sector (8 float32 or 16 bfloat16 keys) from each of
+// 8192 equal strata of the bucket and takes the two sample keys whose ranks lie
+// six standard deviations either side of the expected rank of the k-th largest,
+// rounded outwards to their top 15 bits.  The exact threshold is found
+// afterwards (nsml_list.cuh), which also repairs the rare case of a misleading
 // sample, so the sample only decides how much work is done, never the result.
 //
-// The kernel is one cluster of eight blocks: 8192 threads fetch one scattered
-// element each (one round of memory latency, spread over eight SMs), write the
-// keys into block 0's shared memory through the cluster's distributed shared
-// memory, meet at the cluster barrier, and block 0 selects.
+// What bounds the kernel is latency: launch, one round of scattered reads, the
+// select.  It is one cluster of eight blocks; a block counts its keys' top 15
+// bits (all of a bfloat16 magnitude) in shared memory, then sums an eighth of
+// the bins over the eight blocks through distributed shared memory, so that one
+// counting level and two cluster barriers replace the two levels in a single
+// block that an exact 24-bit select takes.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -35,7 +38,7 @@ __device__ __forceinline__ uint32_t mix32(uint32_t x) {
 
 // Block-wide search from the top over bins held PER per thread (own[] holds
 // this thread's consecutive bins, lowest first): leaves in s_out the digit d
-// with #{digit > d} < rem <= #{digit >= d} and the rank left inside bin d.
+// with #{digit > d} < rem <= #{digit >= d}, the rank left inside bin d and the bin's count.
 // Called by every thread of the block; s_tot needs one word per warp.
 template <int PER, int THREADS>
 __device__ __forceinline__ void find_digit_from_top(const unsigned int (&own)[PER], unsigned int rem,
@@ -61,6 +64,7 @@ __device__ __forceinline__ void find_digit_from_top(const unsigned int (&own)[PE
       if (rem <= above + own[b]) {
         s_out[0] = (unsigned)(t * PER + b);
         s_out[1] = rem - above;
+        s_out[2] = own[b];
         break;
       }
       above += own[b];
@@ -69,66 +73,118 @@ __device__ __forceinline__ void find_digit_from_top(const unsigned int (&own)[PE
   __syncthreads();
 }
 
-// Clears the per-call control region and sets ctl->lo from a stratified
-// sample of the bucket (of bucket + addend when an addend is given).  rank_from_top == 0 means "no sampling" (small bucket, or nearly
-// everything is kept): lo = 0.
+template <int DTYPE>
+__host__ __device__ constexpr int sample_keys() { return DTYPE == NSML_F32 ? 8 : 16; }  // keys per stratum: a 32-byte sector
+constexpr int kSampleBinBits = 15;
+constexpr int kSampleBins = 1 << kSampleBinBits;  // bins of the keys' top bits, 16-bit counters
+constexpr size_t kSampleSmem = kSampleBins * 2;
+
+// Clears the per-call control region and sets ctl->lo and ctl->hi from a stratified sample of the bucket (of
+// bucket + addend when an addend is given).  rank_lo, rank_hi: ranks from the top among the sampled keys.  A rank
+// beyond the non-zero sample keys leaves its bound 0.
 template <int DTYPE>
 __global__ void __cluster_dims__(kSampleBlocks, 1, 1) __launch_bounds__(kSampleThreads)
-k_sample(BucketSrc<DTYPE> src, const float* __restrict__ addend, unsigned long long n, unsigned int rank_from_top,
+k_sample(BucketSrc<DTYPE> src, const float* __restrict__ addend, unsigned long long n, unsigned int rank_lo, unsigned int rank_hi,
          Ctl* ctl, uint4* zero_base, unsigned int zero_vec16, int keep_status) {
   namespace cg = cooperative_groups;
-  __shared__ unsigned int s_keys[kSamples];  // block 0: the sample keys, then (first 4096 words) the histogram
-  unsigned int* s_hist = s_keys;
-  __shared__ unsigned int s_tot[kSampleThreads / 32];
-  __shared__ unsigned int s_out[2];
+  constexpr int KEYS = sample_keys<DTYPE>();
+  extern __shared__ __align__(16) unsigned int s_bins[];  // two 16-bit counters per word
+  __shared__ unsigned int s_scan[kSampleThreads / 32];
+  __shared__ unsigned int s_slice[kSampleBlocks];  // keys in each block's slice of the bins
   cg::cluster_group cluster = cg::this_cluster();
   const unsigned int rank = cluster.block_rank();
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  for (int i = t; i < kSampleBins / 8; i += kSampleThreads) reinterpret_cast<uint4*>(s_bins)[i] = make_uint4(0u, 0u, 0u, 0u);
+  pdl_wait();
+  pdl_launch_dependents();  // the bucket pass may start to load (only now: what the stream did before this kernel is complete)
 
-  if (rank_from_top != 0) {
-    const unsigned long long stratum = (unsigned long long)rank * kSampleThreads + threadIdx.x;
-    const unsigned long long begin = stratum * n / kSamples;
-    const unsigned long long end = (stratum + 1) * n / kSamples;  // > begin because n >= 2 * kSamples
-    const unsigned long long pos = begin + mix32((uint32_t)stratum * 0x9E3779B1u + 0x85EBCA6Bu) % (uint32_t)(end - begin);
+  const unsigned long long stratum = (unsigned long long)rank * kSampleThreads + t;
+  const unsigned long long begin = stratum * n / kSamples;
+  const unsigned long long end = (stratum + 1) * n / kSamples;  // > begin
+  unsigned long long pos = (begin + mix32((uint32_t)stratum * 0x9E3779B1u + 0x85EBCA6Bu) % (uint32_t)(end - begin)) & ~(unsigned long long)(KEYS - 1);
+  if (pos + KEYS > n) pos = (n - KEYS) & ~(unsigned long long)(KEYS - 1);  // (n >= KEYS)
+  uint32_t bits[KEYS / 4][4];
+#pragma unroll
+  for (int q = 0; q < KEYS / 4; ++q) {
+    const BucketSrc<DTYPE> bare{src.grad, addend != nullptr ? nullptr : src.mask};
+    bare.load_full4(pos + q * 4, bits[q]);
+  }
+  if (addend != nullptr) {
     // with an addend (the residual of the local accumulation) the bucket that is selected from is the sum
-    uint32_t bits = src.load1(pos);
-    if (addend != nullptr && !src.pruned(pos)) bits = __float_as_uint(__fadd_rn(__uint_as_float(src.raw1(pos)), addend[pos]));
-    const uint32_t key = bits & 0x7FFFFFFFu;
-    unsigned int* remote = cluster.map_shared_rank(s_keys, 0);
-    remote[stratum] = key;
+#pragma unroll
+    for (int q = 0; q < KEYS / 4; ++q) {
+      const float4 a = *reinterpret_cast<const float4*>(addend + pos + q * 4);
+      const float add[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        bits[q][e] = __float_as_uint(__fadd_rn(__uint_as_float(bits[q][e]), add[e]));
+        if (src.pruned(pos + q * 4 + e)) bits[q][e] = 0;
+      }
+    }
   }
   // keep_status: an error an earlier step of the same call left in the status word stays visible
-  for (unsigned int i = rank * kSampleThreads + threadIdx.x; i < zero_vec16; i += kSamples)
+  for (unsigned int i = rank * kSampleThreads + t; i < zero_vec16; i += kSamples)
     zero_base[i] = make_uint4((i == 0 && keep_status) ? (unsigned int)ctl->status : 0u, 0, 0, 0);
-  cluster.sync();  // release/acquire at cluster scope: keys have landed in block 0, the control region is cleared
-  if (rank != 0) return;
-
-  unsigned int lo = 0;
-  if (rank_from_top != 0) {
-    uint32_t keys[kSampleBlocks];
+  __syncthreads();
+  unsigned int fine_keys = 0;  // keys with any of their low 16 bits set
 #pragma unroll
-    for (int s = 0; s < kSampleBlocks; ++s) keys[s] = s_keys[s * kSampleThreads + threadIdx.x];
-    __syncthreads();  // every key is in registers: the buffer becomes the histogram
-    unsigned int prefix = 0, rem = rank_from_top;
+  for (int q = 0; q < KEYS / 4; ++q)
 #pragma unroll
-    for (int level = 0; level < 2; ++level) {  // 12 + 12 bits
-      const int shift = digit_shift(level);
-      __syncthreads();  // the previous level's bins have been read
-      for (int b = threadIdx.x; b < kMaxBins; b += kSampleThreads) s_hist[b] = 0;
-      __syncthreads();
-#pragma unroll
-      for (int s = 0; s < kSampleBlocks; ++s)
-        if (level == 0 || (keys[s] >> 19) == prefix) atomicAdd(&s_hist[(keys[s] >> shift) & (kMaxBins - 1)], 1u);
-      __syncthreads();
-      unsigned int own[4];
-#pragma unroll
-      for (int b = 0; b < 4; ++b) own[b] = s_hist[threadIdx.x * 4 + b];
-      find_digit_from_top<4, kSampleThreads>(own, rem, s_tot, s_out);
-      prefix = (prefix << 12) | s_out[0];
-      rem = s_out[1];
+    for (int e = 0; e < 4; ++e) {
+      const unsigned int bin = (bits[q][e] & 0x7FFFFFFFu) >> (31 - kSampleBinBits);
+      fine_keys += (bits[q][e] & 0xFFFFu) != 0;
+      if (bin != 0) atomicAdd(&s_bins[bin >> 1], 1u << (16 * (bin & 1)));  // (a block has at most 16384 keys: no overflow)
     }
-    lo = prefix << 7;
+  const int fine_threads = DTYPE == NSML_F32 ? __syncthreads_count(fine_keys != 0) : 0;
+  cluster.sync();  // every block's counts are complete, the control region is cleared
+  // (a float32 key has its low 16 bits zero once in 65536)
+  if (rank == 0 && t == 0) ctl->coarse = fine_threads < kSampleThreads / 16;
+
+  // this block's slice of the bins, four per thread, summed over the blocks
+  constexpr int kSlice = kSampleBins / kSampleBlocks;
+  static_assert(kSlice == 4 * kSampleThreads, "four bins per thread");
+  unsigned int own[4] = {0, 0, 0, 0};
+#pragma unroll
+  for (int b = 0; b < kSampleBlocks; ++b) {
+    const uint2 v = reinterpret_cast<const uint2*>(cluster.map_shared_rank(s_bins, b))[rank * (kSlice / 4) + t];
+    own[0] += v.x & 0xFFFFu; own[1] += v.x >> 16;
+    own[2] += v.y & 0xFFFFu; own[3] += v.y >> 16;
   }
-  if (threadIdx.x == 0) ctl->lo = lo;
+  const unsigned int mine = own[0] + own[1] + own[2] + own[3];
+  unsigned int incl = mine;  // this thread and all higher lanes of the warp
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned int v = __shfl_down_sync(0xFFFFFFFFu, incl, o);
+    if (lane + o < 32) incl += v;
+  }
+  if (lane == 0) s_scan[warp] = incl;
+  __syncthreads();
+  unsigned int above = incl - mine, total = 0;
+#pragma unroll
+  for (int w = 0; w < kSampleThreads / 32; ++w) {
+    const unsigned int c = s_scan[w];
+    if (w > warp) above += c;
+    total += c;
+  }
+  if (t < kSampleBlocks) *cluster.map_shared_rank(&s_slice[rank], t) = total;
+  cluster.sync();  // also: no block leaves while its bins are still read
+  for (int s = rank + 1; s < kSampleBlocks; ++s) above += s_slice[s];
+#pragma unroll
+  for (int which = 0; which < 2; ++which) {
+    const unsigned int j = which == 0 ? rank_lo : rank_hi;
+    if (above < j && j <= above + mine) {  // exactly one thread of the cluster, if any
+      unsigned int a = above;
+#pragma unroll
+      for (int b = 3; b >= 0; --b) {
+        if (a < j && j <= a + own[b]) {
+          const unsigned int bin = rank * kSlice + t * 4 + b;
+          if (which == 0) ctl->lo = bin << (31 - kSampleBinBits);
+          else ctl->hi = (bin + 1) << (31 - kSampleBinBits);
+        }
+        a += own[b];
+      }
+    }
+  }
 }
 
 }  // namespace nsml

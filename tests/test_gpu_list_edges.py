@@ -1,0 +1,103 @@
+"""GPU parity of the list strategy where it can go wrong: tile edges, a threshold bin longer than its list, ties, a
+sample that misleads in either direction, keys without low bits, lists longer than a block's shared memory."""
+import numpy as np
+import pytest
+import torch
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+if torch.cuda.is_available():
+    import paper_2506_16235_b200 as nsml
+    from gpu_util import check_compress, gpu_compress, oracle_compress, assert_payload_equal
+    from test_gpu_compress import sampled_positions
+
+
+def gauss(n, seed, spread=2.0):
+    rng = np.random.default_rng(seed)
+    return (rng.standard_normal(n) * 10.0 ** rng.uniform(-4.0, -4.0 + spread, n)).astype(np.float32)
+
+
+def sampled_sectors(n, keys):
+    """All elements of the sectors the sampler reads (`keys` elements, aligned)."""
+    pos = sampled_positions(n) & ~np.int64(keys - 1)
+    pos = np.where(pos + keys > n, (n - keys) & ~np.int64(keys - 1), pos)
+    return np.unique((pos[:, None] + np.arange(keys)).reshape(-1))
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("n", [8 * 8192 - 1, 8 * 8192, 8 * 8192 + 1, 17 * 4096 + 513, 64 * 4096 + 1])
+def test_tile_and_group_edges(n, dtype):
+    g = gauss(n, n)
+    g[-2:] = [3.0, -4.0]
+    g[4095:4097] = [5.0, -6.0]
+    if dtype == "bf16":
+        g = synth.f32_to_bf16_bits(g)
+    mask = np.random.default_rng(n).random(n) < 0.3
+    for ratio, bits in ((0.002, 8), (0.03, 32), (0.2, 16)):
+        check_compress(g, ratio, bits)
+        check_compress(g, ratio, bits, mask_bool=mask)
+
+
+@pytest.mark.parametrize("ties", [1, 1023, 1024, 1025, 40_000])
+def test_threshold_bin_at_the_length_of_its_list(ties):
+    # `ties` equal magnitudes around the threshold, spread over the bucket; half of them survive
+    n, ratio = 1_000_003, 0.05
+    rng = np.random.default_rng(ties)
+    g = (rng.standard_normal(n) * 1e-3).astype(np.float32)
+    k = nsml.nsml_k_of(n, ratio)
+    order = rng.permutation(n)
+    g[order[:k - (ties + 1) // 2]] = (2.0 + rng.random(k - (ties + 1) // 2)).astype(np.float32)
+    g[order[k - (ties + 1) // 2:k - (ties + 1) // 2 + ties]] = np.float32(0.712345) * rng.choice(np.array([-1, 1], np.float32), ties)
+    check_compress(g, ratio, 8)
+
+
+def test_many_close_keys_in_the_threshold_bin():
+    # 200k keys inside a few thousand float32 steps of one another: the bin is refined
+    n = 2_000_000
+    rng = np.random.default_rng(5)
+    g = (rng.standard_normal(n) * 1e-4).astype(np.float32)
+    where = rng.choice(n, 200_000, replace=False)
+    g[where] = (np.float32(0.5).view(np.uint32) + rng.integers(0, 3000, 200_000).astype(np.uint32)).view(np.float32)
+    for ratio in (0.05, 0.0995):
+        check_compress(g, ratio, 16)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_misleading_samples(dtype):
+    n = 1 << 20
+    rng = np.random.default_rng(3)
+    keys = 8 if dtype == "f32" else 16
+    conv = (lambda x: x) if dtype == "f32" else synth.f32_to_bf16_bits
+    at = sampled_sectors(n, keys)
+    low = gauss(n, 1)
+    low[at] = 0.0                     # the sample sees only zeros: everything non-zero is listed
+    high = gauss(n, 2)
+    high[at] *= np.float32(1e4)       # the sample sees only large values: too short a list
+    hidden = gauss(n, 4)
+    hidden[at] *= np.float32(1e-6)    # the sample sees only small values: the threshold lies above the window
+    for g in (low, high, hidden):
+        check_compress(conv(g), 0.01, 8)
+
+
+def test_float32_bucket_widened_from_bfloat16():
+    n = 3_000_001
+    g = (synth.f32_to_bf16_bits(gauss(n, 8)).astype(np.uint32) << 16).view(np.float32)
+    for ratio in (0.001, 0.02, 0.2):
+        check_compress(g, ratio, 8)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_list_longer_than_the_blocks_shared_memory(dtype):
+    n = 20_000_003
+    g = gauss(n, 9, spread=1.0)
+    if dtype == "bf16":
+        g = synth.f32_to_bf16_bits(g)
+    for bits in (8, 16):
+        check_compress(g, 0.24, bits)
+
+
+def test_all_equal_large_bucket():
+    g = np.full(2_000_001, 0.37, dtype=np.float32)
+    check_compress(g, 0.05, 8)
