@@ -206,12 +206,12 @@ class Workload:
             self.account(acc, "k_clear", 256 + 4 * 4 * 4096)
             self.account(acc, "k_finalize_dense", esize * n + 8 * k + 4 * k + vb * k + s)
             return
-        self.account(acc, "k_sample", 32 * 8192)
+        self.account(acc, "k_sample", 16 * 16384)
         # candidates: 16-bit offset in the tile + value (bfloat16: both in 32 bits)
         entry = 6 if esize == 4 else 4
         self.account(acc, "k_compact_bucket", esize * n + entry * k)
         # list stage: candidates read once; survivors written, for int8 by way of a float32 copy
-        self.account(acc, "k_finalize", entry * k + 4 * k + (8 * k if bits == 8 else 0) + vb * k + s)
+        self.account(acc, "k_emit", entry * k + 4 * k + (8 * k if bits == 8 else 0) + vb * k + s)
 
     def merge_bytes(self, acc, n, ks_bits, zero_first=True):
         total = 4 * n if zero_first else 0

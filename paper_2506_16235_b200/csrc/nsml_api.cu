@@ -19,11 +19,11 @@
 namespace nsml {
 
 enum KernelId {
-  K_SAMPLE = 0, K_COMPACT_BUCKET, K_FINALIZE, K_PARTITION, K_MERGE, K_CLEAR, K_FINALIZE_DENSE,
+  K_SAMPLE = 0, K_COMPACT_BUCKET, K_EMIT, K_PARTITION, K_MERGE, K_CLEAR, K_FINALIZE_DENSE,
   K_SUMSQ, K_FEEDBACK_ADD, K_FEEDBACK_SUBTRACT, K_PRUNE_HIST, K_PRUNE_TIES, K_PRUNE_WRITE, K_PRUNE_WRITE_RANKED, K_PRUNE_SAMPLE, K_PRUNE_COUNT, K_PRUNE_SETTLE, K_PRUNE_MARK, K_PRUNE_FIX, K_COUNT
 };
 
-static const char* const kKernelNames[K_COUNT] = {"k_sample", "k_compact_bucket", "k_finalize", "k_partition", "k_merge",
+static const char* const kKernelNames[K_COUNT] = {"k_sample", "k_compact_bucket", "k_emit", "k_partition", "k_merge",
                                                   "k_clear", "k_finalize_dense", "k_sumsq", "k_feedback_add",
                                                   "k_feedback_subtract", "k_prune_hist", "k_prune_ties", "k_prune_write",
                                                   "k_prune_write_ranked", "k_prune_sample", "k_prune_count",
@@ -106,12 +106,10 @@ static int device_info(const DeviceInfo** out) {
     prepare(k_finalize_dense<NSML_F32, kFinLargeThreads, kFinDenseLargeCache>, kFinLargeThreads, finalize_dyn_smem(kFinDenseLargeCache), &d.dense_large);
     prepare(k_finalize_dense<NSML_BF16, kFinLargeThreads, kFinDenseLargeCache>, kFinLargeThreads, finalize_dyn_smem(kFinDenseLargeCache), &d.dense_large);
     int list_fits = 0;  // every shape of the list stage is resident at least once per SM
-    prepare(k_finalize<NSML_F32, kListSmallCache, true>, kListThreads, list_dyn_smem(kListSmallCache), &list_fits);
-    prepare(k_finalize<NSML_BF16, kListSmallCache, true>, kListThreads, list_dyn_smem(kListSmallCache), &list_fits);
-    prepare(k_finalize<NSML_F32, kListSmallCache, false>, kListThreads, list_dyn_smem(kListSmallCache), &list_fits);
-    prepare(k_finalize<NSML_BF16, kListSmallCache, false>, kListThreads, list_dyn_smem(kListSmallCache), &list_fits);
-    prepare(k_finalize<NSML_F32, kListLargeCache, false>, kListThreads, list_dyn_smem(kListLargeCache), &list_fits);
-    prepare(k_finalize<NSML_BF16, kListLargeCache, false>, kListThreads, list_dyn_smem(kListLargeCache), &list_fits);
+    prepare(k_emit<NSML_F32, kEmitPer>, kEmitThreads, sizeof(EmitShared), &list_fits);
+    prepare(k_emit<NSML_BF16, kEmitPer>, kEmitThreads, sizeof(EmitShared), &list_fits);
+    prepare(k_emit<NSML_F32, 2 * kEmitPer>, kEmitThreads, sizeof(EmitShared), &list_fits);
+    prepare(k_emit<NSML_BF16, 2 * kEmitPer>, kEmitThreads, sizeof(EmitShared), &list_fits);
     prepare(k_sample<NSML_F32>, kSampleThreads, kSampleSmem, &list_fits);
     prepare(k_sample<NSML_BF16>, kSampleThreads, kSampleSmem, &list_fits);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.merge, k_merge<kDenseTileLarge>, kMergeThreads, 0);
@@ -225,13 +223,14 @@ struct SamplePlan {
 
 static SamplePlan sample_plan(int64_t n, int64_t k, int grad_dtype) {
   SamplePlan s;
-  if (n < 2 * (int64_t)kSamples) return s;
+  if (n < (int64_t)kSamples) return s;
   const double keys = (double)kSamples * (grad_dtype == NSML_F32 ? sample_keys<NSML_F32>() : sample_keys<NSML_BF16>());
   const double p = (double)k / (double)n, mean = keys * p, six = 6.0 * std::sqrt(keys * p * (1.0 - p));
   const double lo = std::ceil(mean + six) + 1.0, hi = std::floor(mean - six);
   if (lo >= keys) return s;
   s.rank_lo = (unsigned int)lo;
-  s.rank_hi = hi < 1.0 ? 1u : (unsigned int)hi;
+  // (the largest sampled key, with about n / keys elements above it, where that is safely fewer than k)
+  s.rank_hi = hi >= 1.0 ? (unsigned int)hi : 8.0 * (double)n / keys < (double)k ? 1u : 0u;
   s.expected = (double)n * (mean + six) / keys * 1.04 + 64.0;  // (the bound is rounded down to 15 key bits: a few per cent more)
   return s;
 }
@@ -265,7 +264,6 @@ static int launch_compress(const void* grad, float* residual, const uint32_t* ma
   fp.ctl = ctl;
   fp.hist = reinterpret_cast<unsigned int*>(ws + L.hist);
   fp.block_counts = reinterpret_cast<unsigned long long*>(ws + L.block_counts);
-  fp.bin_list = reinterpret_cast<uint2*>(ws + L.bin_list);
   fp.tiles = (unsigned int)(((unsigned long long)n + tile - 1) / tile);
   fp.list.off = reinterpret_cast<unsigned short*>(ws + L.cand_off);
   fp.list.val = reinterpret_cast<uint32_t*>(ws + L.cand_val);
@@ -273,7 +271,14 @@ static int launch_compress(const void* grad, float* residual, const uint32_t* ma
   fp.list.group_count = reinterpret_cast<unsigned int*>(ws + L.group_count);
   fp.list.window_hist = fp.hist + 3 * kMaxBins;
   fp.list.group_shift = group_shift_of(fp.tiles);
+  fp.list.bins = reinterpret_cast<uint2*>(ws + L.bins);
+  fp.list.bin_room = bin_room_of(n);
+  const size_t chunks = align_up((size_t)n, tile_elems<NSML_BF16>()) / kChunk;
+  fp.list.chunk_sum[0] = reinterpret_cast<unsigned long long*>(ws + L.chunk_sum);
+  fp.list.chunk_sum[1] = fp.list.chunk_sum[0] + chunks;
+  fp.list.block_fill = reinterpret_cast<unsigned int*>(ws + L.block_fill);
   fp.raw_val = reinterpret_cast<float*>(ws + L.raw_val);
+  fp.residual = residual;
   fp.payload = payload;
   fp.P = P;
   cudaError_t le;
@@ -315,22 +320,16 @@ static int launch_compress(const void* grad, float* residual, const uint32_t* ma
                      dim3(fp.tiles), dim3(kCta), 0, st, false, 0, false, true, src, residual, (unsigned long long)n, ctl, fp.list);
     if (le != cudaSuccess) return NSML_ERR_CUDA;
   }
-  LaunchScope scope(K_FINALIZE, st);
-  if (plan.expected <= kListClusterMaxCandidates && fp.tiles >= kListClusterBlocks) {
-    // the blocks of a cluster are co-scheduled by the hardware, so no cooperative launch is needed
-    le = launch_prio(k_finalize<FDTYPE, kListSmallCache, true>, dim3(kListClusterBlocks), dim3(kListThreads), list_dyn_smem(kListSmallCache),
-                     st, false, kListClusterBlocks, true, true, fsrc, fp);
-  } else if (plan.expected / dev.sms <= (double)kListSmallCache) {
-    // short lists: no more blocks than about 4096 candidates each (cheaper barriers)
-    unsigned int grid = (unsigned int)(plan.expected / (double)g_list_block_candidates.load(std::memory_order_relaxed)) + 1;
-    if (grid > (unsigned int)dev.sms) grid = (unsigned int)dev.sms;
-    le = launch_prio(k_finalize<FDTYPE, kListSmallCache, false>, dim3(grid), dim3(kListThreads), list_dyn_smem(kListSmallCache), st, true, 0,
-                     true, true, fsrc, fp);
-  } else {
-    le = launch_prio(k_finalize<FDTYPE, kListLargeCache, false>, dim3(dev.sms), dim3(kListThreads), list_dyn_smem(kListLargeCache), st, true, 0,
-                     true, true, fsrc, fp);
+  {
+    // Blocks draw chunks of the list by ticket; no more blocks than about 4096 candidates each, at most two per SM.
+    LaunchScope scope(K_EMIT, st);
+    const double want = plan.expected / (0.5 * (double)g_list_block_candidates.load(std::memory_order_relaxed)) + 1.0;
+    const unsigned int grid = want < 2.0 * dev.sms ? (unsigned int)want : 2u * dev.sms;
+    // long lists: larger chunks, a block takes several
+    le = launch_prio(plan.expected <= 2.0 * dev.sms * kChunk ? k_emit<FDTYPE, kEmitPer> : k_emit<FDTYPE, 2 * kEmitPer>, dim3(grid), dim3(kEmitThreads), sizeof(EmitShared), st, false, 0, true, true, fsrc, fp);
+    if (le != cudaSuccess) return NSML_ERR_CUDA;
   }
-  return le == cudaSuccess ? NSML_OK : NSML_ERR_CUDA;
+  return NSML_OK;
 }
 
 static int compress_impl(const void* grad, int64_t n, int grad_dtype, double ratio, int bits,
@@ -604,7 +603,7 @@ static int feedback_impl(const void* grad, float* residual, int64_t n, int grad_
       rc = launch_compress<NSML_BF16, NSML_F32>(grad, residual, prune_mask, n, k, bits, ws, pl, L, P, *dev, st);
   }
   if (rc != NSML_OK) return rc;
-  {
+  if (use_dense(n, k)) {  // (the list stage takes what the payload carries out of the residual itself)
     LaunchScope scope(K_FEEDBACK_SUBTRACT, st);
     const unsigned int sgrid = grid_for((unsigned long long)k, kCta, dev->sms * 8);
     k_feedback_subtract<<<sgrid, kCta, 0, st>>>(static_cast<const unsigned char*>(payload), residual,
@@ -657,7 +656,7 @@ int nsml_compress_strategy(int64_t n, double ratio) {
 }
 
 int nsml_set_list_block_candidates(int candidates) {
-  if (candidates < 1024 || candidates > kListSmallCache) return NSML_ERR_ARG;
+  if (candidates < 1024 || candidates > 8192) return NSML_ERR_ARG;
   g_list_block_candidates.store(candidates, std::memory_order_relaxed);
   return NSML_OK;
 }

@@ -17,10 +17,13 @@ __device__ __forceinline__ uint16_t encode_f16(float v) {
 
 __device__ __forceinline__ float decode_f16(uint16_t h) { return __half2float(__ushort_as_half(h)); }
 
-// code = clamp(rint(v / scale), +-127): one IEEE division, half to even.
-__device__ __forceinline__ int encode_i8(float v, float scale) {
+// code = clamp(rint(v / scale), +-127): one IEEE division, half to even.  inv = 1 / scale (any rounding): the product
+// v * inv differs from the quotient by less than 1e-4, so where it is not that close to the middle between two integers
+// it gives the same code without the division.
+__device__ __forceinline__ int encode_i8(float v, float scale, float inv) {
   if (scale == 0.0f) return 0;
-  int c = __float2int_rn(__fdiv_rn(v, scale));
+  const float near = __fmul_rn(v, inv), whole = rintf(near);
+  const int c = fabsf(__fsub_rn(near, whole)) < 0.4999f ? (int)whole : __float2int_rn(__fdiv_rn(v, scale));  // (inf, NaN: the division)
   return max(-127, min(127, c));
 }
 

@@ -28,47 +28,66 @@ struct Ctl {
   int status;                 // first device-detected error (NSML_ERR_*), 0 = ok
   unsigned int lo, hi;        // sampled bounds of the threshold key: probably lo <= T < hi
   unsigned int barrier;       // arrivals at the finalize kernel's grid barriers
-  unsigned int coarse;        // most sampled keys have zeros in their low 16 bits
-  unsigned int listed;        // entries of the threshold's bin appended to the bin list
+  unsigned int grain;         // the sampled keys (nearly all of them) are multiples of 1 << grain: 16, 13 or 0
+  unsigned int ticket;        // chunks of the list handed out
+  unsigned int fallback;      // a bin that was taken for a single key holds others
+  unsigned int done;          // chunks of the list that are finished, where that has to be known
+  unsigned int drawn[5], finished[5];  // general select: units of work of each phase
 };
 static_assert(sizeof(Ctl) <= 256, "control block must fit its 256-byte slot");
 
 // The window of keys the sample leaves open, cut into at most kMaxBins bins of 1 << shift keys.
 struct Window {
   unsigned int lo, hi, shift;  // keys lo .. hi-1; bin (key - lo) >> shift
+  unsigned int grain;          // the keys are (taken to be) multiples of 1 << grain
   bool few;                    // there are at most kFewBins bins
+
+  __device__ __forceinline__ bool single() const { return shift <= grain; }  // a bin holds one key ...
+  __device__ __forceinline__ unsigned int key_of(unsigned int bin) const {   // ... this one
+    return (lo + (bin << shift) + ((1u << grain) - 1u)) & ~((1u << grain) - 1u);
+  }
 };
 constexpr unsigned int kFewBins = 64;
-// TYPE: element type of the keys; the low 16 bits of a bfloat16 key are zero, so a bin need not be narrower than that
-// (and holds one key then).  The same goes for a float32 bucket that was widened from bfloat16, which the sample tells
-// (`coarse`); there a narrower bin only costs a refinement later.
+// TYPE: element type of the keys.  The low 16 bits of a bfloat16 key are zero, so a bin need not be narrower than that
+// and holds one key then; the same goes for float32 buckets widened from bfloat16 or binary16 (13 bits), which the
+// sample tells and the list stage verifies.
 template <int TYPE>
 __host__ __device__ constexpr unsigned int min_bin_shift() { return TYPE == NSML_F32 ? 0 : 16; }
 template <int TYPE>
 __device__ __forceinline__ Window make_window(const Ctl* ctl) {
   Window w;
   const unsigned int hi = ctl->hi;
-  w.lo = max(ctl->lo, 1u);  // zeros are never candidates of the list strategy
+  w.grain = TYPE == NSML_BF16 ? 16u : ctl->grain;
+  w.lo = ctl->lo;  // 0: the sample holds too few non-zero keys; everything is listed, zeros too
   w.hi = hi > w.lo ? hi : 0x80000000u;
   const unsigned int span = (w.hi - w.lo - 1) / kMaxBins;
-  w.shift = max(TYPE == NSML_BF16 || ctl->coarse ? 16u : 0u, span == 0 ? 0u : 32u - __clz(span));
+  w.shift = max(w.grain, span == 0 ? 0u : 32u - __clz(span));
   w.few = (w.hi - w.lo - 1) >> w.shift < kFewBins;
   return w;
 }
 
 constexpr int kSegElems = 512;            // granule of the index ranges that the dense select's blocks own
 constexpr int kTileBytes = 16384;         // bucket bytes per tile of the candidate list: what a block of the bucket pass takes
-constexpr int kMaxGroups = 1024;          // the bucket pass keeps a candidate count per group of tiles
+constexpr int kMaxGroups = 8192;          // the bucket pass keeps a candidate count per group of tiles (of one tile, up to 32M
+                                          // float32 or 64M bfloat16 elements)
 constexpr int kMaxFinalizeBlocks = 1024;  // upper bound on blocks of the finalize kernels
-constexpr unsigned int kBinCap = 1024;    // entries of the threshold's bin that can be settled one by one
+constexpr int kChunk = 2048;              // candidates a block of the list stage takes at a time
+
+// The keys inside the window are also kept by bin, up to this many per bin: four times what is to be expected where the
+// window is widest (kept fraction a quarter: 2 per cent of the bucket over at least 2048 bins).
+inline unsigned int bin_room_of(int64_t n) {
+  unsigned int room = 16;
+  while (room < 2048 && (int64_t)room * 25000 < n) room *= 2;
+  return room;
+}
 
 // elements per tile; TYPE: element type of the stream the tiles cut (a tile of a bucket with a residual holds
 // float32 sums)
 template <int TYPE>
 __host__ __device__ constexpr int tile_elems() { return kTileBytes / (TYPE == NSML_F32 ? 4 : 2); }
-// tiles per group, as a shift: 64, or more where the groups would be too many
+// tiles per group, as a shift
 inline unsigned int group_shift_of(unsigned long long tiles) {
-  unsigned int s = 6;
+  unsigned int s = 0;
   while (((tiles + (1ull << s) - 1) >> s) > (unsigned long long)kMaxGroups) ++s;
   return s;
 }
@@ -78,7 +97,9 @@ struct CompressLayout {  // byte offsets inside a compress workspace
   size_t group_count;   // u32[kMaxGroups]: candidates per group of tiles
   size_t zero_bytes;    // everything before this offset is cleared per call
   size_t block_counts;  // u64[kMaxFinalizeBlocks]: per-block counts exchanged at barriers
-  size_t bin_list;      // uint2[kBinCap]: (key, index) of the candidates in the threshold's bin
+  size_t bins;          // uint2[kMaxBins][bin_room_of(n)]: (key, index) of the candidates inside the window, by bin
+  size_t chunk_sum;     // u64[2][chunks]: survivors of a chunk, and up to it; cleared by the bucket pass
+  size_t block_fill;    // u32[chunks]: values delivered to a payload block of 1024; cleared by the bucket pass
   size_t tile_count;    // u32[tiles]: candidates per tile
   size_t cand_off;      // u16[n]: a candidate's offset inside its tile; tile t's candidates start at t * tile_elems
   size_t cand_val;      // u32[n]: float32 bit patterns (bfloat16 bucket: offset << 16 | bfloat16 bits, and no cand_off)
@@ -98,8 +119,11 @@ inline CompressLayout compress_layout(int64_t n) {
   L.group_count = L.hist + 4 * kMaxBins * sizeof(unsigned int);
   L.zero_bytes = L.group_count + kMaxGroups * sizeof(unsigned int);
   L.block_counts = L.zero_bytes;
-  L.bin_list = L.block_counts + kMaxFinalizeBlocks * 8;
-  L.tile_count = L.bin_list + kBinCap * 8;
+  L.bins = L.block_counts + kMaxFinalizeBlocks * 8;
+  L.chunk_sum = L.bins + (size_t)kMaxBins * bin_room_of(n) * 8;
+  const size_t chunks = npad / kChunk;
+  L.block_fill = L.chunk_sum + align_up(2 * chunks * 8, 256);
+  L.tile_count = L.block_fill + align_up(chunks * 4, 256);
   L.cand_off = L.tile_count + align_up(npad / tile_elems<NSML_F32>() * 4, 256);
   L.cand_val = L.cand_off + npad * 2;
   // The list strategy keeps less than kDenseRatioAny of the bucket; the dense strategy, which may keep all of it,

@@ -3,7 +3,7 @@
 // lower bound is dropped here, in one streaming read).
 //
 // The bucket is cut into tiles of kTileBytes.  A block takes a tile and appends
-// what it keeps (every key >= lo, lo >= 1) to the tile's own slots of the list,
+// what it keeps (every key >= lo) to the tile's own slots of the list,
 // [t * tile, t * tile + count), in index order, so nothing can overflow, nothing
 // is allocated and no block ever waits for another; tiles in increasing order
 // are in index order.  Keys inside the sampled window are counted in 4096 bins
@@ -44,6 +44,10 @@ struct TileList {  // where the bucket pass leaves what it keeps
   unsigned int* tile_count;
   unsigned int* group_count;
   unsigned int* window_hist;
+  uint2* bins;                // (key, index) by bin of the window; not where a bin holds one key
+  unsigned int bin_room;
+  unsigned long long* chunk_sum[2];
+  unsigned int* block_fill;
   unsigned int group_shift;
 };
 
@@ -66,7 +70,7 @@ struct KeepShared {
 // equal bins add once.
 template <int EPL, bool PACKED, class Bits>
 __device__ __forceinline__ void keep_tile(const TileList& out, unsigned long long tile, unsigned int first, const Window& win,
-                                          Ctl* ctl, KeepShared<PACKED>& sh, Bits&& bits_of) {
+                                          Ctl* ctl, KeepShared<PACKED>& sh, unsigned long long n, Bits&& bits_of) {
   constexpr unsigned int FULL = 0xFFFFFFFFu;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned int lt = (1u << lane) - 1u;
@@ -77,6 +81,10 @@ __device__ __forceinline__ void keep_tile(const TileList& out, unsigned long lon
     uint32_t bits[EPL];
     bits_of(r, bits);
     flags[r] = keep_flags<EPL>(bits, t);
+    if (win.lo == 0) {  // everything is kept: not what the bucket's ragged end is padded with
+      const unsigned long long i = tile * (unsigned long long)KeepShared<PACKED>::TILE + first + (r * 32 + lane) * EPL;
+      if (i + EPL > n) flags[r] &= i < n ? (1u << (n - i)) - 1u : 0u;
+    }
     mine += __popc(flags[r]);
   }
   const unsigned int warp_total = __reduce_add_sync(FULL, mine);
@@ -92,7 +100,17 @@ __device__ __forceinline__ void keep_tile(const TileList& out, unsigned long lon
   }
   if (threadIdx.x == 0) {
     out.tile_count[tile] = total;
-    if (total) atomicAdd(out.group_count + (tile >> out.group_shift), total);
+    if (total) {
+      if (out.group_shift == 0) out.group_count[tile] = total;
+      else atomicAdd(out.group_count + (tile >> out.group_shift), total);
+    }
+  }
+  constexpr int kChunksPerTile = KeepShared<PACKED>::TILE / kChunk;
+  if (threadIdx.x < kChunksPerTile) {  // clear the list stage's counters on the way
+    const unsigned long long c = tile * kChunksPerTile + threadIdx.x;
+    out.chunk_sum[0][c] = 0;
+    out.chunk_sum[1][c] = 0;
+    out.block_fill[c] = 0;
   }
   if (total == 0) return;
   if (warp_total != 0) {
@@ -147,25 +165,48 @@ __device__ __forceinline__ void keep_tile(const TileList& out, unsigned long lon
       if (!PACKED) *reinterpret_cast<uint2*>(out.off + base + i) = *reinterpret_cast<const uint2*>(sh.off + (PACKED ? 0 : i));
     }
     const uint32_t e4[4] = {v.x, v.y, v.z, v.w};
+    uint32_t key[4];
+    unsigned int bin[4], slot[4];
+    bool inside[4], nonfinite = false;
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      const uint32_t key = (PACKED ? e4[e] << 16 : e4[e]) & 0x7FFFFFFFu;
+      key[e] = (PACKED ? e4[e] << 16 : e4[e]) & 0x7FFFFFFFu;
       const bool live = i + e < total;
-      if (live && key >= kInfKey) set_status(&ctl->status, NSML_ERR_NONFINITE);
-      const bool inside = live && key < win.hi;  // (key >= lo)
-      const unsigned int bin = (key - win.lo) >> win.shift;
-      unsigned int add = inside ? 1u : 0u;
-      if (crowded) {
-        const unsigned int who = __ballot_sync(FULL, inside);
-        if (inside) {
-          const unsigned int same = __match_any_sync(who, bin);
-          add = (same & lt) == 0 ? (unsigned int)__popc(same) : 0u;
+      nonfinite |= live && key[e] >= kInfKey;
+      inside[e] = live && key[e] < win.hi;  // (key >= lo)
+      bin[e] = (key[e] - win.lo) >> win.shift;
+      slot[e] = 0;
+    }
+    if (nonfinite) set_status(&ctl->status, NSML_ERR_NONFINITE);
+    if (crowded) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const unsigned int who = __ballot_sync(FULL, inside[e]);
+        if (inside[e]) {
+          const unsigned int same = __match_any_sync(who, bin[e]);
+          const int leader = __ffs(same) - 1;
+          unsigned int base_slot = 0;
+          if (lane == leader) {
+            if (win.few) atomicAdd(&sh.few[bin[e]], (unsigned int)__popc(same));
+            else base_slot = atomicAdd(out.window_hist + bin[e], (unsigned int)__popc(same));
+          }
+          slot[e] = __shfl_sync(same, base_slot, leader) + __popc(same & lt);
         }
       }
-      if (add) {
-        if (win.few) atomicAdd(&sh.few[bin], add);
-        else atomicAdd(out.window_hist + bin, add);
-      }
+    } else if (win.few) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (inside[e]) atomicAdd(&sh.few[bin[e]], 1u);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e)  // (the four are in flight together)
+        if (inside[e]) slot[e] = atomicAdd(out.window_hist + bin[e], 1u);
+    }
+    if (!win.single()) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (inside[e] && slot[e] < out.bin_room)
+          out.bins[(size_t)bin[e] * out.bin_room + slot[e]] = make_uint2(key[e], (uint32_t)base + (PACKED ? e4[e] >> 16 : sh.off[PACKED ? 0 : i + e]));
     }
   }
   if (win.few) {
@@ -271,7 +312,7 @@ k_compact_bucket(BucketSrc<DTYPE> src, float* __restrict__ residual, unsigned lo
     }
   }
   const Window win = make_window<FEEDBACK ? NSML_F32 : DTYPE>(ctl);
-  keep_tile<EPL, !FEEDBACK && DTYPE == NSML_BF16>(out, tile, first, win, ctl, sh, [&](int r, uint32_t (&bits)[EPL]) {
+  keep_tile<EPL, !FEEDBACK && DTYPE == NSML_BF16>(out, tile, first, win, ctl, sh, n, [&](int r, uint32_t (&bits)[EPL]) {
     unpack16<FEEDBACK ? NSML_F32 : DTYPE, EPL>(q[r], bits);
     if (MASKED) {
       // this lane's EPL mask bits inside the round's ROUND / 32 words

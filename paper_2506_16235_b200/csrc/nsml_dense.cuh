@@ -30,18 +30,16 @@
 
 namespace nsml {
 
-// s_cache: CACHE values of shared memory; stage: 256 words per warp for the write phase (may be sh.hist);
-// `barriers`: grid barriers passed so far.
-template <int DTYPE, int THREADS, int CACHE, bool CLUSTER>
-__device__ __forceinline__ void dense_select(const BucketSrc<DTYPE>& src, const FinalizeParams& p, FinalizeShared<THREADS>& sh, uint32_t* s_cache,
-                                             uint32_t* stage, unsigned int barriers) {
+template <int DTYPE, int THREADS, int CACHE>
+__device__ __forceinline__ void dense_select(const BucketSrc<DTYPE>& src, const FinalizeParams& p, FinalizeShared<THREADS>& sh, uint32_t* s_cache) {
   static_assert(CACHE % 128 == 0, "a warp step (32 words) is cached as a whole or not at all");
+  unsigned int barriers = 0;
+  const unsigned int G = gridDim.x, blk = blockIdx.x;
   uint4* cache4 = reinterpret_cast<uint4*>(s_cache);
   constexpr int NW = THREADS / 32;
   constexpr unsigned int CW = CACHE / 4;  // cached words
   constexpr unsigned int FULL = 0xFFFFFFFFu;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const unsigned int G = gridDim.x, blk = blockIdx.x;
   const unsigned long long range_lo = ((unsigned long long)blk * p.nseg / G) * kSegElems;  // a multiple of 512
   const unsigned long long range_hi = min(((unsigned long long)(blk + 1) * p.nseg / G) * kSegElems, p.n);
   const unsigned int E = (unsigned int)(range_hi - range_lo);  // >= 1: the grid has at most nseg blocks
@@ -141,7 +139,7 @@ __device__ __forceinline__ void dense_select(const BucketSrc<DTYPE>& src, const 
     if (nonfinite) set_status(&p.ctl->status, NSML_ERR_NONFINITE);
   }
   flush_hist<kMaxBins>(sh, p.hist);
-  if (!grid_barrier<CLUSTER>(p.ctl, ++barriers * G, sh)) return;
+  if (!grid_barrier(p.ctl, ++barriers * G, sh)) return;
 
   // ---------------- phase 1: resolve digit 0, histogram of digit 1 ----------------
   // Digit 0 splits the entries into those above the threshold's bin (survivors whatever T turns out
@@ -210,7 +208,7 @@ __device__ __forceinline__ void dense_select(const BucketSrc<DTYPE>& src, const 
     if (threadIdx.x == 0 && block_zeros != 0) atomicAdd(&sh.hist[0], (unsigned int)block_zeros);
   }
   flush_hist<kMaxBins>(sh, p.hist + 1 * kMaxBins);
-  if (!grid_barrier<CLUSTER>(p.ctl, ++barriers * G, sh)) return;
+  if (!grid_barrier(p.ctl, ++barriers * G, sh)) return;
 
   // Calls f(q, key) for this lane's share of the warp's listed undecided entries.
   auto for_listed = [&](auto&& f) {
@@ -255,7 +253,7 @@ __device__ __forceinline__ void dense_select(const BucketSrc<DTYPE>& src, const 
     if (threadIdx.x == 0 && block_zeros != 0) atomicAdd(&sh.hist[0], (unsigned int)block_zeros);
   }
   flush_hist<128>(sh, p.hist + 2 * kMaxBins);
-  if (!grid_barrier<CLUSTER>(p.ctl, ++barriers * G, sh)) return;
+  if (!grid_barrier(p.ctl, ++barriers * G, sh)) return;
 
   // ---------------- phase 3: T and r; this warp's keys > T and == T, per slice ----------------
   resolve_digit<128>(p.hist + 2 * kMaxBins, rem, sh);
@@ -301,7 +299,7 @@ __device__ __forceinline__ void dense_select(const BucketSrc<DTYPE>& src, const 
   }
   unsigned long long* ac_counts = p.block_counts;
   if (threadIdx.x == 0) ac_counts[blk] = (block_a << 32) | block_c;
-  if (!grid_barrier<CLUSTER>(p.ctl, ++barriers * G, sh)) return;
+  if (!grid_barrier(p.ctl, ++barriers * G, sh)) return;
 
   // ---------------- phase 4: write the survivors in index order ----------------
   unsigned long long a_before = 0, c_before = 0, a_all = 0, c_all = 0;
@@ -323,7 +321,8 @@ __device__ __forceinline__ void dense_select(const BucketSrc<DTYPE>& src, const 
     return;
   }
   uint32_t* out_idx = reinterpret_cast<uint32_t*>(p.payload + p.P.idx_off);
-  uint32_t* stage_idx = stage + warp * 256;  // 128 indices, then 128 values, per warp
+  static_assert(kMaxBins >= NW * 256, "the staging areas of all warps fit the histogram");
+  uint32_t* stage_idx = sh.hist + warp * 256;  // 128 indices, then 128 values, per warp
   uint32_t* stage_val = stage_idx + 128;
 #pragma unroll
   for (int q = 0; q < 2; ++q) {
@@ -365,7 +364,7 @@ __device__ __forceinline__ void dense_select(const BucketSrc<DTYPE>& src, const 
       const unsigned int total = __shfl_sync(FULL, incl, 31);
       const unsigned int a_lane = (incl - mine) & 0xFFFFu, c_lane = (incl - mine) >> 16;  // of this step, in lower lanes
       // Survivors of this step go to consecutive payload positions.  They are first put in order into the
-      // warp's staging area (usually the histogram's shared memory, free in this phase), then written 32 at a time.
+      // warp's staging area (the histogram's shared memory, free in this phase), then written 32 at a time.
       const unsigned int c_room = r > c_here ? r - c_here : 0u;           // ties still to keep from here on
       const unsigned int ta = total & 0xFFFFu, tc = min(total >> 16, c_room);
       const unsigned int step_base = a_here + min(c_here, r);              // payload position of the step's first survivor
@@ -399,7 +398,7 @@ __device__ __forceinline__ void dense_select(const BucketSrc<DTYPE>& src, const 
   // ---------------- phase 5: the header; int8: quantise ----------------
   if (blk == 0 && threadIdx.x == 0) write_header(p);
   if (p.bits != NSML_BITS_INT8) return;  // float32 and fp16 values are in the payload already
-  if (!grid_barrier<CLUSTER>(p.ctl, ++barriers * G, sh)) return;
+  if (!grid_barrier(p.ctl, ++barriers * G, sh)) return;
   quantize_all(p, sh);
 }
 
@@ -408,8 +407,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS)  // at most 64 regist
 k_finalize_dense(BucketSrc<DTYPE> src, FinalizeParams p) {
   __shared__ FinalizeShared<THREADS> sh;
   extern __shared__ __align__(16) uint32_t s_cache[];
-  static_assert(kMaxBins >= THREADS / 32 * 256, "the staging areas of all warps fit the histogram");
-  dense_select<DTYPE, THREADS, CACHE, false>(src, p, sh, s_cache, sh.hist, 0);
+  dense_select<DTYPE, THREADS, CACHE>(src, p, sh, s_cache);
 }
 
 }  // namespace nsml

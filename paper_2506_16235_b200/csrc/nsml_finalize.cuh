@@ -29,10 +29,10 @@ struct FinalizeParams {
   Ctl* ctl;
   unsigned int* hist;                // [3][kMaxBins]
   unsigned long long* block_counts;  // [kMaxFinalizeBlocks]
-  uint2* bin_list;                   // [kBinCap]
   unsigned int tiles;
   TileList list;
   float* raw_val;
+  float* residual;                   // list strategy with local accumulation: holds gradient + residual; what the payload carries is taken out
   unsigned char* payload;
   PayloadLayout P;
 };
@@ -91,15 +91,9 @@ __device__ __forceinline__ unsigned int block_excl_scan(unsigned int v, unsigned
 }
 
 // All blocks arrive, then all leave.  `target` = barrier ordinal * gridDim.x.
-// CLUSTER: the grid is one thread-block cluster and the barrier is the hardware's (release / acquire at
-// cluster scope, which orders the blocks' global-memory traffic as well); it cannot time out.
 // SH: any shared-memory struct with an int member `ok`.  max_polls: polls after which the wait gives up.
-template <bool CLUSTER = false, class SH>
+template <class SH>
 __device__ __forceinline__ bool grid_barrier(Ctl* ctl, unsigned int target, SH& sh, int max_polls = kMaxPolls) {
-  if (CLUSTER) {
-    cooperative_groups::this_cluster().sync();
-    return true;
-  }
   __syncthreads();
   if (threadIdx.x == 0) {
     // Arrive with release, wait with acquire (both at device scope): what the block wrote before the
@@ -182,6 +176,11 @@ __device__ __forceinline__ void put_value(const FinalizeParams& p, unsigned long
   else if (p.bits == NSML_BITS_FP16) reinterpret_cast<uint16_t*>(p.payload + p.P.val_off)[pos] = encode_f16(__uint_as_float(bits));
   else p.raw_val[pos] = __uint_as_float(bits);
 }
+// What a receiver reconstructs of a float32 or fp16 value, taken out of it (one float32 subtraction).
+__device__ __forceinline__ float not_carried(const FinalizeParams& p, uint32_t bits) {
+  const float v = __uint_as_float(bits);
+  return __fsub_rn(v, p.bits == NSML_BITS_FP32 ? v : decode_f16(encode_f16(v)));
+}
 
 // int8: thread group `threadIdx.x >> 8` (256 threads) converts the block of 1024 survivors qb from raw_val
 // into codes and a max-abs scale; live = false: this group has no block this round.  Called by every thread
@@ -214,17 +213,17 @@ __device__ __forceinline__ void quantize_block(const FinalizeParams& p, Finalize
   m = sh.qmax[group * 8];
 #pragma unroll
   for (int w = 1; w < 8; ++w) m = fmaxf(m, sh.qmax[group * 8 + w]);
-  const float scale = __fdiv_rn(m, 127.0f);
+  const float scale = __fdiv_rn(m, 127.0f), inv = __fdiv_rn(1.0f, scale);
   if (live) {
     if (gtid == 0) reinterpret_cast<float*>(p.payload + p.P.scale_off)[qb] = scale;
     signed char* out = reinterpret_cast<signed char*>(p.payload + p.P.val_off);
     if (cnt == 4) {
       uint32_t w = 0;
 #pragma unroll
-      for (int e = 0; e < 4; ++e) w |= ((uint32_t)encode_i8(v[e], scale) & 0xFFu) << (8 * e);
+      for (int e = 0; e < 4; ++e) w |= ((uint32_t)encode_i8(v[e], scale, inv) & 0xFFu) << (8 * e);
       *reinterpret_cast<uint32_t*>(out + j0) = w;
     } else {
-      for (int e = 0; e < cnt; ++e) out[j0 + e] = (signed char)encode_i8(v[e], scale);
+      for (int e = 0; e < cnt; ++e) out[j0 + e] = (signed char)encode_i8(v[e], scale, inv);
     }
   }
 }

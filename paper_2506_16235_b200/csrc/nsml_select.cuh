@@ -4,10 +4,12 @@
 // The bucket is streamed exactly once, by the compaction pass, which needs a
 // key `lo` such that a little more than k keys are >= lo, and counts the keys
 // between lo and a second bound `hi` that a little fewer than k keys exceed.
-// k_sample reads one 32-byte sector (8 float32 or 16 bfloat16 keys) from each of
-// 8192 equal strata of the bucket and takes the two sample keys whose ranks lie
-// six standard deviations either side of the expected rank of the k-th largest,
-// rounded outwards to their top 15 bits.  The exact threshold is found
+// k_sample reads 16 bytes (4 float32 or 8 bfloat16 keys) from each of 16384 equal
+// strata of the bucket and takes the two sample keys whose ranks lie six standard
+// deviations either side of the expected rank of the k-th largest, rounded
+// outwards to their top 15 bits.  (The keys of a stratum lie side by side; where
+// neighbours are alike, as in the rows of a sparse embedding gradient, they count
+// for less than as many independent draws, in the extreme case for one.)  The exact threshold is found
 // afterwards (nsml_list.cuh), which also repairs the rare case of a misleading
 // sample, so the sample only decides how much work is done, never the result.
 //
@@ -27,7 +29,8 @@ namespace nsml {
 
 constexpr int kSampleThreads = 1024;
 constexpr int kSampleBlocks = 8;
-constexpr int kSamples = kSampleThreads * kSampleBlocks;  // 8192 strata
+constexpr int kSampleLoads = 2;  // strata per thread
+constexpr int kSamples = kSampleThreads * kSampleBlocks * kSampleLoads;  // 16384 strata
 
 __device__ __forceinline__ uint32_t mix32(uint32_t x) {
   x ^= x >> 16; x *= 0x7FEB352Du;
@@ -74,7 +77,7 @@ __device__ __forceinline__ void find_digit_from_top(const unsigned int (&own)[PE
 }
 
 template <int DTYPE>
-__host__ __device__ constexpr int sample_keys() { return DTYPE == NSML_F32 ? 8 : 16; }  // keys per stratum: a 32-byte sector
+__host__ __device__ constexpr int sample_keys() { return DTYPE == NSML_F32 ? 4 : 8; }  // keys per stratum: 16 bytes
 constexpr int kSampleBinBits = 15;
 constexpr int kSampleBins = 1 << kSampleBinBits;  // bins of the keys' top bits, 16-bit counters
 constexpr size_t kSampleSmem = kSampleBins * 2;
@@ -96,49 +99,59 @@ k_sample(BucketSrc<DTYPE> src, const float* __restrict__ addend, unsigned long l
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   for (int i = t; i < kSampleBins / 8; i += kSampleThreads) reinterpret_cast<uint4*>(s_bins)[i] = make_uint4(0u, 0u, 0u, 0u);
   pdl_wait();
-  pdl_launch_dependents();  // the bucket pass may start to load (only now: what the stream did before this kernel is complete)
 
-  const unsigned long long stratum = (unsigned long long)rank * kSampleThreads + t;
-  const unsigned long long begin = stratum * n / kSamples;
-  const unsigned long long end = (stratum + 1) * n / kSamples;  // > begin
-  unsigned long long pos = (begin + mix32((uint32_t)stratum * 0x9E3779B1u + 0x85EBCA6Bu) % (uint32_t)(end - begin)) & ~(unsigned long long)(KEYS - 1);
-  if (pos + KEYS > n) pos = (n - KEYS) & ~(unsigned long long)(KEYS - 1);  // (n >= KEYS)
-  uint32_t bits[KEYS / 4][4];
+  uint4 raw[kSampleLoads];
+  float add[kSampleLoads][KEYS];
+  uint32_t pruned[kSampleLoads];  // bit e: key e of the stratum is pruned
 #pragma unroll
-  for (int q = 0; q < KEYS / 4; ++q) {
-    const BucketSrc<DTYPE> bare{src.grad, addend != nullptr ? nullptr : src.mask};
-    bare.load_full4(pos + q * 4, bits[q]);
-  }
-  if (addend != nullptr) {
-    // with an addend (the residual of the local accumulation) the bucket that is selected from is the sum
+  for (int s = 0; s < kSampleLoads; ++s) {
+    const unsigned long long stratum = ((unsigned long long)s * kSampleBlocks + rank) * kSampleThreads + t;
+    const unsigned long long begin = stratum * n / kSamples;
+    const unsigned long long end = (stratum + 1) * n / kSamples;  // > begin
+    unsigned long long pos = (begin + mix32((uint32_t)stratum * 0x9E3779B1u + 0x85EBCA6Bu) % (uint32_t)(end - begin)) & ~(unsigned long long)(KEYS - 1);
+    if (pos + KEYS > n) pos = (n - KEYS) & ~(unsigned long long)(KEYS - 1);  // (n >= KEYS)
+    raw[s] = __ldcs(reinterpret_cast<const uint4*>(static_cast<const unsigned char*>(src.grad) + pos * (DTYPE == NSML_F32 ? 4 : 2)));
 #pragma unroll
-    for (int q = 0; q < KEYS / 4; ++q) {
-      const float4 a = *reinterpret_cast<const float4*>(addend + pos + q * 4);
-      const float add[4] = {a.x, a.y, a.z, a.w};
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        bits[q][e] = __float_as_uint(__fadd_rn(__uint_as_float(bits[q][e]), add[e]));
-        if (src.pruned(pos + q * 4 + e)) bits[q][e] = 0;
-      }
+    for (int e = 0; e < KEYS; e += 4) {
+      const float4 a = addend != nullptr ? *reinterpret_cast<const float4*>(addend + pos + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+      add[s][e] = a.x; add[s][e + 1] = a.y; add[s][e + 2] = a.z; add[s][e + 3] = a.w;
     }
+    pruned[s] = src.mask != nullptr ? __ldg(src.mask + (pos >> 5)) >> (unsigned)(pos & 31) : 0u;
   }
   // keep_status: an error an earlier step of the same call left in the status word stays visible
-  for (unsigned int i = rank * kSampleThreads + t; i < zero_vec16; i += kSamples)
+  for (unsigned int i = rank * kSampleThreads + t; i < zero_vec16; i += kSampleBlocks * kSampleThreads)
     zero_base[i] = make_uint4((i == 0 && keep_status) ? (unsigned int)ctl->status : 0u, 0, 0, 0);
   __syncthreads();
-  unsigned int fine_keys = 0;  // keys with any of their low 16 bits set
+  unsigned int low_bits = 0;
 #pragma unroll
-  for (int q = 0; q < KEYS / 4; ++q)
+  for (int s = 0; s < kSampleLoads; ++s) {
+    uint32_t bits[KEYS];
+    if (DTYPE == NSML_F32) {
+      bits[0] = raw[s].x; bits[1] = raw[s].y; bits[2] = raw[s].z; bits[3] = raw[s].w;
+    } else {
+      bits[0] = raw[s].x << 16; bits[1] = raw[s].x & 0xFFFF0000u;
+      bits[2] = raw[s].y << 16; bits[3] = raw[s].y & 0xFFFF0000u;
+      bits[4 % KEYS] = raw[s].z << 16; bits[5 % KEYS] = raw[s].z & 0xFFFF0000u;
+      bits[6 % KEYS] = raw[s].w << 16; bits[7 % KEYS] = raw[s].w & 0xFFFF0000u;
+    }
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const unsigned int bin = (bits[q][e] & 0x7FFFFFFFu) >> (31 - kSampleBinBits);
-      fine_keys += (bits[q][e] & 0xFFFFu) != 0;
+    for (int e = 0; e < KEYS; ++e) {
+      // with an addend (the residual of the local accumulation) the bucket that is selected from is the sum
+      if (addend != nullptr) bits[e] = __float_as_uint(__fadd_rn(__uint_as_float(bits[e]), add[s][e]));
+      if ((pruned[s] >> e) & 1u) bits[e] = 0;
+      low_bits |= bits[e] & 0xFFFFu;
+      const unsigned int bin = (bits[e] & 0x7FFFFFFFu) >> (31 - kSampleBinBits);
       if (bin != 0) atomicAdd(&s_bins[bin >> 1], 1u << (16 * (bin & 1)));  // (a block has at most 16384 keys: no overflow)
     }
-  const int fine_threads = DTYPE == NSML_F32 ? __syncthreads_count(fine_keys != 0) : 0;
+  }
+  // The bucket pass may start to load: only now, when what the stream did before this kernel is complete, and behind
+  // this kernel's own reads.
+  pdl_launch_dependents();
+  // (a float32 key has its low 13 bits zero once in 8192; a few odd keys do not matter here)
+  const int below16 = DTYPE == NSML_F32 && addend == nullptr ? __syncthreads_count(low_bits != 0) : kSampleThreads;
+  const int below13 = DTYPE == NSML_F32 && addend == nullptr ? __syncthreads_count((low_bits & 0x1FFFu) != 0) : kSampleThreads;
   cluster.sync();  // every block's counts are complete, the control region is cleared
-  // (a float32 key has its low 16 bits zero once in 65536)
-  if (rank == 0 && t == 0) ctl->coarse = fine_threads < kSampleThreads / 16;
+  if (rank == 0 && t == 0) ctl->grain = below16 < kSampleThreads / 16 ? 16 : below13 < kSampleThreads / 16 ? 13 : 0;
 
   // this block's slice of the bins, four per thread, summed over the blocks
   constexpr int kSlice = kSampleBins / kSampleBlocks;

@@ -19,15 +19,15 @@ def gauss(n, seed, spread=2.0):
     return (rng.standard_normal(n) * 10.0 ** rng.uniform(-4.0, -4.0 + spread, n)).astype(np.float32)
 
 
-def sampled_sectors(n, keys):
-    """All elements of the sectors the sampler reads (`keys` elements, aligned)."""
-    pos = sampled_positions(n) & ~np.int64(keys - 1)
+def sampled_elements(n, keys):
+    """All elements the sampler reads: `keys` neighbours (aligned) from each of 16384 strata."""
+    pos = sampled_positions(n, 16384) & ~np.int64(keys - 1)
     pos = np.where(pos + keys > n, (n - keys) & ~np.int64(keys - 1), pos)
     return np.unique((pos[:, None] + np.arange(keys)).reshape(-1))
 
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
-@pytest.mark.parametrize("n", [8 * 8192 - 1, 8 * 8192, 8 * 8192 + 1, 17 * 4096 + 513, 64 * 4096 + 1])
+@pytest.mark.parametrize("n", [97 * 4096 - 1, 97 * 4096, 97 * 4096 + 1, 113 * 4096 + 513, 128 * 4096 + 1])
 def test_tile_and_group_edges(n, dtype):
     g = gauss(n, n)
     g[-2:] = [3.0, -4.0]
@@ -68,9 +68,9 @@ def test_many_close_keys_in_the_threshold_bin():
 def test_misleading_samples(dtype):
     n = 1 << 20
     rng = np.random.default_rng(3)
-    keys = 8 if dtype == "f32" else 16
+    keys = 4 if dtype == "f32" else 8
     conv = (lambda x: x) if dtype == "f32" else synth.f32_to_bf16_bits
-    at = sampled_sectors(n, keys)
+    at = sampled_elements(n, keys)
     low = gauss(n, 1)
     low[at] = 0.0                     # the sample sees only zeros: everything non-zero is listed
     high = gauss(n, 2)
@@ -101,3 +101,41 @@ def test_list_longer_than_the_blocks_shared_memory(dtype):
 def test_all_equal_large_bucket():
     g = np.full(2_000_001, 0.37, dtype=np.float32)
     check_compress(g, 0.05, 8)
+
+
+@pytest.mark.parametrize("codes", [127, 3])
+def test_quantised_gradient(codes):
+    # few distinct magnitudes with full mantissas: the threshold's bin is one key with a great many ties
+    n = 2_500_001
+    rng = np.random.default_rng(codes)
+    g = (np.rint(rng.standard_normal(n) * codes / 3).astype(np.float32) * np.float32(0.0123457))
+    for ratio in (0.02, 0.2):
+        check_compress(g, ratio, 8)
+
+
+def test_equal_keys_beside_a_few_others_in_the_threshold_bin():
+    # the bin overflows with one key, but holds others: found out while the list is read, and done over
+    n, ratio = 1_000_003, 0.05
+    rng = np.random.default_rng(11)
+    g = (rng.standard_normal(n) * 1e-3).astype(np.float32)
+    k = nsml.nsml_k_of(n, ratio)
+    order = rng.permutation(n)
+    g[order[:k - 2000]] = (2.0 + rng.random(k - 2000)).astype(np.float32)
+    g[order[k - 2000:k + 3000]] = np.float32(0.712345)
+    late = np.sort(order[k - 2000:k + 3000])[-3:]
+    g[late] = np.nextafter(np.float32(0.712345), np.float32(1))
+    check_compress(g, ratio, 8)
+
+
+def test_feedback_when_ties_fill_the_threshold_bin():
+    n, ratio = 600_011, 0.05
+    rng = np.random.default_rng(12)
+    g = (np.rint(rng.standard_normal(n) * 2).astype(np.float32) * np.float32(0.0123457))
+    from oracle.adaptive import error_feedback_step
+    residual = torch.zeros(n, device="cuda")
+    want = np.zeros(n, dtype=np.float32)
+    for bits in (8, 16, 32):
+        payload = nsml.nsml_compress_feedback(torch.from_numpy(g).cuda(), residual, ratio, bits)
+        ref, want = error_feedback_step(g, want, ratio, bits)
+        assert_payload_equal(payload, ref)
+        assert np.array_equal(residual.cpu().numpy().view(np.uint32), want.view(np.uint32))
