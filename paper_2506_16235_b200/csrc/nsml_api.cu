@@ -15,19 +15,20 @@
 #include "nsml_dense.cuh"
 #include "nsml_list.cuh"
 #include "nsml_select.cuh"
+#include "nsml_small.cuh"
 
 namespace nsml {
 
 enum KernelId {
   K_SAMPLE = 0, K_COMPACT_BUCKET, K_EMIT, K_PARTITION, K_MERGE, K_CLEAR, K_FINALIZE_DENSE,
-  K_SUMSQ, K_FEEDBACK_ADD, K_FEEDBACK_SUBTRACT, K_PRUNE_HIST, K_PRUNE_TIES, K_PRUNE_WRITE, K_PRUNE_WRITE_RANKED, K_PRUNE_SAMPLE, K_PRUNE_COUNT, K_PRUNE_SETTLE, K_PRUNE_MARK, K_PRUNE_FIX, K_COUNT
+  K_SUMSQ, K_FEEDBACK_ADD, K_FEEDBACK_SUBTRACT, K_PRUNE_HIST, K_PRUNE_TIES, K_PRUNE_WRITE, K_PRUNE_WRITE_RANKED, K_PRUNE_SAMPLE, K_PRUNE_COUNT, K_PRUNE_SETTLE, K_PRUNE_MARK, K_PRUNE_FIX, K_SELECT_SMALL, K_COUNT
 };
 
 static const char* const kKernelNames[K_COUNT] = {"k_sample", "k_compact_bucket", "k_emit", "k_partition", "k_merge",
                                                   "k_clear", "k_finalize_dense", "k_sumsq", "k_feedback_add",
                                                   "k_feedback_subtract", "k_prune_hist", "k_prune_ties", "k_prune_write",
                                                   "k_prune_write_ranked", "k_prune_sample", "k_prune_count",
-                                                  "k_prune_settle", "k_prune_mark", "k_prune_fix"};
+                                                  "k_prune_settle", "k_prune_mark", "k_prune_fix", "k_select_small"};
 
 static std::atomic<int64_t> g_launches{0};
 
@@ -110,6 +111,10 @@ static int device_info(const DeviceInfo** out) {
     prepare(k_emit<NSML_BF16, kEmitPer>, kEmitThreads, sizeof(EmitShared), &list_fits);
     prepare(k_emit<NSML_F32, 2 * kEmitPer>, kEmitThreads, sizeof(EmitShared), &list_fits);
     prepare(k_emit<NSML_BF16, 2 * kEmitPer>, kEmitThreads, sizeof(EmitShared), &list_fits);
+    prepare(k_select_small<NSML_F32, 1>, kSmallThreads, kSmallOneBlock * 4, &list_fits);
+    prepare(k_select_small<NSML_BF16, 1>, kSmallThreads, kSmallOneBlock * 4, &list_fits);
+    prepare(k_select_small<NSML_F32, kSmallBlocks>, kSmallThreads, kSmallPerBlock * 4, &list_fits);
+    prepare(k_select_small<NSML_BF16, kSmallBlocks>, kSmallThreads, kSmallPerBlock * 4, &list_fits);
     prepare(k_sample<NSML_F32>, kSampleThreads, kSampleSmem, &list_fits);
     prepare(k_sample<NSML_BF16>, kSampleThreads, kSampleSmem, &list_fits);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.merge, k_merge<kDenseTileLarge>, kMergeThreads, 0);
@@ -245,6 +250,9 @@ static bool use_dense(int64_t n, int64_t k) {
   return p_keep >= kDenseRatioAny || sample_plan(n, k, NSML_F32).rank_lo == 0;
 }
 
+// Small mode: the whole bucket is held in the shared memory of one block or cluster.
+static bool use_small(int64_t n) { return n <= kSmallMaxN; }
+
 // DTYPE: element type of `grad` (what the sample and the bucket pass read).  FDTYPE: element type of the
 // bucket the later stages re-read; with a residual (local accumulation fused into the bucket pass, list
 // strategy only) that bucket is the residual buffer, float32, which then holds gradient + residual.
@@ -282,6 +290,17 @@ static int launch_compress(const void* grad, float* residual, const uint32_t* ma
   fp.payload = payload;
   fp.P = P;
   cudaError_t le;
+  if (use_small(n)) {
+    fp.raw_val = reinterpret_cast<float*>(ws + dense_raw_val(L));
+    LaunchScope scope(K_SELECT_SMALL, st);
+    const bool one = n <= (int64_t)kSmallOneBlock;
+    const unsigned int blocks = one ? 1 : kSmallBlocks;
+    const unsigned int per_block = (unsigned int)align_up(((size_t)n + blocks - 1) / blocks, 128);
+    auto kernel = one ? k_select_small<DTYPE, 1> : k_select_small<DTYPE, kSmallBlocks>;
+    le = launch_prio(kernel, dim3(blocks), dim3(kSmallThreads), (size_t)per_block * 4, st, false, one ? 0 : kSmallBlocks, true, true, src, fp,
+                     per_block, keep_status ? 1 : 0);
+    return le == cudaSuccess ? NSML_OK : NSML_ERR_CUDA;
+  }
   if (use_dense(n, k)) {
     fp.raw_val = reinterpret_cast<float*>(ws + dense_raw_val(L));
     const bool small_shape = (unsigned long long)n <= (unsigned long long)dev.sms * kFinSmallCache;
@@ -577,7 +596,7 @@ static int feedback_impl(const void* grad, float* residual, int64_t n, int grad_
   const DeviceInfo* dev = nullptr;
   int rc = device_info(&dev);
   if (rc != NSML_OK) return rc;
-  if (use_dense(n, k)) {
+  if (use_dense(n, k) && !use_small(n)) {
     // dense strategy (no bucket pass to fuse the add into): residual <- grad + residual first, then the select
     // over the residual buffer
     const unsigned int grid = stream_grid(n, *dev, dev->feedback_add < 8 ? dev->feedback_add : 8, 1u << 16);
@@ -603,7 +622,7 @@ static int feedback_impl(const void* grad, float* residual, int64_t n, int grad_
       rc = launch_compress<NSML_BF16, NSML_F32>(grad, residual, prune_mask, n, k, bits, ws, pl, L, P, *dev, st);
   }
   if (rc != NSML_OK) return rc;
-  if (use_dense(n, k)) {  // (the list stage takes what the payload carries out of the residual itself)
+  if (use_dense(n, k) && !use_small(n)) {  // (the other strategies take what the payload carries out of the residual themselves)
     LaunchScope scope(K_FEEDBACK_SUBTRACT, st);
     const unsigned int sgrid = grid_for((unsigned long long)k, kCta, dev->sms * 8);
     k_feedback_subtract<<<sgrid, kCta, 0, st>>>(static_cast<const unsigned char*>(payload), residual,
