@@ -291,7 +291,6 @@ static int launch_compress(const void* grad, float* residual, const uint32_t* ma
   fp.P = P;
   cudaError_t le;
   if (use_small(n)) {
-    fp.raw_val = reinterpret_cast<float*>(ws + dense_raw_val(L));
     LaunchScope scope(K_SELECT_SMALL, st);
     const bool one = n <= (int64_t)kSmallOneBlock;
     const unsigned int blocks = one ? 1 : kSmallBlocks;
@@ -302,7 +301,6 @@ static int launch_compress(const void* grad, float* residual, const uint32_t* ma
     return le == cudaSuccess ? NSML_OK : NSML_ERR_CUDA;
   }
   if (use_dense(n, k)) {
-    fp.raw_val = reinterpret_cast<float*>(ws + dense_raw_val(L));
     const bool small_shape = (unsigned long long)n <= (unsigned long long)dev.sms * kFinSmallCache;
     unsigned long long cap = (unsigned long long)dev.sms * (small_shape || dev.dense_large < 2 ? 1 : 2);
     if (cap > (unsigned long long)kMaxFinalizeBlocks) cap = kMaxFinalizeBlocks;

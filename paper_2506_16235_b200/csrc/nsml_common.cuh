@@ -103,7 +103,7 @@ struct CompressLayout {  // byte offsets inside a compress workspace
   size_t tile_count;    // u32[tiles]: candidates per tile
   size_t cand_off;      // u16[n]: a candidate's offset inside its tile; tile t's candidates start at t * tile_elems
   size_t cand_val;      // u32[n]: float32 bit patterns (bfloat16 bucket: offset << 16 | bfloat16 bits, and no cand_off)
-  size_t raw_val;       // f32[k]: survivor values before int8 quantisation
+  size_t raw_val;       // f32[n]: survivor values before int8 quantisation
   size_t total;
 };
 
@@ -126,13 +126,10 @@ inline CompressLayout compress_layout(int64_t n) {
   L.tile_count = L.block_fill + align_up(chunks * 4, 256);
   L.cand_off = L.tile_count + align_up(npad / tile_elems<NSML_F32>() * 4, 256);
   L.cand_val = L.cand_off + npad * 2;
-  // The list strategy keeps less than kDenseRatioAny of the bucket; the dense strategy, which may keep all of it,
-  // has no candidate list, so its survivors' values start where the list would.
   L.raw_val = L.cand_val + npad * 4;
-  L.total = L.raw_val + align_up((size_t)((double)n * kDenseRatioAny) * 4 + 4, 256);
+  L.total = L.raw_val + npad * 4;
   return L;
 }
-inline size_t dense_raw_val(const CompressLayout& L) { return L.cand_off; }  // npad * 6 bytes: room for n values
 
 struct PayloadLayout {
   int64_t k;
