@@ -15,6 +15,7 @@ if the library has not been built.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 from typing import List, Optional, Sequence
 
@@ -216,6 +217,7 @@ def nsml_compress_strategy(n: int, ratio: float) -> int:
     return rc
 
 
+@functools.lru_cache(maxsize=1024)
 def nsml_payload_bytes(n: int, ratio: float, bits: int) -> int:
     return int(lib.nsml_payload_bytes(int(n), float(ratio), int(bits)))
 
@@ -231,16 +233,29 @@ def nsml_accumulate_workspace_bytes(n: int, W: int) -> int:
 # --------------------------------------------------------------------------
 # device operations
 # --------------------------------------------------------------------------
-def _torch():
-    import torch
+_torch_module = None
+_raw_stream = None  # () -> the current stream as an integer
 
-    return torch
+
+def _torch():
+    global _torch_module, _raw_stream
+    if _torch_module is None:
+        import torch
+
+        # torch.cuda.current_stream() builds a Stream object on every call (3 us, a quarter of a small call's host time)
+        get, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+        if get is not None and device is not None:
+            _raw_stream = lambda: get(device())  # noqa: E731
+        else:
+            _raw_stream = lambda: int(torch.cuda.current_stream().cuda_stream)  # noqa: E731
+        _torch_module = torch
+    return _torch_module
 
 
 def _stream_ptr(stream) -> int:
-    torch = _torch()
     if stream is None:
-        stream = torch.cuda.current_stream()
+        _torch()
+        return _raw_stream()
     return int(stream.cuda_stream)
 
 
@@ -251,6 +266,16 @@ def _grad_dtype(t) -> int:
     if t.dtype == torch.bfloat16:
         return NSML_BF16
     raise TypeError("gradient bucket must be float32 or bfloat16")
+
+
+def _front(payload, need: int):
+    """The first `need` bytes of a payload buffer (the buffer itself if that is all of it)."""
+    return payload if payload.numel() == need and payload.dim() == 1 else payload[:need]
+
+
+@functools.lru_cache(maxsize=None)
+def _array_type(element, count: int):
+    return element * count
 
 
 def alloc_bytes(nbytes: int, device):
@@ -289,7 +314,7 @@ def nsml_compress(grad, ratio: float, bits: int = NSML_BITS_INT8, prune_mask=Non
                            payload.data_ptr(), payload.numel(), workspace.data_ptr(), workspace.numel(),
                            _stream_ptr(stream))
     _check(rc, "nsml_compress")
-    return payload[:need]
+    return _front(payload, need)
 
 
 def nsml_decompress_accumulate(payloads: Sequence, dense, zero_first: bool = True, workspace=None, stream=None,
@@ -306,9 +331,9 @@ def nsml_decompress_accumulate(payloads: Sequence, dense, zero_first: bool = Tru
     n = dense.numel()
     if workspace is None:
         workspace = alloc_bytes(nsml_accumulate_workspace_bytes(n, max(1, min(W, NSML_MAX_WORKERS))), dense.device)
-    ptrs = (ctypes.c_void_p * max(W, 1))(*[p.data_ptr() for p in payloads])
+    ptrs = _array_type(ctypes.c_void_p, max(W, 1))(*[p.data_ptr() for p in payloads])
     if sized:
-        sizes = (ctypes.c_size_t * max(W, 1))(*[p.numel() * p.element_size() for p in payloads])
+        sizes = _array_type(ctypes.c_size_t, max(W, 1))(*[p.numel() * p.element_size() for p in payloads])
         rc = lib.nsml_decompress_accumulate_sized(ptrs, sizes, W, dense.data_ptr(), n, 1 if zero_first else 0,
                                                   workspace.data_ptr(), workspace.numel(), _stream_ptr(stream))
     else:
@@ -330,7 +355,7 @@ def nsml_decompress_accumulate_static(payloads: Sequence, dense, zero_first: boo
     calls on one device must not overlap.  With want_status the call
     synchronises the stream and returns the device-detected status."""
     W = len(payloads)
-    ptrs = (ctypes.c_void_p * max(W, 1))(*[p.data_ptr() for p in payloads])
+    ptrs = _array_type(ctypes.c_void_p, max(W, 1))(*[p.data_ptr() for p in payloads])
     status = ctypes.c_int(0)
     rc = lib.nsml_decompress_accumulate_static(ptrs, W, dense.data_ptr(), dense.numel(), 1 if zero_first else 0,
                                                _stream_ptr(stream), ctypes.byref(status) if want_status else None)
@@ -410,7 +435,7 @@ def nsml_compress_feedback(grad, residual, ratio: float, bits: int = NSML_BITS_I
                                     None if prune_mask is None else prune_mask.data_ptr(), payload.data_ptr(),
                                     payload.numel(), workspace.data_ptr(), workspace.numel(), _stream_ptr(stream))
     _check(rc, "nsml_compress_feedback")
-    return payload[:need]
+    return _front(payload, need)
 
 
 def nsml_compress_adaptive(grad, ratio: float, tr_q: float, tr_d: float, plain_bits: int = NSML_BITS_FP32,
@@ -437,7 +462,7 @@ def nsml_compress_adaptive(grad, ratio: float, tr_q: float, tr_d: float, plain_b
                                     _stream_ptr(stream), ctypes.byref(r), ctypes.byref(b), ctypes.byref(l2))
     _check(rc, "nsml_compress_adaptive")
     need = nsml_payload_bytes(n, r.value, b.value)
-    return payload[:need], r.value, b.value, (l2.value if l2.value >= 0.0 else None), prune_mask
+    return _front(payload, need), r.value, b.value, (l2.value if l2.value >= 0.0 else None), prune_mask
 
 
 def nsml_last_status(workspace, stream=None) -> int:
@@ -465,7 +490,7 @@ def nsml_decompress_accumulate_host(payloads_host: Sequence, dense_host, zero_fi
                                     stream=None):
     W = len(payloads_host)
     ptrs = (ctypes.c_void_p * max(W, 1))(*[p.data_ptr() for p in payloads_host])
-    sizes = (ctypes.c_size_t * max(W, 1))(*[p.numel() * p.element_size() for p in payloads_host])
+    sizes = _array_type(ctypes.c_size_t, max(W, 1))(*[p.numel() * p.element_size() for p in payloads_host])
     rc = lib.nsml_decompress_accumulate_host(ptrs, sizes, W, dense_host.data_ptr(), dense_host.numel(),
                                              1 if zero_first else 0, device_scratch.data_ptr(),
                                              device_scratch.numel(), _stream_ptr(stream))
