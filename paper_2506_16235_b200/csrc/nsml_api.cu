@@ -21,14 +21,12 @@ namespace nsml {
 
 enum KernelId {
   K_SAMPLE = 0, K_COMPACT_BUCKET, K_EMIT, K_PARTITION, K_MERGE, K_CLEAR, K_FINALIZE_DENSE,
-  K_SUMSQ, K_FEEDBACK_ADD, K_FEEDBACK_SUBTRACT, K_PRUNE_HIST, K_PRUNE_TIES, K_PRUNE_WRITE, K_PRUNE_WRITE_RANKED, K_PRUNE_SAMPLE, K_PRUNE_COUNT, K_PRUNE_SETTLE, K_PRUNE_MARK, K_PRUNE_FIX, K_SELECT_SMALL, K_COUNT
+  K_SUMSQ, K_FEEDBACK_ADD, K_FEEDBACK_SUBTRACT, K_PRUNE_PASS, K_PRUNE_FINISH, K_SELECT_SMALL, K_COUNT
 };
 
 static const char* const kKernelNames[K_COUNT] = {"k_sample", "k_compact_bucket", "k_emit", "k_partition", "k_merge",
                                                   "k_clear", "k_finalize_dense", "k_sumsq", "k_feedback_add",
-                                                  "k_feedback_subtract", "k_prune_hist", "k_prune_ties", "k_prune_write",
-                                                  "k_prune_write_ranked", "k_prune_sample", "k_prune_count",
-                                                  "k_prune_settle", "k_prune_mark", "k_prune_fix", "k_select_small"};
+                                                  "k_feedback_subtract", "k_prune_pass", "k_prune_finish", "k_select_small"};
 
 static std::atomic<int64_t> g_launches{0};
 
@@ -83,7 +81,7 @@ struct DeviceInfo {
   bool ready = false;
   int sms = 0;
   int dense_small = 0, dense_large = 0, merge = 0;  // resident blocks per SM
-  int sumsq = 0, feedback_add = 0, prune_hist = 0, prune_write = 0, prune_write_ranked = 0;  // the same, streaming kernels
+  int sumsq = 0, feedback_add = 0;  // the same, streaming kernels
 };
 static DeviceInfo g_dev[64];
 static std::mutex g_dev_mutex;
@@ -129,13 +127,7 @@ static int device_info(const DeviceInfo** out) {
     resident(k_sumsq<NSML_BF16>, &d.sumsq);
     resident(k_feedback_add<NSML_F32>, &d.feedback_add);
     resident(k_feedback_add<NSML_BF16>, &d.feedback_add);
-    resident(k_prune_hist<0>, &d.prune_hist);
-    resident(k_prune_hist<1>, &d.prune_hist);
-    resident(k_prune_hist<2>, &d.prune_hist);
-    resident(k_prune_ties, &d.prune_hist);
-    resident(k_prune_write, &d.prune_write);
-    resident(k_prune_write_ranked, &d.prune_write_ranked);
-    if (e == cudaSuccess && (d.sumsq < 1 || d.feedback_add < 1 || d.prune_hist < 1 || d.prune_write < 1 || d.prune_write_ranked < 1)) e = cudaErrorUnknown;
+    if (e == cudaSuccess && (d.sumsq < 1 || d.feedback_add < 1)) e = cudaErrorUnknown;
     int coop = 0;
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
     if (e != cudaSuccess || d.dense_small < 1 || d.dense_large < 1 || list_fits < 1 || d.merge < 1 || !coop) {
@@ -232,8 +224,7 @@ static SamplePlan sample_plan(int64_t n, int64_t k, int grad_dtype) {
   const double keys = (double)kSamples * (grad_dtype == NSML_F32 ? sample_keys<NSML_F32>() : sample_keys<NSML_BF16>());
   const double p = (double)k / (double)n, mean = keys * p, six = 6.0 * std::sqrt(keys * p * (1.0 - p));
   const double lo = std::ceil(mean + six) + 1.0, hi = std::floor(mean - six);
-  if (lo >= keys) return s;
-  s.rank_lo = (unsigned int)lo;
+  if (lo < keys) s.rank_lo = (unsigned int)lo;
   // (the largest sampled key, with about n / keys elements above it, where that is safely fewer than k)
   s.rank_hi = hi >= 1.0 ? (unsigned int)hi : 8.0 * (double)n / keys < (double)k ? 1u : 0u;
   s.expected = (double)n * (mean + six) / keys * 1.04 + 64.0;  // (the bound is rounded down to 15 key bits: a few per cent more)
@@ -496,84 +487,39 @@ static int prune_impl(const float* weights, int64_t n, double ratio, uint32_t* m
   int rc = device_info(&dev);
   if (rc != NSML_OK) return rc;
   unsigned char* ws = static_cast<unsigned char*>(workspace);
-  if (cudaMemsetAsync(ws, 0, L.tie_list, st) != cudaSuccess) return NSML_ERR_CUDA;  // status, ctl, histograms
   if (m == 0) {  // ratio 1: nothing is pruned
+    if (cudaMemsetAsync(ws, 0, 256, st) != cudaSuccess) return NSML_ERR_CUDA;
     if (cudaMemsetAsync(mask, 0, (size_t)((n + 31) / 32) * 4, st) != cudaSuccess) return NSML_ERR_CUDA;
     return NSML_OK;
   }
-  PruneCtl* ctl = reinterpret_cast<PruneCtl*>(ws);
-  unsigned int* hist = reinterpret_cast<unsigned int*>(ws + L.hist);
-  unsigned int* tile_ties = reinterpret_cast<unsigned int*>(ws + L.tile_ties);
-  uint2* tie_list = reinterpret_cast<uint2*>(ws + L.tie_list);
+  Ctl* ctl = reinterpret_cast<Ctl*>(ws);
+  uint2* list = reinterpret_cast<uint2*>(ws + L.list);
   const BucketSrc<NSML_F32> src{weights, nullptr};
-  const unsigned int grid = stream_grid(n, *dev, dev->prune_hist < 8 ? dev->prune_hist : 8, 1u << 16);
-  const unsigned int wgrid = stream_grid(n, *dev, dev->prune_write < 8 ? dev->prune_write : 8, 1u << 16);
-  const unsigned long long un = (unsigned long long)n;
-  bool two_pass = false;
-  // Two passes where a sample can bracket the threshold: ranks (from the top, among the complemented keys of
-  // kPruneSamples weights) six standard deviations either side of the expected rank of the m-th largest.
-  if (n >= 2 * (int64_t)kPruneSamples) {
-    const double p = (double)m / (double)n, mean = kPruneSamples * p, six = 6.0 * std::sqrt(kPruneSamples * p * (1.0 - p));
-    const double r_lo = std::ceil(mean + six) + 1.0, r_hi = std::floor(mean - six);
-    if (r_lo < (double)kPruneSamples && r_hi >= 1.0) {
-      two_pass = true;
-      unsigned int* fine = reinterpret_cast<unsigned int*>(ws + L.fine);
-      {
-        LaunchScope scope(K_PRUNE_SAMPLE, st);
-        launch_prio(k_prune_sample, dim3(1), dim3(1024), 0, st, false, 0, true, false, src, un, (unsigned int)r_lo, (unsigned int)r_hi, ctl);
-      }
-      {
-        LaunchScope scope(K_PRUNE_COUNT, st);
-        k_prune_count<<<grid, kCta, 0, st>>>(src, un, ctl, fine);
-      }
-      {
-        LaunchScope scope(K_PRUNE_SETTLE, st);
-        launch_prio(k_prune_settle, dim3(1), dim3(kCta), 0, st, false, 0, true, false, (unsigned int)m, ctl, fine);
-      }
-      {
-        LaunchScope scope(K_PRUNE_MARK, st);
-        // a block per 16 KB tile: short-lived blocks on one moving window read faster than persistent ones
-        const unsigned long long mark_tiles = (un + kStreamTile - 1) / kStreamTile;
-        k_prune_mark<<<(unsigned int)mark_tiles, kCta, 0, st>>>(src, un, ctl, tie_list, mask);
-      }
-      {
-        LaunchScope scope(K_PRUNE_FIX, st);
-        launch_prio(k_prune_fix, dim3(kPruneFixBlocks), dim3(kCta), 0, st, false, 0, true, false, ctl, tie_list, mask);
-      }
+  const bool sampled = n >= (int64_t)kSamples;
+  cudaError_t le;
+  if (sampled) {
+    // bracket of the (n - m + 1)-th largest magnitude; also clears the control block and the histograms
+    const SamplePlan plan = sample_plan(n, n - m + 1, NSML_F32);
+    {
+      LaunchScope scope(K_SAMPLE, st);
+      le = launch_prio(k_sample<NSML_F32>, dim3(kSampleBlocks), dim3(kSampleThreads), kSampleSmem, st, false, 0, true, true, src, nullptr,
+                       (unsigned long long)n, plan.rank_lo, plan.rank_hi, ctl, reinterpret_cast<uint4*>(ws), (unsigned int)(L.zero_bytes / 16), 0);
+      if (le != cudaSuccess) return NSML_ERR_CUDA;
     }
-  }
-  // The four-pass build: every kernel of it leaves at once when the two passes above have built the mask.  Behind
-  // the two-pass path it is the rare fallback, so it gets small grids (two blocks per SM): what counts there is
-  // how little the six launches cost when they have nothing to do; they are then launched at high priority
-  // like the other short kernels, so that they do not queue behind other streams' passes.
-  const unsigned int small = (unsigned int)dev->sms * 2;
-  const unsigned int fgrid = two_pass && grid > small ? small : grid;
-  const unsigned int fwgrid = two_pass && wgrid > small ? small : wgrid;
-  {
-    LaunchScope scope(K_PRUNE_HIST, st);
-    launch_prio(k_prune_hist<0>, dim3(fgrid), dim3(kCta), 0, st, false, 0, two_pass, false, src, un, (unsigned int)m, ctl, hist, tie_list);
+    LaunchScope scope(K_PRUNE_PASS, st);
+    le = launch_prio(k_prune_pass, dim3((unsigned int)((n + kPruneTile - 1) / kPruneTile)), dim3(kCta), 0, st, false, 0, false, true, src,
+                     (unsigned long long)n, ctl, list, (unsigned int)L.cap, mask);
+    if (le != cudaSuccess) return NSML_ERR_CUDA;
+  } else if (cudaMemsetAsync(ws, 0, L.zero_bytes, st) != cudaSuccess) {
+    return NSML_ERR_CUDA;
   }
   {
-    LaunchScope scope(K_PRUNE_HIST, st);
-    launch_prio(k_prune_hist<1>, dim3(fgrid), dim3(kCta), 0, st, false, 0, two_pass, false, src, un, (unsigned int)m, ctl, hist, tie_list);
-  }
-  {
-    LaunchScope scope(K_PRUNE_HIST, st);
-    launch_prio(k_prune_hist<2>, dim3(fgrid), dim3(kCta), 0, st, false, 0, two_pass, false, src, un, (unsigned int)m, ctl, hist, tie_list);
-  }
-  {
-    LaunchScope scope(K_PRUNE_TIES, st);
-    launch_prio(k_prune_ties, dim3(fgrid), dim3(kCta), 0, st, false, 0, two_pass, false, src, un, ctl, hist, tie_list, tile_ties);
-  }
-  {
-    LaunchScope scope(K_PRUNE_WRITE, st);
-    launch_prio(k_prune_write, dim3(fwgrid), dim3(kCta), 0, st, false, 0, two_pass, false, src, un, ctl, tile_ties, mask);
-  }
-  {
-    LaunchScope scope(K_PRUNE_WRITE_RANKED, st);  // returns at once unless ties have to be ranked
-    unsigned int rgrid = stream_grid(n, *dev, dev->prune_write_ranked < 8 ? dev->prune_write_ranked : 8, 1u << 16);
-    if (two_pass && rgrid > small) rgrid = small;
-    launch_prio(k_prune_write_ranked, dim3(rgrid), dim3(kCta), 0, st, false, 0, two_pass, false, src, un, ctl, tile_ties, mask);
+    LaunchScope scope(K_PRUNE_FINISH, st);
+    const unsigned int grid = grid_for((unsigned long long)n, kPruneUnit, 2 * dev->sms);
+    le = launch_prio(k_prune_finish, dim3(grid), dim3(kPruneThreads), 0, st, false, 0, true, sampled, src, (unsigned int)n, (unsigned int)m, ctl,
+                     reinterpret_cast<unsigned int*>(ws + L.hist), list, (unsigned int)L.cap, reinterpret_cast<uint2*>(ws + L.bin_list),
+                     reinterpret_cast<unsigned int*>(ws + L.unit_ties), mask, sampled ? 1 : 0);
+    if (le != cudaSuccess) return NSML_ERR_CUDA;
   }
   if (cudaGetLastError() != cudaSuccess) return NSML_ERR_CUDA;
   return NSML_OK;

@@ -32,7 +32,8 @@ struct Ctl {
   unsigned int ticket;        // chunks of the list handed out
   unsigned int fallback;      // a bin that was taken for a single key holds others
   unsigned int done;          // chunks of the list that are finished, where that has to be known
-  unsigned int drawn[5], finished[5];  // general select: units of work of each phase
+  unsigned long long below_listed;     // mask build: weights below the bracket << 32 | weights listed inside it
+  unsigned int drawn[9], finished[9];  // general select, mask build: units of work of each phase
 };
 static_assert(sizeof(Ctl) <= 256, "control block must fit its 256-byte slot");
 

@@ -446,7 +446,8 @@ __device__ __forceinline__ bool emit_chunks(const FinalizeParams& p, EmitShared&
 }
 
 // Waits (bounded) until a counter has reached `target`; called by the whole block.
-__device__ __forceinline__ bool wait_count(const unsigned int* at, unsigned int target, Ctl* ctl, EmitShared& sh) {
+template <class SH>  // (with a word sh.done[0])
+__device__ __forceinline__ bool wait_count(const unsigned int* at, unsigned int target, Ctl* ctl, SH& sh) {
   if (threadIdx.x == 0) {
     unsigned int ok = 0;
     for (int polls = 0; polls < kMaxPolls && !ok; ++polls) {
@@ -467,8 +468,8 @@ __device__ __forceinline__ bool wait_count(const unsigned int* at, unsigned int 
 // A phase of the general select: blocks draw its units of work by ticket; it is over when all units are finished.
 // Whoever waits has no unit left to do, and every unit that is not finished has been drawn by a running block, so the
 // phases need no co-resident grid.
-template <class Work, class Last>
-__device__ __forceinline__ bool run_phase(Ctl* ctl, int phase, unsigned int units, EmitShared& sh, Work&& work, Last&& last) {
+template <class SH, class Work, class Last>
+__device__ __forceinline__ bool run_phase(Ctl* ctl, int phase, unsigned int units, SH& sh, Work&& work, Last&& last) {
   unsigned int mine = 0;
   for (;;) {
     __syncthreads();
