@@ -198,77 +198,96 @@ inline PruneLayout prune_layout(int64_t n) {
   return L;
 }
 
-// A block per 4096 weights, all loads issued at once (short-lived blocks on one moving window read fastest).
-__global__ void __launch_bounds__(kCta, 5)
+// A block per 4096 weights, all loads issued at once (short-lived blocks on one moving window read fastest).  Bound by
+// instructions once the loads are in flight: two compares with two flag updates and one add per weight, the mask words by
+// a three-step exchange among eight lanes, places in the list by one shared and one global add per warp and block (the
+// list has no order).
+__global__ void __launch_bounds__(kCta, 6)
 k_prune_pass(BucketSrc<NSML_F32> src, unsigned long long n, Ctl* ctl, uint2* __restrict__ list, unsigned int cap, uint32_t* __restrict__ mask) {
-  __shared__ unsigned int s_below[kCta / 32], s_inside[kCta / 32], s_base;
+  __shared__ unsigned int s_count, s_base;  // count: below the bracket << 16 | inside it
   constexpr unsigned int FULL = 0xFFFFFFFFu;
   pdl_launch_dependents();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned long long i0 = (unsigned long long)blockIdx.x * kPruneTile + warp * 512;  // the warp's 512 weights
   uint32_t b[4][4];
-  int cnt[4];
+  const bool whole = i0 + 512 <= n;
+  if (whole) {
 #pragma unroll
-  for (int r = 0; r < 4; ++r) cnt[r] = src.load_vals4(i0 + r * 128 + lane * 4, n, b[r]);
+    for (int r = 0; r < 4; ++r) src.load_full4(i0 + r * 128 + lane * 4, b[r]);
+  }
+  if (threadIdx.x == 0) s_count = 0;
+  __syncthreads();
   pdl_wait();
+  if (!whole) {
+#pragma unroll
+    for (int r = 0; r < 4; ++r) src.load_vals4(i0 + r * 128 + lane * 4, n, b[r]);
+  }
   const unsigned int lo = ctl->lo, hi = ctl->hi > lo ? ctl->hi : 0x80000000u;
   // (on the weight itself: key < E  <=>  |w| < float(E); NaN is not below anything)
   const float t_lo = __uint_as_float(min(lo, kInfKey)), t_hi = __uint_as_float(min(hi, kInfKey));
-  unsigned int below = 0, flags = 0;  // flags: bit r * 4 + e = inside the bracket
-  bool nonfinite = false;
+  unsigned int under = 0, inside = 0;  // bit r * 4 + e
+  float bad = 0.f;                     // becomes NaN with the first weight that is not finite
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    unsigned int f = 0;
+  for (int r = 0; r < 4; ++r)
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      const float a = fabsf(__uint_as_float(b[r][e]));
-      const bool here = e < cnt[r], under = a < t_lo;
-      f |= (unsigned int)(here && under) << e;
-      flags |= (unsigned int)(here && !under && a < t_hi) << (r * 4 + e);
-      nonfinite |= !(a < __uint_as_float(kInfKey));  // (missing weights read as 0)
+      const float w = __uint_as_float(b[r][e]);
+      if (fabsf(w) < t_lo) under |= 1u << (r * 4 + e);
+      if (fabsf(w) < t_hi) inside |= 1u << (r * 4 + e);
+      bad = __fmaf_rn(w, 0.f, bad);
     }
-    below += __popc(f);
-    // the 4-bit flags of eight neighbouring lanes make one mask word
-    unsigned int x = f << (4 * (lane & 7));
-    x |= __shfl_xor_sync(FULL, x, 1);
-    x |= __shfl_xor_sync(FULL, x, 2);
-    x |= __shfl_xor_sync(FULL, x, 4);
-    const unsigned long long word = i0 / 32 + r * 4 + (lane >> 3);
-    if ((lane & 7) == 0 && word < (n + 31) / 32) mask[word] = x;
+  inside &= ~under;
+  if (!(bad == 0.f)) set_status(&ctl->status, NSML_ERR_NONFINITE);
+  if (!whole) {  // missing weights were read as 0
+    unsigned int here = 0;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const unsigned long long i = i0 + r * 128 + lane * 4;
+      here |= (i + 4 <= n ? 15u : i < n ? (1u << (n - i)) - 1u : 0u) << (r * 4);
+    }
+    under &= here;
+    inside &= here;
   }
-  if (nonfinite) set_status(&ctl->status, NSML_ERR_NONFINITE);
-  const unsigned int mine = __popc(flags);
-  unsigned int incl = mine;
+  const unsigned int mine = __popc(inside);
+  unsigned int count = (unsigned int)__popc(under) << 16 | mine, incl = count;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const unsigned int up = __shfl_up_sync(FULL, incl, o);
     if (lane >= o) incl += up;
   }
-  below = __reduce_add_sync(FULL, below);
-  if (lane == 31) s_inside[warp] = incl;
-  if (lane == 0) s_below[warp] = below;
-  __syncthreads();
-  unsigned int before = 0, inside = 0, all_below = 0;
-#pragma unroll
-  for (int w = 0; w < kCta / 32; ++w) {
-    if (w < warp) before += s_inside[w];
-    inside += s_inside[w];
-    all_below += s_below[w];
+  unsigned int at = 0;
+  if (lane == 31 && incl != 0) at = atomicAdd(&s_count, incl);  // (at most 4096 of either kind: the halves do not meet)
+  // A mask word is the nibbles of eight neighbouring lanes.  Each step hands half of the rounds to a partner and
+  // doubles what is held of the others: 4 rounds of 4 bits, 2 of 8, 1 of 16, 1 of 32.
+  {
+    const bool odd = lane & 1, odd2 = lane & 2;
+    const unsigned int give = odd ? under & 0xFFu : under >> 8, got = __shfl_xor_sync(FULL, give, 1);
+    const unsigned int keep = odd ? under >> 8 : under;  // rounds 2, 3 in odd lanes, 0, 1 in even ones
+    const unsigned int low = odd ? got : keep, high = odd ? keep : got;
+    const unsigned int two = (low & 15u) | (high & 15u) << 4 | (low & 0xF0u) << 4 | (high & 0xF0u) << 8;
+    const unsigned int got2 = __shfl_xor_sync(FULL, odd2 ? two & 0xFFu : two >> 8, 2), keep2 = (odd2 ? two >> 8 : two) & 0xFFu;
+    const unsigned int one = odd2 ? got2 | keep2 << 8 : keep2 | got2 << 8;
+    const unsigned int word = one | __shfl_down_sync(FULL, one, 4) << 16;
+    const unsigned long long at_word = i0 / 32 + (((lane & 1) << 1) | (lane >> 1 & 1)) * 4 + (lane >> 3);
+    if ((lane & 4) == 0 && at_word < (n + 31) / 32) mask[at_word] = word;
   }
-  if (threadIdx.x == 0) {
-    s_base = (unsigned int)atomicAdd(&ctl->below_listed, (unsigned long long)all_below << 32 | inside);
-  }
-  if (inside == 0) return;
   __syncthreads();
-  unsigned int at = s_base + before + incl - mine;
+  const unsigned int all = s_count;
+  if (threadIdx.x == 0 && all != 0)
+    s_base = (unsigned int)atomicAdd(&ctl->below_listed, (unsigned long long)(all >> 16) << 32 | (all & 0xFFFFu));
+  if ((all & 0xFFFFu) == 0) return;
+  __syncthreads();
+  at = s_base + (__shfl_sync(FULL, at, 31) & 0xFFFFu) + ((incl - count) & 0xFFFFu);
 #pragma unroll
-  for (int r = 0; r < 4; ++r)
+  for (int r = 0; r < 4; ++r) {
+    if ((inside >> (r * 4) & 15u) == 0) continue;
 #pragma unroll
     for (int e = 0; e < 4; ++e)
-      if (flags & (1u << (r * 4 + e))) {
+      if (inside & (1u << (r * 4 + e))) {
         if (at < cap) list[at] = make_uint2(b[r][e] & 0x7FFFFFFFu, (uint32_t)i0 + r * 128 + lane * 4 + e);
         ++at;
       }
+  }
 }
 
 struct PruneShared {
