@@ -416,7 +416,7 @@ static unsigned int stream_grid(int64_t n, const DeviceInfo& dev, int per_sm, un
 }
 
 static int sumsq_impl(const void* grad, int64_t n, int grad_dtype, void* workspace, size_t workspace_bytes,
-                      cudaStream_t st) {
+                      cudaStream_t st, SumsqCtl* to_host = nullptr) {
   if (grad == nullptr || workspace == nullptr) return NSML_ERR_ARG;
   if (grad_dtype != NSML_F32 && grad_dtype != NSML_BF16) return NSML_ERR_ARG;
   if (n < 1 || n > NSML_MAX_N) return NSML_ERR_ARG;
@@ -433,21 +433,44 @@ static int sumsq_impl(const void* grad, int64_t n, int grad_dtype, void* workspa
   {
     LaunchScope scope(K_SUMSQ, st);
     if (grad_dtype == NSML_F32)
-      k_sumsq<NSML_F32><<<grid, kCta, 0, st>>>(BucketSrc<NSML_F32>{grad, nullptr}, (unsigned long long)n, ctl, partials);
+      k_sumsq<NSML_F32><<<grid, kCta, 0, st>>>(BucketSrc<NSML_F32>{grad, nullptr}, (unsigned long long)n, ctl, partials, to_host);
     else
-      k_sumsq<NSML_BF16><<<grid, kCta, 0, st>>>(BucketSrc<NSML_BF16>{grad, nullptr}, (unsigned long long)n, ctl, partials);
+      k_sumsq<NSML_BF16><<<grid, kCta, 0, st>>>(BucketSrc<NSML_BF16>{grad, nullptr}, (unsigned long long)n, ctl, partials, to_host);
   }
   if (cudaGetLastError() != cudaSuccess) return NSML_ERR_CUDA;
   return NSML_OK;
 }
 
-// Synchronises the stream and reads the status word and the sum of squares left by sumsq_impl.
-static int sumsq_read(const void* workspace, cudaStream_t st, double* sumsq) {
-  SumsqCtl host;
-  if (cudaMemcpyAsync(&host, workspace, sizeof(host), cudaMemcpyDeviceToHost, st) != cudaSuccess) return NSML_ERR_CUDA;
+// A few bytes of page-locked host memory that kernels of any device can write; one per calling thread, freed with it.
+struct HostSlot {
+  SumsqCtl* at = nullptr;
+  HostSlot() {
+    // (allowed while another thread captures a stream)
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return;
+    void* p = nullptr;
+    if (cudaHostAlloc(&p, sizeof(SumsqCtl), cudaHostAllocPortable | cudaHostAllocMapped) == cudaSuccess) at = static_cast<SumsqCtl*>(p);
+    else cudaGetLastError();
+    cudaThreadExchangeStreamCaptureMode(&mode);
+  }
+  ~HostSlot() { if (at != nullptr) cudaFreeHost(at); }
+};
+
+// Sum of squares, waited for: synchronises the stream.
+static int sumsq_wait(const void* grad, int64_t n, int grad_dtype, void* workspace, size_t workspace_bytes, cudaStream_t st,
+                      double* sumsq) {
+  static thread_local HostSlot slot;
+  const int rc = sumsq_impl(grad, n, grad_dtype, workspace, workspace_bytes, st, slot.at);
+  if (rc != NSML_OK) return rc;
+  SumsqCtl pageable;
+  SumsqCtl* host = slot.at;
+  if (host == nullptr) {
+    host = &pageable;
+    if (cudaMemcpyAsync(host, workspace, sizeof(*host), cudaMemcpyDeviceToHost, st) != cudaSuccess) return NSML_ERR_CUDA;
+  }
   if (cudaStreamSynchronize(st) != cudaSuccess) return NSML_ERR_CUDA;
-  if (host.status != NSML_OK) return host.status;
-  *sumsq = host.sumsq;
+  if (host->status != NSML_OK) return host->status;
+  *sumsq = host->sumsq;
   return NSML_OK;
 }
 
@@ -684,10 +707,9 @@ size_t nsml_l2_workspace_bytes(void) { return kSumsqWorkspace; }
 int nsml_grad_l2(const void* grad, int64_t n, int grad_dtype, void* workspace, size_t workspace_bytes, void* stream,
                  double* l2_out) {
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  int rc = sumsq_impl(grad, n, grad_dtype, workspace, workspace_bytes, st);
-  if (rc != NSML_OK || l2_out == nullptr) return rc;
+  if (l2_out == nullptr) return sumsq_impl(grad, n, grad_dtype, workspace, workspace_bytes, st);
   double sumsq = 0.0;
-  rc = sumsq_read(workspace, st, &sumsq);
+  const int rc = sumsq_wait(grad, n, grad_dtype, workspace, workspace_bytes, st, &sumsq);
   if (rc != NSML_OK) return rc;
   *l2_out = std::sqrt(sumsq);
   return NSML_OK;
@@ -755,10 +777,8 @@ int nsml_compress_adaptive(const void* grad, int64_t n, int grad_dtype, double r
   double use_ratio = ratio, l2 = -1.0;
   int use_bits = plain_bits;
   if (ratio < tr_q) {
-    int rc = sumsq_impl(grad, n, grad_dtype, workspace, workspace_bytes, st);
-    if (rc != NSML_OK) return rc;
     double sumsq = 0.0;
-    rc = sumsq_read(workspace, st, &sumsq);
+    int rc = sumsq_wait(grad, n, grad_dtype, workspace, workspace_bytes, st, &sumsq);
     if (rc != NSML_OK) return rc;
     l2 = std::sqrt(sumsq);
     rc = gate(ratio, l2, tr_q, tr_d, plain_bits, &use_ratio, &use_bits);

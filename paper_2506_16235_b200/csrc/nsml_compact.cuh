@@ -16,7 +16,7 @@
 namespace nsml {
 
 // |v| >= t on floats equals key >= lo for finite v; written as !(|v| < t) so
-// that NaN is kept too (the finalize kernel reports non-finite candidates).
+// that NaN is kept too (k_emit reports non-finite candidates).
 template <int EPL>
 __device__ __forceinline__ unsigned int keep_flags(const uint32_t (&bits)[EPL], float t) {
   unsigned int f = 0;

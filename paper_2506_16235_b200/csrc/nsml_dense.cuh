@@ -16,14 +16,14 @@
 // cached words and its own slice of the uncached ones, so that block order,
 // warp order and lane order together are index order.
 //
-// Phases, separated by grid barriers (same protocol and bounds as k_finalize):
+// Phases, separated by grid barriers (nsml_finalize.cuh):
 //   0  load the range, keep the shared-memory copy, histogram of digit 0   | barrier
 //   1  resolve digit 0; histogram of digit 1                               | barrier
 //   2  resolve digit 1; histogram of digit 2                               | barrier
 //   3  resolve digit 2 -> T, r; per-warp counts of keys > T and == T       | barrier
 //   4  prefix over blocks and warps; write survivors in index order
 //      (float32 and fp16 values straight into the payload)
-//   5  int8 only, behind one more barrier: quantise (shared with k_finalize)
+//   5  int8 only, behind one more barrier: quantise
 #pragma once
 
 #include "nsml_finalize.cuh"
