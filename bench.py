@@ -762,16 +762,15 @@ class Alg2Workload(Workload):
                 nsml.nsml_decompress_accumulate([p], lane.dense, zero_first=True, workspace=lane.aws, stream=lane.stream)
                 if acc is not None:
                     self.account(acc, "k_sumsq", 4 * n)
-                    # mask build in two passes (sampled window); the four-pass kernels behind them leave at once
-                    self.account(acc, "k_prune_sample", 4 * 8192)
-                    self.account(acc, "k_prune_count", 4 * n)
-                    self.account(acc, "k_prune_settle", 4 * 4096)
-                    self.account(acc, "k_prune_mark", 4 * n + n // 8)
-                    self.account(acc, "k_prune_fix", 8 * 1024)
-                    self.account(acc, "k_feedback_subtract", 13 * k)
+                    # mask build: sample, one pass (lists about 3 % of the weights as key and index), list read twice
+                    self.account(acc, "k_sample", 16 * 16384)
+                    self.account(acc, "k_prune_pass", 4 * n + n // 8 + 8 * n // 32)
+                    self.account(acc, "k_prune_finish", 2 * 8 * n // 32)
                     self.compress_bytes(acc, n, 4, self.RATIO, self.BITS)
-                    # the bucket pass also reads the mask and the residual and writes gradient + residual back
+                    # the bucket pass also reads the mask and the residual and writes gradient + residual back; the list
+                    # stage takes what the payload carries out of the residual
                     self.account(acc, "k_compact_bucket", n // 8 + 8 * n)
+                    self.account(acc, "k_emit", 8 * k)
                     self.merge_bytes(acc, n, [(k, self.BITS)])
 
             yield ((i * self.STATE + b) % self.GRADS, b), nsml.nsml_payload_bytes(n, self.RATIO, self.BITS), enqueue

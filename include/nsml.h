@@ -23,7 +23,7 @@
  *     caller before and after the call.  "host pointer" = ordinary memory.
  *   - Device work is enqueued on `stream` (a cudaStream_t passed as void*, NULL
  *     = the default stream) and the call returns without synchronising.  The
- *     short, latency-bound kernels of a call (sample, gather, list stage,
+ *     short, latency-bound kernels of a call (sample, list stage,
  *     partition) are launched at the device's highest stream priority, whatever
  *     the priority of `stream`: with several buckets in flight on several
  *     streams they are then placed between the blocks of other buckets'
@@ -212,11 +212,14 @@ int nsml_compress(const void* grad, int64_t n, int grad_dtype, double ratio, int
 /* Which of its two internal strategies nsml_compress takes for (n, ratio) on
  * the current device.  Both give the same payload; this is information for
  * byte accounting (the paper prescribes no strategy).
- *   NSML_STRATEGY_LIST   a stratified sample bounds the threshold from below,
- *                        one streaming pass keeps the candidates above the
- *                        bound, an exact radix select runs on that list
- *   NSML_STRATEGY_DENSE  the radix select runs over the bucket itself (high
+ *   NSML_STRATEGY_LIST   a stratified sample bounds the threshold from both
+ *                        sides, one streaming pass keeps the candidates above
+ *                        the lower bound, the exact threshold is found among
+ *                        the few keys of one bin between the bounds
+ *   NSML_STRATEGY_DENSE  a radix select runs over the bucket itself (high
  *                        kept fractions, and buckets too small to sample)
+ * (Buckets of up to 163,840 elements are taken by one kernel of their own,
+ * whichever of the two this names.)
  * Returns the strategy, or NSML_ERR_ARG / NSML_ERR_CUDA. */
 #define NSML_STRATEGY_LIST 0
 #define NSML_STRATEGY_DENSE 1
@@ -228,13 +231,9 @@ int nsml_compress_strategy(int64_t n, double ratio);
  * of nsml_compress does not depend on it.  Fewer candidates per block = more
  * blocks = a shorter list stage for a call that has the GPU to itself; more
  * candidates per block = fewer SMs held while the stage waits for memory, which
- * is what counts when several buckets are compressed on several streams at
- * once.  Above the default the gather kernel in front of the list stage also
- * runs as one block per group of segments instead of two, and long lists get
- * one list-stage block per SM instead of two.  Measured on one
- * B200, 25M-element buckets, ratio 0.01, int8: 2048 -> a lone call 65 us;
- * 4096 -> 68 us, the eight-stream step of 20 calls and 5 sums 0.70 ms;
- * 8192 -> 81 us and 0.63 ms.
+ * is what counts when several calls run on several streams at once.  (A block
+ * takes chunks by ticket; the grid has a block per half the given number of
+ * candidates, at most two per SM.)
  *   candidates   1024 ... 8192; the default is 4096
  * Returns NSML_OK, or NSML_ERR_ARG for a value out of range (nothing changes).
  * Takes effect for calls made after it returns. */
