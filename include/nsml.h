@@ -231,9 +231,12 @@ int nsml_compress_strategy(int64_t n, double ratio);
  * of nsml_compress does not depend on it.  Fewer candidates per block = more
  * blocks = a shorter list stage for a call that has the GPU to itself; more
  * candidates per block = fewer SMs held while the stage waits for memory, which
- * is what counts when several calls run on several streams at once.  (A block
- * takes chunks by ticket; the grid has a block per half the given number of
- * candidates, at most two per SM.)
+ * is what counts when several calls run on several streams at once.  (Blocks
+ * take chunks by ticket.  Up to the default the grid has a block per half the
+ * given number of candidates, at most two per SM; above it, far fewer blocks
+ * for short lists and at most one per SM for long ones.)  Measured on one
+ * B200, 25M-element buckets, ratio 0.01, int8, eight streams, a step of 20 calls
+ * and 5 sums: 0.68 ms with 80 blocks per call, 0.63 ms with the 10 of 8192.
  *   candidates   1024 ... 8192; the default is 4096
  * Returns NSML_OK, or NSML_ERR_ARG for a value out of range (nothing changes).
  * Takes effect for calls made after it returns. */

@@ -174,9 +174,9 @@ k_feedback_subtract(const unsigned char* __restrict__ payload, float* __restrict
 // ties), the same kernel does a radix select over the weights instead (12 + 12 +
 // 7 bits, then the ties by their rank): the result is exact either way.
 //
-// Measured (25M weights, ratio 0.02): 86 us in eleven launches before (two passes
-// over the weights, 35 and 25 us; six kernels of the fallback, which left at once,
-// 17 us).
+// Measured (24.4M weights): 11 + 34 + 18 us (sample, pass, finish), less what they
+// overlap; before, eleven launches, 102 us: two passes over the weights (35 and 25
+// us), a sample in one block (14), six kernels of the fallback that left at once (17).
 // ------------------------------------------------------------------------
 constexpr int kPruneTile = kCta * 16;       // weights per block of the pass
 constexpr int kPruneThreads = 512;
