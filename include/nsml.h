@@ -169,6 +169,8 @@ int nsml_ctrl_load(nsml_ctrl* c, const void* buf, size_t bytes);
 int64_t nsml_k_of(int64_t n, double ratio);
 /* Exact size in bytes of the payload nsml_compress writes for (n, ratio, bits). */
 size_t nsml_payload_bytes(int64_t n, double ratio, int bits);
+/* The workspace sizes, here and below, never shrink as n or W grows: a workspace
+ * sized for the largest bucket (and the most workers) serves every smaller one. */
 /* Scratch needed by nsml_compress for a bucket of n elements (any ratio, bits). */
 size_t nsml_workspace_bytes(int64_t n, int grad_dtype);
 /* Scratch needed by nsml_decompress_accumulate for (n, W). */

@@ -30,14 +30,18 @@ struct PayloadTable {
 
 struct AccumulateLayout {
   size_t offsets;  // u32[W][tiles + 1]
-  size_t total;
+  size_t total;    // what a sum of n elements uses
+  size_t ask;      // what a caller is told to bring: enough for every smaller n, too (one workspace serves buckets of
+                   // several sizes), although the table is shorter right above kDenseTileSmallMaxN than below it
 };
 
 inline AccumulateLayout accumulate_layout(int64_t n, int W) {
   AccumulateLayout L;
   const size_t tile = (size_t)dense_tile(n), tiles = ((size_t)n + tile - 1) / tile;
+  const size_t most_small = ((size_t)kDenseTileSmallMaxN + kDenseTileSmall - 1) / kDenseTileSmall;
   L.offsets = 256;
   L.total = L.offsets + align_up((size_t)W * (tiles + 1) * 4, 256);
+  L.ask = n <= kDenseTileSmallMaxN || tiles >= most_small ? L.total : L.offsets + align_up((size_t)W * (most_small + 1) * 4, 256);
   return L;
 }
 

@@ -668,7 +668,7 @@ size_t nsml_workspace_bytes(int64_t n, int grad_dtype) {
 
 size_t nsml_accumulate_workspace_bytes(int64_t n, int W) {
   if (n < 1 || n > NSML_MAX_N || W < 1 || W > NSML_MAX_WORKERS) return 0;
-  return accumulate_layout(n, W).total;
+  return accumulate_layout(n, W).ask;
 }
 
 int nsml_compress(const void* grad, int64_t n, int grad_dtype, double ratio, int bits, const uint32_t* prune_mask,

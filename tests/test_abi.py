@@ -119,3 +119,31 @@ def test_list_block_candidates_knob_checks_its_range(nsml):
         assert nsml.lib.nsml_set_list_block_candidates(bad) == nsml.NSML_ERR_ARG
     for good in (1024, 8192, 4096):  # leaves the default in place
         assert nsml.lib.nsml_set_list_block_candidates(good) == nsml.NSML_OK
+
+
+def test_workspace_sizes_never_shrink_with_n_or_w(nsml):
+    # one workspace, sized for the largest bucket and the most workers, has to serve every smaller one: around every
+    # size at which a layout changes (tiles of the sum and the bucket pass, bins, groups of tiles) and in between
+    largest = 2_147_483_647  # NSML_MAX_N
+    at = {1, largest}
+    for base in (2048, 4096, 8192, 16_384, 163_840, 400_000, 2_424_832, 9_699_328, 1 << 24, 33_554_432, 1 << 26, 1 << 30):
+        at.update(base + d for d in (-1, 0, 1))
+    at.update(int(1.13 ** i) for i in range(1, 176) if int(1.13 ** i) <= largest)
+    sizes = sorted(at)
+    queries = {
+        "compress f32": lambda n: nsml.nsml_workspace_bytes(n, nsml.NSML_F32),
+        "compress bf16": lambda n: nsml.nsml_workspace_bytes(n, nsml.NSML_BF16),
+        "prune": nsml.nsml_prune_workspace_bytes,
+        "adaptive": lambda n: nsml.lib.nsml_adaptive_workspace_bytes(n, nsml.NSML_F32),
+        "host sum": lambda n: nsml.lib.nsml_accumulate_host_scratch_bytes(n, 8, 1 << 20),
+        "host compress": lambda n: nsml.lib.nsml_compress_host_scratch_bytes(n, nsml.NSML_F32, 0.5, 8),
+    }
+    for W in (1, 2, 3, 8, 63, 64):
+        queries[f"sum of {W}"] = lambda n, W=W: nsml.nsml_accumulate_workspace_bytes(n, W)
+    for what, query in queries.items():
+        got = [query(n) for n in sizes]
+        shrinks = [(a, b) for a, b, x, y in zip(sizes, sizes[1:], got, got[1:]) if y < x]
+        assert min(got) > 0 and not shrinks, f"{what}: shrinks between {shrinks}"
+    for n in sizes:
+        per_w = [nsml.nsml_accumulate_workspace_bytes(n, W) for W in range(1, 65)]
+        assert per_w == sorted(per_w)

@@ -9,6 +9,7 @@ import oracle
 pytestmark = pytest.mark.gpu
 
 if torch.cuda.is_available():
+    import paper_2506_16235_b200 as nsml
     from gpu_util import check_accumulate, payload_to_device
 
 SWITCH = 296 * 8192  # largest bucket that takes the small tile
@@ -38,3 +39,17 @@ def test_many_workers_most_of_them_sparse(W):
     n = 100_003
     want = [crowded_payload(n, 1 if w % 3 else 5000, 8, w) for w in range(W)]
     check_accumulate([payload_to_device(p) for p in want], want, n, zero_first=True)
+
+
+def test_one_workspace_sized_for_the_largest_bucket_serves_them_all():
+    # a gradient set in 25 MB buckets: the shorter ones need more room for their (smaller) tiles than the longest one
+    W, sizes = 8, (6_553_600, SWITCH, 2_000_000, 12_289)
+    ws = nsml.alloc_bytes(nsml.nsml_accumulate_workspace_bytes(max(sizes), W), "cuda")
+    for n in sizes:
+        want = [crowded_payload(n, 1500, 8, n + w) for w in range(W)]
+        dense = torch.full((n,), 7.0, device="cuda")
+        nsml.nsml_decompress_accumulate([payload_to_device(p) for p in want], dense, workspace=ws)
+        assert nsml.nsml_last_status(ws) == 0
+        ref = oracle.decompress_sum(want, n)
+        largest = max(float(np.abs(p.raw).max()) for p in want)
+        assert float(np.abs(dense.cpu().numpy().astype(np.float64) - ref).max()) <= 1e-6 * largest
