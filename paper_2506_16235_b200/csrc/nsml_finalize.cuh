@@ -176,7 +176,9 @@ __device__ __forceinline__ void put_value(const FinalizeParams& p, unsigned long
   else if (p.bits == NSML_BITS_FP16) reinterpret_cast<uint16_t*>(p.payload + p.P.val_off)[pos] = encode_f16(__uint_as_float(bits));
   else p.raw_val[pos] = __uint_as_float(bits);
 }
-// What a receiver reconstructs of a float32 or fp16 value, taken out of it (one float32 subtraction).
+// What a receiver reconstructs of a float32 or fp16 value, taken out of it (one float32 subtraction).  Callers leave
+// out +0.0 only: there nothing changes, and it may stand for a pruned parameter, whose sum in the residual stays.
+// -0.0 is a sum like any other and leaves -0.0 - (-0.0) = +0.0.
 __device__ __forceinline__ float not_carried(const FinalizeParams& p, uint32_t bits) {
   const float v = __uint_as_float(bits);
   return __fsub_rn(v, p.bits == NSML_BITS_FP32 ? v : decode_f16(encode_f16(v)));

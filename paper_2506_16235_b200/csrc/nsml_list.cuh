@@ -253,7 +253,7 @@ __device__ __forceinline__ unsigned int tied_of(unsigned long long s) { return (
 
 // 128 threads (four warps) turn values get(j), j < cnt <= 1024, into the codes and the scale of payload block qb; with a
 // residual, what the codes do not carry stays at the values' indices index(j) (a zero leaves its place alone: it may be a
-// pruned parameter's, whose sum stays).
+// pruned parameter's, whose sum stays; and code 0 is +0.0, which taken out of -0.0 leaves -0.0).
 // Called by every thread of the block (it holds block barriers); live: the group has a block.
 template <class Get, class Index>
 __device__ __forceinline__ void quantize_group(const FinalizeParams& p, float* residual, float* s_qmax, unsigned int qb, bool live, unsigned int cnt,
@@ -385,7 +385,7 @@ __device__ __forceinline__ bool emit_chunks(const FinalizeParams& p, EmitShared&
             sh.kept.idx[at - p0] = idx[u];
           } else {
             put_value(p, at, v[u]);
-            if (take_out && (v[u] & 0x7FFFFFFFu) != 0) p.residual[idx[u]] = not_carried(p, v[u]);
+            if (take_out && v[u] != 0) p.residual[idx[u]] = not_carried(p, v[u]);  // (+0.0: see not_carried)
           }
         }
       }

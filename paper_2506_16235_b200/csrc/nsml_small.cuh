@@ -223,7 +223,7 @@ k_select_small(BucketSrc<DTYPE> src, FinalizeParams p, unsigned int per_block, i
         if (at < k) {
           out_idx[at] = idx;
           put_value(p, at, b[e]);
-          if (p.residual != nullptr && p.bits != NSML_BITS_INT8 && (b[e] & 0x7FFFFFFFu) != 0) p.residual[idx] = not_carried(p, b[e]);
+          if (p.residual != nullptr && p.bits != NSML_BITS_INT8 && b[e] != 0) p.residual[idx] = not_carried(p, b[e]);
         }
       }
       s_mine += is_sure;

@@ -10,7 +10,7 @@ pytestmark = pytest.mark.gpu
 
 if torch.cuda.is_available():
     import paper_2506_16235_b200 as nsml
-    from gpu_util import check_compress, gpu_compress, oracle_compress, assert_payload_equal
+    from gpu_util import check_compress, gpu_compress, mask_words, oracle_compress, assert_payload_equal
     from test_gpu_compress import sampled_positions
 
 
@@ -139,3 +139,29 @@ def test_feedback_when_ties_fill_the_threshold_bin():
         ref, want = error_feedback_step(g, want, ratio, bits)
         assert_payload_equal(payload, ref)
         assert np.array_equal(residual.cpu().numpy().view(np.uint32), want.view(np.uint32))
+
+
+# one block, one cluster, the list (its ties settled at once; a list shorter than k), the bucket itself
+@pytest.mark.parametrize("n,ratio,hidden", [(5000, 0.4, False), (100_003, 0.1, False), (700_001, 0.1, False), (1 << 20, 0.1, True),
+                                            (900_001, 0.5, False)])
+@pytest.mark.parametrize("bits", [8, 16, 32])
+def test_feedback_takes_selected_negative_zeros_out(n, ratio, hidden, bits):
+    # fewer non-zero sums than survivors, all zero sums -0.0: a selected one leaves +0.0 where the payload carries its sign
+    from oracle.adaptive import error_feedback_step
+    rng = np.random.default_rng(n + bits)
+    g = rng.standard_normal(n).astype(np.float32)
+    zero = rng.random(n) >= 0.5 * ratio
+    if hidden:  # (the sampler sees no zero, so the list holds the sampled elements only)
+        zero[:] = True
+        zero[sampled_elements(n, 4)] = False
+    g[zero] = -0.0
+    mask = rng.random(n) < 0.2
+    start = np.where(zero, np.float32(-0.0), np.float32(0.5)).astype(np.float32)
+    words = torch.from_numpy(mask_words(mask).view(np.int32)).cuda()
+    for masked in (False, True):
+        residual, want = torch.from_numpy(start.copy()).cuda(), start
+        for _ in range(2):
+            payload = nsml.nsml_compress_feedback(torch.from_numpy(g).cuda(), residual, ratio, bits, prune_mask=words if masked else None)
+            ref, want = error_feedback_step(g, want, ratio, bits, prune_mask_=mask if masked else None)
+            assert_payload_equal(payload, ref)
+            assert np.array_equal(residual.cpu().numpy().view(np.uint32), want.view(np.uint32))
