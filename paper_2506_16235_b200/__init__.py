@@ -217,7 +217,6 @@ def nsml_compress_strategy(n: int, ratio: float) -> int:
     return rc
 
 
-@functools.lru_cache(maxsize=1024)
 def nsml_payload_bytes(n: int, ratio: float, bits: int) -> int:
     return int(lib.nsml_payload_bytes(int(n), float(ratio), int(bits)))
 

@@ -56,6 +56,19 @@ def test_k_rule_and_sizes(nsml):
     assert nsml.nsml_accumulate_workspace_bytes(1 << 20, 65) == 0
 
 
+def test_payload_size_follows_a_ratio_that_changes_in_place(nsml):
+    # a ratio kept as a 0-d tensor or array, as a training loop may hold it, is read on every call
+    import numpy as np
+    import torch
+
+    want = {r: nsml.nsml_payload_bytes(100_000, r, 8) for r in (0.01, 0.5)}
+    tensor, array = torch.tensor(0.01, dtype=torch.float64), np.array(0.01)
+    assert nsml.nsml_payload_bytes(100_000, tensor, 8) == nsml.nsml_payload_bytes(100_000, array, 8) == want[0.01]
+    tensor.fill_(0.5)
+    array[...] = 0.5
+    assert nsml.nsml_payload_bytes(100_000, tensor, 8) == nsml.nsml_payload_bytes(100_000, array, 8) == want[0.5]
+
+
 def test_header_struct_is_64_bytes(nsml):
     import numpy as np
 
