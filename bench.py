@@ -866,7 +866,7 @@ def serial_compress(nsml, torch, grad, ratio, bits, ws, payload, esize, peak, re
     last bucket of a backward pass, say) gets.  The algorithmic bytes of the call are one read of the bucket plus
     the payload written."""
     n = grad.numel()
-    nsml.nsml_set_list_block_candidates(2048)  # the setting for a call that has the GPU to itself (default 4096: 3 us more)
+    nsml.nsml_set_list_block_candidates(4096)  # the default: a call that has the GPU to itself
     for _ in range(5):
         nsml.nsml_compress(grad, ratio, bits, payload=payload, workspace=ws)
     torch.cuda.synchronize()
@@ -882,7 +882,7 @@ def serial_compress(nsml, torch, grad, ratio, bits, ws, payload, esize, peak, re
     gbs = nbytes / (us * 1e-6) / 1e9
     return {"us_per_call": us, "algorithmic_bytes": nbytes, "algorithmic_GBps": gbs, "frac_of_measured": gbs / peak,
             "frac_of_nominal_8TBps": gbs / 8000.0, "n": n, "ratio": ratio, "bits": bits,
-            "list_block_candidates": 2048,
+            "list_block_candidates": 4096,
             "note": "one call at a time on one stream, eager launches; the same bucket every time, so a bucket that "
                     "fits the 126 MB L2 is partly served from it"}
 
@@ -1057,8 +1057,8 @@ def main():
     kwargs = {}
     if args.workload == "gpt2" and args.buckets:
         kwargs["buckets"] = list(range(args.buckets))
-    # several buckets in flight: the list stage takes more candidates per block (fewer SMs held while it waits
-    # for memory); the one-call-at-a-time measurement below goes back to the library's default
+    # several buckets in flight: the list stage gets few blocks that take many chunks each (fewer SMs held while it
+    # waits for memory); the one-call-at-a-time measurement below goes back to the library's default
     if args.list_block_candidates is None:
         args.list_block_candidates = 8192 if args.workload in ("gpt2", "decoder") else 4096
     nsml.nsml_set_list_block_candidates(args.list_block_candidates)
@@ -1157,7 +1157,7 @@ def main():
         nl, graphs = max(1, args.streams), not args.no_graphs
         del wl
         torch.cuda.empty_cache()
-        # (key, workload, candidates per list-stage block: the legs with few calls in flight keep the library's default)
+        # (key, workload, nsml_set_list_block_candidates: the legs with few calls in flight keep the library's default)
         for key, make, candidates in (
             ("ratio_0.1_25M", lambda: Gpt2Workload(nsml, torch, device, rank, buckets=[2, 3], nlanes=nl, ratio=0.1, workers=2),
              args.list_block_candidates),

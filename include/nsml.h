@@ -228,17 +228,17 @@ int nsml_compress(const void* grad, int64_t n, int grad_dtype, double ratio, int
 int nsml_compress_strategy(int64_t n, double ratio);
 
 /* nsml_set_list_block_candidates -- a tuning knob of the list strategy, for the
- * whole process: about how many candidates one thread block of the list stage
- * takes when the list is short (up to about a million candidates).  The result
- * of nsml_compress does not depend on it.  Fewer candidates per block = more
- * blocks = a shorter list stage for a call that has the GPU to itself; more
- * candidates per block = fewer SMs held while the stage waits for memory, which
- * is what counts when several calls run on several streams at once.  (Blocks
- * take chunks by ticket.  Up to the default the grid has a block per half the
- * given number of candidates, at most two per SM; above it, far fewer blocks
- * for short lists and at most one per SM for long ones.)  Measured on one
- * B200, 25M-element buckets, ratio 0.01, int8, eight streams, a step of 20 calls
- * and 5 sums: 0.68 ms with 80 blocks per call, 0.63 ms with the 10 of 8192.
+ * whole process: whether the list stage is laid out for a call that has the GPU
+ * to itself (the default, and every value below it) or for several calls on
+ * several streams at once (values above it).  The result of nsml_compress does
+ * not depend on it.  Blocks of the list stage take chunks of 2048 candidates
+ * (long lists: 4096) by ticket; up to the default there is a block per chunk, at
+ * most two per SM.  Above it a short list (up to about 600,000 candidates) gets
+ * fewer blocks, by the fourth power of the excess and not below ten, and a long one at
+ * most one block per SM, so that fewer SMs are held while the stage waits for
+ * memory: a lone call takes longer, several at once are done sooner.  Measured on
+ * one B200, 25M-element buckets, ratio 0.01, int8, eight streams, a step of 20
+ * calls and 5 sums: 0.73 ms with 148 blocks per call, 0.63 ms with the 10 of 8192.
  *   candidates   1024 ... 8192; the default is 4096
  * Returns NSML_OK, or NSML_ERR_ARG for a value out of range (nothing changes).
  * Takes effect for calls made after it returns. */

@@ -205,7 +205,8 @@ def nsml_k_of(n: int, ratio: float) -> int:
 
 
 def nsml_set_list_block_candidates(candidates: int) -> None:
-    """Tuning knob of the list stage (1024 ... 8192, default 4096); the results do not depend on it."""
+    """Tuning knob of the list stage (1024 ... 8192; above the default 4096: for many calls in flight); the results do not
+    depend on it."""
     _check(lib.nsml_set_list_block_candidates(int(candidates)), "nsml_set_list_block_candidates")
 
 

@@ -231,8 +231,9 @@ static SamplePlan sample_plan(int64_t n, int64_t k, int grad_dtype) {
   return s;
 }
 
-// Candidates per block of the list stage's small shape (nsml_set_list_block_candidates).
+// nsml_set_list_block_candidates: up to the default a block of the list stage per chunk of a short list, above it few.
 constexpr int kListBlockCandidates = 4096;  // default of the knob
+constexpr double kListFewBlocks = 10;       // blocks for a short list where the knob is well above it
 static std::atomic<int> g_list_block_candidates{kListBlockCandidates};
 
 // Dense mode: the select runs over the bucket itself, with no sample and no bucket pass.
@@ -330,14 +331,23 @@ static int launch_compress(const void* grad, float* residual, const uint32_t* ma
     if (le != cudaSuccess) return NSML_ERR_CUDA;
   }
   {
-    // Blocks draw chunks of the list by ticket, so the grid is free: a block per half the knob's candidates, at most two
-    // per SM, is fastest alone.  A knob above the default says that other calls fill the GPU: a block that waits for
-    // memory then holds what their passes need, so short lists get a few blocks that take many chunks (25M elements at
-    // ratio 0.01, eight streams, per step of 20 calls: 80 blocks 0.68 ms, 40 0.65, 20 0.64, 10 0.63) and long ones one per SM.
+    // Blocks draw chunks of the list by ticket, so the grid is free.  For a call that has the GPU to itself a block per
+    // chunk, at most two per SM, is fastest (more would find no chunk).  A knob above the default says that other calls
+    // fill the GPU: a block that waits for memory then holds what their passes need, so short lists get a few blocks
+    // that take many chunks each and long ones one block per SM.  25M-element buckets, eight streams, knob 8192, ms per
+    // step with 2 / 5 / 10 / 20 / 40 / 80 / 148 blocks: kept fraction 0.001 (2 buckets, 2 workers) 0.115 / 0.112 / 0.109
+    // / 0.110 / 0.112 / 0.116 / 0.124, 0.003 0.133 / 0.122 / 0.121 / 0.118 / 0.119 / 0.124 / 0.131, 0.01 (5 buckets, 4
+    // workers) 0.698 / 0.631 / 0.630 / 0.638 / 0.645 / 0.678 / 0.731: kListFewBlocks is near the best of all three.  A
+    // block per 32768 candidates alone (the fourth power of the excess at 8192) is right at 0.01 only (two blocks at 0.001).
+    // Long lists, 0.1: 1.14 / 0.549 / 0.382 / 0.363 / 0.357 / 0.352 / 0.355, with 296 0.378.
     LaunchScope scope(K_EMIT, st);
     const bool short_list = plan.expected <= 2.0 * dev.sms * kChunk;
-    const double knob = (double)g_list_block_candidates.load(std::memory_order_relaxed), over = knob / kListBlockCandidates;
-    const double want = plan.expected / (0.5 * knob * (short_list && over > 1.0 ? over * over * over : 1.0)) + 1.0;
+    const double over = (double)g_list_block_candidates.load(std::memory_order_relaxed) / kListBlockCandidates;
+    double want = plan.expected / kChunk + 1.0;  // a block per chunk
+    if (over > 1.0 && short_list && want > kListFewBlocks) {
+      want /= over * over * over * over;
+      if (want < kListFewBlocks) want = kListFewBlocks;
+    }
     const unsigned int cap = (over > 1.0 ? 1u : 2u) * dev.sms;
     const unsigned int grid = want < (double)cap ? (unsigned int)want : cap;
     // long lists: larger chunks, a block takes several
