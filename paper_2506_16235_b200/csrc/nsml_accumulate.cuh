@@ -15,12 +15,16 @@
 
 namespace nsml {
 
-// Dense elements per tile (the block's unit of work; 32 or 8 KB of shared memory).  The small tile is for
-// buckets that would otherwise give the large one fewer tiles than two per SM of work: what counts there is
-// that a tile's entries, and the round trips they take, are spread over many blocks.
+// Dense elements per tile (the block's unit of work; 32 or 8 KB of shared memory).  The small tile spreads a short
+// bucket's entries, and the round trips they take, over more blocks; it is taken while its blocks are one wave (1024
+// tiles; 7 blocks on each of 148 SMs are 1036), with a margin of a few.  Measured (us per sum, several in a row, small /
+// large tile).  Overwriting, W = 4 at 0.01 int8: 300k elements 7.9 / 8.4, 1M 10.0 / 9.9, 2.0M 11.9 / 11.5, 2.4M (a second
+// wave) 14.5 / 11.9; W = 2 at 0.3 float32: 1M 14.3 / 17.7, 2.0M 18.2 / 20.6.  Adding, W = 4 at 0.01: 300k 8.8 / 11.6, 1M
+// 12.4 / 18.1, 2.0M 14.6 / 20.0, 2.4M 19.5 / 20.1.  The large one's lead where a bucket of 1 to 2M elements is
+// overwritten with few entries is 7 per cent at most, the small one's where it is added to 30.
 constexpr int kDenseTileLarge = 8192;
 constexpr int kDenseTileSmall = 2048;
-constexpr int64_t kDenseTileSmallMaxN = 296LL * kDenseTileLarge;
+constexpr int64_t kDenseTileSmallMaxN = 1024LL * kDenseTileSmall;
 inline int dense_tile(int64_t n) { return n <= kDenseTileSmallMaxN ? kDenseTileSmall : kDenseTileLarge; }
 
 struct PayloadTable {

@@ -80,7 +80,7 @@ struct LaunchScope {  // brackets one kernel launch
 struct DeviceInfo {
   bool ready = false;
   int sms = 0;
-  int dense_small = 0, dense_large = 0, merge = 0;  // resident blocks per SM
+  int dense_small = 0, dense_large = 0, merge_small = 0, merge_large = 0;  // resident blocks per SM
   int sumsq = 0, feedback_add = 0;  // the same, streaming kernels
 };
 static DeviceInfo g_dev[64];
@@ -115,7 +115,8 @@ static int device_info(const DeviceInfo** out) {
     prepare(k_select_small<NSML_BF16, kSmallBlocks>, kSmallThreads, kSmallPerBlock * 4, &list_fits);
     prepare(k_sample<NSML_F32>, kSampleThreads, kSampleSmem, &list_fits);
     prepare(k_sample<NSML_BF16>, kSampleThreads, kSampleSmem, &list_fits);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.merge, k_merge<kDenseTileLarge>, kMergeThreads, 0);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.merge_small, k_merge<kDenseTileSmall>, kMergeThreads, 0);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.merge_large, k_merge<kDenseTileLarge>, kMergeThreads, 0);
     // The streaming kernels run as one wave of resident blocks (a second, partial wave would read
     // with a fraction of the SMs' loads in flight).
     auto resident = [&](auto kernel, int* out) {
@@ -130,7 +131,7 @@ static int device_info(const DeviceInfo** out) {
     if (e == cudaSuccess && (d.sumsq < 1 || d.feedback_add < 1)) e = cudaErrorUnknown;
     int coop = 0;
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-    if (e != cudaSuccess || d.dense_small < 1 || d.dense_large < 1 || list_fits < 1 || d.merge < 1 || !coop) {
+    if (e != cudaSuccess || d.dense_small < 1 || d.dense_large < 1 || list_fits < 1 || d.merge_small < 1 || d.merge_large < 1 || !coop) {
       cudaGetLastError();
       return NSML_ERR_CUDA;
     }
@@ -417,8 +418,9 @@ static int accumulate_impl(const void* const* payloads, const size_t* payload_by
   }
   {
     LaunchScope scope(K_MERGE, st, timed);
-    const unsigned int grid = grid_for(tiles, 1, dev->sms * dev->merge);
-    auto kernel = tile == kDenseTileLarge ? k_merge<kDenseTileLarge> : k_merge<kDenseTileSmall>;
+    const bool large = tile == kDenseTileLarge;
+    const unsigned int grid = grid_for(tiles, 1, dev->sms * (large ? dev->merge_large : dev->merge_small));
+    auto kernel = large ? k_merge<kDenseTileLarge> : k_merge<kDenseTileSmall>;
     launch_prio(kernel, dim3(grid), dim3(kMergeThreads), 0, st, false, 0, false, true, table, W, dense, (unsigned long long)n, zero_first, tiles, offsets, status);
   }
   if (cudaGetLastError() != cudaSuccess) return NSML_ERR_CUDA;

@@ -139,7 +139,7 @@ def test_workspace_sizes_never_shrink_with_n_or_w(nsml):
     # size at which a layout changes (tiles of the sum and the bucket pass, bins, groups of tiles) and in between
     largest = 2_147_483_647  # NSML_MAX_N
     at = {1, largest}
-    for base in (2048, 4096, 8192, 16_384, 163_840, 400_000, 2_424_832, 9_699_328, 1 << 24, 33_554_432, 1 << 26, 1 << 30):
+    for base in (2048, 4096, 8192, 16_384, 163_840, 400_000, 1 << 21, 2_424_832, 1 << 23, 9_699_328, 1 << 24, 33_554_432, 1 << 26, 1 << 30):
         at.update(base + d for d in (-1, 0, 1))
     at.update(int(1.13 ** i) for i in range(1, 176) if int(1.13 ** i) <= largest)
     sizes = sorted(at)

@@ -12,7 +12,7 @@ if torch.cuda.is_available():
     import paper_2506_16235_b200 as nsml
     from gpu_util import check_accumulate, payload_to_device
 
-SWITCH = 296 * 8192  # largest bucket that takes the small tile
+SWITCH = 1024 * 2048  # largest bucket that takes the small tile
 
 
 def crowded_payload(n, k, bits, seed):
@@ -27,7 +27,7 @@ def crowded_payload(n, k, bits, seed):
 
 
 @pytest.mark.parametrize("zero_first", [True, False])
-@pytest.mark.parametrize("n", [2047, 2048, 2049, SWITCH, SWITCH + 1, SWITCH + 8191])
+@pytest.mark.parametrize("n", [2047, 2048, 2049, SWITCH - 1, SWITCH, SWITCH + 1, SWITCH + 8191, 296 * 8192, 296 * 8192 + 1])
 def test_tile_edges(n, zero_first):
     want = [crowded_payload(n, min(n, 20_011), bits, n + bits) for bits in (8, 16, 32)]
     init = None if zero_first else np.random.default_rng(1).standard_normal(n).astype(np.float32)
@@ -43,7 +43,7 @@ def test_many_workers_most_of_them_sparse(W):
 
 def test_one_workspace_sized_for_the_largest_bucket_serves_them_all():
     # a gradient set in 25 MB buckets: the shorter ones need more room for their (smaller) tiles than the longest one
-    W, sizes = 8, (6_553_600, SWITCH, 2_000_000, 12_289)
+    W, sizes = 8, (6_553_600, 2_424_832, SWITCH, 2_000_000, 12_289)
     ws = nsml.alloc_bytes(nsml.nsml_accumulate_workspace_bytes(max(sizes), W), "cuda")
     for n in sizes:
         want = [crowded_payload(n, 1500, 8, n + w) for w in range(W)]
