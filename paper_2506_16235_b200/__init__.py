@@ -297,7 +297,8 @@ def nsml_compress(grad, ratio: float, bits: int = NSML_BITS_INT8, prune_mask=Non
         raise ValueError("grad must be a contiguous 1-D CUDA tensor")
     n = grad.numel()
     dtype = _grad_dtype(grad)
-    need = nsml_payload_bytes(n, ratio, bits)
+    ratio, bits = float(ratio), int(bits)  # (read once: a ratio may be a 0-d tensor)
+    need = lib.nsml_payload_bytes(n, ratio, bits)
     if need == 0:
         raise NsmlError(NSML_ERR_ARG, "nsml_compress")
     if payload is None:
@@ -310,7 +311,7 @@ def nsml_compress(grad, ratio: float, bits: int = NSML_BITS_INT8, prune_mask=Non
                 and prune_mask.numel() >= (n + 31) // 32):
             raise ValueError("prune_mask must be a contiguous CUDA tensor of ceil(n/32) 32-bit words")
         mask_ptr = prune_mask.data_ptr()
-    rc = lib.nsml_compress(grad.data_ptr(), n, dtype, float(ratio), int(bits), mask_ptr,
+    rc = lib.nsml_compress(grad.data_ptr(), n, dtype, ratio, bits, mask_ptr,
                            payload.data_ptr(), payload.numel(), workspace.data_ptr(), workspace.numel(),
                            _stream_ptr(stream))
     _check(rc, "nsml_compress")
@@ -424,14 +425,15 @@ def nsml_compress_feedback(grad, residual, ratio: float, bits: int = NSML_BITS_I
     n = grad.numel()
     if residual.dtype != torch.float32 or residual.numel() != n:
         raise ValueError("residual must be float32 with one element per gradient element")
-    need = nsml_payload_bytes(n, ratio, bits)
+    ratio, bits = float(ratio), int(bits)  # (read once: a ratio may be a 0-d tensor)
+    need = lib.nsml_payload_bytes(n, ratio, bits)
     if need == 0:
         raise NsmlError(NSML_ERR_ARG, "nsml_compress_feedback")
     if payload is None:
         payload = alloc_bytes(need, grad.device)
     if workspace is None:
         workspace = alloc_bytes(nsml_workspace_bytes(n, NSML_F32), grad.device)
-    rc = lib.nsml_compress_feedback(grad.data_ptr(), residual.data_ptr(), n, _grad_dtype(grad), float(ratio), int(bits),
+    rc = lib.nsml_compress_feedback(grad.data_ptr(), residual.data_ptr(), n, _grad_dtype(grad), ratio, bits,
                                     None if prune_mask is None else prune_mask.data_ptr(), payload.data_ptr(),
                                     payload.numel(), workspace.data_ptr(), workspace.numel(), _stream_ptr(stream))
     _check(rc, "nsml_compress_feedback")
@@ -477,8 +479,9 @@ def nsml_compress_host(grad_host, ratio: float, bits: int, payload_host, device_
     asynchronous copies), device_scratch a uint8 CUDA tensor.  Returns the payload size."""
     n = grad_host.numel()
     dtype = _grad_dtype(grad_host)
-    need = nsml_payload_bytes(n, ratio, bits)
-    rc = lib.nsml_compress_host(grad_host.data_ptr(), n, dtype, float(ratio), int(bits),
+    ratio, bits = float(ratio), int(bits)  # (read once: a ratio may be a 0-d tensor)
+    need = lib.nsml_payload_bytes(n, ratio, bits)
+    rc = lib.nsml_compress_host(grad_host.data_ptr(), n, dtype, ratio, bits,
                                 None if prune_mask_host is None else prune_mask_host.data_ptr(),
                                 payload_host.data_ptr(), payload_host.numel(),
                                 device_scratch.data_ptr(), device_scratch.numel(), _stream_ptr(stream))
