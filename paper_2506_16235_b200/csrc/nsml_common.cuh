@@ -59,7 +59,10 @@ __device__ __forceinline__ Window make_window(const Ctl* ctl) {
   Window w;
   const unsigned int hi = ctl->hi;
   w.grain = TYPE == NSML_BF16 ? 16u : ctl->grain;
-  w.lo = ctl->lo;  // 0: the sample holds too few non-zero keys; everything is listed, zeros too
+  // 0: the sample holds too few non-zero keys; everything is listed, zeros too.  At most infinity: a bucket with many
+  // NaN has a NaN's key here, and the bucket pass compares floats with it, so that it would list every key and count
+  // those below `lo` in bins that do not exist.
+  w.lo = min(ctl->lo, kInfKey);
   w.hi = hi > w.lo ? hi : 0x80000000u;
   const unsigned int span = (w.hi - w.lo - 1) / kMaxBins;
   w.shift = max(w.grain, span == 0 ? 0u : 32u - __clz(span));

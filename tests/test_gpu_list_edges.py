@@ -10,7 +10,7 @@ pytestmark = pytest.mark.gpu
 
 if torch.cuda.is_available():
     import paper_2506_16235_b200 as nsml
-    from gpu_util import check_compress, gpu_compress, mask_words, oracle_compress, assert_payload_equal
+    from gpu_util import check_compress, gpu_compress, mask_words, oracle_compress, to_device_grad, assert_payload_equal
     from test_gpu_compress import sampled_positions
 
 
@@ -165,3 +165,33 @@ def test_feedback_takes_selected_negative_zeros_out(n, ratio, hidden, bits):
             ref, want = error_feedback_step(g, want, ratio, bits, prune_mask_=mask if masked else None)
             assert_payload_equal(payload, ref)
             assert np.array_equal(residual.cpu().numpy().view(np.uint32), want.view(np.uint32))
+
+
+# more NaN (or infinities) than survivors: the sample's bounds are then themselves keys of NaN
+@pytest.mark.parametrize("word", [0x7FC00000, 0x7F810000, 0x7FFF0000, 0xFFC00000, 0x7F800000])
+@pytest.mark.parametrize("share", [0.03, 0.6, 1.0])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_many_nonfinite_values_are_reported_and_nothing_else_is_touched(dtype, share, word):
+    n, ratio = 700_001, 0.02
+    rng = np.random.default_rng(int(share * 100))
+    clean = gauss(n, 6)
+    bad = clean.view(np.uint32).copy()
+    bad[rng.random(n) < share] = word
+    bad = bad.view(np.float32)
+    if dtype == "bf16":
+        clean, bad = synth.f32_to_bf16_bits(clean), (bad.view(np.uint32) >> 16).astype(np.uint16)
+    need, room = nsml.nsml_payload_bytes(n, ratio, 8), nsml.nsml_workspace_bytes(n)
+    payload = torch.full((need + 4096,), 0xA5, dtype=torch.uint8, device="cuda")
+    ws = torch.full((room + (1 << 20),), 0xA5, dtype=torch.uint8, device="cuda")
+    residual = torch.zeros(n, device="cuda")
+    for call in ("plain", "residual"):
+        if call == "plain":
+            nsml.nsml_compress(to_device_grad(bad), ratio, 8, payload=payload, workspace=ws)
+        else:
+            nsml.nsml_compress_feedback(to_device_grad(bad), residual, ratio, 8, payload=payload, workspace=ws)
+        assert nsml.nsml_last_status(ws) == nsml.NSML_ERR_NONFINITE
+        assert bool((payload[need:] == 0xA5).all()) and bool((ws[room:] == 0xA5).all())
+    # and the workspace serves an ordinary call
+    out = nsml.nsml_compress(to_device_grad(clean), ratio, 8, payload=payload, workspace=ws)
+    assert nsml.nsml_last_status(ws) == 0
+    assert_payload_equal(out, oracle_compress(clean, ratio, 8))
