@@ -73,6 +73,35 @@ def payload_to_device(want: oracle.Payload) -> torch.Tensor:
     return torch.from_numpy(raw).cuda()
 
 
+def took_the_fallback(workspace: torch.Tensor) -> bool:
+    """Whether the last list-strategy compress, or mask build, on this workspace settled its threshold by rounds over the
+    list, the bucket or the weights because the sample did not cover it: units of work drawn in phase 3 of those rounds
+    (control block at the start of the workspace, `drawn` at byte 40)."""
+    return int(workspace[52:56].view(torch.int32).item()) != 0
+
+
+def sampled_positions(n, strata=16384):
+    """First positions the library's stratified sampler reads (one per stratum, a hashed offset inside it), restated from
+    its description so that a test can build a bucket on which the sample is misleading."""
+    s = np.arange(strata, dtype=np.uint64)
+    begin = s * np.uint64(n) // np.uint64(strata)
+    end = (s + np.uint64(1)) * np.uint64(n) // np.uint64(strata)
+    x = (s * np.uint64(0x9E3779B1) + np.uint64(0x85EBCA6B)) & np.uint64(0xFFFFFFFF)
+    x ^= x >> np.uint64(16)
+    x = (x * np.uint64(0x7FEB352D)) & np.uint64(0xFFFFFFFF)
+    x ^= x >> np.uint64(15)
+    x = (x * np.uint64(0x846CA68B)) & np.uint64(0xFFFFFFFF)
+    x ^= x >> np.uint64(16)
+    return (begin + x % (end - begin)).astype(np.int64)
+
+
+def sampled_elements(n, keys):
+    """All elements the sampler reads: `keys` neighbours (16 bytes, aligned) from each of 16384 strata."""
+    pos = sampled_positions(n) & ~np.int64(keys - 1)
+    pos = np.where(pos + keys > n, (n - keys) & ~np.int64(keys - 1), pos)
+    return np.unique((pos[:, None] + np.arange(keys)).reshape(-1))
+
+
 def check_accumulate(payload_tensors, oracle_payloads, n, zero_first, dense_init=None, max_abs=None):
     """GPU sum vs oracle: within 1e-6 of the bucket's largest magnitude."""
     if dense_init is None:

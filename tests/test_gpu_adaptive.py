@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 if torch.cuda.is_available():
     import paper_2506_16235_b200 as nsml
     from gpu_util import (CANARY, assert_payload_equal, check_accumulate, check_compress, mask_words,
-                          payload_to_device, to_device_grad)
+                          payload_to_device, sampled_elements, took_the_fallback, to_device_grad)
 
 L2_RTOL = 1e-12  # float64 sums of exact squares in another order: ~sqrt(n) * 2^-53 at worst
 
@@ -51,19 +51,20 @@ def test_l2_norm_reports_nonfinite():
 
 
 # ------------------------------------------------------------------ Step 2
-def gpu_mask(w, ratio):
+def gpu_mask(w, ratio, ws=None):
     n = w.size
     words = (n + 31) // 32
     buf = torch.full((words + 64,), -1515870811, dtype=torch.int32, device="cuda")  # 0xA5A5A5A5
-    ws = nsml.alloc_bytes(nsml.nsml_prune_workspace_bytes(n), "cuda")
+    if ws is None:
+        ws = nsml.alloc_bytes(nsml.nsml_prune_workspace_bytes(n), "cuda")
     nsml.nsml_prune_mask_build(torch.from_numpy(w).cuda(), ratio, prune_mask=buf, workspace=ws)
     status = nsml.nsml_last_status(ws)
     assert bool((buf[words:] == -1515870811).all()), "wrote past the end of the mask"
     return buf[:words].cpu().numpy().view(np.uint32), status
 
 
-def check_mask(w, ratio):
-    got, status = gpu_mask(w, ratio)
+def check_mask(w, ratio, ws=None):
+    got, status = gpu_mask(w, ratio, ws)
     assert status == 0, nsml.nsml_strerror(status)
     want = mask_words(oracle.prune_mask(w, ratio))
     assert np.array_equal(got, want), f"mask differs (n={w.size}, ratio={ratio})"
@@ -128,32 +129,22 @@ def test_prune_mask_25m_bucket():
     check_mask(w, 0.01)
 
 
-def prune_sampled_positions(n, strata=8192):
-    """Positions the mask build's stratified sampler reads (one per stratum, a hashed offset inside it),
-    restated from its description so that a test can build weights on which the sample misleads."""
-    s = np.arange(strata, dtype=np.uint64)
-    width = np.uint64(n // strata)
-    x = (s * np.uint64(0x9E3779B1) + np.uint64(0x85EBCA6B)) & np.uint64(0xFFFFFFFF)
-    x ^= x >> np.uint64(16)
-    x = (x * np.uint64(0x7FEB352D)) & np.uint64(0xFFFFFFFF)
-    x ^= x >> np.uint64(15)
-    x = (x * np.uint64(0x846CA68B)) & np.uint64(0xFFFFFFFF)
-    x ^= x >> np.uint64(16)
-    return (s * width + ((x * width) >> np.uint64(32))).astype(np.int64)
-
-
 @pytest.mark.parametrize("n", [70_001, 1 << 20])
 def test_prune_mask_misleading_sample_still_exact(n):
-    # tiny (then huge) magnitudes exactly where the sampler looks: the sampled window misses the threshold and
-    # the four-pass build has to produce the mask
+    # tiny (then huge) magnitudes exactly where the sampler looks: the bracket misses the threshold and the radix
+    # select over the weights has to produce the mask
     rng = np.random.default_rng(n)
     w = rng.standard_normal(n).astype(np.float32)
-    pos = prune_sampled_positions(n)
+    pos = sampled_elements(n, 4)
+    ws = nsml.alloc_bytes(nsml.nsml_prune_workspace_bytes(n), "cuda")
+    check_mask(w, 0.01, ws)
+    assert not took_the_fallback(ws)
     for fill in (1e-9, 1e9):
         w2 = w.copy()
         w2[pos] = (fill * (1.0 + rng.random(pos.size))).astype(np.float32)
         for ratio in (0.01, 0.5):
-            check_mask(w2, ratio)
+            check_mask(w2, ratio, ws)
+            assert took_the_fallback(ws)
 
 
 def test_prune_mask_two_pass_path_with_ties_in_the_threshold_bin():
@@ -174,11 +165,11 @@ def test_prune_mask_reports_nonfinite():
     assert status == nsml.NSML_ERR_NONFINITE
 
 
-@pytest.mark.parametrize("ratio", [0.01, 0.5])  # list strategy and dense strategy of Step 3
-def test_whole_algorithm_keeps_the_mask_build_error_visible(ratio):
+@pytest.mark.parametrize("n", [100_000, 400_000])  # Step 3 in one kernel; by the list (0.01) and over the bucket (0.5)
+@pytest.mark.parametrize("ratio", [0.01, 0.5])
+def test_whole_algorithm_keeps_the_mask_build_error_visible(ratio, n):
     # Steps 2 and 3 share one workspace: non-finite weights found while the mask is built (Step 2) must
     # still be reported after Step 3 has run on the same workspace
-    n = 100_000
     rng = np.random.default_rng(17)
     g = rng.standard_normal(n).astype(np.float32)
     w = rng.standard_normal(n).astype(np.float32)
@@ -269,9 +260,9 @@ def test_feedback_steps(bits, n):
     run_feedback(gs, 0.03, bits)
 
 
-def test_feedback_with_mask_bf16_and_dense_strategy():
+@pytest.mark.parametrize("n", [150_001, 400_001])  # one kernel; list and dense strategy
+def test_feedback_with_mask_bf16_and_dense_strategy(n):
     rng = np.random.default_rng(8)
-    n = 150_001
     mask = rng.random(n) < 0.4
     gs = [(rng.standard_normal(n).astype(np.float32).view(np.uint32) >> 16).astype(np.uint16) for _ in range(3)]
     run_feedback(gs, 0.02, 16, mask_bool=mask)
@@ -343,8 +334,8 @@ def test_prune_mask_small_tie_group_at_the_threshold():
 
 
 def test_feedback_when_fewer_than_k_sums_are_nonzero():
-    # list strategy whose candidate list comes out short: the list stage rebuilds it from the bucket, which
-    # here is the residual buffer holding gradient + residual
+    # list strategy whose sample finds too few non-zero keys: everything is listed, zeros too, and the zeros that fill
+    # the payload up are ranked by index
     rng = np.random.default_rng(41)
     n = 300_001
     gs = []

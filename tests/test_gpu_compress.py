@@ -11,7 +11,8 @@ pytestmark = pytest.mark.gpu
 
 if torch.cuda.is_available():
     import paper_2506_16235_b200 as nsml
-    from gpu_util import (assert_payload_equal, check_compress, gpu_compress, oracle_compress, to_device_grad)
+    from gpu_util import (assert_payload_equal, check_compress, gpu_compress, oracle_compress, sampled_elements,
+                          took_the_fallback, to_device_grad)
 
 SIZES = [1, 2, 3, 4, 5, 7, 31, 32, 33, 127, 128, 129, 511, 512, 513, 4095, 4096, 4097, 8191, 12289, 100003]
 
@@ -106,50 +107,47 @@ def test_bf16_buckets(n):
             check_compress(g, ratio, bits)
 
 
-def sampled_positions(n, strata=8192):
-    """Positions the library's stratified sampler reads (one per stratum, a
-    hashed offset inside it), restated from its description so that a test can
-    build a bucket on which the sample is misleading."""
-    s = np.arange(strata, dtype=np.uint64)
-    begin = s * np.uint64(n) // np.uint64(strata)
-    end = (s + np.uint64(1)) * np.uint64(n) // np.uint64(strata)
-    x = (s * np.uint64(0x9E3779B1) + np.uint64(0x85EBCA6B)) & np.uint64(0xFFFFFFFF)
-    x ^= x >> np.uint64(16)
-    x = (x * np.uint64(0x7FEB352D)) & np.uint64(0xFFFFFFFF)
-    x ^= x >> np.uint64(15)
-    x = (x * np.uint64(0x846CA68B)) & np.uint64(0xFFFFFFFF)
-    x ^= x >> np.uint64(16)
-    return (begin + x % (end - begin)).astype(np.int64)
-
-
 @pytest.mark.parametrize("n", [20000, 200000, 1 << 20])
 def test_misleading_sample_still_gives_the_exact_result(n):
-    # large magnitudes exactly where the sampler looks, small ones elsewhere:
-    # the sampled bracket then keeps far fewer than k elements and the repeat
-    # pass has to produce the list
+    # large magnitudes exactly where the sampler looks, small ones elsewhere: the list then holds far fewer than k
+    # elements and the result has to come from the bucket (20000 elements are taken without a sample)
+    ws = nsml.alloc_bytes(nsml.nsml_workspace_bytes(n), "cuda")
+
+    def check(g, ratio, bits):
+        payload = nsml.nsml_compress(to_device_grad(g), ratio, bits, workspace=ws)
+        assert nsml.nsml_last_status(ws) == 0
+        assert_payload_equal(payload, oracle_compress(g, ratio, bits))
+        return n > 163_840 and took_the_fallback(ws)
+
     rng = np.random.default_rng(n)
     g = (rng.standard_normal(n) * 1e-3).astype(np.float32)
-    pos = sampled_positions(n)
-    g[pos] = (100.0 + rng.random(pos.size)).astype(np.float32) * rng.choice(np.array([-1.0, 1.0], np.float32), pos.size)
-    for ratio in (0.1, 0.5):
-        check_compress(g, ratio, 8)
-    # and the opposite: zeros where the sampler looks (bracket starts at key 0)
+    assert not check(g, 0.1, 8)
+    pos = sampled_elements(n, 4)
+    g[pos] = (10.0 ** rng.uniform(2, 5, pos.size)).astype(np.float32) * rng.choice(np.array([-1.0, 1.0], np.float32), pos.size)
+    assert check(g, 0.1, 8) == (n > 163_840)
+    check(g, 0.5, 8)
+    # and the opposite: zeros where the sampler looks (everything is listed, the window is all keys)
     g = rng.standard_normal(n).astype(np.float32)
     g[pos] = 0.0
-    check_compress(g, 0.05, 16)
+    if np.count_nonzero(g) >= nsml.nsml_k_of(n, 0.05):
+        assert check(g, 0.05, 16) == (n > 163_840)
+    else:
+        check(g, 0.05, 16)
 
 
-def test_nonfinite_is_reported_not_trapped():
+# one kernel for the whole bucket; the sampled list; the bucket itself
+@pytest.mark.parametrize("n,ratio", [(9000, 0.1), (300_001, 0.1), (300_001, 0.5)])
+def test_nonfinite_is_reported_not_trapped(n, ratio):
     rng = np.random.default_rng(2)
     for bad in (np.inf, -np.inf, np.nan):
-        g = rng.standard_normal(9000).astype(np.float32)
+        g = rng.standard_normal(n).astype(np.float32)
         g[4321] = bad
-        _, status = gpu_compress(g, 0.1, 8)
+        _, status = gpu_compress(g, ratio, 8)
         assert status == nsml.NSML_ERR_NONFINITE
         with pytest.raises(oracle.NonFiniteGradient):
-            oracle_compress(g, 0.1, 8)
-    # the same workspace is usable afterwards
-    check_compress(rng.standard_normal(9000).astype(np.float32), 0.1, 8)
+            oracle_compress(g, ratio, 8)
+    # the next call is a clean one
+    check_compress(rng.standard_normal(n).astype(np.float32), ratio, 8)
 
 
 def test_payload_is_bit_reproducible():
@@ -275,11 +273,13 @@ def test_bounded_wait_runs_out_and_reports_timeout():
     assert nsml.nsml_last_status(ws) == 0
     assert_payload_equal(payload, oracle.compress(g, 0.01, 8))
 
-# The bucket pass gives every warp 2 KB of the bucket (one float32 segment of 512 elements, two bfloat16
-# segments) and every block eight warps: sizes at and around the segment, warp and block boundaries, with the
-# ragged last segment falling to the first, a middle and the last warp of a block, with and without a mask.
-PASS_EDGE_SIZES = [16384, 16385, 16384 + 511, 16384 + 512, 16384 + 513, 16384 + 1024 + 1, 20480 - 1, 20480, 20480 + 1,
+# The bucket pass gives every warp 2 KB of the bucket (512 float32 or 1024 bfloat16 elements) and every block eight
+# warps: sizes at and around the boundaries of warps and blocks, with the ragged end falling to the first, a middle and
+# the last warp of a block, with and without a mask.  The same sizes as they are (one kernel takes those, without a pass)
+# and 40 tiles on.
+EDGE_SIZES = [16384, 16385, 16384 + 511, 16384 + 512, 16384 + 513, 16384 + 1024 + 1, 20480 - 1, 20480, 20480 + 1,
                    24576 + 7 * 512 + 3, 8 * 4096 - 512 + 5, 8 * 4096 + 1]
+PASS_EDGE_SIZES = EDGE_SIZES + [163_840 + n for n in EDGE_SIZES]
 
 
 @pytest.mark.parametrize("n", PASS_EDGE_SIZES)
@@ -306,10 +306,10 @@ def test_list_block_candidates_knob_does_not_change_the_payload(candidates):
     g = (rng.standard_normal(n) * 10.0 ** rng.uniform(-4, -1, n)).astype(np.float32)
     nsml.nsml_set_list_block_candidates(candidates)
     try:
-        for ratio in (0.002, 0.02, 0.2):  # cluster shape and small shape of the list stage
+        for ratio in (0.002, 0.02, 0.2):  # seven chunks of 2048 candidates to four hundred
             check_compress(g, ratio, 8)
             check_compress(g, ratio, 16)
-        # the large shape (more than about 1.2M expected candidates): one block per SM above the default setting
+        # long lists (more than about 600,000 expected candidates): one block per SM above the default setting
         big = (rng.standard_normal(8_000_003) * 10.0 ** rng.uniform(-4, -1, 8_000_003)).astype(np.float32)
         check_compress(big, 0.2, 8)
     finally:

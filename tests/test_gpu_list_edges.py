@@ -4,26 +4,20 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 import synth
 
 pytestmark = pytest.mark.gpu
 
 if torch.cuda.is_available():
     import paper_2506_16235_b200 as nsml
-    from gpu_util import check_compress, gpu_compress, mask_words, oracle_compress, to_device_grad, assert_payload_equal
-    from test_gpu_compress import sampled_positions
+    from gpu_util import (assert_payload_equal, check_compress, gpu_compress, mask_words, oracle_compress, sampled_elements,
+                          took_the_fallback, to_device_grad)
 
 
 def gauss(n, seed, spread=2.0):
     rng = np.random.default_rng(seed)
     return (rng.standard_normal(n) * 10.0 ** rng.uniform(-4.0, -4.0 + spread, n)).astype(np.float32)
-
-
-def sampled_elements(n, keys):
-    """All elements the sampler reads: `keys` neighbours (aligned) from each of 16384 strata."""
-    pos = sampled_positions(n, 16384) & ~np.int64(keys - 1)
-    pos = np.where(pos + keys > n, (n - keys) & ~np.int64(keys - 1), pos)
-    return np.unique((pos[:, None] + np.arange(keys)).reshape(-1))
 
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
@@ -195,3 +189,48 @@ def test_many_nonfinite_values_are_reported_and_nothing_else_is_touched(dtype, s
     out = nsml.nsml_compress(to_device_grad(clean), ratio, 8, payload=payload, workspace=ws)
     assert nsml.nsml_last_status(ws) == 0
     assert_payload_equal(out, oracle_compress(clean, ratio, 8))
+
+
+# buckets of more than 8192 tiles (float32: 33,554,432 elements, bfloat16 twice as many): the list counts candidates per
+# group of two or four tiles.  even: a run of 128 list entries spans more tiles than one round of 64 covers; crowded: all
+# of them in a few tiles; close: the threshold's bin overflows and is refined over the list.
+@pytest.mark.parametrize("n,dtype,kind", [(33_554_433, "f32", "even"), (33_554_433, "f32", "crowded"), (33_554_433, "f32", "close"),
+                                          (67_108_865, "bf16", "even"), (67_112_961, "f32", "crowded")])
+def test_buckets_of_more_tiles_than_groups(n, dtype, kind):
+    rng = np.random.default_rng(n)
+    g = rng.standard_normal(n, dtype=np.float32)
+    ratios = (0.00005, 0.01, 0.2)
+    if kind == "crowded":
+        g[n // 3:n // 3 + n // 50] *= np.float32(1000.0)
+        g[-4097:] *= np.float32(1000.0)
+    if kind == "close":
+        ratios = (0.01,)
+        g *= np.float32(1e-4)
+        where = rng.choice(n, 600_000, replace=False)
+        g[where] = (np.float32(0.5).view(np.uint32) + rng.integers(0, 3000, where.size).astype(np.uint32)).view(np.float32)
+    raw = synth.f32_to_bf16_bits(g) if dtype == "bf16" else g
+    wants = oracle.compress_many(oracle.widen_bf16(raw) if dtype == "bf16" else g, ratios, 8)
+    grad, ws = to_device_grad(raw), nsml.alloc_bytes(nsml.nsml_workspace_bytes(n), "cuda")
+    for ratio, want in zip(ratios, wants):
+        payload = nsml.nsml_compress(grad, ratio, 8, workspace=ws)
+        assert nsml.nsml_last_status(ws) == 0
+        assert took_the_fallback(ws) == (kind == "close")
+        assert_payload_equal(payload, want)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_feedback_on_more_tiles_than_groups(dtype):
+    from oracle.adaptive import error_feedback_step
+    n = 33_554_433 + 5000
+    rng = np.random.default_rng(n)
+    g = rng.standard_normal(n, dtype=np.float32)
+    raw = g
+    if dtype == "bf16":
+        raw = synth.f32_to_bf16_bits(g)
+        g = oracle.widen_bf16(raw)
+    start = rng.standard_normal(n, dtype=np.float32)
+    residual = torch.from_numpy(start.copy()).cuda()
+    payload = nsml.nsml_compress_feedback(to_device_grad(raw), residual, 0.01, 16)
+    want, left = error_feedback_step(g, start, 0.01, 16)
+    assert_payload_equal(payload, want)
+    assert np.array_equal(residual.cpu().numpy().view(np.uint32), left.view(np.uint32))

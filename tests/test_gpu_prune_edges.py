@@ -3,7 +3,7 @@ import numpy as np
 import pytest
 
 from test_gpu_adaptive import check_mask
-from test_gpu_list_edges import sampled_elements
+from gpu_util import sampled_elements
 
 pytestmark = pytest.mark.gpu
 
