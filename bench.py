@@ -201,6 +201,9 @@ class Workload:
         k = self.nsml.nsml_k_of(n, ratio)
         vb = 1 if bits == 8 else 2
         s = 4 * ((k + 1023) // 1024) if bits == 8 else 0
+        if n <= 163_840:  # one kernel that holds the bucket in shared memory
+            self.account(acc, "k_select_small", esize * n + 4 * k + vb * k + s)
+            return
         if self.nsml.nsml_compress_strategy(n, ratio) == 1:
             # dense strategy: the select reads the bucket itself once, survivors written and re-read
             self.account(acc, "k_clear", 256 + 4 * 4 * 4096)
@@ -220,7 +223,7 @@ class Workload:
             if not zero_first:
                 total += 8 * k
         self.account(acc, "k_merge", total)
-        self.account(acc, "k_partition", 4 * len(ks_bits) * (n // 8192 + 2))
+        self.account(acc, "k_partition", 4 * len(ks_bits) * (n // (2048 if n <= 1 << 21 else 8192) + 2))
 
 
 class Lanes:

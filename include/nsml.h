@@ -23,8 +23,8 @@
  *     caller before and after the call.  "host pointer" = ordinary memory.
  *   - Device work is enqueued on `stream` (a cudaStream_t passed as void*, NULL
  *     = the default stream) and the call returns without synchronising.  The
- *     short, latency-bound kernels of a call (sample, list stage,
- *     partition) are launched at the device's highest stream priority, whatever
+ *     short, latency-bound kernels of a call (sample, list stage, small
+ *     buckets, partition) are launched at the device's highest stream priority, whatever
  *     the priority of `stream`: with several buckets in flight on several
  *     streams they are then placed between the blocks of other buckets'
  *     streaming passes instead of behind them.  Order within `stream` is kept.
@@ -33,6 +33,9 @@
  *     ran out) are written to a status word at the start of `workspace`; read it
  *     with nsml_last_status().
  *   - The library allocates no device memory: scratch comes in as `workspace`.
+ *     A calling thread's first nsml_grad_l2 that waits for the norm, or
+ *     nsml_compress_adaptive that needs it, allocates a few bytes of page-locked
+ *     host memory, which the thread keeps until it ends.
  *     Two calls that share a workspace must not overlap on the GPU.
  */
 #ifndef NSML_H
@@ -211,17 +214,17 @@ int nsml_compress(const void* grad, int64_t n, int grad_dtype, double ratio, int
                   const uint32_t* prune_mask, void* payload, size_t payload_capacity,
                   void* workspace, size_t workspace_bytes, void* stream);
 
-/* Which of its two internal strategies nsml_compress takes for (n, ratio) on
- * the current device.  Both give the same payload; this is information for
- * byte accounting (the paper prescribes no strategy).
+/* Which of its two strategies for large buckets nsml_compress takes for
+ * (n, ratio) on the current device.  Both give the same payload; this is
+ * information for byte accounting (the paper prescribes no strategy).
  *   NSML_STRATEGY_LIST   a stratified sample bounds the threshold from both
  *                        sides, one streaming pass keeps the candidates above
  *                        the lower bound, the exact threshold is found among
  *                        the few keys of one bin between the bounds
  *   NSML_STRATEGY_DENSE  a radix select runs over the bucket itself (high
- *                        kept fractions, and buckets too small to sample)
- * (Buckets of up to 163,840 elements are taken by one kernel of their own,
- * whichever of the two this names.)
+ *                        kept fractions)
+ * Buckets of up to 163,840 elements are taken by one kernel that holds them in
+ * shared memory, whichever of the two this names for them.
  * Returns the strategy, or NSML_ERR_ARG / NSML_ERR_CUDA. */
 #define NSML_STRATEGY_LIST 0
 #define NSML_STRATEGY_DENSE 1

@@ -211,7 +211,8 @@ def nsml_set_list_block_candidates(candidates: int) -> None:
 
 
 def nsml_compress_strategy(n: int, ratio: float) -> int:
-    """0 = sampled candidate list, 1 = dense select over the bucket (current device)."""
+    """0 = sampled candidate list, 1 = dense select over the bucket (current device; up to 163,840 elements one kernel takes
+    the call whatever this says)."""
     rc = int(lib.nsml_compress_strategy(int(n), float(ratio)))
     if rc < 0:
         raise NsmlError(rc, "nsml_compress_strategy")

@@ -5,9 +5,11 @@
 //           (k_sample, k_prune_pass, k_prune_finish)
 //   Step 3  "accumulate the local filtered gradients": the bucket that is
 //           compressed is gradient + residual, and the residual keeps what the
-//           payload does not carry (k_feedback_add, k_feedback_subtract)
-// All of them stream the bucket with 16-byte loads, block-cyclically, so that
-// the grid reads one moving window of memory.
+//           payload does not carry (k_feedback_add, k_feedback_subtract: around
+//           the dense select; the other strategies do both themselves)
+// The streaming kernels read with 16-byte loads on one moving window of memory:
+// k_sumsq and k_feedback_add as one wave of blocks that take tiles block-cyclically,
+// k_prune_pass with a short-lived block per tile.
 #pragma once
 
 #include "nsml_accumulate.cuh"

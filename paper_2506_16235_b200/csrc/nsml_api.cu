@@ -151,12 +151,12 @@ static inline unsigned int grid_for(unsigned long long work_items, unsigned long
   return (unsigned int)blocks;
 }
 
-// The short, latency-bound kernels (sample, gather, list stage, partition) are launched at the highest stream
-// priority.  When several buckets are in flight on several streams, every bucket pass that is ready sits in
+// The short, latency-bound kernels (sample, list stage, small select, mask finish, partition) are launched at the
+// highest stream priority.  When several buckets are in flight on several streams, every bucket pass that is ready sits in
 // front of the device's block scheduler with thousands of blocks to place; a list-stage kernel that becomes
 // ready later is otherwise placed only after all of them, so the passes of a step ran first, back to back,
-// and the list stages afterwards with nothing to overlap them (measured with a timer in every kernel:
-// 250 us of an 800 us step).  At high priority its few blocks are placed as soon as blocks of the running pass
+// and the list stages afterwards with nothing to overlap them (measured with a timer in every kernel, before the list
+// stage was rebuilt: 250 us of an 800 us step).  At high priority its few blocks are placed as soon as blocks of the running pass
 // retire, and it runs beside the next pass.
 static int high_priority() {
   static const int p = [] {
@@ -238,7 +238,8 @@ constexpr double kListFewBlocks = 10;       // blocks for a short list where the
 static std::atomic<int> g_list_block_candidates{kListBlockCandidates};
 
 // Dense mode: the select runs over the bucket itself, with no sample and no bucket pass.
-// Taken when the bucket cannot be sampled and when the candidate list would be about as large as the bucket.
+// Taken when the candidate list would be about as large as the bucket.  (What cannot be sampled is taken by use_small,
+// which is asked first.)
 static bool use_dense(int64_t n, int64_t k) {
   const double p_keep = (double)k / (double)n;
   return p_keep >= kDenseRatioAny || sample_plan(n, k, NSML_F32).rank_lo == 0;

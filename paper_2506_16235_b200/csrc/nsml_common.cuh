@@ -27,7 +27,7 @@ constexpr int kMaxPolls = 1 << 22;
 struct Ctl {
   int status;                 // first device-detected error (NSML_ERR_*), 0 = ok
   unsigned int lo, hi;        // sampled bounds of the threshold key: probably lo <= T < hi
-  unsigned int barrier;       // arrivals at the finalize kernel's grid barriers
+  unsigned int barrier;       // arrivals at the dense select's grid barriers
   unsigned int grain;         // the sampled keys (nearly all of them) are multiples of 1 << grain: 16, 13 or 0
   unsigned int ticket;        // chunks of the list handed out
   unsigned int fallback;      // a bin that was taken for a single key holds others
@@ -74,8 +74,8 @@ constexpr int kSegElems = 512;            // granule of the index ranges that th
 constexpr int kTileBytes = 16384;         // bucket bytes per tile of the candidate list: what a block of the bucket pass takes
 constexpr int kMaxGroups = 8192;          // the bucket pass keeps a candidate count per group of tiles (of one tile, up to 32M
                                           // float32 or 64M bfloat16 elements)
-constexpr int kMaxFinalizeBlocks = 1024;  // upper bound on blocks of the finalize kernels
-constexpr int kChunk = 2048;              // candidates a block of the list stage takes at a time
+constexpr int kMaxFinalizeBlocks = 1024;  // upper bound on blocks of the dense select
+constexpr int kChunk = 2048;              // candidates a block of the list stage takes at a time (long lists: twice that)
 
 // The keys inside the window are also kept by bin, up to this many per bin: four times what is to be expected where the
 // window is widest (kept fraction a quarter: 2 per cent of the bucket over at least 2048 bins).

@@ -1,8 +1,8 @@
 // Bucket -> payload without a candidate list, in one cooperative kernel.
 //
-// For calls that keep a large fraction of the bucket (or whose bucket is too
-// small to sample) a candidate list would be about as large as the bucket, so
-// the radix select (12 + 12 + 7 bits of the magnitude key; Alg. 2 Step 3 read
+// For calls that keep a large fraction of a bucket (and one that is not held in
+// shared memory as a whole, nsml_small.cuh) a candidate list would be about as
+// large as the bucket, so the radix select (12 + 12 + 7 bits of the magnitude key; Alg. 2 Step 3 read
 // as: keep the k largest |g|, ties by lower index) runs over the bucket itself.
 // Block b owns the index range of its share of the 512-element segments: entry
 // j of the block is element range_start + j, zeros and pruned elements included

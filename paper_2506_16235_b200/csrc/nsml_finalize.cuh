@@ -1,11 +1,14 @@
-// What the two select kernels share (nsml_list.cuh: the exact top-k of a candidate
-// list; nsml_dense.cuh: of the bucket itself): grid barriers, block-wide sums and
-// scans, the resolution of a key digit, the payload header, the quantisation
-// (Alg. 2 Step 1 "quantize" for fp16; int8 per block of 1024 survivors).
+// What the select kernels share (nsml_list.cuh: the exact top-k of a candidate
+// list; nsml_small.cuh: of a bucket in shared memory; nsml_dense.cuh: of a large
+// bucket): their parameters, the payload header and a survivor's value on its way
+// out (Alg. 2 Step 1 "quantize" for fp16); and what the dense select alone uses:
+// grid barriers, block-wide sums, the resolution of a key digit, the int8
+// quantisation per block of 1024 survivors.
 //
-// All blocks of a select kernel are co-resident (cooperative launch, or one
-// thread-block cluster).  Every barrier wait is bounded: when it runs out the
-// block records NSML_ERR_TIMEOUT and leaves; the others then time out as well.
+// The dense select is the only kernel whose blocks meet at grid barriers and have
+// to be co-resident (cooperative launch).  Every barrier wait is bounded: when it
+// runs out the block records NSML_ERR_TIMEOUT and leaves; the others then time out
+// as well.
 #pragma once
 
 #include "nsml_codec.cuh"
@@ -15,7 +18,7 @@
 
 namespace nsml {
 
-// Shapes of the dense select: small buckets run as 256-thread blocks with 8192 cached values, large ones as two
+// Shapes of the dense select: up to 8192 elements per SM run as 256-thread blocks with 8192 cached values, more as two
 // 512-thread blocks per SM that hold 2 x 23040 values, 6.8M elements over 148 SMs (a 25 MB float32 bucket stays on
 // chip).
 constexpr int kFinSmallThreads = 256, kFinSmallCache = 8192;
@@ -32,7 +35,7 @@ struct FinalizeParams {
   unsigned int tiles;
   TileList list;
   float* raw_val;
-  float* residual;                   // list strategy with local accumulation: holds gradient + residual; what the payload carries is taken out
+  float* residual;                   // local accumulation in one call: holds gradient + residual; what the payload carries is taken out (dense select: by kernels of its own)
   unsigned char* payload;
   PayloadLayout P;
 };
@@ -45,7 +48,6 @@ struct FinalizeShared {
   unsigned short und[THREADS / 32][kUndCap];
   unsigned long long red[(THREADS / 32)];
   unsigned long long run[2 * (THREADS / 32)];  // write phase: survivors per (warp, run)
-  unsigned int scan[(THREADS / 32)];
   unsigned int tot[(THREADS / 32)];
   unsigned int out[3];
   float qmax[(THREADS / 32)];
@@ -64,30 +66,6 @@ __device__ __forceinline__ unsigned long long block_sum(unsigned long long v, Fi
 #pragma unroll
   for (int w = 0; w < (THREADS / 32); ++w) s += sh.red[w];
   return s;
-}
-
-// Exclusive prefix over the block in thread order; `total` = sum over the block.
-template <int THREADS>
-__device__ __forceinline__ unsigned int block_excl_scan(unsigned int v, unsigned int& total, FinalizeShared<THREADS>& sh) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  unsigned int incl = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const unsigned int up = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-    if (lane >= o) incl += up;
-  }
-  __syncthreads();  // sh.scan may still be read from an earlier call
-  if (lane == 31) sh.scan[warp] = incl;
-  __syncthreads();
-  unsigned int before = 0, all = 0;
-#pragma unroll
-  for (int w = 0; w < (THREADS / 32); ++w) {
-    const unsigned int c = sh.scan[w];
-    if (w < warp) before += c;
-    all += c;
-  }
-  total = all;
-  return before + incl - v;
 }
 
 // All blocks arrive, then all leave.  `target` = barrier ordinal * gridDim.x.
@@ -148,7 +126,7 @@ __device__ __forceinline__ void resolve_digit(const unsigned int* ghist, unsigne
 }
 
 // Clears the control block and the histograms of a workspace (what the sample
-// kernel does on the list path) ahead of a dense-mode finalize.
+// kernel does on the list path) ahead of the dense select.
 __global__ void __launch_bounds__(kCta) k_clear(uint4* __restrict__ region, unsigned int count16, int keep_status) {
   for (unsigned int i = blockIdx.x * kCta + threadIdx.x; i < count16; i += gridDim.x * kCta)
     region[i] = make_uint4((i == 0 && keep_status) ? reinterpret_cast<const unsigned int*>(region)[0] : 0u, 0u, 0u, 0u);
@@ -231,10 +209,7 @@ __device__ __forceinline__ void quantize_block(const FinalizeParams& p, Finalize
 }
 
 // int8 only, after a grid barrier behind the write phase: every block of 1024 survivors parked in raw_val
-// becomes codes and a scale, a group of 256 threads per block.  (Measured against letting whichever thread
-// block delivers a payload block's last survivor quantise it, with no barrier: the atomic, the fences and the
-// read-back cost that variant as much as the barrier costs this one, 34.9 against 33.2 us for the list stage
-// of a 25M-element bucket.)
+// becomes codes and a scale, a group of 256 threads per block.
 template <int THREADS>
 __device__ __forceinline__ void quantize_all(const FinalizeParams& p, FinalizeShared<THREADS>& sh) {
   const unsigned long long qblocks = (p.k + NSML_QBLOCK - 1) / NSML_QBLOCK;
