@@ -204,10 +204,10 @@ class Workload:
         if n <= 163_840:  # one kernel that holds the bucket in shared memory
             self.account(acc, "k_select_small", esize * n + 4 * k + vb * k + s)
             return
-        if self.nsml.nsml_compress_strategy(n, ratio) == 1:
-            # dense strategy: the select reads the bucket itself once, survivors written and re-read
-            self.account(acc, "k_clear", 256 + 4 * 4 * 4096)
-            self.account(acc, "k_finalize_dense", esize * n + 8 * k + 4 * k + vb * k + s)
+        if self.nsml.nsml_compress_strategy(n, ratio) == 1 or (esize == 2 and ratio >= 0.1):
+            # dense strategy: the select reads the bucket itself once
+            self.account(acc, "k_clear", 256 + 4 * 4 * 4096 + 4 * 8192)
+            self.account(acc, "k_select_grid", esize * n + 4 * k + vb * k + s)
             return
         self.account(acc, "k_sample", 16 * 16384)
         # candidates: 16-bit offset in the tile + value (bfloat16: both in 32 bits)

@@ -221,8 +221,11 @@ int nsml_compress(const void* grad, int64_t n, int grad_dtype, double ratio, int
  *                        sides, one streaming pass keeps the candidates above
  *                        the lower bound, the exact threshold is found among
  *                        the few keys of one bin between the bounds
- *   NSML_STRATEGY_DENSE  a radix select runs over the bucket itself (high
- *                        kept fractions)
+ *   NSML_STRATEGY_DENSE  one cooperative kernel selects from the bucket itself,
+ *                        which it holds in shared memory as far as that goes
+ *                        (kept fractions from 0.125 on; bfloat16 buckets are
+ *                        taken this way from 0.1 on, which this function, not
+ *                        told the type, does not say)
  * Buckets of up to 163,840 elements are taken by one kernel that holds them in
  * shared memory, whichever of the two this names for them.
  * Returns the strategy, or NSML_ERR_ARG / NSML_ERR_CUDA. */

@@ -3,13 +3,12 @@
 //   Step 2  the pruning mask built from the weights: the ceil(0.5*(1-ratio)*n)
 //           parameters of smallest magnitude, ties by lower index
 //           (k_sample, k_prune_pass, k_prune_finish)
-//   Step 3  "accumulate the local filtered gradients": the bucket that is
-//           compressed is gradient + residual, and the residual keeps what the
-//           payload does not carry (k_feedback_add, k_feedback_subtract: around
-//           the dense select; the other strategies do both themselves)
+// (Step 3, "accumulate the local filtered gradients", is part of the compress
+// kernels: the bucket is gradient + residual, and the residual keeps what the
+// payload does not carry.)
 // The streaming kernels read with 16-byte loads on one moving window of memory:
-// k_sumsq and k_feedback_add as one wave of blocks that take tiles block-cyclically,
-// k_prune_pass with a short-lived block per tile.
+// k_sumsq as one wave of blocks that take tiles block-cyclically, k_prune_pass
+// with a short-lived block per tile.
 #pragma once
 
 #include "nsml_accumulate.cuh"
@@ -96,70 +95,6 @@ k_sumsq(BucketSrc<DTYPE> src, unsigned long long n, SumsqCtl* ctl, double* __res
       to_host->sumsq = total;
       to_host->status = __ldcg(&ctl->status);
     }
-  }
-}
-
-// ------------------------------------------------------------------------
-// Step 3, local accumulation.  residual <- gradient + residual (one float32
-// add per element); the sum is what gets compressed.
-// ------------------------------------------------------------------------
-template <int DTYPE>
-__global__ void __launch_bounds__(kCta)
-k_feedback_add(BucketSrc<DTYPE> src, float* __restrict__ residual, unsigned long long n) {
-  const unsigned long long tiles = (n + kStreamTile - 1) / kStreamTile;
-  for (unsigned long long tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-    const unsigned long long base = tile * kStreamTile;
-    if (base + kStreamTile <= n) {
-      uint32_t g[kStreamLoads][4];
-      float4 r[kStreamLoads];
-#pragma unroll
-      for (int u = 0; u < kStreamLoads; ++u) {
-        const unsigned long long i0 = base + (unsigned long long)(u * kCta + threadIdx.x) * 4;
-        src.load_full4(i0, g[u]);
-        r[u] = *reinterpret_cast<const float4*>(residual + i0);
-      }
-#pragma unroll
-      for (int u = 0; u < kStreamLoads; ++u) {
-        const unsigned long long i0 = base + (unsigned long long)(u * kCta + threadIdx.x) * 4;
-        float4 s;
-        s.x = __fadd_rn(__uint_as_float(g[u][0]), r[u].x);
-        s.y = __fadd_rn(__uint_as_float(g[u][1]), r[u].y);
-        s.z = __fadd_rn(__uint_as_float(g[u][2]), r[u].z);
-        s.w = __fadd_rn(__uint_as_float(g[u][3]), r[u].w);
-        *reinterpret_cast<float4*>(residual + i0) = s;
-      }
-    } else {
-      for (unsigned long long i = base + threadIdx.x; i < n; i += kCta)
-        residual[i] = __fadd_rn(__uint_as_float(src.load1(i)), residual[i]);
-    }
-  }
-}
-
-// residual[idx_j] <- residual[idx_j] - v'_j for every payload entry, v' being the
-// value a receiver reconstructs (one float32 subtraction).  Indices are unique,
-// so entries do not interfere.
-__global__ void __launch_bounds__(kCta)
-k_feedback_subtract(const unsigned char* __restrict__ payload, float* __restrict__ residual, unsigned long long n,
-                    int* status) {
-  const nsml_payload_header* h = reinterpret_cast<const nsml_payload_header*>(payload);
-  if (!header_ok(h, n)) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) set_status(status, NSML_ERR_PAYLOAD);
-    return;
-  }
-  const unsigned long long k = h->k;
-  const uint32_t* idx = reinterpret_cast<const uint32_t*>(payload + h->idx_off);
-  const unsigned char* val = payload + h->val_off;
-  const float* scale = reinterpret_cast<const float*>(payload + h->scale_off);
-  const int bits = (int)h->bits;
-  for (unsigned long long j = (unsigned long long)blockIdx.x * kCta + threadIdx.x; j < k;
-       j += (unsigned long long)gridDim.x * kCta) {
-    const uint32_t i = idx[j];
-    float v;
-    if (bits == NSML_BITS_INT8) v = decode_i8(reinterpret_cast<const signed char*>(val)[j], scale[j >> 10]);
-    else if (bits == NSML_BITS_FP16) v = decode_f16(reinterpret_cast<const uint16_t*>(val)[j]);
-    else v = reinterpret_cast<const float*>(val)[j];
-    if (i < n) residual[i] = __fsub_rn(residual[i], v);
-    else set_status(status, NSML_ERR_PAYLOAD);
   }
 }
 

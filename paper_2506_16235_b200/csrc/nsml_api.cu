@@ -12,7 +12,7 @@
 #include "nsml_common.cuh"
 #include "nsml_compact.cuh"
 #include "nsml_finalize.cuh"
-#include "nsml_dense.cuh"
+#include "nsml_grid.cuh"
 #include "nsml_list.cuh"
 #include "nsml_select.cuh"
 #include "nsml_small.cuh"
@@ -20,13 +20,13 @@
 namespace nsml {
 
 enum KernelId {
-  K_SAMPLE = 0, K_COMPACT_BUCKET, K_EMIT, K_PARTITION, K_MERGE, K_CLEAR, K_FINALIZE_DENSE,
-  K_SUMSQ, K_FEEDBACK_ADD, K_FEEDBACK_SUBTRACT, K_PRUNE_PASS, K_PRUNE_FINISH, K_SELECT_SMALL, K_COUNT
+  K_SAMPLE = 0, K_COMPACT_BUCKET, K_EMIT, K_PARTITION, K_MERGE, K_CLEAR, K_SELECT_GRID,
+  K_SUMSQ, K_PRUNE_PASS, K_PRUNE_FINISH, K_SELECT_SMALL, K_COUNT
 };
 
 static const char* const kKernelNames[K_COUNT] = {"k_sample", "k_compact_bucket", "k_emit", "k_partition", "k_merge",
-                                                  "k_clear", "k_finalize_dense", "k_sumsq", "k_feedback_add",
-                                                  "k_feedback_subtract", "k_prune_pass", "k_prune_finish", "k_select_small"};
+                                                  "k_clear", "k_select_grid", "k_sumsq", "k_prune_pass", "k_prune_finish",
+                                                  "k_select_small"};
 
 static std::atomic<int64_t> g_launches{0};
 
@@ -80,8 +80,7 @@ struct LaunchScope {  // brackets one kernel launch
 struct DeviceInfo {
   bool ready = false;
   int sms = 0;
-  int dense_small = 0, dense_large = 0, merge_small = 0, merge_large = 0;  // resident blocks per SM
-  int sumsq = 0, feedback_add = 0;  // the same, streaming kernels
+  int merge_small = 0, merge_large = 0, grid = 0, sumsq = 0;  // resident blocks per SM
 };
 static DeviceInfo g_dev[64];
 static std::mutex g_dev_mutex;
@@ -100,10 +99,14 @@ static int device_info(const DeviceInfo** out) {
       if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, kernel, threads, smem);
       if (*resident == 0 || r < *resident) *resident = r;
     };
-    prepare(k_finalize_dense<NSML_F32, kFinSmallThreads, kFinSmallCache>, kFinSmallThreads, finalize_dyn_smem(kFinSmallCache), &d.dense_small);
-    prepare(k_finalize_dense<NSML_BF16, kFinSmallThreads, kFinSmallCache>, kFinSmallThreads, finalize_dyn_smem(kFinSmallCache), &d.dense_small);
-    prepare(k_finalize_dense<NSML_F32, kFinLargeThreads, kFinDenseLargeCache>, kFinLargeThreads, finalize_dyn_smem(kFinDenseLargeCache), &d.dense_large);
-    prepare(k_finalize_dense<NSML_BF16, kFinLargeThreads, kFinDenseLargeCache>, kFinLargeThreads, finalize_dyn_smem(kFinDenseLargeCache), &d.dense_large);
+    prepare(k_select_grid<NSML_F32, false, false>, kGridThreads, kGridSmem, &d.grid);
+    prepare(k_select_grid<NSML_F32, false, true>, kGridThreads, kGridSmem, &d.grid);
+    prepare(k_select_grid<NSML_F32, true, false>, kGridThreads, kGridSmem, &d.grid);
+    prepare(k_select_grid<NSML_F32, true, true>, kGridThreads, kGridSmem, &d.grid);
+    prepare(k_select_grid<NSML_BF16, false, false>, kGridThreads, kGridSmem, &d.grid);
+    prepare(k_select_grid<NSML_BF16, false, true>, kGridThreads, kGridSmem, &d.grid);
+    prepare(k_select_grid<NSML_BF16, true, false>, kGridThreads, kGridSmem, &d.grid);
+    prepare(k_select_grid<NSML_BF16, true, true>, kGridThreads, kGridSmem, &d.grid);
     int list_fits = 0;  // every shape of the list stage is resident at least once per SM
     prepare(k_emit<NSML_F32, kEmitPer>, kEmitThreads, sizeof(EmitShared), &list_fits);
     prepare(k_emit<NSML_BF16, kEmitPer>, kEmitThreads, sizeof(EmitShared), &list_fits);
@@ -117,8 +120,8 @@ static int device_info(const DeviceInfo** out) {
     prepare(k_sample<NSML_BF16>, kSampleThreads, kSampleSmem, &list_fits);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.merge_small, k_merge<kDenseTileSmall>, kMergeThreads, 0);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.merge_large, k_merge<kDenseTileLarge>, kMergeThreads, 0);
-    // The streaming kernels run as one wave of resident blocks (a second, partial wave would read
-    // with a fraction of the SMs' loads in flight).
+    // The norm runs as one wave of resident blocks (a second, partial wave would read with a
+    // fraction of the SMs' loads in flight).
     auto resident = [&](auto kernel, int* out) {
       int r = 0;
       if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, kernel, kCta, 0);
@@ -126,12 +129,10 @@ static int device_info(const DeviceInfo** out) {
     };
     resident(k_sumsq<NSML_F32>, &d.sumsq);
     resident(k_sumsq<NSML_BF16>, &d.sumsq);
-    resident(k_feedback_add<NSML_F32>, &d.feedback_add);
-    resident(k_feedback_add<NSML_BF16>, &d.feedback_add);
-    if (e == cudaSuccess && (d.sumsq < 1 || d.feedback_add < 1)) e = cudaErrorUnknown;
+    if (e == cudaSuccess && d.sumsq < 1) e = cudaErrorUnknown;
     int coop = 0;
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-    if (e != cudaSuccess || d.dense_small < 1 || d.dense_large < 1 || list_fits < 1 || d.merge_small < 1 || d.merge_large < 1 || !coop) {
+    if (e != cudaSuccess || d.grid < 1 || list_fits < 1 || d.merge_small < 1 || d.merge_large < 1 || !coop) {
       cudaGetLastError();
       return NSML_ERR_CUDA;
     }
@@ -151,7 +152,7 @@ static inline unsigned int grid_for(unsigned long long work_items, unsigned long
   return (unsigned int)blocks;
 }
 
-// The short, latency-bound kernels (sample, list stage, small select, mask finish, partition) are launched at the
+// The short, latency-bound kernels (sample, clear, list stage, small select, mask finish, partition) are launched at the
 // highest stream priority.  When several buckets are in flight on several streams, every bucket pass that is ready sits in
 // front of the device's block scheduler with thousands of blocks to place; a list-stage kernel that becomes
 // ready later is otherwise placed only after all of them, so the passes of a step ran first, back to back,
@@ -211,7 +212,7 @@ static int64_t k_of(int64_t n, double ratio) {
   return k;
 }
 
-// What the sample of a call is asked for: the ranks (from the top, 1-based) of the two sample keys six standard
+// What the sample of a call is asked for: the ranks (from the top, 1-based) of the two sample keys `sigmas` standard
 // deviations either side of the expected rank of the k-th largest, and the number of candidates to expect above
 // the lower one.  rank_lo = 0: do not sample (small bucket, or nearly everything is kept).
 struct SamplePlan {
@@ -219,11 +220,11 @@ struct SamplePlan {
   double expected = 0.0;
 };
 
-static SamplePlan sample_plan(int64_t n, int64_t k, int grad_dtype) {
+static SamplePlan sample_plan(int64_t n, int64_t k, int grad_dtype, double sigmas = 6.0) {
   SamplePlan s;
   if (n < (int64_t)kSamples) return s;
   const double keys = (double)kSamples * (grad_dtype == NSML_F32 ? sample_keys<NSML_F32>() : sample_keys<NSML_BF16>());
-  const double p = (double)k / (double)n, mean = keys * p, six = 6.0 * std::sqrt(keys * p * (1.0 - p));
+  const double p = (double)k / (double)n, mean = keys * p, six = sigmas * std::sqrt(keys * p * (1.0 - p));
   const double lo = std::ceil(mean + six) + 1.0, hi = std::floor(mean - six);
   if (lo < keys) s.rank_lo = (unsigned int)lo;
   // (the largest sampled key, with about n / keys elements above it, where that is safely fewer than k)
@@ -237,20 +238,19 @@ constexpr int kListBlockCandidates = 4096;  // default of the knob
 constexpr double kListFewBlocks = 10;       // blocks for a short list where the knob is well above it
 static std::atomic<int> g_list_block_candidates{kListBlockCandidates};
 
-// Dense mode: the select runs over the bucket itself, with no sample and no bucket pass.
-// Taken when the candidate list would be about as large as the bucket.  (What cannot be sampled is taken by use_small,
-// which is asked first.)
-static bool use_dense(int64_t n, int64_t k) {
-  const double p_keep = (double)k / (double)n;
-  return p_keep >= kDenseRatioAny || sample_plan(n, k, NSML_F32).rank_lo == 0;
+// Dense mode: the select runs over the bucket itself, with no candidate list.  (What cannot be sampled is taken by
+// use_small, which is asked first.)
+static unsigned int grid_blocks(const DeviceInfo& dev) { return (unsigned int)(dev.sms < kGridMaxBlocks ? dev.sms / 2 * 2 : kGridMaxBlocks); }
+template <int VT>
+static bool use_dense(int64_t n, int64_t k, const DeviceInfo& dev) {
+  return (double)k >= dense_from<VT>() * (double)n && n <= (int64_t)grid_max_rows<VT>() * grid_blocks(dev) * grid_seg<VT>();
 }
 
 // Small mode: the whole bucket is held in the shared memory of one block or cluster.
 static bool use_small(int64_t n) { return n <= kSmallMaxN; }
 
 // DTYPE: element type of `grad` (what the sample and the bucket pass read).  FDTYPE: element type of the
-// bucket the later stages re-read; with a residual (local accumulation fused into the bucket pass, list
-// strategy only) that bucket is the residual buffer, float32, which then holds gradient + residual.
+// bucket the later stages re-read; with a residual (local accumulation fused into the pass) that bucket is the residual buffer, float32, which then holds gradient + residual.
 template <int DTYPE, int FDTYPE>
 static int launch_compress(const void* grad, float* residual, const uint32_t* mask, int64_t n, int64_t k, int bits,
                            unsigned char* ws, unsigned char* payload, const CompressLayout& L, const PayloadLayout& P,
@@ -263,10 +263,8 @@ static int launch_compress(const void* grad, float* residual, const uint32_t* ma
   fp.n = (unsigned long long)n;
   fp.k = (unsigned long long)k;
   fp.bits = bits;
-  fp.nseg = ((unsigned long long)n + kSegElems - 1) / kSegElems;
   fp.ctl = ctl;
   fp.hist = reinterpret_cast<unsigned int*>(ws + L.hist);
-  fp.block_counts = reinterpret_cast<unsigned long long*>(ws + L.block_counts);
   fp.tiles = (unsigned int)(((unsigned long long)n + tile - 1) / tile);
   fp.list.off = reinterpret_cast<unsigned short*>(ws + L.cand_off);
   fp.list.val = reinterpret_cast<uint32_t*>(ws + L.cand_val);
@@ -295,25 +293,33 @@ static int launch_compress(const void* grad, float* residual, const uint32_t* ma
                      per_block, keep_status ? 1 : 0);
     return le == cudaSuccess ? NSML_OK : NSML_ERR_CUDA;
   }
-  if (use_dense(n, k)) {
-    const bool small_shape = (unsigned long long)n <= (unsigned long long)dev.sms * kFinSmallCache;
-    unsigned long long cap = (unsigned long long)dev.sms * (small_shape || dev.dense_large < 2 ? 1 : 2);
-    if (cap > (unsigned long long)kMaxFinalizeBlocks) cap = kMaxFinalizeBlocks;
-    unsigned long long want = (unsigned long long)n / 4096 + 1;  // at least about 4096 elements per block
-    if (want > fp.nseg) want = fp.nseg;
-    const unsigned int grid = (unsigned int)(want < cap ? want : cap);
+  if (use_dense<FDTYPE>(n, k, dev)) {
+    // Bounds four standard deviations either side of the threshold's expected rank: one call in 16,000 takes another round
+    // (3 us), the others have a window a third narrower than with six.
+    const SamplePlan plan = sample_plan(n, k, DTYPE, 4.0);
+    const unsigned int segs = (unsigned int)(((unsigned long long)n + grid_seg<FDTYPE>() - 1) / grid_seg<FDTYPE>());
+    const unsigned int most = grid_blocks(dev), grid = segs < most ? segs : most, rows = (segs + grid - 1) / grid;
+    // room for twice the keys that are to be expected inside the window, the rest of the shared memory for slices
+    const double keys = (double)kSamples * (DTYPE == NSML_F32 ? sample_keys<NSML_F32>() : sample_keys<NSML_BF16>());
+    const double window = plan.rank_lo == 0 ? 0.05 : (double)(plan.rank_lo - plan.rank_hi) / keys;
+    const double entries = window * (double)n / ((double)grid * kGridWarps) * 2.0 + 64.0;
+    const unsigned int cap = entries < (double)kGridMaxCap ? (unsigned int)entries / 8 * 8 : kGridMaxCap;
+    const size_t fixed = grid_smem<FDTYPE>(rows, cap, 0);
+    unsigned int room = (unsigned int)((kGridSmem - fixed) / kGridSliceBytes);
+    if (room > rows * kGridWarps) room = rows * kGridWarps;
     {
       LaunchScope scope(K_CLEAR, st);
-      k_clear<<<4, kCta, 0, st>>>(reinterpret_cast<uint4*>(ws), (unsigned int)(L.group_count / 16), keep_status ? 1 : 0);
+      le = launch_prio(k_clear, dim3(8), dim3(kCta), 0, st, false, 0, true, true, reinterpret_cast<uint4*>(ws), (unsigned int)(L.zero_bytes / 16),
+                       keep_status ? 1 : 0);
+      if (le != cudaSuccess) return NSML_ERR_CUDA;
     }
-    LaunchScope scope(K_FINALIZE_DENSE, st);
+    LaunchScope scope(K_SELECT_GRID, st);
+    const bool fb = residual != nullptr, masked = mask != nullptr;
     // cooperative: every block co-resident; normal priority, it streams the whole bucket
-    if (small_shape)
-      le = launch_prio(k_finalize_dense<FDTYPE, kFinSmallThreads, kFinSmallCache>, dim3(grid), dim3(kFinSmallThreads),
-                       finalize_dyn_smem(kFinSmallCache), st, true, 0, false, false, fsrc, fp);
-    else
-      le = launch_prio(k_finalize_dense<FDTYPE, kFinLargeThreads, kFinDenseLargeCache>, dim3(grid), dim3(kFinLargeThreads),
-                       finalize_dyn_smem(kFinDenseLargeCache), st, true, 0, false, false, fsrc, fp);
+    le = launch_prio(fb ? (masked ? k_select_grid<DTYPE, true, true> : k_select_grid<DTYPE, true, false>)
+                        : (masked ? k_select_grid<DTYPE, false, true> : k_select_grid<DTYPE, false, false>),
+                     dim3(grid), dim3(kGridThreads), fixed + (size_t)room * kGridSliceBytes, st, true, 0, false, true, src, fp, segs, rows, cap,
+                     room, plan.rank_lo, plan.rank_hi);
     return le == cudaSuccess ? NSML_OK : NSML_ERR_CUDA;
   }
   const SamplePlan plan = sample_plan(n, k, DTYPE);
@@ -583,38 +589,17 @@ static int feedback_impl(const void* grad, float* residual, int64_t n, int grad_
   const DeviceInfo* dev = nullptr;
   int rc = device_info(&dev);
   if (rc != NSML_OK) return rc;
-  if (use_dense(n, k) && !use_small(n)) {
-    // dense strategy (no bucket pass to fuse the add into): residual <- grad + residual first, then the select
-    // over the residual buffer
-    const unsigned int grid = stream_grid(n, *dev, dev->feedback_add < 8 ? dev->feedback_add : 8, 1u << 16);
-    {
-      LaunchScope scope(K_FEEDBACK_ADD, st);
-      if (grad_dtype == NSML_F32)
-        k_feedback_add<NSML_F32><<<grid, kCta, 0, st>>>(BucketSrc<NSML_F32>{grad, nullptr}, residual, (unsigned long long)n);
-      else
-        k_feedback_add<NSML_BF16><<<grid, kCta, 0, st>>>(BucketSrc<NSML_BF16>{grad, nullptr}, residual, (unsigned long long)n);
-    }
-    rc = compress_impl(residual, n, NSML_F32, ratio, bits, prune_mask, payload, payload_capacity, workspace,
-                       workspace_bytes, st);
-  } else {
-    // list strategy: the bucket pass adds the residual as it streams the gradient and leaves the sum in it
-    if (prune_mask != nullptr && !aligned(prune_mask, 4)) return NSML_ERR_ARG;
-    unsigned char* ws = static_cast<unsigned char*>(workspace);
-    unsigned char* pl = static_cast<unsigned char*>(payload);
-    const PayloadLayout P = payload_layout(k, bits);
-    const CompressLayout L = compress_layout(n);
-    if (grad_dtype == NSML_F32)
-      rc = launch_compress<NSML_F32, NSML_F32>(grad, residual, prune_mask, n, k, bits, ws, pl, L, P, *dev, st);
-    else
-      rc = launch_compress<NSML_BF16, NSML_F32>(grad, residual, prune_mask, n, k, bits, ws, pl, L, P, *dev, st);
-  }
+  // the kernels that read the gradient add the residual to it, leave the sum there and take out what the payload carries
+  if (prune_mask != nullptr && !aligned(prune_mask, 4)) return NSML_ERR_ARG;
+  unsigned char* ws = static_cast<unsigned char*>(workspace);
+  unsigned char* pl = static_cast<unsigned char*>(payload);
+  const PayloadLayout P = payload_layout(k, bits);
+  const CompressLayout L = compress_layout(n);
+  if (grad_dtype == NSML_F32)
+    rc = launch_compress<NSML_F32, NSML_F32>(grad, residual, prune_mask, n, k, bits, ws, pl, L, P, *dev, st);
+  else
+    rc = launch_compress<NSML_BF16, NSML_F32>(grad, residual, prune_mask, n, k, bits, ws, pl, L, P, *dev, st);
   if (rc != NSML_OK) return rc;
-  if (use_dense(n, k) && !use_small(n)) {  // (the other strategies take what the payload carries out of the residual themselves)
-    LaunchScope scope(K_FEEDBACK_SUBTRACT, st);
-    const unsigned int sgrid = grid_for((unsigned long long)k, kCta, dev->sms * 8);
-    k_feedback_subtract<<<sgrid, kCta, 0, st>>>(static_cast<const unsigned char*>(payload), residual,
-                                                (unsigned long long)n, static_cast<int*>(workspace));
-  }
   if (cudaGetLastError() != cudaSuccess) return NSML_ERR_CUDA;
   return NSML_OK;
 }
@@ -658,7 +643,7 @@ int nsml_compress_strategy(int64_t n, double ratio) {
   const DeviceInfo* dev = nullptr;
   const int rc = device_info(&dev);
   if (rc != NSML_OK) return rc;
-  return use_dense(n, k) ? NSML_STRATEGY_DENSE : NSML_STRATEGY_LIST;
+  return use_dense<NSML_F32>(n, k, *dev) ? NSML_STRATEGY_DENSE : NSML_STRATEGY_LIST;
 }
 
 int nsml_set_list_block_candidates(int candidates) {

@@ -27,13 +27,15 @@ constexpr int kMaxPolls = 1 << 22;
 struct Ctl {
   int status;                 // first device-detected error (NSML_ERR_*), 0 = ok
   unsigned int lo, hi;        // sampled bounds of the threshold key: probably lo <= T < hi
-  unsigned int barrier;       // arrivals at the dense select's grid barriers
+  unsigned int barrier;       // arrivals at the grid barriers of a cooperative kernel
   unsigned int grain;         // the sampled keys (nearly all of them) are multiples of 1 << grain: 16, 13 or 0
   unsigned int ticket;        // chunks of the list handed out
   unsigned int fallback;      // a bin that was taken for a single key holds others
   unsigned int done;          // chunks of the list that are finished, where that has to be known
   unsigned long long below_listed;     // mask build: weights below the bracket << 32 | weights listed inside it
   unsigned int drawn[9], finished[9];  // general select, mask build: units of work of each phase
+  unsigned long long listed_above;  // grid select: candidates << 32 | those above the window
+  unsigned int sampled, members;    // grid select: sampler blocks done; keys of the threshold's bin
 };
 static_assert(sizeof(Ctl) <= 256, "control block must fit its 256-byte slot");
 
@@ -70,11 +72,9 @@ __device__ __forceinline__ Window make_window(const Ctl* ctl) {
   return w;
 }
 
-constexpr int kSegElems = 512;            // granule of the index ranges that the dense select's blocks own
 constexpr int kTileBytes = 16384;         // bucket bytes per tile of the candidate list: what a block of the bucket pass takes
 constexpr int kMaxGroups = 8192;          // the bucket pass keeps a candidate count per group of tiles (of one tile, up to 32M
                                           // float32 or 64M bfloat16 elements)
-constexpr int kMaxFinalizeBlocks = 1024;  // upper bound on blocks of the dense select
 constexpr int kChunk = 2048;              // candidates a block of the list stage takes at a time (long lists: twice that)
 
 // The keys inside the window are also kept by bin, up to this many per bin: four times what is to be expected where the
@@ -100,7 +100,6 @@ struct CompressLayout {  // byte offsets inside a compress workspace
   size_t hist;          // u32[4][kMaxBins]: digit histograms; the last one counts the candidates inside the sampled window
   size_t group_count;   // u32[kMaxGroups]: candidates per group of tiles
   size_t zero_bytes;    // everything before this offset is cleared per call
-  size_t block_counts;  // u64[kMaxFinalizeBlocks]: per-block counts exchanged at barriers
   size_t bins;          // uint2[kMaxBins][bin_room_of(n)]: (key, index) of the candidates inside the window, by bin
   size_t chunk_sum;     // u64[2][chunks]: survivors of a chunk, and up to it; cleared by the bucket pass
   size_t block_fill;    // u32[chunks]: values delivered to a payload block of 1024; cleared by the bucket pass
@@ -113,8 +112,16 @@ struct CompressLayout {  // byte offsets inside a compress workspace
 
 __host__ __device__ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-// Kept fraction from which the select runs over the bucket itself.
-constexpr double kDenseRatioAny = 0.25;
+// Kept fraction from which the select runs over the bucket itself (k_select_grid) and not over a candidate list.  Two
+// states in turn, us, list / grid select, buckets of tensors of different scales | of one scale throughout (every 512
+// bytes of the bucket then hold a candidate, the worst case of the grid select):
+//   float32  16M: 0.1 82 / 64 | 72 / 84, 0.15 97 / 68 | 89 / 89, 0.2 106 / 75 | 93 / 94
+//            64M: 0.1 227 / 181 | 220 / 275, 0.15 289 / 195 | 296 / 289, 0.2 415 / 217 | 327 / 299
+//   bfloat16 32M: 0.05 58 / 55 | 61 / 86, 0.1 75 / 60 | 76 / 89, 0.15 97 / 69 | 102 / 94, 0.2 113 / 76 | 117 / 96
+//            67M: 0.05 91 / 88 | 99 / 155, 0.1 128 / 103 | 135 / 158, 0.15 170 / 115 | 184 / 170, 0.2 208 / 123 | 221 / 173
+// The lines are where several scales gain a fifth or more and one scale loses no more than that.
+template <int VT>  // element type of what is selected from
+constexpr double dense_from() { return VT == NSML_F32 ? 0.125 : 0.1; }
 
 inline CompressLayout compress_layout(int64_t n) {
   CompressLayout L;
@@ -122,8 +129,7 @@ inline CompressLayout compress_layout(int64_t n) {
   L.hist = 256;
   L.group_count = L.hist + 4 * kMaxBins * sizeof(unsigned int);
   L.zero_bytes = L.group_count + kMaxGroups * sizeof(unsigned int);
-  L.block_counts = L.zero_bytes;
-  L.bins = L.block_counts + kMaxFinalizeBlocks * 8;
+  L.bins = L.zero_bytes;
   L.chunk_sum = L.bins + (size_t)kMaxBins * bin_room_of(n) * 8;
   const size_t chunks = npad / kChunk;
   L.block_fill = L.chunk_sum + align_up(2 * chunks * 8, 256);

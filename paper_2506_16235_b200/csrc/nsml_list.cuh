@@ -27,7 +27,7 @@
 // a bin of many keys that turn out not to be one key) take more rounds (general_select).
 #pragma once
 
-#include "nsml_dense.cuh"
+#include "nsml_finalize.cuh"
 
 namespace nsml {
 

@@ -59,8 +59,8 @@ __device__ __forceinline__ void find_digit_from_top(const unsigned int (&own)[PE
   __syncthreads();  // s_tot and s_out may still be read from an earlier call
   if (lane == 0) s_tot[warp] = incl;
   __syncthreads();
-  unsigned int above = incl - mine;
-  for (int w = warp + 1; w < THREADS / 32; ++w) above += s_tot[w];
+  static_assert(THREADS <= 1024, "a warp's lanes hold all warps' counts");
+  unsigned int above = incl - mine + __reduce_add_sync(0xFFFFFFFFu, lane > warp && lane < THREADS / 32 ? s_tot[lane] : 0u);
   if (above < rem && rem <= above + mine) {  // exactly one thread
 #pragma unroll
     for (int b = PER - 1; b >= 0; --b) {
