@@ -25,6 +25,7 @@ namespace nsml {
 constexpr int kDenseTileLarge = 8192;
 constexpr int kDenseTileSmall = 2048;
 constexpr int64_t kDenseTileSmallMaxN = 1024LL * kDenseTileSmall;
+static_assert(kDenseTileLarge == 1 << 13 && kDenseTileSmall == 1 << 11, "tiles by shift");
 inline int dense_tile(int64_t n) { return n <= kDenseTileSmallMaxN ? kDenseTileSmall : kDenseTileLarge; }
 
 struct PayloadTable {
@@ -74,22 +75,39 @@ __host__ __device__ inline bool header_ok(const nsml_payload_header* h, unsigned
 
 // offsets[w][b] = first payload entry of worker w whose index is >= b * tile.
 //
-// A block settles kPartBounds consecutive boundaries of one worker, a thread each.  What a search costs is its
-// chain of dependent reads of the index array (about 1 us each, the array is in DRAM) and, where boundaries are
-// many, the 64 bytes that every read fetches.  So kPartProbes evenly spaced indices of the whole array go to
-// shared memory (and, where the block's boundaries lie in a small part of it, as many of that part: about one
+// What bounds the kernel is its chain of dependent reads (about 1 us each from DRAM).  Payloads of few entries are read
+// as a whole (kPartScan): a thread compares the tiles of four neighbouring entries and writes the boundaries between
+// them, so that there are two reads in a row, header and indices; and the indices are in L2 when the sum reads them.
+// Where that is more to read than a search (every entry against some 200 bytes per boundary), a block settles
+// kPartBounds consecutive boundaries of one worker, a thread each: kPartProbes evenly spaced indices of the whole array go
+// to shared memory (and, where the block's boundaries lie in a small part of it, as many of that part: about one
 // probe per boundary); every thread finds the two probes around its boundary there, interpolates between them and
 // counts in the 16 entries around the guess, which settles the boundary in one read wherever the indices are
 // locally even, and gallops from the guess where they are not: three or four dependent reads with the payload
 // header's.  (350M elements, 8 workers, 342k boundaries: 54 us with a binary search per thread, 43 us now;
-// 25M elements, 4 workers: 12.3 -> 11 us.)
+// 25M elements, 4 workers of 250k entries: 12.3 us with a binary search, 10.4 with the probes, 6 read as a whole; 1M, 2
+// workers of 52k: 6.2 with the probes, 3.5.  The launch may start under the kernel before it.  Sum as a whole: 25M 35.2 ->
+// 29.1 us, 1M added to 12.3 -> 9.6.)
 //
 // The kernel also clears the call's status word (no separate clearing step is needed); payload errors are
 // reported by the merge kernel: a worker with a bad header gets all-zero offsets, so nothing of its payload
-// is read.
+// is read.  A corrupt payload whose indices do not ascend leaves boundaries unwritten or written twice: the merge
+// kernel takes no offset beyond the number of entries and checks every index against its tile.
 constexpr int kPartBounds = 1024;
 constexpr unsigned int kPartProbes = kPartBounds;  // one per thread
 constexpr unsigned int kPartWindow = 16;
+constexpr unsigned int kPartScan = 8u << 20;  // entries of all workers up to which they are read as a whole: 32 MB, 5 us
+constexpr unsigned int kPartParts = 64;       // blocks per worker for that, at most
+// Blocks per worker: 8192 entries each of the largest payload, as far as the buffers' sizes tell (an entry takes five bytes
+// at least), otherwise of a 16th of the bucket.  No more than that, because blocks that find nothing to do still hold an SM's
+// threads until the header is there: 64 of them for each of eight workers made four streams' steps 20 % longer.
+inline unsigned int partition_blocks(int64_t n, unsigned int tiles, unsigned long long largest_payload) {
+  const unsigned int search = tiles / kPartBounds + 1;
+  const unsigned long long entries = largest_payload != 0 ? largest_payload / 5 : (unsigned long long)n / 16;
+  const unsigned long long scan = entries / 8192 + 1;
+  const unsigned int parts = scan < kPartParts ? (unsigned int)scan : kPartParts;
+  return search > parts ? search : parts;
+}
 
 // [lo, hi] of the first entry whose index is >= target: entries below lo are below it, entry hi is not (or hi is
 // the end).  The probes in shared memory are every gap-th entry from `base` on, `count` of them.
@@ -105,21 +123,65 @@ __device__ __forceinline__ unsigned int probe_bracket(const uint32_t* s_probe, u
   return a;
 }
 
+// Writes `value` for boundaries b .. last, by a warp.
+__device__ __forceinline__ void fill_bounds(unsigned int* out, unsigned int b, unsigned int last, unsigned int value) {
+  for (b += threadIdx.x & 31; b <= last; b += 32) out[b] = value;
+}
+
+// Boundaries of a payload that is read as a whole; part: the block's of `parts`.
+__device__ __forceinline__ void scan_bounds(const uint32_t* idx, unsigned int k, unsigned int tiles, unsigned int shift, unsigned int part,
+                                            unsigned int parts, unsigned int* out) {
+  constexpr unsigned int FULL = 0xFFFFFFFFu;
+  const unsigned int lane = threadIdx.x & 31, quads = (k + 3) / 4, per = (quads + parts - 1) / parts;
+  const unsigned int begin = part * per, end = min(quads, begin + per);
+  for (unsigned int q0 = begin + (threadIdx.x & ~31u); q0 < end; q0 += kPartBounds) {  // uniform over the warp
+    const unsigned int q = q0 + lane;
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if (q < end) v = __ldg(reinterpret_cast<const uint4*>(idx) + q);  // (the section is padded)
+    unsigned int before = __shfl_up_sync(FULL, v.w, 1);
+    if (lane == 0 && q0 != 0) before = __ldg(idx + 4ull * q0 - 1);
+    const uint32_t e[4] = {v.x, v.y, v.z, v.w};
+    unsigned int next = q == 0 ? 0u : min(before >> shift, tiles) + 1;  // the first boundary behind the entry before
+#pragma unroll
+    for (unsigned int i = 0; i < 4; ++i) {
+      const unsigned int j = 4 * q + i, reach = q < end && j < k ? min(e[i] >> shift, tiles) + 1 : next;  // boundaries next .. reach - 1 are the entry's
+      const bool many = reach > next + 4;
+      if (!many)
+        for (unsigned int b = next; b < reach; ++b) out[b] = j;
+      for (unsigned int left = __ballot_sync(FULL, many); left != 0; left &= left - 1) {
+        const int who = __ffs(left) - 1;
+        fill_bounds(out, __shfl_sync(FULL, next, who), __shfl_sync(FULL, reach, who) - 1, __shfl_sync(FULL, j, who));
+      }
+      if (q < end && j < k) next = reach;
+    }
+    const unsigned int last = __ballot_sync(FULL, q < end && q == quads - 1);  // behind the last entry
+    if (last != 0) fill_bounds(out, __shfl_sync(FULL, next, __ffs(last) - 1), tiles, k);
+  }
+}
+
 __global__ void __launch_bounds__(kPartBounds)
-k_partition(PayloadTable table, int W, unsigned long long n, unsigned int tiles, unsigned int tile_elems,
+k_partition(PayloadTable table, int W, unsigned long long n, unsigned int tiles, unsigned int tile_shift,
             unsigned int* __restrict__ offsets, int* status) {
   __shared__ uint32_t s_probe[kPartProbes];
+  pdl_wait();
   pdl_launch_dependents();
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *status = NSML_OK;
   const int w = blockIdx.y;
-  const unsigned int first = blockIdx.x * kPartBounds, count = min((unsigned)kPartBounds, tiles + 1 - first);
-  unsigned int* out = offsets + (unsigned long long)w * (tiles + 1ull) + first;
+  const unsigned int first = blockIdx.x * kPartBounds, count = first > tiles ? 0u : min((unsigned)kPartBounds, tiles + 1 - first);
+  const unsigned int tile_elems = 1u << tile_shift;
+  unsigned int* all = offsets + (unsigned long long)w * (tiles + 1ull);
+  unsigned int* out = all + first;
   const nsml_payload_header* h = reinterpret_cast<const nsml_payload_header*>(table.p[w]);
   if (!header_ok(h, n, table.bytes[w])) {  // uniform over the block
     if (threadIdx.x < count) out[threadIdx.x] = 0;
     return;
   }
   const uint32_t* idx = reinterpret_cast<const uint32_t*>(table.p[w] + h->idx_off);
+  if (h->k * (unsigned long long)W <= kPartScan) {
+    if (blockIdx.x < kPartParts) scan_bounds(idx, (unsigned int)h->k, tiles, tile_shift, blockIdx.x, min(gridDim.x, kPartParts), all);
+    return;
+  }
+  if (count == 0) return;
   unsigned int base = 0, end = (unsigned int)h->k;  // k <= n < 2^31; so is every target below: (tiles + 1) * tile < 2^32
   unsigned int gap, probes, from, to, a;
   auto probe = [&]() {
@@ -250,6 +312,7 @@ k_merge(PayloadTable table, int W, float* __restrict__ dense, unsigned long long
   __shared__ uint2 s_range[2][NSML_MAX_WORKERS];  // the tile's entries of every worker; double-buffered
   const unsigned long long per = (unsigned long long)tiles + 1;
   bool bad = false;
+  unsigned int entries = 0;  // of worker threadIdx.x
   if (threadIdx.x < W) {
     // Headers are checked here (the partition kernel cleared the status word).  A worker with a bad
     // header has all-zero offsets, so its view is never used.
@@ -261,6 +324,7 @@ k_merge(PayloadTable table, int W, float* __restrict__ dense, unsigned long long
       v.val = pbase + h->val_off;
       v.scale = reinterpret_cast<const float*>(pbase + h->scale_off);
       v.bits = (int)h->bits;
+      entries = (unsigned int)h->k;
     } else {
       bad = blockIdx.x == 0;
     }
@@ -268,7 +332,7 @@ k_merge(PayloadTable table, int W, float* __restrict__ dense, unsigned long long
   }
   pdl_wait();  // the offsets are complete
   const unsigned int* my_offsets = offsets + threadIdx.x * per;  // thread w looks after worker w's ranges
-  if (threadIdx.x < W && blockIdx.x < tiles) s_range[0][threadIdx.x] = make_uint2(__ldcg(my_offsets + blockIdx.x), __ldcg(my_offsets + blockIdx.x + 1));
+  if (threadIdx.x < W && blockIdx.x < tiles) s_range[0][threadIdx.x] = make_uint2(min(entries, __ldcg(my_offsets + blockIdx.x)), min(entries, __ldcg(my_offsets + blockIdx.x + 1)));
   int buf = 0;
   for (unsigned int tile = blockIdx.x; tile < tiles; tile += gridDim.x, buf ^= 1) {
     const unsigned long long lo = (unsigned long long)tile * TILE;
@@ -362,7 +426,7 @@ k_merge(PayloadTable table, int W, float* __restrict__ dense, unsigned long long
         if ((u + 1 == kMergeUnits ? w : unit_w[u + 1]) != unit_w[u]) __syncthreads();  // uniform over the block
       }
     }
-    if (fetch) s_range[buf ^ 1][threadIdx.x] = ahead;
+    if (fetch) s_range[buf ^ 1][threadIdx.x] = make_uint2(min(entries, ahead.x), min(entries, ahead.y));
     if (!staged) continue;
     if (len == TILE) {
       fence_async_shared();

@@ -418,10 +418,12 @@ static int accumulate_impl(const void* const* payloads, const size_t* payload_by
   unsigned int* offsets = reinterpret_cast<unsigned int*>(ws + L.offsets);
   const unsigned int tile = (unsigned int)dense_tile(n);
   const unsigned int tiles = (unsigned int)((n + tile - 1) / tile);
+  unsigned long long largest = 0;  // payload, in bytes; 0 = not known
+  for (int w = 0; w < W; ++w) largest = table.bytes[w] > largest ? table.bytes[w] : largest;
   {
     LaunchScope scope(K_PARTITION, st, timed);  // also clears the status word
-    launch_prio(k_partition, dim3(tiles / kPartBounds + 1, W), dim3(kPartBounds), 0, st, false, 0, true, false, table, W, (unsigned long long)n,
-                tiles, tile, offsets, status);
+    launch_prio(k_partition, dim3(partition_blocks(n, tiles, largest), W), dim3(kPartBounds), 0, st, false, 0, true, true, table, W, (unsigned long long)n,
+                tiles, tile == kDenseTileLarge ? 13u : 11u, offsets, status);
   }
   {
     LaunchScope scope(K_MERGE, st, timed);

@@ -53,3 +53,54 @@ def test_one_workspace_sized_for_the_largest_bucket_serves_them_all():
         ref = oracle.decompress_sum(want, n)
         largest = max(float(np.abs(p.raw).max()) for p in want)
         assert float(np.abs(dense.cpu().numpy().astype(np.float64) - ref).max()) <= 1e-6 * largest
+
+
+# The partition reads payloads of few entries (8M over all workers) as a whole, four entries per thread: numbers of entries
+# around a quad, a warp and a block; gaps of one, a few and all tiles; the first and the last tiles empty; both sides of
+# the line (64 workers: 131072 entries each), workers on different sides of it in one call.
+def _payload(n, idx, bits, seed):
+    rng = np.random.default_rng(seed)
+    k = idx.size
+    vals = rng.standard_normal(k).astype(np.float32)
+    if bits == 32:
+        return nsml.pack_payload(n, 32, idx, f32=vals), vals.astype(np.float64)
+    half = vals.astype(np.float16)
+    return nsml.pack_payload(n, 16, idx, half=half.view(np.uint16)), half.astype(np.float64)
+
+
+def _check_sum(n, index_sets, zero_first=True, sized=False):
+    want = np.zeros(n) if zero_first else np.full(n, 0.5)
+    payloads, most = [], 1.0
+    for w, idx in enumerate(index_sets):
+        raw, vals = _payload(n, np.asarray(idx, dtype=np.uint32), 16 if w % 2 else 32, w)
+        want[np.asarray(idx, dtype=np.int64)] += vals
+        most = max(most, float(np.abs(vals).max()))
+        payloads.append(torch.from_numpy(raw).cuda())
+    dense = torch.full((n,), 0.5, device="cuda")
+    ws = torch.full((nsml.nsml_accumulate_workspace_bytes(n, len(payloads)),), 0xFF, dtype=torch.uint8, device="cuda")
+    nsml.nsml_decompress_accumulate(payloads, dense, zero_first=zero_first, workspace=ws, sized=sized)
+    assert nsml.nsml_last_status(ws) == 0
+    # W float32 adds: at most W - 1 roundings of a running sum of at most W * most
+    bound = len(payloads) ** 2 * most * 2.0 ** -24 + 1e-12
+    assert float(np.abs(dense.cpu().numpy().astype(np.float64) - want).max()) <= bound
+
+
+@pytest.mark.parametrize("n", [5000, 300_001, 3_000_001])
+@pytest.mark.parametrize("sized", [False, True])
+def test_partition_reads_whole_payloads(n, sized):
+    rng = np.random.default_rng(n)
+    sizes = [1, 2, 3, 4, 5, 127, 128, 129, 4095, 4096, 4097]
+    sets = [np.sort(rng.choice(n, k, replace=False)) for k in sizes if k < n]
+    _check_sum(n, sets, sized=sized)
+    _check_sum(n, sets, zero_first=False, sized=sized)
+    tail = min(n, 1000)
+    gaps = [np.arange(tail), np.arange(n - tail, n), np.r_[0, n - 1], np.r_[0, 1, n // 2, n - 2, n - 1],
+            np.arange(0, n, max(1, n // 37)), np.r_[np.arange(tail // 2), np.arange(n - tail // 2, n)]]
+    _check_sum(n, gaps, sized=sized)
+
+
+def test_partition_on_both_sides_of_its_line():
+    n, W, line = 400_000, 64, (8 << 20) // 64
+    rng = np.random.default_rng(4)
+    for sizes in ([line] * W, [line + 1] * W, [line - 1 + w % 3 for w in range(W)], [line * 2 if w % 2 else 77 for w in range(W)]):
+        _check_sum(n, [np.sort(rng.choice(n, k, replace=False)) for k in sizes])
