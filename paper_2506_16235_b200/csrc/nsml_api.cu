@@ -116,8 +116,8 @@ static int device_info(const DeviceInfo** out) {
     prepare(k_select_small<NSML_BF16, 1>, kSmallThreads, kSmallOneBlock * 4, &list_fits);
     prepare(k_select_small<NSML_F32, kSmallBlocks>, kSmallThreads, kSmallPerBlock * 4, &list_fits);
     prepare(k_select_small<NSML_BF16, kSmallBlocks>, kSmallThreads, kSmallPerBlock * 4, &list_fits);
-    prepare(k_sample<NSML_F32>, kSampleThreads, kSampleSmem, &list_fits);
-    prepare(k_sample<NSML_BF16>, kSampleThreads, kSampleSmem, &list_fits);
+    prepare(k_sample<NSML_F32>, kSampleThreads, 0, &list_fits);
+    prepare(k_sample<NSML_BF16>, kSampleThreads, 0, &list_fits);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.merge_small, k_merge<kDenseTileSmall>, kMergeThreads, 0);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.merge_large, k_merge<kDenseTileLarge>, kMergeThreads, 0);
     // The norm runs as one wave of resident blocks (a second, partial wave would read with a
@@ -229,7 +229,7 @@ static SamplePlan sample_plan(int64_t n, int64_t k, int grad_dtype, double sigma
   if (lo < keys) s.rank_lo = (unsigned int)lo;
   // (the largest sampled key, with about n / keys elements above it, where that is safely fewer than k)
   s.rank_hi = hi >= 1.0 ? (unsigned int)hi : 8.0 * (double)n / keys < (double)k ? 1u : 0u;
-  s.expected = (double)n * (mean + six) / keys * 1.04 + 64.0;  // (the bound is rounded down to 15 key bits: a few per cent more)
+  s.expected = (double)n * (mean + six) / keys * 1.04 + 64.0;  // (the bound is rounded down to 14 key bits: a few per cent more)
   return s;
 }
 
@@ -325,7 +325,7 @@ static int launch_compress(const void* grad, float* residual, const uint32_t* ma
   const SamplePlan plan = sample_plan(n, k, DTYPE);
   {
     LaunchScope scope(K_SAMPLE, st);  // one cluster of kSampleBlocks blocks (the cluster shape is part of the kernel's definition)
-    le = launch_prio(k_sample<DTYPE>, dim3(kSampleBlocks), dim3(kSampleThreads), kSampleSmem, st, false, 0, true, true, src, residual,
+    le = launch_prio(k_sample<DTYPE>, dim3(kSampleBlocks), dim3(kSampleThreads), 0, st, false, 0, true, true, src, residual,
                      (unsigned long long)n, plan.rank_lo, plan.rank_hi, ctl, reinterpret_cast<uint4*>(ws),
                      (unsigned int)(L.zero_bytes / 16), keep_status ? 1 : 0);
     if (le != cudaSuccess) return NSML_ERR_CUDA;
@@ -555,7 +555,7 @@ static int prune_impl(const float* weights, int64_t n, double ratio, uint32_t* m
     const SamplePlan plan = sample_plan(n, n - m + 1, NSML_F32);
     {
       LaunchScope scope(K_SAMPLE, st);
-      le = launch_prio(k_sample<NSML_F32>, dim3(kSampleBlocks), dim3(kSampleThreads), kSampleSmem, st, false, 0, true, true, src, nullptr,
+      le = launch_prio(k_sample<NSML_F32>, dim3(kSampleBlocks), dim3(kSampleThreads), 0, st, false, 0, true, true, src, nullptr,
                        (unsigned long long)n, plan.rank_lo, plan.rank_hi, ctl, reinterpret_cast<uint4*>(ws), (unsigned int)(L.zero_bytes / 16), 0);
       if (le != cudaSuccess) return NSML_ERR_CUDA;
     }

@@ -7,15 +7,15 @@
 // k_sample reads 16 bytes (4 float32 or 8 bfloat16 keys) from each of 16384 equal
 // strata of the bucket and takes the two sample keys whose ranks lie six standard
 // deviations either side of the expected rank of the k-th largest, rounded
-// outwards to their top 15 bits.  (The keys of a stratum lie side by side; where
+// outwards to their top 14 bits.  (The keys of a stratum lie side by side; where
 // neighbours are alike, as in the rows of a sparse embedding gradient, they count
 // for less than as many independent draws, in the extreme case for one.)  The exact threshold is found
 // afterwards (nsml_list.cuh), which also repairs the rare case of a misleading
 // sample, so the sample only decides how much work is done, never the result.
 //
 // What bounds the kernel is latency: launch, one round of scattered reads, the
-// select.  It is one cluster of eight blocks; a block counts its keys' top 15
-// bits (all of a bfloat16 magnitude) in shared memory, then sums an eighth of
+// select.  It is one cluster of eight blocks; a block counts its keys' top 14
+// bits in shared memory, then sums an eighth of
 // the bins over the eight blocks through distributed shared memory, so that one
 // counting level and two cluster barriers replace the two levels in a single
 // block that an exact 24-bit select takes.
@@ -78,9 +78,16 @@ __device__ __forceinline__ void find_digit_from_top(const unsigned int (&own)[PE
 
 template <int DTYPE>
 __host__ __device__ constexpr int sample_keys() { return DTYPE == NSML_F32 ? 4 : 8; }  // keys per stratum: 16 bytes
-constexpr int kSampleBinBits = 15;
-constexpr int kSampleBins = 1 << kSampleBinBits;  // bins of the keys' top bits, 16-bit counters
-constexpr size_t kSampleSmem = kSampleBins * 2;
+// Keys are counted by their top 14 bits (64 bins per octave), those of 128 octaves from 2^-96 on, in 16-bit counters: 16 KB
+// that eight blocks read from one another.  (All of the top 15 bits, 64 KB: the sum over the blocks took 3 us, now 1.)  A
+// bound that lies below them is 0.
+constexpr int kSampleShift = 17;
+constexpr unsigned int kSampleBins = 8192, kSampleBase = 31u << 6;
+__device__ __forceinline__ unsigned int sample_bin(uint32_t key) {  // 0: not counted
+  return min(max(key >> kSampleShift, kSampleBase) - kSampleBase, kSampleBins - 1);
+}
+__device__ __forceinline__ uint32_t sample_bin_begin(unsigned int bin) { return (bin + kSampleBase) << kSampleShift; }
+__device__ __forceinline__ uint32_t sample_bin_end(unsigned int bin) { return bin + 1 < kSampleBins ? sample_bin_begin(bin + 1) : 0x80000000u; }
 
 // Clears the per-call control region and sets ctl->lo and ctl->hi from a stratified sample of the bucket (of
 // bucket + addend when an addend is given).  rank_lo, rank_hi: ranks from the top among the sampled keys.  A rank
@@ -91,13 +98,14 @@ k_sample(BucketSrc<DTYPE> src, const float* __restrict__ addend, unsigned long l
          Ctl* ctl, uint4* zero_base, unsigned int zero_vec16, int keep_status) {
   namespace cg = cooperative_groups;
   constexpr int KEYS = sample_keys<DTYPE>();
-  extern __shared__ __align__(16) unsigned int s_bins[];  // two 16-bit counters per word
+  __shared__ __align__(16) unsigned int s_bins[kSampleBins / 2];  // two 16-bit counters per word
   __shared__ unsigned int s_scan[kSampleThreads / 32];
   __shared__ unsigned int s_slice[kSampleBlocks];  // keys in each block's slice of the bins
   cg::cluster_group cluster = cg::this_cluster();
   const unsigned int rank = cluster.block_rank();
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  for (int i = t; i < kSampleBins / 8; i += kSampleThreads) reinterpret_cast<uint4*>(s_bins)[i] = make_uint4(0u, 0u, 0u, 0u);
+  static_assert(kSampleBins / 8 == kSampleThreads, "eight counters per thread");
+  reinterpret_cast<uint4*>(s_bins)[t] = make_uint4(0u, 0u, 0u, 0u);
   pdl_wait();
 
   uint4 raw[kSampleLoads];
@@ -140,7 +148,7 @@ k_sample(BucketSrc<DTYPE> src, const float* __restrict__ addend, unsigned long l
       if (addend != nullptr) bits[e] = __float_as_uint(__fadd_rn(__uint_as_float(bits[e]), add[s][e]));
       if ((pruned[s] >> e) & 1u) bits[e] = 0;
       low_bits |= bits[e] & 0xFFFFu;
-      const unsigned int bin = (bits[e] & 0x7FFFFFFFu) >> (31 - kSampleBinBits);
+      const unsigned int bin = sample_bin(bits[e] & 0x7FFFFFFFu);
       if (bin != 0) atomicAdd(&s_bins[bin >> 1], 1u << (16 * (bin & 1)));  // (a block has at most 16384 keys: no overflow)
     }
   }
@@ -153,17 +161,21 @@ k_sample(BucketSrc<DTYPE> src, const float* __restrict__ addend, unsigned long l
   cluster.sync();  // every block's counts are complete, the control region is cleared
   if (rank == 0 && t == 0) ctl->grain = below16 < kSampleThreads / 16 ? 16 : below13 < kSampleThreads / 16 ? 13 : 0;
 
-  // this block's slice of the bins, four per thread, summed over the blocks
-  constexpr int kSlice = kSampleBins / kSampleBlocks;
-  static_assert(kSlice == 4 * kSampleThreads, "four bins per thread");
-  unsigned int own[4] = {0, 0, 0, 0};
+  // this block's slice of the bins, two per thread of the lower half, summed over the blocks
+  constexpr unsigned int kSlice = kSampleBins / kSampleBlocks;
+  static_assert(kSlice == kSampleThreads, "a word of two bins for every other thread");
+  unsigned int own[2] = {0, 0};
+  if (t < (int)kSlice / 2) {
+    unsigned int v[kSampleBlocks];
 #pragma unroll
-  for (int b = 0; b < kSampleBlocks; ++b) {
-    const uint2 v = reinterpret_cast<const uint2*>(cluster.map_shared_rank(s_bins, b))[rank * (kSlice / 4) + t];
-    own[0] += v.x & 0xFFFFu; own[1] += v.x >> 16;
-    own[2] += v.y & 0xFFFFu; own[3] += v.y >> 16;
+    for (int b = 0; b < kSampleBlocks; ++b) v[b] = cluster.map_shared_rank(s_bins, b)[rank * (kSlice / 2) + t];
+#pragma unroll
+    for (int b = 0; b < kSampleBlocks; ++b) {
+      own[0] += v[b] & 0xFFFFu;
+      own[1] += v[b] >> 16;
+    }
   }
-  const unsigned int mine = own[0] + own[1] + own[2] + own[3];
+  const unsigned int mine = own[0] + own[1];
   unsigned int incl = mine;  // this thread and all higher lanes of the warp
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -172,13 +184,8 @@ k_sample(BucketSrc<DTYPE> src, const float* __restrict__ addend, unsigned long l
   }
   if (lane == 0) s_scan[warp] = incl;
   __syncthreads();
-  unsigned int above = incl - mine, total = 0;
-#pragma unroll
-  for (int w = 0; w < kSampleThreads / 32; ++w) {
-    const unsigned int c = s_scan[w];
-    if (w > warp) above += c;
-    total += c;
-  }
+  const unsigned int of_warp = s_scan[lane], total = __reduce_add_sync(0xFFFFFFFFu, of_warp);
+  unsigned int above = incl - mine + __reduce_add_sync(0xFFFFFFFFu, lane > warp ? of_warp : 0u);
   if (t < kSampleBlocks) *cluster.map_shared_rank(&s_slice[rank], t) = total;
   cluster.sync();  // also: no block leaves while its bins are still read
   for (int s = rank + 1; s < kSampleBlocks; ++s) above += s_slice[s];
@@ -188,11 +195,11 @@ k_sample(BucketSrc<DTYPE> src, const float* __restrict__ addend, unsigned long l
     if (above < j && j <= above + mine) {  // exactly one thread of the cluster, if any
       unsigned int a = above;
 #pragma unroll
-      for (int b = 3; b >= 0; --b) {
+      for (int b = 1; b >= 0; --b) {
         if (a < j && j <= a + own[b]) {
-          const unsigned int bin = rank * kSlice + t * 4 + b;
-          if (which == 0) ctl->lo = bin << (31 - kSampleBinBits);
-          else ctl->hi = (bin + 1) << (31 - kSampleBinBits);
+          const unsigned int bin = rank * kSlice + t * 2 + b;
+          if (which == 0) ctl->lo = sample_bin_begin(bin);
+          else ctl->hi = sample_bin_end(bin);
         }
         a += own[b];
       }
