@@ -9,9 +9,10 @@
 // summed through distributed shared memory, and the barriers are the cluster's.
 //
 // Measured (one B200, whole call, int8, kept fraction 0.001 / 0.1 / 0.5): 12,289 elements 25 / 27 / 27 us with the other
-// strategies, 12-13 us here (the host's share of a call is about 12); 65,536 elements 19 / 26 / 29 -> 13.5 / 16 / 18;
+// strategies, 12-13 us here; 65,536 elements 19 / 26 / 29 -> 13.5 / 16 / 18;
 // 131,072 elements 19 / 28 / 29 -> 17 / 19 / 24; at 200,000 elements it is even, hence the limit.  One block instead of
-// the cluster pays up to about 8,000 elements.
+// the cluster pays up to about 8,000 elements.  The keys of the first digit's bin by themselves where they are few, instead
+// of two more digits: 8,192 elements at 0.1 11.0 -> 10.0, 12,289 12.1 -> 10.9, 40,000 14.6 -> 13.1, 163,840 at 0.001 19.1 -> 16.9.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -25,10 +26,11 @@ constexpr int kSmallBlocks = 8;
 constexpr unsigned int kSmallOneBlock = 8192;      // largest bucket that one block takes on its own
 constexpr unsigned int kSmallPerBlock = 20480;     // elements a block holds at most
 constexpr int64_t kSmallMaxN = (int64_t)kSmallBlocks * kSmallPerBlock;
+constexpr unsigned int kSmallKeys = kSmallThreads;  // keys of the first digit's bin that are looked at one per thread
 
 struct SmallShared {
   unsigned int hist[kMaxBins];
-  unsigned int tot[kSmallThreads / 32], out[3], slice[kSmallBlocks];
+  unsigned int tot[kSmallThreads / 32], out[3], slice[kSmallBlocks], listed;
   uint2 warp_sum[kSmallThreads / 32], block_sum[kSmallBlocks];
   float qmax[kSmallThreads / 32];
 };
@@ -53,6 +55,7 @@ k_select_small(BucketSrc<DTYPE> src, FinalizeParams p, unsigned int per_block, i
   pdl_wait();
   pdl_launch_dependents();
   if (rank == 0 && t == 0 && !keep_status) p.ctl->status = NSML_OK;
+  if (t == 0) sh.listed = 0;
 
   // ---------------- load; histogram of digit 0 ----------------
   bool nonfinite = false;
@@ -127,6 +130,7 @@ k_select_small(BucketSrc<DTYPE> src, FinalizeParams p, unsigned int per_block, i
           unsigned int* out = cluster.map_shared_rank(sh.out, b);
           out[0] = rank * slice + t;
           out[1] = rem - above;
+          out[2] = own;
         }
       }
       if (level < 2)
@@ -136,6 +140,44 @@ k_select_small(BucketSrc<DTYPE> src, FinalizeParams p, unsigned int per_block, i
     prefix = (prefix << digit_bits(level)) | sh.out[0];
     rem = sh.out[1];
     if (level == 2) break;
+    if (level == 0 && sh.out[2] <= kSmallKeys) {
+      // The bin's keys, each block's in its histogram's place, then one per thread of every block: the threshold bit by
+      // bit.  (Two more digits take six barriers of the cluster and two passes over the elements.  Up to four keys per
+      // thread: 4 us slower than one, whatever the bin holds.)
+      const unsigned int in_bin = sh.out[2];
+      if (BLOCKS == 1) __syncthreads();
+      for (unsigned int i = t * 4; i < E; i += THREADS * 4) {
+        const uint4 q = *reinterpret_cast<const uint4*>(s_val + i);
+        const uint32_t b[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const uint32_t key = b[e] & 0x7FFFFFFFu;
+          if (i + e < E && (key >> digit_shift(0)) == prefix) sh.hist[atomicAdd(&sh.listed, 1u)] = key;
+        }
+      }
+      sync_all();
+      uint32_t key = 0;
+      if (BLOCKS == 1) {
+        if ((unsigned)t < in_bin) key = sh.hist[t];
+      } else {
+        const unsigned int count = lane < BLOCKS ? *cluster.map_shared_rank(&sh.listed, lane) : 0u;
+        unsigned int at = t, from = 0;
+#pragma unroll
+        for (int b = 0; b < BLOCKS; ++b) {
+          const unsigned int c = __shfl_sync(FULL, count, b);
+          if (from == (unsigned)b && at >= c) {
+            at -= c;
+            ++from;
+          }
+        }
+        if ((unsigned)t < in_bin) key = cluster.map_shared_rank(sh.hist, from)[at];
+      }
+      prefix <<= digit_shift(0);
+      for (uint32_t bit = 1u << (digit_shift(0) - 1); bit != 0; bit >>= 1)
+        if ((unsigned)__syncthreads_count((unsigned)t < in_bin && key >= (prefix | bit)) >= rem) prefix |= bit;
+      rem -= __syncthreads_count((unsigned)t < in_bin && key > prefix);
+      break;
+    }
     if (BLOCKS == 1) {
       for (int b = t; b < kMaxBins; b += THREADS) sh.hist[b] = 0;
       __syncthreads();

@@ -57,3 +57,24 @@ def test_feedback(n, dtype):
         ref, want = error_feedback_step(g, want, ratio, bits, prune_mask_=mask)
         assert_payload_equal(payload, ref)
         assert np.array_equal(residual.cpu().numpy().view(np.uint32), want.view(np.uint32))
+
+
+# the threshold's bin (a sixteenth of an octave) with as many keys as are looked at one per thread, one fewer and one more;
+# all in one block's part or spread over the cluster's, distinct or equal
+@pytest.mark.parametrize("n", [6000, 8192, 8193, 60_000])
+@pytest.mark.parametrize("count", [1, 2, 1023, 1024, 1025])
+@pytest.mark.parametrize("kind", ["spread", "together", "equal", "zeros"])
+def test_keys_of_the_first_digits_bin(n, count, kind):
+    rng = np.random.default_rng(n + count)
+    g = (rng.random(n) * 1e-3 + 1e-6).astype(np.float32)
+    order = np.arange(n) if kind == "together" else rng.permutation(n)
+    if kind == "zeros":
+        g[order[:count]] = 0.0  # (pruned parameters and empty rows share the lowest bin)
+        ratios = [(n - count + take) / n for take in {1, (count + 1) // 2, count}]
+    else:
+        g[order[:count]] = 1.01 if kind == "equal" else 1.0 + rng.random(count) * 0.06
+        g[order[count:count + 100]] = 8.0 + rng.random(100).astype(np.float32)
+        ratios = [(100 + take) / n for take in {1, (count + 1) // 2, count}]
+    g *= rng.choice(np.array([-1.0, 1.0], np.float32), n)
+    for ratio in ratios:
+        check_compress(g, ratio * (1 - 1e-9), 8)
