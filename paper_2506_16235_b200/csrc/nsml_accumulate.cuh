@@ -76,7 +76,7 @@ __host__ __device__ inline bool header_ok(const nsml_payload_header* h, unsigned
 // offsets[w][b] = first payload entry of worker w whose index is >= b * tile.
 //
 // What bounds the kernel is its chain of dependent reads (about 1 us each from DRAM).  Payloads of few entries are read
-// as a whole (kPartScan): a thread compares the tiles of four neighbouring entries and writes the boundaries between
+// as a whole (kPartScan, kPartShare): a thread compares the tiles of four neighbouring entries and writes the boundaries between
 // them, so that there are two reads in a row, header and indices; and the indices are in L2 when the sum reads them.
 // Where that is more to read than a search (every entry against some 200 bytes per boundary), a block settles
 // kPartBounds consecutive boundaries of one worker, a thread each: kPartProbes evenly spaced indices of the whole array go
@@ -98,14 +98,16 @@ constexpr unsigned int kPartProbes = kPartBounds;  // one per thread
 constexpr unsigned int kPartWindow = 16;
 constexpr unsigned int kPartScan = 8u << 20;  // entries of all workers up to which they are read as a whole: 32 MB, 5 us
 constexpr unsigned int kPartParts = 64;       // blocks per worker for that, at most
+constexpr unsigned int kPartShare = 16384;    // ... and entries per block: four rounds of its threads
 // Blocks per worker: 8192 entries each of the largest payload, as far as the buffers' sizes tell (an entry takes five bytes
-// at least), otherwise of a 16th of the bucket.  No more than that, because blocks that find nothing to do still hold an SM's
-// threads until the header is there: 64 of them for each of eight workers made four streams' steps 20 % longer.
-inline unsigned int partition_blocks(int64_t n, unsigned int tiles, unsigned long long largest_payload) {
+// at least), otherwise of an 8th of the bucket.  At most 128 for all workers, because blocks that find little to do still hold half an
+// SM each until the kernel before them is done and the header is there: 64 for each of eight workers made four streams' steps
+// 20 % longer and sums of eight dense payloads 5 %.  (many_calls: nsml_set_list_block_candidates above its default.)
+inline unsigned int partition_blocks(int64_t n, unsigned int tiles, int W, unsigned long long largest_payload, bool many_calls) {
   const unsigned int search = tiles / kPartBounds + 1;
-  const unsigned long long entries = largest_payload != 0 ? largest_payload / 5 : (unsigned long long)n / 16;
+  const unsigned long long entries = largest_payload != 0 ? largest_payload / 5 : (unsigned long long)n / 8;
   const unsigned long long scan = entries / 8192 + 1;
-  const unsigned int parts = scan < kPartParts ? (unsigned int)scan : kPartParts;
+  const unsigned int each = 128u / W < 1 ? 1u : 128u / W < kPartParts ? 128u / W : kPartParts, most = many_calls ? (each + 3) / 4 : each, parts = scan < most ? (unsigned int)scan : most;
   return search > parts ? search : parts;
 }
 
@@ -177,8 +179,9 @@ k_partition(PayloadTable table, int W, unsigned long long n, unsigned int tiles,
     return;
   }
   const uint32_t* idx = reinterpret_cast<const uint32_t*>(table.p[w] + h->idx_off);
-  if (h->k * (unsigned long long)W <= kPartScan) {
-    if (blockIdx.x < kPartParts) scan_bounds(idx, (unsigned int)h->k, tiles, tile_shift, blockIdx.x, min(gridDim.x, kPartParts), all);
+  const unsigned int parts = min(gridDim.x, kPartParts);
+  if (h->k * (unsigned long long)W <= kPartScan && h->k <= parts * (unsigned long long)kPartShare) {
+    if (blockIdx.x < parts) scan_bounds(idx, (unsigned int)h->k, tiles, tile_shift, blockIdx.x, parts, all);
     return;
   }
   if (count == 0) return;

@@ -424,7 +424,9 @@ static int accumulate_impl(const void* const* payloads, const size_t* payload_by
   for (int w = 0; w < W; ++w) largest = table.bytes[w] > largest ? table.bytes[w] : largest;
   {
     LaunchScope scope(K_PARTITION, st, timed);  // also clears the status word
-    launch_prio(k_partition, dim3(partition_blocks(n, tiles, largest), W), dim3(kPartBounds), 0, st, false, 0, true, true, table, W, (unsigned long long)n,
+    // (where many calls are in flight, blocks that wait for the kernel before them would hold what the others need)
+    const bool many = g_list_block_candidates.load(std::memory_order_relaxed) > kListBlockCandidates;
+    launch_prio(k_partition, dim3(partition_blocks(n, tiles, W, largest, many), W), dim3(kPartBounds), 0, st, false, 0, true, !many, table, W, (unsigned long long)n,
                 tiles, tile == kDenseTileLarge ? 13u : 11u, offsets, status);
   }
   {

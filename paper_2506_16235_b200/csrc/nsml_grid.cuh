@@ -23,8 +23,8 @@
 // A sample that misled costs more rounds: a threshold above the window, a histogram of
 // what lies there; fewer than k candidates, a second stream with lo = 0.
 //
-// What bounds it: instructions, about 300 per 128 elements (75 in the stream, 200 where
-// the survivors are written), and four or five steps in which every block waits for the
+// What bounds it: instructions, about 580 per 128 elements at 0.5 by the counters, the
+// walk that writes the survivors and the stream before all, and four or five steps in which every block waits for the
 // others (2 to 4 us each).  Measured (one B200, whole call, before / now; before: a radix
 // select in three digits over a shared-memory copy, every element looked at by every
 // phase, add and subtract of a residual as kernels of their own): 6.55M float32 elements
@@ -631,7 +631,7 @@ k_select_grid(BucketSrc<DTYPE> src, FinalizeParams p, unsigned int segs, unsigne
           const unsigned int row = r0 + r * NW;
           unsigned int a = 0, e = 0;
 #pragma unroll
-          for (int j = 0; j < LOADS; ++j) {  // (at most LOADS * 4096 in either half)
+          for (int j = 0; j < LOADS; ++j) {  // (at most LOADS * 8192 in either half)
             const unsigned int b = j * 64 + lane * 2;
             a += w[r][j];
             e += b + 1 < blk ? w[r][j] : b < blk ? w[r][j] & 0xFFFFu : 0u;
