@@ -19,6 +19,14 @@
 
 namespace nsml {
 
+// A CUDA call failed: what the call returns.  The runtime keeps the error of a refused launch or copy for the thread's next
+// cudaGetLastError, which is not to meet it again: the calls that follow have nothing to do with it.  (Every launch is
+// checked by its own return code.)
+static int cuda_error() {
+  cudaGetLastError();
+  return NSML_ERR_CUDA;
+}
+
 enum KernelId {
   K_SAMPLE = 0, K_COMPACT_BUCKET, K_EMIT, K_PARTITION, K_MERGE, K_CLEAR, K_SELECT_GRID,
   K_SUMSQ, K_PRUNE_PASS, K_PRUNE_FINISH, K_SELECT_SMALL, K_COUNT
@@ -87,11 +95,11 @@ static std::mutex g_dev_mutex;
 
 static int device_info(const DeviceInfo** out) {
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return NSML_ERR_CUDA;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cuda_error();
   std::lock_guard<std::mutex> lock(g_dev_mutex);
   DeviceInfo& d = g_dev[dev];
   if (!d.ready) {
-    if (cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return NSML_ERR_CUDA;
+    if (cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return cuda_error();
     cudaError_t e = cudaSuccess;
     auto prepare = [&](auto kernel, int threads, size_t smem, int* resident) {
       if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -133,8 +141,7 @@ static int device_info(const DeviceInfo** out) {
     int coop = 0;
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
     if (e != cudaSuccess || d.grid < 1 || list_fits < 1 || d.merge_small < 1 || d.merge_large < 1 || !coop) {
-      cudaGetLastError();
-      return NSML_ERR_CUDA;
+      return cuda_error();
     }
     d.ready = true;
   }
@@ -200,6 +207,16 @@ static cudaError_t launch_prio(void (*kernel)(KArgs...), dim3 grid, dim3 block, 
   }
   cfg.attrs = attr;
   cfg.numAttrs = na;
+  return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+
+// without any attribute: at the priority of the stream
+template <class... KArgs, class... Args>
+static cudaError_t launch_plain(void (*kernel)(KArgs...), unsigned int grid, unsigned int block, cudaStream_t st, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.stream = st;
   return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
 }
 
@@ -291,7 +308,7 @@ static int launch_compress(const void* grad, float* residual, const uint32_t* ma
     auto kernel = one ? k_select_small<DTYPE, 1> : k_select_small<DTYPE, kSmallBlocks>;
     le = launch_prio(kernel, dim3(blocks), dim3(kSmallThreads), (size_t)per_block * 4, st, false, one ? 0 : kSmallBlocks, true, true, src, fp,
                      per_block, keep_status ? 1 : 0);
-    return le == cudaSuccess ? NSML_OK : NSML_ERR_CUDA;
+    return le == cudaSuccess ? NSML_OK : cuda_error();
   }
   if (use_dense<FDTYPE>(n, k, dev)) {
     // Bounds four standard deviations either side of the threshold's expected rank: one call in 16,000 takes another round
@@ -311,7 +328,7 @@ static int launch_compress(const void* grad, float* residual, const uint32_t* ma
       LaunchScope scope(K_CLEAR, st);
       le = launch_prio(k_clear, dim3(8), dim3(kCta), 0, st, false, 0, true, true, reinterpret_cast<uint4*>(ws), (unsigned int)(L.zero_bytes / 16),
                        keep_status ? 1 : 0);
-      if (le != cudaSuccess) return NSML_ERR_CUDA;
+      if (le != cudaSuccess) return cuda_error();
     }
     LaunchScope scope(K_SELECT_GRID, st);
     const bool fb = residual != nullptr, masked = mask != nullptr;
@@ -320,7 +337,7 @@ static int launch_compress(const void* grad, float* residual, const uint32_t* ma
                         : (masked ? k_select_grid<DTYPE, false, true> : k_select_grid<DTYPE, false, false>),
                      dim3(grid), dim3(kGridThreads), fixed + (size_t)room * kGridSliceBytes, st, true, 0, false, true, src, fp, segs, rows, cap,
                      room, plan.rank_lo, plan.rank_hi);
-    return le == cudaSuccess ? NSML_OK : NSML_ERR_CUDA;
+    return le == cudaSuccess ? NSML_OK : cuda_error();
   }
   const SamplePlan plan = sample_plan(n, k, DTYPE);
   {
@@ -328,7 +345,7 @@ static int launch_compress(const void* grad, float* residual, const uint32_t* ma
     le = launch_prio(k_sample<DTYPE>, dim3(kSampleBlocks), dim3(kSampleThreads), 0, st, false, 0, true, true, src, residual,
                      (unsigned long long)n, plan.rank_lo, plan.rank_hi, ctl, reinterpret_cast<uint4*>(ws),
                      (unsigned int)(L.zero_bytes / 16), keep_status ? 1 : 0);
-    if (le != cudaSuccess) return NSML_ERR_CUDA;
+    if (le != cudaSuccess) return cuda_error();
   }
   {
     LaunchScope scope(K_COMPACT_BUCKET, st);  // a block per tile
@@ -336,7 +353,7 @@ static int launch_compress(const void* grad, float* residual, const uint32_t* ma
     le = launch_prio(fb ? (masked ? k_compact_bucket<DTYPE, true, true> : k_compact_bucket<DTYPE, true, false>)
                         : (masked ? k_compact_bucket<DTYPE, false, true> : k_compact_bucket<DTYPE, false, false>),
                      dim3(fp.tiles), dim3(kCta), 0, st, false, 0, false, true, src, residual, (unsigned long long)n, ctl, fp.list);
-    if (le != cudaSuccess) return NSML_ERR_CUDA;
+    if (le != cudaSuccess) return cuda_error();
   }
   {
     // Blocks draw chunks of the list by ticket, so the grid is free.  For a call that has the GPU to itself a block per
@@ -362,7 +379,7 @@ static int launch_compress(const void* grad, float* residual, const uint32_t* ma
     const unsigned int grid = want < (double)cap ? (unsigned int)want : cap;
     // long lists: larger chunks, a block takes several
     le = launch_prio(short_list ? k_emit<FDTYPE, kEmitPer> : k_emit<FDTYPE, 2 * kEmitPer>, dim3(grid), dim3(kEmitThreads), sizeof(EmitShared), st, false, 0, true, true, fsrc, fp);
-    if (le != cudaSuccess) return NSML_ERR_CUDA;
+    if (le != cudaSuccess) return cuda_error();
   }
   return NSML_OK;
 }
@@ -388,7 +405,6 @@ static int compress_impl(const void* grad, int64_t n, int grad_dtype, double rat
   if (grad_dtype == NSML_F32) rc = launch_compress<NSML_F32, NSML_F32>(grad, nullptr, prune_mask, n, k, bits, ws, pl, L, P, *dev, st, keep_status);
   else rc = launch_compress<NSML_BF16, NSML_BF16>(grad, nullptr, prune_mask, n, k, bits, ws, pl, L, P, *dev, st, keep_status);
   if (rc != NSML_OK) return rc;
-  if (cudaGetLastError() != cudaSuccess) return NSML_ERR_CUDA;
   return NSML_OK;
 }
 
@@ -422,21 +438,23 @@ static int accumulate_impl(const void* const* payloads, const size_t* payload_by
   const unsigned int tiles = (unsigned int)((n + tile - 1) / tile);
   unsigned long long largest = 0;  // payload, in bytes; 0 = not known
   for (int w = 0; w < W; ++w) largest = table.bytes[w] > largest ? table.bytes[w] : largest;
+  cudaError_t le;
   {
     LaunchScope scope(K_PARTITION, st, timed);  // also clears the status word
     // (where many calls are in flight, blocks that wait for the kernel before them would hold what the others need)
     const bool many = g_list_block_candidates.load(std::memory_order_relaxed) > kListBlockCandidates;
-    launch_prio(k_partition, dim3(partition_blocks(n, tiles, W, largest, many), W), dim3(kPartBounds), 0, st, false, 0, true, !many, table, W, (unsigned long long)n,
+    le = launch_prio(k_partition, dim3(partition_blocks(n, tiles, W, largest, many), W), dim3(kPartBounds), 0, st, false, 0, true, !many, table, W, (unsigned long long)n,
                 tiles, tile == kDenseTileLarge ? 13u : 11u, offsets, status);
+    if (le != cudaSuccess) return cuda_error();
   }
   {
     LaunchScope scope(K_MERGE, st, timed);
     const bool large = tile == kDenseTileLarge;
     const unsigned int grid = grid_for(tiles, 1, dev->sms * (large ? dev->merge_large : dev->merge_small));
     auto kernel = large ? k_merge<kDenseTileLarge> : k_merge<kDenseTileSmall>;
-    launch_prio(kernel, dim3(grid), dim3(kMergeThreads), 0, st, false, 0, false, true, table, W, dense, (unsigned long long)n, zero_first, tiles, offsets, status);
+    le = launch_prio(kernel, dim3(grid), dim3(kMergeThreads), 0, st, false, 0, false, true, table, W, dense, (unsigned long long)n, zero_first, tiles, offsets, status);
+    if (le != cudaSuccess) return cuda_error();
   }
-  if (cudaGetLastError() != cudaSuccess) return NSML_ERR_CUDA;
   return NSML_OK;
 }
 
@@ -458,18 +476,19 @@ static int sumsq_impl(const void* grad, int64_t n, int grad_dtype, void* workspa
   int rc = device_info(&dev);
   if (rc != NSML_OK) return rc;
   unsigned char* ws = static_cast<unsigned char*>(workspace);
-  if (cudaMemsetAsync(ws, 0, 256, st) != cudaSuccess) return NSML_ERR_CUDA;
+  if (cudaMemsetAsync(ws, 0, 256, st) != cudaSuccess) return cuda_error();
   SumsqCtl* ctl = reinterpret_cast<SumsqCtl*>(ws);
   double* partials = reinterpret_cast<double*>(ws + 256);
   const unsigned int grid = stream_grid(n, *dev, dev->sumsq < 8 ? dev->sumsq : 8, kSumsqMaxBlocks);
   {
     LaunchScope scope(K_SUMSQ, st);
+    cudaError_t le;
     if (grad_dtype == NSML_F32)
-      k_sumsq<NSML_F32><<<grid, kCta, 0, st>>>(BucketSrc<NSML_F32>{grad, nullptr}, (unsigned long long)n, ctl, partials, to_host);
+      le = launch_plain(k_sumsq<NSML_F32>, grid, kCta, st, BucketSrc<NSML_F32>{grad, nullptr}, (unsigned long long)n, ctl, partials, to_host);
     else
-      k_sumsq<NSML_BF16><<<grid, kCta, 0, st>>>(BucketSrc<NSML_BF16>{grad, nullptr}, (unsigned long long)n, ctl, partials, to_host);
+      le = launch_plain(k_sumsq<NSML_BF16>, grid, kCta, st, BucketSrc<NSML_BF16>{grad, nullptr}, (unsigned long long)n, ctl, partials, to_host);
+    if (le != cudaSuccess) return cuda_error();
   }
-  if (cudaGetLastError() != cudaSuccess) return NSML_ERR_CUDA;
   return NSML_OK;
 }
 
@@ -498,9 +517,9 @@ static int sumsq_wait(const void* grad, int64_t n, int grad_dtype, void* workspa
   SumsqCtl* host = slot.at;
   if (host == nullptr) {
     host = &pageable;
-    if (cudaMemcpyAsync(host, workspace, sizeof(*host), cudaMemcpyDeviceToHost, st) != cudaSuccess) return NSML_ERR_CUDA;
+    if (cudaMemcpyAsync(host, workspace, sizeof(*host), cudaMemcpyDeviceToHost, st) != cudaSuccess) return cuda_error();
   }
-  if (cudaStreamSynchronize(st) != cudaSuccess) return NSML_ERR_CUDA;
+  if (cudaStreamSynchronize(st) != cudaSuccess) return cuda_error();
   if (host->status != NSML_OK) return host->status;
   *sumsq = host->sumsq;
   return NSML_OK;
@@ -543,8 +562,8 @@ static int prune_impl(const float* weights, int64_t n, double ratio, uint32_t* m
   if (rc != NSML_OK) return rc;
   unsigned char* ws = static_cast<unsigned char*>(workspace);
   if (m == 0) {  // ratio 1: nothing is pruned
-    if (cudaMemsetAsync(ws, 0, 256, st) != cudaSuccess) return NSML_ERR_CUDA;
-    if (cudaMemsetAsync(mask, 0, (size_t)((n + 31) / 32) * 4, st) != cudaSuccess) return NSML_ERR_CUDA;
+    if (cudaMemsetAsync(ws, 0, 256, st) != cudaSuccess) return cuda_error();
+    if (cudaMemsetAsync(mask, 0, (size_t)((n + 31) / 32) * 4, st) != cudaSuccess) return cuda_error();
     return NSML_OK;
   }
   Ctl* ctl = reinterpret_cast<Ctl*>(ws);
@@ -559,14 +578,14 @@ static int prune_impl(const float* weights, int64_t n, double ratio, uint32_t* m
       LaunchScope scope(K_SAMPLE, st);
       le = launch_prio(k_sample<NSML_F32>, dim3(kSampleBlocks), dim3(kSampleThreads), 0, st, false, 0, true, true, src, nullptr,
                        (unsigned long long)n, plan.rank_lo, plan.rank_hi, ctl, reinterpret_cast<uint4*>(ws), (unsigned int)(L.zero_bytes / 16), 0);
-      if (le != cudaSuccess) return NSML_ERR_CUDA;
+      if (le != cudaSuccess) return cuda_error();
     }
     LaunchScope scope(K_PRUNE_PASS, st);
     le = launch_prio(k_prune_pass, dim3((unsigned int)((n + kPruneTile - 1) / kPruneTile)), dim3(kCta), 0, st, false, 0, false, true, src,
                      (unsigned long long)n, ctl, list, (unsigned int)L.cap, mask);
-    if (le != cudaSuccess) return NSML_ERR_CUDA;
+    if (le != cudaSuccess) return cuda_error();
   } else if (cudaMemsetAsync(ws, 0, L.zero_bytes, st) != cudaSuccess) {
-    return NSML_ERR_CUDA;
+    return cuda_error();
   }
   {
     LaunchScope scope(K_PRUNE_FINISH, st);
@@ -574,9 +593,8 @@ static int prune_impl(const float* weights, int64_t n, double ratio, uint32_t* m
     le = launch_prio(k_prune_finish, dim3(grid), dim3(kPruneThreads), 0, st, false, 0, true, sampled, src, (unsigned int)n, (unsigned int)m, ctl,
                      reinterpret_cast<unsigned int*>(ws + L.hist), list, (unsigned int)L.cap, reinterpret_cast<uint2*>(ws + L.bin_list),
                      reinterpret_cast<unsigned int*>(ws + L.unit_ties), mask, sampled ? 1 : 0);
-    if (le != cudaSuccess) return NSML_ERR_CUDA;
+    if (le != cudaSuccess) return cuda_error();
   }
-  if (cudaGetLastError() != cudaSuccess) return NSML_ERR_CUDA;
   return NSML_OK;
 }
 
@@ -606,7 +624,6 @@ static int feedback_impl(const void* grad, float* residual, int64_t n, int grad_
   else
     rc = launch_compress<NSML_BF16, NSML_F32>(grad, residual, prune_mask, n, k, bits, ws, pl, L, P, *dev, st);
   if (rc != NSML_OK) return rc;
-  if (cudaGetLastError() != cudaSuccess) return NSML_ERR_CUDA;
   return NSML_OK;
 }
 
@@ -621,13 +638,12 @@ static std::mutex g_static_mutex;
 
 static int static_scratch(void** out) {
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return NSML_ERR_CUDA;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cuda_error();
   std::lock_guard<std::mutex> lock(g_static_mutex);
   if (g_static_scratch_addr[dev] == nullptr) {
     void* addr = nullptr;
     if (cudaGetSymbolAddress(&addr, g_static_scratch) != cudaSuccess || addr == nullptr) {
-      cudaGetLastError();
-      return NSML_ERR_CUDA;
+      return cuda_error();
     }
     g_static_scratch_addr[dev] = addr;
   }
@@ -706,8 +722,8 @@ int nsml_decompress_accumulate_static(const void* const* payloads, int W, float*
   rc = accumulate_impl(payloads, nullptr, W, dense, n, zero_first, scratch, NSML_STATIC_SCRATCH_BYTES, st, /*timed=*/false);
   if (rc != NSML_OK || status_out == nullptr) return rc;
   int value = 0;
-  if (cudaMemcpyAsync(&value, scratch, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess) return NSML_ERR_CUDA;
-  if (cudaStreamSynchronize(st) != cudaSuccess) return NSML_ERR_CUDA;
+  if (cudaMemcpyAsync(&value, scratch, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess) return cuda_error();
+  if (cudaStreamSynchronize(st) != cudaSuccess) return cuda_error();
   *status_out = value;
   return NSML_OK;
 }
@@ -836,15 +852,15 @@ int nsml_compress_host(const void* grad_host, int64_t n, int grad_dtype, double 
   unsigned char* d_grad = base + ws;
   unsigned char* d_mask = d_grad + align_up(gbytes, 256);
   unsigned char* d_payload = d_mask + align_up(mbytes, 256);
-  if (cudaMemcpyAsync(d_grad, grad_host, gbytes, cudaMemcpyHostToDevice, st) != cudaSuccess) return NSML_ERR_CUDA;
+  if (cudaMemcpyAsync(d_grad, grad_host, gbytes, cudaMemcpyHostToDevice, st) != cudaSuccess) return cuda_error();
   if (prune_mask_host != nullptr &&
       cudaMemcpyAsync(d_mask, prune_mask_host, mbytes, cudaMemcpyHostToDevice, st) != cudaSuccess)
-    return NSML_ERR_CUDA;
+    return cuda_error();
   int rc = compress_impl(d_grad, n, grad_dtype, ratio, bits,
                          prune_mask_host ? reinterpret_cast<const uint32_t*>(d_mask) : nullptr, d_payload, pb, base, ws,
                          st);
   if (rc != NSML_OK) return rc;
-  if (cudaMemcpyAsync(payload_host, d_payload, pb, cudaMemcpyDeviceToHost, st) != cudaSuccess) return NSML_ERR_CUDA;
+  if (cudaMemcpyAsync(payload_host, d_payload, pb, cudaMemcpyDeviceToHost, st) != cudaSuccess) return cuda_error();
   return NSML_OK;
 }
 
@@ -879,17 +895,17 @@ int nsml_decompress_accumulate_host(const void* const* payloads_host, const size
   const void* d_payloads[NSML_MAX_WORKERS];
   for (int w = 0; w < W; ++w) {
     if (cudaMemcpyAsync(cursor, payloads_host[w], payload_bytes[w], cudaMemcpyHostToDevice, st) != cudaSuccess)
-      return NSML_ERR_CUDA;
+      return cuda_error();
     d_payloads[w] = cursor;
     cursor += align_up(payload_bytes[w], 256);
   }
   if (!zero_first &&
       cudaMemcpyAsync(d_dense, dense_host, (size_t)n * 4, cudaMemcpyHostToDevice, st) != cudaSuccess)
-    return NSML_ERR_CUDA;
+    return cuda_error();
   int rc = accumulate_impl(d_payloads, payload_bytes, W, d_dense, n, zero_first, base, ws, st);
   if (rc != NSML_OK) return rc;
   if (cudaMemcpyAsync(dense_host, d_dense, (size_t)n * 4, cudaMemcpyDeviceToHost, st) != cudaSuccess)
-    return NSML_ERR_CUDA;
+    return cuda_error();
   return NSML_OK;
 }
 
@@ -897,8 +913,8 @@ int nsml_last_status(const void* workspace, void* stream, int* status_out) {
   if (workspace == nullptr || status_out == nullptr) return NSML_ERR_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   int value = 0;
-  if (cudaMemcpyAsync(&value, workspace, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess) return NSML_ERR_CUDA;
-  if (cudaStreamSynchronize(st) != cudaSuccess) return NSML_ERR_CUDA;
+  if (cudaMemcpyAsync(&value, workspace, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess) return cuda_error();
+  if (cudaStreamSynchronize(st) != cudaSuccess) return cuda_error();
   *status_out = value;
   return NSML_OK;
 }
@@ -907,9 +923,8 @@ int nsml_selftest_bounded_wait(void* workspace, size_t workspace_bytes, int max_
   if (workspace == nullptr || !aligned(workspace, 256) || max_polls < 1 || max_polls > (1 << 16)) return NSML_ERR_ARG;
   if (workspace_bytes < 256) return NSML_ERR_CAPACITY;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (cudaMemsetAsync(workspace, 0, 256, st) != cudaSuccess) return NSML_ERR_CUDA;
-  k_barrier_probe<<<2, 32, 0, st>>>(static_cast<Ctl*>(workspace), max_polls);
-  if (cudaGetLastError() != cudaSuccess) return NSML_ERR_CUDA;
+  if (cudaMemsetAsync(workspace, 0, 256, st) != cudaSuccess) return cuda_error();
+  if (launch_plain(k_barrier_probe, 2, 32, st, static_cast<Ctl*>(workspace), max_polls) != cudaSuccess) return cuda_error();
   return NSML_OK;
 }
 
