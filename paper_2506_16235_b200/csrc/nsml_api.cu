@@ -313,11 +313,12 @@ static int launch_compress(const void* grad, float* residual, const uint32_t* ma
   if (use_dense<FDTYPE>(n, k, dev)) {
     // Bounds four standard deviations either side of the threshold's expected rank: one call in 16,000 takes another round
     // (3 us), the others have a window a third narrower than with six.
-    const SamplePlan plan = sample_plan(n, k, DTYPE, 4.0);
+    SamplePlan plan = sample_plan(n, k, DTYPE, 4.0);
     const unsigned int segs = (unsigned int)(((unsigned long long)n + grid_seg<FDTYPE>() - 1) / grid_seg<FDTYPE>());
     const unsigned int most = grid_blocks(dev), grid = segs < most ? segs : most, rows = (segs + grid - 1) / grid;
     // room for twice the keys that are to be expected inside the window, the rest of the shared memory for slices
     const double keys = (double)kSamples * (DTYPE == NSML_F32 ? sample_keys<NSML_F32>() : sample_keys<NSML_BF16>());
+    if (plan.rank_lo == 0 && k != n) plan.rank_lo = (unsigned int)keys + 1;  // nearly everything is kept: an upper bound alone
     const double window = plan.rank_lo == 0 ? 0.05 : (double)(plan.rank_lo - plan.rank_hi) / keys;
     const double entries = window * (double)n / ((double)grid * kGridWarps) * 2.0 + 64.0;
     const unsigned int cap = entries < (double)kGridMaxCap ? (unsigned int)entries / 8 * 8 : kGridMaxCap;

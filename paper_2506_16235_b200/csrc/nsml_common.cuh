@@ -36,6 +36,7 @@ struct Ctl {
   unsigned int drawn[9], finished[9];  // general select, mask build: units of work of each phase
   unsigned long long listed_above;  // grid select: candidates << 32 | those above the window
   unsigned int sampled, members;    // grid select: sampler blocks done; keys of the threshold's bin
+  unsigned int zeros[4];            // grid select: zeros among the keys that the histogram of a round counted
 };
 static_assert(sizeof(Ctl) <= 256, "control block must fit its 256-byte slot");
 

@@ -21,7 +21,9 @@
 //           magnitude of every 1024 survivors
 //   write   indices and values; int8 behind one more barrier
 // A sample that misled costs more rounds: a threshold above the window, a histogram of
-// what lies there; fewer than k candidates, a second stream with lo = 0.
+// what lies there; fewer than k candidates, a second stream with lo = 0.  A sample with
+// fewer non-zero keys than its ranks says that the threshold is zero: the keys above it
+// are counted in the stream, the others are ties, and there is no window.
 //
 // What bounds it: instructions, about 580 per 128 elements at 0.5 by the counters, the
 // walk that writes the survivors and the stream before all, and four or five steps in which every block waits for the
@@ -47,7 +49,15 @@ constexpr unsigned int kGridMembers = 2048;  // keys of the threshold's bin that
 constexpr int kGridMaxBlocks = 192;
 constexpr size_t kGridSmem = 232448;         // 227 KB
 constexpr unsigned int kGridMaxCap = 384;    // window entries of a warp, at most
-constexpr unsigned int kGridFewBins = 256;   // a window of no more bins is counted in shared memory first
+// The window's histogram.  Adds to one global address run at one per nanosecond, and the keys of a bin may be any number (a
+// repeated value; a window from zero on): a block counts in shared memory and adds a bin's count once.  (With an add per
+// key, 25M float32 elements of which 54 % are zero took 18 ms at 0.5, now 0.12; of one value 16, now 0.20.)  In a short
+// float32 bucket, whose window has a few keys per warp and most bins fewer than kGridDirect per block, those few are added
+// at once and the pass over the bins behind them is left out; lists of kGridShareCap and more entries pay for it.  us, pass
+// left out / not: 6.55M at 0.5 57.2 / 58.2, 12M 80.8 / 79.1, 25M 150 / 142.
+constexpr unsigned int kGridFewBins = 256, kGridShareCap = 128;
+constexpr unsigned int kGridDirect = 4;                // a bin's first keys, counted in the upper three bits of its word, too
+constexpr unsigned int kGridCounted = (1u << 29) - 1;  // all its keys
 constexpr int kGridPitch = kGridWarps + 1;   // words between the rows of the tables
 
 template <int VT>
@@ -69,10 +79,11 @@ struct GridShared {
   unsigned long long listed;  // candidates << 32 | those above the window
   unsigned int tot[kGridWarps], out[3];
   unsigned int lo, hi, pool;
+  unsigned int zeros, heavy;  // zeros among the keys counted; bins hold keys that have not been added to the grid's
   int ok;
 };
-// The sample counts keys by their top 15 bits (of bfloat16: all), those of 64 octaves from 2^-49 on; a bound that lies
-// below them is 0.
+// The sample counts keys by their top 15 bits (of bfloat16: all), those of 64 octaves from 2^-49 on, all smaller ones that
+// are not zero in its first bin.
 constexpr unsigned int kGridSampleBins = 8192, kGridSampleBase = 78u << 7;
 constexpr unsigned int kGridSliceBytes = 512;
 template <int VT>
@@ -101,6 +112,7 @@ k_select_grid(BucketSrc<DTYPE> src, FinalizeParams p, unsigned int segs, unsigne
   constexpr int OFF_BITS = grid_off_bits<VT>();
   constexpr unsigned int SLOTS = grid_slots<VT>();
   static_assert(SEG == kGridThreads * EPL && SLICE == 1u << OFF_BITS, "a lane has EPL elements of a segment");
+  constexpr unsigned int UNIT = VT == NSML_BF16 ? 65536u : 1u;  // the smallest key that is not zero; keys are multiples of it
   constexpr int DEPTH = FEEDBACK ? 4 : 6;  // rows whose loads are in flight
   constexpr int PAIR = 2;                  // rows that are looked at together
   constexpr int THREADS = kGridThreads, NW = kGridWarps, PITCH = kGridPitch;
@@ -176,7 +188,7 @@ k_select_grid(BucketSrc<DTYPE> src, FinalizeParams p, unsigned int segs, unsigne
   for (unsigned int i = t; i < kMaxBins; i += THREADS) sh.hist[i] = 0;
   for (unsigned int i = t; i < rows * SLOTS; i += THREADS) qm[i] = 0;
   for (unsigned int i = t; i < rows; i += THREADS) extra[i] = row_t[i] = part_t[i] = 0;
-  if (t == 0) sh.lo = sh.hi = sh.pool = 0, sh.listed = 0;
+  if (t == 0) sh.lo = sh.hi = sh.pool = sh.zeros = sh.heavy = 0, sh.listed = 0;
   __syncthreads();
   if (sampler) {
     uint32_t b[KEYS];
@@ -185,8 +197,8 @@ k_select_grid(BucketSrc<DTYPE> src, FinalizeParams p, unsigned int segs, unsigne
     for (int e = 0; e < KEYS; ++e) {
       if (FEEDBACK) b[e] = __float_as_uint(__fadd_rn(__uint_as_float(b[e]), reinterpret_cast<const float*>(addend)[e]));
       if (MASKED && ((sample_mask >> e) & 1u)) b[e] = 0;
-      const unsigned int top = (b[e] & 0x7FFFFFFFu) >> 16, bin = min(max(top, kGridSampleBase) - kGridSampleBase, kGridSampleBins - 1);
-      if (bin != 0) atomicAdd(&sh.hist[bin >> 1], 1u << (16 * (bin & 1)));  // (a block has at most 8192 keys)
+      const unsigned int key = b[e] & 0x7FFFFFFFu, bin = min(max(key >> 16, kGridSampleBase) - kGridSampleBase, kGridSampleBins - 1);
+      if (key != 0) atomicAdd(&sh.hist[bin >> 1], 1u << (16 * (bin & 1)));  // (a block has at most 8192 keys)
     }
   }
   pdl_wait();  // the control block and the histograms are cleared
@@ -244,14 +256,18 @@ k_select_grid(BucketSrc<DTYPE> src, FinalizeParams p, unsigned int segs, unsigne
 #pragma unroll
     for (int b = PER - 1; b >= 0; --b) {
       const unsigned int bin = t * PER + b;
-      if (above < rank_lo && rank_lo <= above + own[b]) sh.lo = (bin + kGridSampleBase) << 16;
-      if (above < rank_hi && rank_hi <= above + own[b]) sh.hi = bin + 1 < kGridSampleBins ? (bin + 1 + kGridSampleBase) << 16 : 0u;
+      if (above < rank_lo && rank_lo <= above + own[b]) sh.lo = bin == 0 ? UNIT : (bin + kGridSampleBase) << 16;
+      if (above < rank_hi && rank_hi <= above + own[b]) sh.hi = bin + 1 < kGridSampleBins ? (bin + 1 + kGridSampleBase) << 16 : 0x80000000u;
       above += own[b];
     }
     __syncthreads();
   }
   unsigned int lo = min(sh.lo, kInfKey), hi = sh.hi;  // (as make_window)
-  if (hi <= lo) hi = 0x80000000u;
+  // The sample holds fewer keys that are not zero than either rank, or everything is kept and there was no sample: the
+  // threshold is taken for zero, with no window; the number of other keys will tell.
+  auto all_sure = [&]() { return (sh.lo | sh.hi) == 0; };
+  if (all_sure()) hi = lo = UNIT;
+  else if (hi <= lo) hi = 0x80000000u;
 
   // ---------------- what a warp keeps ----------------
   unsigned int len = 0;  // keys inside the window; more than cap: they are not all in the list
@@ -343,8 +359,9 @@ k_select_grid(BucketSrc<DTYPE> src, FinalizeParams p, unsigned int segs, unsigne
     if (VT == NSML_BF16) shift = max(shift, 16u);
   };
   set_window(lo, hi);
+  if (all_sure()) lo = 0;
   unsigned int rem = k, in_bin = 0;
-  bool single = false;
+  bool single = false, zero = false;     // the bin is one key; that is zero, and all other keys have been counted
   bool again = false, streaming = true;  // the stream is repeated, with lo = 0; it is still to be done
   unsigned int above = 0;                // of the lane: keys above the window
   bool nonfinite = false;
@@ -476,23 +493,45 @@ k_select_grid(BucketSrc<DTYPE> src, FinalizeParams p, unsigned int segs, unsigne
     // ---------------- histogram of the window ----------------
     unsigned int* ghist = p.hist + level * kMaxBins;
     {
-      const bool few = (whi - wlo - 1) >> shift < kGridFewBins;
-      auto into_bin = [&](uint32_t key) {
-        if (few) atomicAdd(&sh.hist[(key - wlo) >> shift], 1u);
-        else atomicAdd(ghist + ((key - wlo) >> shift), 1u);
-      };
+      const unsigned int direct = (whi - wlo - 1) >> shift < kGridFewBins || cap >= kGridShareCap ? 0u : kGridDirect;
+      unsigned int zeros = 0;  // of the lane: a window from zero on may hold little else, so they are added together
+      if (level != 0) {
+        for (unsigned int b = t; b < kMaxBins; b += THREADS) sh.hist[b] = 0;
+        __syncthreads();
+      }
       if (len > cap) {
         walk_slices(all_slices, [&](unsigned int, const uint32_t (&bits)[EPL], int here, unsigned int) {
 #pragma unroll
           for (int e = 0; e < EPL; ++e) {
             const uint32_t key = bits[e] & 0x7FFFFFFFu;
-            if (e < here && key - wlo < whi - wlo) into_bin(key);
+            if (e >= here || key - wlo >= whi - wlo) continue;
+            if (key == 0) ++zeros;
+            else atomicAdd(&sh.hist[(key - wlo) >> shift], 1u);
           }
         });
+        if (!PACKED && lane == 0) sh.heavy = 1;
       } else {
         walk_list([&](bool live, unsigned int, uint32_t key, unsigned int) {
-          if (live && key - wlo < whi - wlo) into_bin(key);
+          if (live && key - wlo < whi - wlo) {
+            const unsigned int bin = (key - wlo) >> shift;
+            zeros += key == 0;
+            if (PACKED) {
+              atomicAdd(&sh.hist[bin], 1u);
+            } else if ((atomicAdd(&sh.hist[bin], 1u) & kGridCounted) < direct) {
+              atomicAdd(ghist + bin, 1u);
+              atomicAdd(&sh.hist[bin], kGridCounted + 1u);
+            } else {
+              sh.heavy = 1;
+            }
+          }
         });
+      }
+      if (wlo == 0) {
+        zeros = __reduce_add_sync(FULL, zeros);
+        if (lane == 0 && zeros != 0) {
+          if (len > cap) atomicAdd(&sh.hist[0], zeros);
+          atomicAdd(&sh.zeros, zeros);
+        }
       }
       if (level == 0) {
         const unsigned int sure = __reduce_add_sync(FULL, above);
@@ -501,12 +540,13 @@ k_select_grid(BucketSrc<DTYPE> src, FinalizeParams p, unsigned int segs, unsigne
       }
       __syncthreads();
       if (level == 0 && t == 0) atomicAdd(&p.ctl->listed_above, sh.listed);
-      if (few) {
-        for (int b = t; b < (int)kGridFewBins; b += THREADS)
-          if (sh.hist[b]) {
-            atomicAdd(ghist + b, sh.hist[b]);
-            sh.hist[b] = 0;
-          }
+      if (t == 0 && sh.zeros != 0) {
+        atomicAdd(&p.ctl->zeros[level], sh.zeros);
+        sh.zeros = 0;
+      }
+      if (wlo != whi && (PACKED || sh.heavy)) {
+        for (unsigned int b = t; b <= (whi - wlo - 1) >> shift; b += THREADS)
+          if (const unsigned int c = (sh.hist[b] & kGridCounted) - (sh.hist[b] >> 29)) atomicAdd(ghist + b, c);
       }
     }
     if ((level == 1 || (lo == 0 && rank_lo != 0)) && blk == 0 && t == 0) p.ctl->drawn[3] = 1;  // (the sample was not enough)
@@ -520,7 +560,7 @@ k_select_grid(BucketSrc<DTYPE> src, FinalizeParams p, unsigned int segs, unsigne
     }
     if (level == 0) {  // (all decisions here are uniform over the grid)
       const unsigned long long both = __ldcg(&p.ctl->listed_above);
-      const unsigned int listed = (unsigned int)(both >> 32), higher = (unsigned int)both;
+      const unsigned int listed = all_sure() ? n : (unsigned int)(both >> 32), higher = (unsigned int)both;
       if (listed < k) {  // the sample misled: keep everything; the threshold lies below lo
         rem = k - listed;
         set_window(0, lo);
@@ -532,20 +572,34 @@ k_select_grid(BucketSrc<DTYPE> src, FinalizeParams p, unsigned int segs, unsigne
         load_first();
         continue;
       }
-      if (higher >= k) {  // the threshold lies above the window
+      if (higher >= k && k != n) {  // the threshold lies above the window
         set_window(whi, 0x80000000u);
         len = cap + 1;  // (the list is of no use)
         continue;
       }
       rem = k - higher;
+      if (all_sure()) {  // (rem of the zeros are kept: of k = n elements all, if there are any)
+        set_window(0, UNIT);
+        single = zero = true;
+        break;
+      }
     }
     find_digit_from_top<PER, THREADS>(own, rem, sh.tot, sh.out);
     const unsigned int from = wlo + (sh.out[0] << shift), width = 1u << shift;
     set_window(from, min(whi, from + width));
     rem = sh.out[1];
     in_bin = sh.out[2];
-    if (width == (VT == NSML_BF16 ? 65536u : 1u)) {
-      single = true;  // one key (of bfloat16 the multiple of 65536): its ties are kept up to the last one's index
+    if (from == 0) {
+      const unsigned int larger = in_bin - __ldcg(&p.ctl->zeros[level]);
+      if (rem > larger) {  // the threshold is zero
+        set_window(0, UNIT);
+        rem -= larger;
+        single = true;
+        break;
+      }
+    }
+    if (width == UNIT) {
+      single = true;  // one key: its ties are kept up to the last one's index
       break;
     }
     if (in_bin <= kGridMembers) break;
@@ -560,7 +614,10 @@ k_select_grid(BucketSrc<DTYPE> src, FinalizeParams p, unsigned int segs, unsigne
     const unsigned int slot = atomicAdd(&p.ctl->members, 1u);
     if (slot < kGridMembers) p.list.bins[slot] = make_uint2(key, idx);
   };
-  if (len > cap) {
+  if (zero) {  // a slice's other elements are ties
+    for (unsigned int row = lane; row < rows; row += 32)
+      if (row_index(row) < n) cnt[row * PITCH + warp] |= (min(n - row_index(row), SLICE) - cnt[row * PITCH + warp]) << 16;
+  } else if (len > cap) {
     walk_slices(all_slices, [&](unsigned int row, const uint32_t (&bits)[EPL], int here, unsigned int) {
       unsigned int c = 0;
 #pragma unroll
@@ -731,7 +788,7 @@ k_select_grid(BucketSrc<DTYPE> src, FinalizeParams p, unsigned int segs, unsigne
     __syncwarp();
     if (cut_row != FULL) {  // (one warp of the grid)
       unsigned int seen = 0;
-      if (len > cap) {
+      if (len > cap || T == 0) {  // (zeros may not be listed)
         walk_slices([&](unsigned int row) { return row == cut_row; }, [&](unsigned int row, const uint32_t (&bits)[EPL], int here, unsigned int) {
           unsigned int mine = 0, all, at = FULL;
 #pragma unroll
