@@ -229,39 +229,12 @@ static int64_t k_of(int64_t n, double ratio) {
   return k;
 }
 
-// What the sample of a call is asked for: the ranks (from the top, 1-based) of the two sample keys `sigmas` standard
-// deviations either side of the expected rank of the k-th largest, and the number of candidates to expect above
-// the lower one.  rank_lo = 0: do not sample (small bucket, or nearly everything is kept).
-struct SamplePlan {
-  unsigned int rank_lo = 0, rank_hi = 0;
-  double expected = 0.0;
-};
-
-static SamplePlan sample_plan(int64_t n, int64_t k, int grad_dtype, double sigmas = 6.0) {
-  SamplePlan s;
-  if (n < (int64_t)kSamples) return s;
-  const double keys = (double)kSamples * (grad_dtype == NSML_F32 ? sample_keys<NSML_F32>() : sample_keys<NSML_BF16>());
-  const double p = (double)k / (double)n, mean = keys * p, six = sigmas * std::sqrt(keys * p * (1.0 - p));
-  const double lo = std::ceil(mean + six) + 1.0, hi = std::floor(mean - six);
-  if (lo < keys) s.rank_lo = (unsigned int)lo;
-  // (the largest sampled key, with about n / keys elements above it, where that is safely fewer than k)
-  s.rank_hi = hi >= 1.0 ? (unsigned int)hi : 8.0 * (double)n / keys < (double)k ? 1u : 0u;
-  s.expected = (double)n * (mean + six) / keys * 1.04 + 64.0;  // (the bound is rounded down to 14 key bits: a few per cent more)
-  return s;
-}
-
 // nsml_set_list_block_candidates: up to the default a block of the list stage per chunk of a short list, above it few.
 constexpr int kListBlockCandidates = 4096;  // default of the knob
 constexpr double kListFewBlocks = 10;       // blocks for a short list where the knob is well above it
 static std::atomic<int> g_list_block_candidates{kListBlockCandidates};
 
-// Dense mode: the select runs over the bucket itself, with no candidate list.  (What cannot be sampled is taken by
-// use_small, which is asked first.)
 static unsigned int grid_blocks(const DeviceInfo& dev) { return (unsigned int)(dev.sms < kGridMaxBlocks ? dev.sms / 2 * 2 : kGridMaxBlocks); }
-template <int VT>
-static bool use_dense(int64_t n, int64_t k, const DeviceInfo& dev) {
-  return (double)k >= dense_from<VT>() * (double)n && n <= (int64_t)grid_max_rows<VT>() * grid_blocks(dev) * grid_seg<VT>();
-}
 
 // Small mode: the whole bucket is held in the shared memory of one block or cluster.
 static bool use_small(int64_t n) { return n <= kSmallMaxN; }
@@ -310,21 +283,8 @@ static int launch_compress(const void* grad, float* residual, const uint32_t* ma
                      per_block, keep_status ? 1 : 0);
     return le == cudaSuccess ? NSML_OK : cuda_error();
   }
-  if (use_dense<FDTYPE>(n, k, dev)) {
-    // Bounds four standard deviations either side of the threshold's expected rank: one call in 16,000 takes another round
-    // (3 us), the others have a window a third narrower than with six.
-    SamplePlan plan = sample_plan(n, k, DTYPE, 4.0);
-    const unsigned int segs = (unsigned int)(((unsigned long long)n + grid_seg<FDTYPE>() - 1) / grid_seg<FDTYPE>());
-    const unsigned int most = grid_blocks(dev), grid = segs < most ? segs : most, rows = (segs + grid - 1) / grid;
-    // room for twice the keys that are to be expected inside the window, the rest of the shared memory for slices
-    const double keys = (double)kSamples * (DTYPE == NSML_F32 ? sample_keys<NSML_F32>() : sample_keys<NSML_BF16>());
-    if (plan.rank_lo == 0 && k != n) plan.rank_lo = (unsigned int)keys + 1;  // nearly everything is kept: an upper bound alone
-    const double window = plan.rank_lo == 0 ? 0.05 : (double)(plan.rank_lo - plan.rank_hi) / keys;
-    const double entries = window * (double)n / ((double)grid * kGridWarps) * 2.0 + 64.0;
-    const unsigned int cap = entries < (double)kGridMaxCap ? (unsigned int)entries / 8 * 8 : kGridMaxCap;
-    const size_t fixed = grid_smem<FDTYPE>(rows, cap, 0);
-    unsigned int room = (unsigned int)((kGridSmem - fixed) / kGridSliceBytes);
-    if (room > rows * kGridWarps) room = rows * kGridWarps;
+  // Dense mode: the select runs over the bucket itself, with no candidate list.
+  if (const GridPlan g = grid_plan<FDTYPE>(n, k, DTYPE, grid_blocks(dev)); g.grid != 0) {
     {
       LaunchScope scope(K_CLEAR, st);
       le = launch_prio(k_clear, dim3(8), dim3(kCta), 0, st, false, 0, true, true, reinterpret_cast<uint4*>(ws), (unsigned int)(L.zero_bytes / 16),
@@ -336,8 +296,7 @@ static int launch_compress(const void* grad, float* residual, const uint32_t* ma
     // cooperative: every block co-resident; normal priority, it streams the whole bucket
     le = launch_prio(fb ? (masked ? k_select_grid<DTYPE, true, true> : k_select_grid<DTYPE, true, false>)
                         : (masked ? k_select_grid<DTYPE, false, true> : k_select_grid<DTYPE, false, false>),
-                     dim3(grid), dim3(kGridThreads), fixed + (size_t)room * kGridSliceBytes, st, true, 0, false, true, src, fp, segs, rows, cap,
-                     room, plan.rank_lo, plan.rank_hi);
+                     dim3(g.grid), dim3(kGridThreads), g.smem, st, true, 0, false, true, src, fp, g.segs, g.rows, g.cap, g.room, g.rank_lo, g.rank_hi);
     return le == cudaSuccess ? NSML_OK : cuda_error();
   }
   const SamplePlan plan = sample_plan(n, k, DTYPE);
@@ -666,7 +625,7 @@ int nsml_compress_strategy(int64_t n, double ratio) {
   const DeviceInfo* dev = nullptr;
   const int rc = device_info(&dev);
   if (rc != NSML_OK) return rc;
-  return use_dense<NSML_F32>(n, k, *dev) ? NSML_STRATEGY_DENSE : NSML_STRATEGY_LIST;
+  return grid_plan<NSML_F32>(n, k, NSML_F32, grid_blocks(*dev)).grid != 0 ? NSML_STRATEGY_DENSE : NSML_STRATEGY_LIST;
 }
 
 int nsml_set_list_block_candidates(int candidates) {

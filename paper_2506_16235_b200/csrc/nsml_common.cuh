@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "nsml.h"
+#include "nsml_plan.h"
 
 namespace nsml {
 
@@ -110,19 +111,6 @@ struct CompressLayout {  // byte offsets inside a compress workspace
   size_t raw_val;       // f32[n]: survivor values before int8 quantisation
   size_t total;
 };
-
-__host__ __device__ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
-
-// Kept fraction from which the select runs over the bucket itself (k_select_grid) and not over a candidate list.  Two
-// states in turn, us, list / grid select, buckets of tensors of different scales | of one scale throughout (every 512
-// bytes of the bucket then hold a candidate, the worst case of the grid select):
-//   float32  16M: 0.1 82 / 64 | 72 / 84, 0.15 97 / 68 | 89 / 89, 0.2 106 / 75 | 93 / 94
-//            64M: 0.1 227 / 181 | 220 / 275, 0.15 289 / 195 | 296 / 289, 0.2 415 / 217 | 327 / 299
-//   bfloat16 32M: 0.05 58 / 55 | 61 / 86, 0.1 75 / 60 | 76 / 89, 0.15 97 / 69 | 102 / 94, 0.2 113 / 76 | 117 / 96
-//            67M: 0.05 91 / 88 | 99 / 155, 0.1 128 / 103 | 135 / 158, 0.15 170 / 115 | 184 / 170, 0.2 208 / 123 | 221 / 173
-// The lines are where several scales gain a fifth or more and one scale loses no more than that.
-template <int VT>  // element type of what is selected from
-constexpr double dense_from() { return VT == NSML_F32 ? 0.125 : 0.1; }
 
 inline CompressLayout compress_layout(int64_t n) {
   CompressLayout L;

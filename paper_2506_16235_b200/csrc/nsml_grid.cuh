@@ -43,12 +43,8 @@
 
 namespace nsml {
 
-constexpr int kGridThreads = 1024, kGridWarps = kGridThreads / 32;
 constexpr int kGridSamplers = kSamples / kGridThreads;  // blocks that take the sample, a stratum per thread
 constexpr unsigned int kGridMembers = 2048;  // keys of the threshold's bin that are exchanged
-constexpr int kGridMaxBlocks = 192;
-constexpr size_t kGridSmem = 232448;         // 227 KB
-constexpr unsigned int kGridMaxCap = 384;    // window entries of a warp, at most
 // The window's histogram.  Adds to one global address run at one per nanosecond, and the keys of a bin may be any number (a
 // repeated value; a window from zero on): a block counts in shared memory and adds a bin's count once.  (With an add per
 // key, 25M float32 elements of which 54 % are zero took 18 ms at 0.5, now 0.12; of one value 16, now 0.20.)  In a short
@@ -58,17 +54,6 @@ constexpr unsigned int kGridMaxCap = 384;    // window entries of a warp, at mos
 constexpr unsigned int kGridFewBins = 256, kGridShareCap = 128;
 constexpr unsigned int kGridDirect = 4;                // a bin's first keys, counted in the upper three bits of its word, too
 constexpr unsigned int kGridCounted = (1u << 29) - 1;  // all its keys
-constexpr int kGridPitch = kGridWarps + 1;   // words between the rows of the tables
-
-template <int VT>
-__host__ __device__ constexpr unsigned int grid_seg() { return kGridThreads * (VT == NSML_F32 ? 4 : 8); }  // elements of a segment
-// An entry's place in its warp's part of the bucket has 16 bits: the row and the offset inside the row's slice.
-template <int VT>
-__host__ __device__ constexpr int grid_off_bits() { return VT == NSML_F32 ? 7 : 8; }
-template <int VT>
-__host__ __device__ constexpr unsigned int grid_max_rows() { return 1u << (16 - grid_off_bits<VT>()); }
-template <int VT>
-__host__ __device__ constexpr unsigned int grid_slots() { return grid_seg<VT>() / NSML_QBLOCK + 1; }  // payload blocks of 1024 a segment can touch
 
 struct GridShared {
   union {
@@ -82,21 +67,10 @@ struct GridShared {
   unsigned int zeros, heavy;  // zeros among the keys counted; bins hold keys that have not been added to the grid's
   int ok;
 };
+static_assert(sizeof(GridShared) == kGridSharedBytes, "the plan counts on it");
 // The sample counts keys by their top 15 bits (of bfloat16: all), those of 64 octaves from 2^-49 on, all smaller ones that
 // are not zero in its first bin.
 constexpr unsigned int kGridSampleBins = 8192, kGridSampleBase = 78u << 7;
-constexpr unsigned int kGridSliceBytes = 512;
-template <int VT>
-__host__ __device__ constexpr size_t grid_entry_bytes() { return VT == NSML_F32 ? 6 : 4; }  // of the window's list
-// what of the shared memory a row takes: three tables, six words, the maxima (scales) of its payload blocks and their
-// inverses, where its slices are
-template <int VT>
-__host__ __device__ constexpr size_t grid_row_bytes() { return (3 * kGridPitch + 6 + 2 * grid_slots<VT>()) * 4 + kGridWarps * 2; }
-// cap: window entries a warp has room for; room: slices the block has room for
-template <int VT>
-__host__ __device__ inline size_t grid_smem(unsigned int rows, unsigned int cap, unsigned int room) {
-  return align_up(sizeof(GridShared) + (size_t)rows * grid_row_bytes<VT>() + (size_t)kGridWarps * cap * grid_entry_bytes<VT>(), 16) + (size_t)room * kGridSliceBytes;
-}
 
 struct SliceScale { float scale, inv; unsigned int slots; bool one; };  // one: the slice's survivors share a payload block
 

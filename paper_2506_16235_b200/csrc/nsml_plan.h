@@ -1,0 +1,124 @@
+// What a call is launched with, worked out on the host: the ranks the sample is asked for, and whether and how the grid
+// select (nsml_grid.cuh) takes the call.  Plain C++, so that every size can be gone through without a GPU.
+#pragma once
+
+#include <cmath>
+#include <cstddef>
+#include <cstdint>
+
+#include "nsml.h"
+
+#ifdef __CUDACC__
+#define NSML_HD __host__ __device__
+#else
+#define NSML_HD
+#endif
+
+namespace nsml {
+
+NSML_HD inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
+
+// ---- the sample ----
+constexpr int kSamples = 16384;  // strata
+template <int DTYPE>
+NSML_HD constexpr int sample_keys() { return DTYPE == NSML_F32 ? 4 : 8; }  // keys per stratum: 16 bytes
+inline double sampled_keys(int grad_dtype) { return (double)kSamples * (grad_dtype == NSML_F32 ? sample_keys<NSML_F32>() : sample_keys<NSML_BF16>()); }
+
+// What the sample of a call is asked for: the ranks (from the top, 1-based) of the two sample keys `sigmas` standard
+// deviations either side of the expected rank of the k-th largest, and the number of candidates to expect above
+// the lower one.  rank_lo = 0: do not sample (small bucket, or nearly everything is kept).
+struct SamplePlan {
+  unsigned int rank_lo = 0, rank_hi = 0;
+  double expected = 0.0;
+};
+
+inline SamplePlan sample_plan(int64_t n, int64_t k, int grad_dtype, double sigmas = 6.0) {
+  SamplePlan s;
+  if (n < (int64_t)kSamples) return s;
+  const double keys = sampled_keys(grad_dtype);
+  const double p = (double)k / (double)n, mean = keys * p, spread = sigmas * std::sqrt(keys * p * (1.0 - p));
+  const double lo = std::ceil(mean + spread) + 1.0, hi = std::floor(mean - spread);
+  if (lo < keys) s.rank_lo = (unsigned int)lo;
+  // (the largest sampled key, with about n / keys elements above it, where that is safely fewer than k)
+  s.rank_hi = hi >= 1.0 ? (unsigned int)hi : 8.0 * (double)n / keys < (double)k ? 1u : 0u;
+  s.expected = (double)n * (mean + spread) / keys * 1.04 + 64.0;  // (the bound is rounded down to 14 key bits: a few per cent more)
+  return s;
+}
+
+// ---- the grid select ----
+constexpr int kGridThreads = 1024, kGridWarps = kGridThreads / 32;
+constexpr int kGridMaxBlocks = 192;
+constexpr size_t kGridSmem = 232448;          // 227 KB
+constexpr size_t kGridSharedBytes = 24752;    // of GridShared
+constexpr unsigned int kGridMaxCap = 384;     // window entries of a warp, at most
+constexpr int kGridPitch = kGridWarps + 1;    // words between the rows of the tables
+constexpr unsigned int kGridSliceBytes = 512;
+
+template <int VT>
+NSML_HD constexpr unsigned int grid_seg() { return kGridThreads * (VT == NSML_F32 ? 4 : 8); }  // elements of a segment
+// An entry's place in its warp's part of the bucket has 16 bits: the row and the offset inside the row's slice.
+template <int VT>
+NSML_HD constexpr int grid_off_bits() { return VT == NSML_F32 ? 7 : 8; }
+template <int VT>
+NSML_HD constexpr unsigned int grid_max_rows() { return 1u << (16 - grid_off_bits<VT>()); }
+template <int VT>
+NSML_HD constexpr unsigned int grid_slots() { return grid_seg<VT>() / NSML_QBLOCK + 1; }  // payload blocks of 1024 a segment can touch
+template <int VT>
+NSML_HD constexpr size_t grid_entry_bytes() { return VT == NSML_F32 ? 6 : 4; }  // of the window's list
+// what of the shared memory a row takes: three tables, six words, the maxima (scales) of its payload blocks and their
+// inverses, where its slices are
+template <int VT>
+NSML_HD constexpr size_t grid_row_bytes() { return (3 * kGridPitch + 6 + 2 * grid_slots<VT>()) * 4 + kGridWarps * 2; }
+// cap: window entries a warp has room for; room: slices the block has room for
+template <int VT>
+NSML_HD inline size_t grid_smem(unsigned int rows, unsigned int cap, unsigned int room) {
+  return align_up(kGridSharedBytes + (size_t)rows * grid_row_bytes<VT>() + (size_t)kGridWarps * cap * grid_entry_bytes<VT>(), 16) +
+         (size_t)room * kGridSliceBytes;
+}
+
+// Kept fraction from which the select runs over the bucket itself (k_select_grid) and not over a candidate list.  Two
+// states in turn, us, list / grid select, buckets of tensors of different scales | of one scale throughout (every 512
+// bytes of the bucket then hold a candidate, the worst case of the grid select):
+//   float32  16M: 0.1 82 / 64 | 72 / 84, 0.15 97 / 68 | 89 / 89, 0.2 106 / 75 | 93 / 94
+//            64M: 0.1 227 / 181 | 220 / 275, 0.15 289 / 195 | 296 / 289, 0.2 415 / 217 | 327 / 299
+//   bfloat16 32M: 0.05 58 / 55 | 61 / 86, 0.1 75 / 60 | 76 / 89, 0.15 97 / 69 | 102 / 94, 0.2 113 / 76 | 117 / 96
+//            67M: 0.05 91 / 88 | 99 / 155, 0.1 128 / 103 | 135 / 158, 0.15 170 / 115 | 184 / 170, 0.2 208 / 123 | 221 / 173
+// The lines are where several scales gain a fifth or more and one scale loses no more than that.
+template <int VT>  // element type of what is selected from
+constexpr double dense_from() { return VT == NSML_F32 ? 0.125 : 0.1; }
+
+// What k_select_grid is launched with.  grid = 0: it does not take the call.
+struct GridPlan {
+  unsigned int grid = 0, segs = 0, rows = 0, cap = 0, room = 0, rank_lo = 0, rank_hi = 0;
+  size_t smem = 0;
+};
+
+// VT: element type of what is selected from (float32 where a residual is added); grad_dtype: of the bucket; blocks: those
+// that are resident at once, an even number.  The one place that decides: a call is taken if the launch fits.
+template <int VT>
+inline GridPlan grid_plan(int64_t n, int64_t k, int grad_dtype, unsigned int blocks) {
+  GridPlan g;
+  if ((double)k < dense_from<VT>() * (double)n) return g;
+  // Bounds four standard deviations either side of the threshold's expected rank: one call in 16,000 takes another round
+  // (3 us), the others have a window a third narrower than with six.
+  const SamplePlan plan = sample_plan(n, k, grad_dtype, 4.0);
+  const double keys = sampled_keys(grad_dtype);
+  g.rank_lo = plan.rank_lo == 0 && k != n ? (unsigned int)keys + 1 : plan.rank_lo;  // (nearly everything is kept: an upper bound alone)
+  g.rank_hi = plan.rank_hi;
+  g.segs = (unsigned int)(((unsigned long long)n + grid_seg<VT>() - 1) / grid_seg<VT>());
+  const unsigned int grid = g.segs < blocks ? g.segs : blocks;
+  g.rows = (g.segs + grid - 1) / grid;
+  // room for twice the keys that are to be expected inside the window, the rest of the shared memory for slices
+  const double window = g.rank_lo == 0 ? 0.05 : (double)(g.rank_lo - g.rank_hi) / keys;
+  const double entries = window * (double)n / ((double)grid * kGridWarps) * 2.0 + 64.0;
+  g.cap = entries < (double)kGridMaxCap ? (unsigned int)entries / 8 * 8 : kGridMaxCap;
+  const size_t fixed = grid_smem<VT>(g.rows, g.cap, 0);
+  if (g.rows > grid_max_rows<VT>() || fixed > kGridSmem) return g;
+  const size_t room = (kGridSmem - fixed) / kGridSliceBytes, slices = (size_t)g.rows * kGridWarps;
+  g.room = (unsigned int)(room < slices ? room : slices);
+  g.smem = fixed + (size_t)g.room * kGridSliceBytes;
+  g.grid = grid;
+  return g;
+}
+
+}  // namespace nsml

@@ -30,7 +30,7 @@ namespace nsml {
 constexpr int kSampleThreads = 1024;
 constexpr int kSampleBlocks = 8;
 constexpr int kSampleLoads = 2;  // strata per thread
-constexpr int kSamples = kSampleThreads * kSampleBlocks * kSampleLoads;  // 16384 strata
+static_assert(kSamples == kSampleThreads * kSampleBlocks * kSampleLoads, "every stratum has a thread");
 
 __device__ __forceinline__ uint32_t mix32(uint32_t x) {
   x ^= x >> 16; x *= 0x7FEB352Du;
@@ -76,8 +76,6 @@ __device__ __forceinline__ void find_digit_from_top(const unsigned int (&own)[PE
   __syncthreads();
 }
 
-template <int DTYPE>
-__host__ __device__ constexpr int sample_keys() { return DTYPE == NSML_F32 ? 4 : 8; }  // keys per stratum: 16 bytes
 // Keys are counted by their top 14 bits (64 bins per octave), those of 128 octaves from 2^-96 on, in 16-bit counters: 16 KB
 // that eight blocks read from one another.  (All of the top 15 bits, 64 KB: the sum over the blocks took 3 us, now 1.)  A
 // bound that lies below them is 0.
