@@ -17,13 +17,13 @@ INCLUDE = os.path.join(ROOT, "include")
 LIB_PATH = os.path.join(PKG_DIR, "libnsml.so")
 STAMP_PATH = LIB_PATH + ".stamp"
 
-SOURCES = ["nsml_api.cu", "nsml_controller.cpp"]
+SOURCES = ["nsml_api.cu", "nsml_grid_large.cu", "nsml_controller.cpp"]
 FLAGS = [
     "-O3", "-std=c++17", "-lineinfo",
     "-gencode", "arch=compute_100a,code=sm_100a",
     "-ftz=false", "-prec-div=true", "-prec-sqrt=true", "-fmad=false",
     "-Xcompiler", "-fPIC", "-Xcompiler", "-ffp-contract=off",
-    "-shared", "-cudart", "static",
+    "-shared", "-cudart", "static", "--threads", "2",
 ]
 
 

@@ -84,6 +84,13 @@ struct LaunchScope {  // brackets one kernel launch
   }
 };
 
+template <int DTYPE>
+static GridKernel<DTYPE> grid_kernel(bool feedback, bool masked, bool large) {
+  if (large) return large_grid_kernel<DTYPE>(feedback, masked);
+  return feedback ? (masked ? k_select_grid<DTYPE, true, true, false> : k_select_grid<DTYPE, true, false, false>)
+                  : (masked ? k_select_grid<DTYPE, false, true, false> : k_select_grid<DTYPE, false, false, false>);
+}
+
 // ---- per-device launch geometry -------------------------------------------
 struct DeviceInfo {
   bool ready = false;
@@ -107,14 +114,12 @@ static int device_info(const DeviceInfo** out) {
       if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, kernel, threads, smem);
       if (*resident == 0 || r < *resident) *resident = r;
     };
-    prepare(k_select_grid<NSML_F32, false, false>, kGridThreads, kGridSmem, &d.grid);
-    prepare(k_select_grid<NSML_F32, false, true>, kGridThreads, kGridSmem, &d.grid);
-    prepare(k_select_grid<NSML_F32, true, false>, kGridThreads, kGridSmem, &d.grid);
-    prepare(k_select_grid<NSML_F32, true, true>, kGridThreads, kGridSmem, &d.grid);
-    prepare(k_select_grid<NSML_BF16, false, false>, kGridThreads, kGridSmem, &d.grid);
-    prepare(k_select_grid<NSML_BF16, false, true>, kGridThreads, kGridSmem, &d.grid);
-    prepare(k_select_grid<NSML_BF16, true, false>, kGridThreads, kGridSmem, &d.grid);
-    prepare(k_select_grid<NSML_BF16, true, true>, kGridThreads, kGridSmem, &d.grid);
+    for (const bool feedback : {false, true})
+      for (const bool masked : {false, true})
+        for (const bool large : {false, true}) {
+          prepare(grid_kernel<NSML_F32>(feedback, masked, large), kGridThreads, kGridSmem, &d.grid);
+          prepare(grid_kernel<NSML_BF16>(feedback, masked, large), kGridThreads, kGridSmem, &d.grid);
+        }
     int list_fits = 0;  // every shape of the list stage is resident at least once per SM
     prepare(k_emit<NSML_F32, kEmitPer>, kEmitThreads, sizeof(EmitShared), &list_fits);
     prepare(k_emit<NSML_BF16, kEmitPer>, kEmitThreads, sizeof(EmitShared), &list_fits);
@@ -292,11 +297,9 @@ static int launch_compress(const void* grad, float* residual, const uint32_t* ma
       if (le != cudaSuccess) return cuda_error();
     }
     LaunchScope scope(K_SELECT_GRID, st);
-    const bool fb = residual != nullptr, masked = mask != nullptr;
     // cooperative: every block co-resident; normal priority, it streams the whole bucket
-    le = launch_prio(fb ? (masked ? k_select_grid<DTYPE, true, true> : k_select_grid<DTYPE, true, false>)
-                        : (masked ? k_select_grid<DTYPE, false, true> : k_select_grid<DTYPE, false, false>),
-                     dim3(g.grid), dim3(kGridThreads), g.smem, st, true, 0, false, true, src, fp, g.segs, g.rows, g.cap, g.room, g.rank_lo, g.rank_hi);
+    le = launch_prio(grid_kernel<DTYPE>(residual != nullptr, mask != nullptr, g.large), dim3(g.grid), dim3(kGridThreads), g.smem, st, true, 0, false,
+                     true, src, fp, g.segs, g.rows, g.cap, g.room, g.rank_lo, g.rank_hi);
     return le == cudaSuccess ? NSML_OK : cuda_error();
   }
   const SamplePlan plan = sample_plan(n, k, DTYPE);

@@ -57,14 +57,14 @@ __device__ __forceinline__ bool grid_barrier(Ctl* ctl, unsigned int target, SH& 
 // than the grid can deliver, so each wait runs out after max_polls polls, the status word becomes
 // NSML_ERR_TIMEOUT and the kernel returns by itself.
 struct BarrierProbeShared { int ok; };
-__global__ void __launch_bounds__(32) k_barrier_probe(Ctl* ctl, int max_polls) {
+static __global__ void __launch_bounds__(32) k_barrier_probe(Ctl* ctl, int max_polls) {
   __shared__ BarrierProbeShared sh;
   grid_barrier(ctl, gridDim.x + 1u, sh, max_polls);
 }
 
 // Clears the control block and the histograms of a workspace (what the sample
 // kernel does on the list path) ahead of the grid select.
-__global__ void __launch_bounds__(kCta) k_clear(uint4* __restrict__ region, unsigned int count16, int keep_status) {
+static __global__ void __launch_bounds__(kCta) k_clear(uint4* __restrict__ region, unsigned int count16, int keep_status) {
   pdl_wait();
   pdl_launch_dependents();
   for (unsigned int i = blockIdx.x * kCta + threadIdx.x; i < count16; i += gridDim.x * kCta)

@@ -24,6 +24,9 @@
 // what lies there; fewer than k candidates, a second stream with lo = 0.  A sample with
 // fewer non-zero keys than its ranks says that the threshold is zero: the keys above it
 // are counted in the stream, the others are ties, and there is no window.
+// LARGE: tables and lists lie in the workspace (grid_plan says when), so that no bucket is too
+// large: 200M float32 elements at 0.5 take 1.19 ms, 310M 1.8 (the candidate list, which
+// took such calls for a while, 2.8 and 6.1; the radix select before 1.72 and 2.7).
 //
 // What bounds it: instructions, about 580 per 128 elements at 0.5 by the counters, the
 // walk that writes the survivors and the stream before all, and four or five steps in which every block waits for the
@@ -39,7 +42,9 @@
 // instead of 332 at 64M), 512 threads twice per SM (3-4 us more in the shared steps).
 #pragma once
 
-#include "nsml_list.cuh"
+#include <type_traits>
+
+#include "nsml_finalize.cuh"
 
 namespace nsml {
 
@@ -74,12 +79,14 @@ constexpr unsigned int kGridSampleBins = 8192, kGridSampleBase = 78u << 7;
 
 struct SliceScale { float scale, inv; unsigned int slots; bool one; };  // one: the slice's survivors share a payload block
 
-template <int DTYPE, bool FEEDBACK, bool MASKED>
+template <int DTYPE, bool FEEDBACK, bool MASKED, bool LARGE>
 __global__ void __launch_bounds__(kGridThreads, 1)
 k_select_grid(BucketSrc<DTYPE> src, FinalizeParams p, unsigned int segs, unsigned int rows, unsigned int cap, unsigned int room,
               unsigned int rank_lo, unsigned int rank_hi) {
   constexpr int VT = FEEDBACK ? NSML_F32 : DTYPE;  // what the list holds
-  constexpr bool PACKED = VT == NSML_BF16;         // list entries are bfloat16 keys << 16 | place
+  constexpr bool PACKED = VT == NSML_BF16;         // slices hold bfloat16 values
+  constexpr bool SHORT = PACKED && !LARGE;         // list entries are bfloat16 keys << 16 | place
+  using Place = typename std::conditional<LARGE, unsigned int, unsigned short>::type;  // an entry's: row and offset in its slice
   constexpr int ESIZE = DTYPE == NSML_F32 ? 4 : 2;
   constexpr int EPL = FEEDBACK ? 4 : 16 / ESIZE;   // elements of a lane's load
   constexpr unsigned int SEG = grid_seg<VT>(), SLICE = SEG / kGridWarps;  // elements of a segment, of a warp's part
@@ -94,7 +101,8 @@ k_select_grid(BucketSrc<DTYPE> src, FinalizeParams p, unsigned int segs, unsigne
   extern __shared__ __align__(16) unsigned char s_raw[];
   GridShared& sh = *reinterpret_cast<GridShared*>(s_raw);
   // per row and warp: survivors | ties << 16; place of the slice's first survivor; largest key
-  unsigned int* cnt = reinterpret_cast<unsigned int*>(s_raw + sizeof(GridShared));
+  unsigned char* tables = LARGE ? reinterpret_cast<unsigned char*>(p.list.off) + blockIdx.x * grid_table_bytes<VT>(rows) : s_raw + sizeof(GridShared);
+  unsigned int* cnt = reinterpret_cast<unsigned int*>(tables);
   unsigned int* base = cnt + rows * PITCH;
   unsigned int* top = base + rows * PITCH;
   unsigned int* row_s = top + rows * PITCH;     // per row: survivors, ties; those in the segments before the block's
@@ -111,9 +119,10 @@ k_select_grid(BucketSrc<DTYPE> src, FinalizeParams p, unsigned int segs, unsigne
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const unsigned int lt = (1u << lane) - 1u, G = gridDim.x, blk = blockIdx.x;
   const unsigned int n = (unsigned int)p.n, k = (unsigned int)p.k;
-  uint32_t* s_val = reinterpret_cast<uint32_t*>(lists) + warp * cap;  // the warp's list: keys, and places in its part
-  unsigned short* s_pos = reinterpret_cast<unsigned short*>(lists + (size_t)NW * cap * 4) + (PACKED ? 0 : warp * cap);
-  uint4* s_slice = reinterpret_cast<uint4*>(s_raw + grid_smem<VT>(rows, cap, 0));  // the block's slices
+  const size_t list = LARGE ? ((size_t)blk * NW + warp) * cap : warp * cap;  // the warp's list: keys, and places in its part
+  uint32_t* s_val = (LARGE ? p.list.val : reinterpret_cast<uint32_t*>(lists)) + list;
+  Place* s_pos = (LARGE ? reinterpret_cast<Place*>(p.raw_val) : reinterpret_cast<Place*>(lists + (size_t)NW * cap * 4)) + (SHORT ? 0 : list);
+  uint4* s_slice = reinterpret_cast<uint4*>(s_raw + grid_smem<VT>(LARGE ? 0 : rows, LARGE ? 0 : cap, 0));  // the block's slices
   float* residual = p.residual;
   unsigned int barriers = 0;
 
@@ -319,8 +328,8 @@ k_select_grid(BucketSrc<DTYPE> src, FinalizeParams p, unsigned int segs, unsigne
 #pragma unroll 1
     for (unsigned int i = lane; i - lane < len; i += 32) {
       const uint32_t v = i < len ? s_val[i] : 0u;
-      const unsigned int pos = PACKED ? v & 0xFFFFu : i < len ? s_pos[PACKED ? 0 : i] : 0u;
-      f(i < len, pos >> OFF_BITS, PACKED ? v & 0xFFFF0000u : v, pos & (SLICE - 1));
+      const unsigned int pos = SHORT ? v & 0xFFFFu : i < len ? s_pos[SHORT ? 0 : i] : 0u;
+      f(i < len, pos >> OFF_BITS, SHORT ? v & 0xFFFF0000u : v, pos & (SLICE - 1));
     }
   };
 
@@ -372,8 +381,8 @@ k_select_grid(BucketSrc<DTYPE> src, FinalizeParams p, unsigned int segs, unsigne
       for (int e = 0; e < EPL; ++e)
         if (inside & (1u << e)) {
           const unsigned int pos = row << OFF_BITS | (lane * EPL + e);
-          s_val[rank] = PACKED ? (bits[e] & 0x7FFF0000u) | pos : bits[e] & 0x7FFFFFFFu;
-          if (!PACKED) s_pos[rank] = (unsigned short)pos;
+          s_val[rank] = SHORT ? (bits[e] & 0x7FFF0000u) | pos : bits[e] & 0x7FFFFFFFu;
+          if (!SHORT) s_pos[rank] = (Place)pos;
           ++rank;
         }
     }
@@ -859,7 +868,7 @@ k_select_grid(BucketSrc<DTYPE> src, FinalizeParams p, unsigned int segs, unsigne
     if (mine != 0) {
       const unsigned int first = base[row * PITCH + warp], last = first + mine - 1;
       if (first / NSML_QBLOCK == last / NSML_QBLOCK && last < k)
-        atomicMax(qm + row * SLOTS + first / NSML_QBLOCK - row_at[row] / NSML_QBLOCK, top[row * PITCH + warp]);
+        atomicMax(qm + (row * SLOTS + first / NSML_QBLOCK - row_at[row] / NSML_QBLOCK), top[row * PITCH + warp]);
     }
   }
   walk_slices([&](unsigned int row) {
@@ -870,7 +879,7 @@ k_select_grid(BucketSrc<DTYPE> src, FinalizeParams p, unsigned int segs, unsigne
     unsigned int all, at = base[row * PITCH + warp] + lanes_before(__popc(flags), all);
 #pragma unroll
     for (int e = 0; e < EPL; ++e)
-      if (flags & (1u << e)) atomicMax(qm + slots + at++ / NSML_QBLOCK, bits[e] & 0x7FFFFFFFu);
+      if (flags & (1u << e)) atomicMax(qm + (slots + at++ / NSML_QBLOCK), bits[e] & 0x7FFFFFFFu);  // (slots may be below zero)
   });
   __syncthreads();
   for (unsigned int i = t; i < rows * SLOTS; i += THREADS)
@@ -899,5 +908,11 @@ k_select_grid(BucketSrc<DTYPE> src, FinalizeParams p, unsigned int segs, unsigne
       if (FEEDBACK && v != 0.0f) residual[idx] = __fsub_rn(v, decode_i8(code, scale));  // (a zero: as in quantize_group)
     });
 }
+
+template <int DTYPE>
+using GridKernel = void (*)(BucketSrc<DTYPE>, FinalizeParams, unsigned int, unsigned int, unsigned int, unsigned int, unsigned int, unsigned int);
+// The instances for large buckets are compiled beside the others, in nsml_grid_large.cu.
+template <int DTYPE>
+GridKernel<DTYPE> large_grid_kernel(bool feedback, bool masked);
 
 }  // namespace nsml

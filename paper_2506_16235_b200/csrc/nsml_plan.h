@@ -50,7 +50,8 @@ constexpr int kGridThreads = 1024, kGridWarps = kGridThreads / 32;
 constexpr int kGridMaxBlocks = 192;
 constexpr size_t kGridSmem = 232448;          // 227 KB
 constexpr size_t kGridSharedBytes = 24752;    // of GridShared
-constexpr unsigned int kGridMaxCap = 384;     // window entries of a warp, at most
+constexpr unsigned int kGridMaxCap = 384;     // window entries of a warp in shared memory, at most
+constexpr double kGridListMargin = 1.25;      // ... and how many times as many as expected there has to be room for
 constexpr int kGridPitch = kGridWarps + 1;    // words between the rows of the tables
 constexpr unsigned int kGridSliceBytes = 512;
 
@@ -69,7 +70,8 @@ NSML_HD constexpr size_t grid_entry_bytes() { return VT == NSML_F32 ? 6 : 4; }  
 // inverses, where its slices are
 template <int VT>
 NSML_HD constexpr size_t grid_row_bytes() { return (3 * kGridPitch + 6 + 2 * grid_slots<VT>()) * 4 + kGridWarps * 2; }
-// cap: window entries a warp has room for; room: slices the block has room for
+// cap: window entries a warp has room for; room: slices the block has room for.  (Tables and lists in the workspace: none
+// of either here.)
 template <int VT>
 NSML_HD inline size_t grid_smem(unsigned int rows, unsigned int cap, unsigned int room) {
   return align_up(kGridSharedBytes + (size_t)rows * grid_row_bytes<VT>() + (size_t)kGridWarps * cap * grid_entry_bytes<VT>(), 16) +
@@ -91,10 +93,14 @@ constexpr double dense_from() { return VT == NSML_F32 ? 0.125 : 0.1; }
 struct GridPlan {
   unsigned int grid = 0, segs = 0, rows = 0, cap = 0, room = 0, rank_lo = 0, rank_hi = 0;
   size_t smem = 0;
+  bool large = false;  // tables and lists lie in the workspace
 };
+// a block's tables in the workspace
+template <int VT>
+NSML_HD inline size_t grid_table_bytes(unsigned int rows) { return align_up(rows * grid_row_bytes<VT>(), 16); }
 
 // VT: element type of what is selected from (float32 where a residual is added); grad_dtype: of the bucket; blocks: those
-// that are resident at once, an even number.  The one place that decides: a call is taken if the launch fits.
+// that are resident at once, an even number.  The one place that decides: every size is taken, in a form that fits.
 template <int VT>
 inline GridPlan grid_plan(int64_t n, int64_t k, int grad_dtype, unsigned int blocks) {
   GridPlan g;
@@ -110,10 +116,20 @@ inline GridPlan grid_plan(int64_t n, int64_t k, int grad_dtype, unsigned int blo
   g.rows = (g.segs + grid - 1) / grid;
   // room for twice the keys that are to be expected inside the window, the rest of the shared memory for slices
   const double window = g.rank_lo == 0 ? 0.05 : (double)(g.rank_lo - g.rank_hi) / keys;
-  const double entries = window * (double)n / ((double)grid * kGridWarps) * 2.0 + 64.0;
-  g.cap = entries < (double)kGridMaxCap ? (unsigned int)entries / 8 * 8 : kGridMaxCap;
-  const size_t fixed = grid_smem<VT>(g.rows, g.cap, 0);
-  if (g.rows > grid_max_rows<VT>() || fixed > kGridSmem) return g;
+  const double entries = window * (double)n / ((double)grid * kGridWarps), twice = entries * 2.0 + 64.0;
+  g.cap = twice < (double)kGridMaxCap ? (unsigned int)twice / 8 * 8 : kGridMaxCap;
+  // Large buckets, whose tables (or places in the lists, 16 bits) do not fit, or whose lists would overflow (every phase then
+  // walks all slices again), have both in the workspace: the tables, 0.14 bytes an element, in the place of the candidate
+  // list's offsets, the lists, eight bytes an entry, in that of its values and of the raw values.  us, in shared memory / in
+  // the workspace, by the entries a warp is to expect (there is room for 384): 64M float32 at 0.5 (216) 306 / 407, 100M at
+  // 0.2 (264) 505 / 541, 100M at 0.5 (337) 631 / 589, 120M at 0.5 (405) 824 / 736, 150M at 0.2 (411) 977 / 801; bfloat16 at
+  // 0.2 134M (254) 228 / 287, 270M (509) 568 / 516.
+  g.large = g.rows > grid_max_rows<VT>() || grid_smem<VT>(g.rows, g.cap, 0) > kGridSmem || entries * kGridListMargin > (double)kGridMaxCap;
+  if (g.large) {
+    const double most = (double)n / ((double)grid * kGridWarps);
+    g.cap = (unsigned int)(twice < most ? twice : most) / 8 * 8;
+  }
+  const size_t fixed = g.large ? grid_smem<VT>(0, 0, 0) : grid_smem<VT>(g.rows, g.cap, 0);
   const size_t room = (kGridSmem - fixed) / kGridSliceBytes, slices = (size_t)g.rows * kGridWarps;
   g.room = (unsigned int)(room < slices ? room : slices);
   g.smem = fixed + (size_t)g.room * kGridSliceBytes;

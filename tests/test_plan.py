@@ -14,7 +14,7 @@ PROGRAM = r"""
 #include "nsml_plan.h"
 using namespace nsml;
 
-static long taken = 0, left = 0, wrong = 0;
+static long taken = 0, left = 0, large = 0, wrong = 0;
 
 // what the kernel relies on, beside that the driver accepts the launch
 template <int VT>
@@ -22,17 +22,28 @@ static void check(int64_t n, double ratio, int grad_dtype, unsigned int blocks) 
   int64_t k = (int64_t)std::ceil(ratio * (double)n);
   if (k > n) k = n;
   const GridPlan g = grid_plan<VT>(n, k, grad_dtype, blocks);
-  if (g.grid == 0) { ++left; return; }
+  if (g.grid == 0) {  // less is kept
+    wrong += (double)k >= dense_from<VT>() * (double)n;
+    ++left;
+    return;
+  }
   ++taken;
   const uint64_t seg = grid_seg<VT>();
-  bool ok = g.smem <= kGridSmem && g.smem == grid_smem<VT>(g.rows, g.cap, g.room);
+  bool ok = g.smem <= kGridSmem && g.smem == grid_smem<VT>(g.large ? 0 : g.rows, g.large ? 0 : g.cap, g.room);
   ok &= g.grid <= blocks && (g.grid % 2 == 0 || g.rows == 1);
   ok &= (uint64_t)g.segs * seg >= (uint64_t)n && (uint64_t)(g.segs - 1) * seg < (uint64_t)n;
   ok &= (uint64_t)g.rows * g.grid >= g.segs && g.rows >= 1;
   ok &= (uint64_t)g.rows * g.grid * seg < (1ull << 32);               // element indices of any row
-  ok &= g.rows <= grid_max_rows<VT>();  // an entry's place in 16 bits
+  if (g.large) {                                                      // in the workspace: 2 bytes an element, 4 and 4
+    ok &= (uint64_t)g.grid * grid_table_bytes<VT>(g.rows) <= 2ull * n;
+    ok &= (uint64_t)g.grid * kGridWarps * g.cap <= (uint64_t)n;
+  } else {
+    ok &= g.rows <= grid_max_rows<VT>();                              // an entry's place in 16 bits
+    ok &= g.cap <= kGridMaxCap;
+  }
   ok &= g.room <= g.rows * kGridWarps && g.room < 0xFFFFu;            // a slice's place + 1 in 16 bits, 0xFFFF apart
   ok &= (g.rank_lo == 0) == (k == n) && (g.rank_lo == 0 || g.rank_hi < g.rank_lo);
+  large += g.large;
   if (!ok && wrong++ < 10)
     std::printf("n %lld ratio %g type %d of %d blocks %u: grid %u segs %u rows %u cap %u room %u smem %zu ranks %u %u\n", (long long)n, ratio, VT,
                 grad_dtype, blocks, g.grid, g.segs, g.rows, g.cap, g.room, g.smem, g.rank_lo, g.rank_hi);
@@ -56,8 +67,8 @@ int main() {
       }
     }
   }
-  std::printf("%ld taken, %ld left, %ld wrong\n", taken, left, wrong);
-  return wrong == 0 && taken > 0 && left > 0 ? 0 : 1;
+  std::printf("%ld taken, %ld of them large, %ld left, %ld wrong\n", taken, large, left, wrong);
+  return wrong == 0 && taken > large && large > 0 && left > 0 ? 0 : 1;
 }
 """
 
