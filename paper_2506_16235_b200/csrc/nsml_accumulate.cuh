@@ -91,8 +91,11 @@ __host__ __device__ inline bool header_ok(const nsml_payload_header* h, unsigned
 //
 // The kernel also clears the call's status word (no separate clearing step is needed); payload errors are
 // reported by the merge kernel: a worker with a bad header gets all-zero offsets, so nothing of its payload
-// is read.  A corrupt payload whose indices do not ascend leaves boundaries unwritten or written twice: the merge
-// kernel takes no offset beyond the number of entries and checks every index against its tile.
+// is read.  In a corrupt payload, whose indices do not ascend or lie beyond the last tile, boundaries may be written more
+// than once, by any of several entries, but each is written: on the way from before the first tile to behind the last one
+// the indices pass it upwards.  Boundary 0 is 0, so if the last one is the number of entries, the ranges of the tiles cover
+// every entry, in whichever order they run, and an entry in a range that is not its tile's is found by the merge kernel,
+// which also takes no offset beyond the number of entries.
 constexpr int kPartBounds = 1024;
 constexpr unsigned int kPartProbes = kPartBounds;  // one per thread
 constexpr unsigned int kPartWindow = 16;
@@ -335,6 +338,7 @@ k_merge(PayloadTable table, int W, float* __restrict__ dense, unsigned long long
   }
   pdl_wait();  // the offsets are complete
   const unsigned int* my_offsets = offsets + threadIdx.x * per;  // thread w looks after worker w's ranges
+  if (threadIdx.x < W && blockIdx.x == 0) bad |= __ldcg(my_offsets + tiles) != entries;  // (there are entries behind the last tile)
   if (threadIdx.x < W && blockIdx.x < tiles) s_range[0][threadIdx.x] = make_uint2(min(entries, __ldcg(my_offsets + blockIdx.x)), min(entries, __ldcg(my_offsets + blockIdx.x + 1)));
   int buf = 0;
   for (unsigned int tile = blockIdx.x; tile < tiles; tile += gridDim.x, buf ^= 1) {
