@@ -89,6 +89,11 @@ __host__ __device__ inline bool header_ok(const nsml_payload_header* h, unsigned
 // workers of 52k: 6.2 with the probes, 3.5.  The launch may start under the kernel before it.  Sum as a whole: 25M 35.2 ->
 // 29.1 us, 1M added to 12.3 -> 9.6.)
 //
+// The sum's kernel may be launched once the blocks with nothing to do have left: placed around them (16 of 17 where the
+// payloads turn out to be searched, each holding half an SM's registers) its blocks are spread unevenly.  Eight payloads of
+// 655k entries, searched, in 6.55M elements: 63.8 -> 59.2 us, of 10M in 25M 229.8 -> 221; read as a whole, 250k in 25M: 29.2 ->
+// 28.5.
+//
 // The kernel also clears the call's status word (no separate clearing step is needed); payload errors are
 // reported by the merge kernel: a worker with a bad header gets all-zero offsets, so nothing of its payload
 // is read.  In a corrupt payload, whose indices do not ascend or lie beyond the last tile, boundaries may be written more
@@ -109,8 +114,12 @@ constexpr unsigned int kPartShare = 16384;    // ... and entries per block: four
 inline unsigned int partition_blocks(int64_t n, unsigned int tiles, int W, unsigned long long largest_payload, bool many_calls) {
   const unsigned int search = tiles / kPartBounds + 1;
   const unsigned long long entries = largest_payload != 0 ? largest_payload / 5 : (unsigned long long)n / 8;
+  unsigned int most = 128u / W;
+  if (most < 1) most = 1;
+  if (most > kPartParts) most = kPartParts;
+  if (many_calls) most = (most + 3) / 4;
   const unsigned long long scan = entries / 8192 + 1;
-  const unsigned int each = 128u / W < 1 ? 1u : 128u / W < kPartParts ? 128u / W : kPartParts, most = many_calls ? (each + 3) / 4 : each, parts = scan < most ? (unsigned int)scan : most;
+  const unsigned int parts = scan < most ? (unsigned int)scan : most;
   return search > parts ? search : parts;
 }
 
@@ -169,7 +178,6 @@ k_partition(PayloadTable table, int W, unsigned long long n, unsigned int tiles,
             unsigned int* __restrict__ offsets, int* status) {
   __shared__ uint32_t s_probe[kPartProbes];
   pdl_wait();
-  pdl_launch_dependents();
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *status = NSML_OK;
   const int w = blockIdx.y;
   const unsigned int first = blockIdx.x * kPartBounds, count = first > tiles ? 0u : min((unsigned)kPartBounds, tiles + 1 - first);
@@ -184,10 +192,13 @@ k_partition(PayloadTable table, int W, unsigned long long n, unsigned int tiles,
   const uint32_t* idx = reinterpret_cast<const uint32_t*>(table.p[w] + h->idx_off);
   const unsigned int parts = min(gridDim.x, kPartParts);
   if (h->k * (unsigned long long)W <= kPartScan && h->k <= parts * (unsigned long long)kPartShare) {
-    if (blockIdx.x < parts) scan_bounds(idx, (unsigned int)h->k, tiles, tile_shift, blockIdx.x, parts, all);
+    if (blockIdx.x >= parts) return;
+    pdl_launch_dependents();
+    scan_bounds(idx, (unsigned int)h->k, tiles, tile_shift, blockIdx.x, parts, all);
     return;
   }
   if (count == 0) return;
+  pdl_launch_dependents();
   unsigned int base = 0, end = (unsigned int)h->k;  // k <= n < 2^31; so is every target below: (tiles + 1) * tile < 2^32
   unsigned int gap, probes, from, to, a;
   auto probe = [&]() {
