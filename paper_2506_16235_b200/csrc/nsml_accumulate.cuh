@@ -104,7 +104,8 @@ __host__ __device__ inline bool header_ok(const nsml_payload_header* h, unsigned
 constexpr int kPartBounds = 1024;
 constexpr unsigned int kPartProbes = kPartBounds;  // one per thread
 constexpr unsigned int kPartWindow = 16;
-constexpr unsigned int kPartScan = 8u << 20;  // entries of all workers up to which they are read as a whole: 32 MB, 5 us
+constexpr unsigned int kPartScan = 8u << 20;  // entries of all workers up to which they are read as a whole: 32 MB, 5 us (the
+                                              // line below is lower, but for 8 workers from 537M elements on, 64 from 67M)
 constexpr unsigned int kPartParts = 64;       // blocks per worker for that, at most
 constexpr unsigned int kPartShare = 16384;    // ... and entries per block: four rounds of its threads
 // Blocks per worker: 8192 entries each of the largest payload, as far as the buffers' sizes tell (an entry takes five bytes

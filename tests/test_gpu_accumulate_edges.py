@@ -55,9 +55,9 @@ def test_one_workspace_sized_for_the_largest_bucket_serves_them_all():
         assert float(np.abs(dense.cpu().numpy().astype(np.float64) - ref).max()) <= 1e-6 * largest
 
 
-# The partition reads payloads of few entries (8M over all workers) as a whole, four entries per thread: numbers of entries
-# around a quad, a warp and a block; gaps of one, a few and all tiles; the first and the last tiles empty; both sides of
-# the line (64 workers: 131072 entries each), workers on different sides of it in one call.
+# The partition reads payloads of few entries (16,384 per block) as a whole, four entries per thread: numbers of entries
+# around a quad, a warp and a block; gaps of one, a few and all tiles; the first and the last tiles empty; long payloads of 64
+# workers, which are searched, beside short ones; both sides of the line, workers on different sides of it in one call.
 def _payload(n, idx, bits, seed):
     rng = np.random.default_rng(seed)
     k = idx.size
@@ -104,3 +104,30 @@ def test_partition_on_both_sides_of_its_line():
     rng = np.random.default_rng(4)
     for sizes in ([line] * W, [line + 1] * W, [line - 1 + w % 3 for w in range(W)], [line * 2 if w % 2 else 77 for w in range(W)]):
         _check_sum(n, [np.sort(rng.choice(n, k, replace=False)) for k in sizes])
+
+
+def _line(n, W, many_calls=False):
+    """Entries up to which a payload is read as a whole: 16,384 per block that the sum launches for a worker (sizes not
+    told, or larger than an 8th of the bucket: as many blocks as there may be)."""
+    blocks = max(1, min(64, 128 // W))
+    return 16_384 * ((blocks + 3) // 4 if many_calls else blocks)
+
+
+@pytest.mark.parametrize("sized", [False, True])
+@pytest.mark.parametrize("many_calls", [False, True])
+@pytest.mark.parametrize("W,n", [(1, 4_300_000), (2, 4_300_000), (8, 1_100_000), (64, 140_000)])
+def test_payloads_around_the_line_between_reading_and_searching(W, n, many_calls, sized):
+    line = _line(n, W, many_calls)
+    rng = np.random.default_rng(W)
+
+    def payloads(sizes):
+        return [np.sort(rng.permutation(n)[:k]) for k in sizes]
+
+    nsml.nsml_set_list_block_candidates(8192 if many_calls else 4096)
+    try:
+        for extra in (-1, 0, 1):
+            _check_sum(n, payloads([line + extra] * W), sized=sized)
+        _check_sum(n, payloads([line + w % 3 - 1 for w in range(W)]), sized=sized)
+        _check_sum(n, payloads([line + 4097 if w % 2 else 77 for w in range(W)]), zero_first=False, sized=sized)
+    finally:
+        nsml.nsml_set_list_block_candidates(4096)
