@@ -76,16 +76,26 @@ __device__ __forceinline__ void find_digit_from_top(const unsigned int (&own)[PE
   __syncthreads();
 }
 
-// Keys are counted by their top 14 bits (64 bins per octave), those of 128 octaves from 2^-96 on, in 16-bit counters: 16 KB
-// that eight blocks read from one another.  (All of the top 15 bits, 64 KB: the sum over the blocks took 3 us, now 1.)  A
-// bound that lies below them is 0.
-constexpr int kSampleShift = 17;
-constexpr unsigned int kSampleBins = 8192, kSampleBase = 31u << 6;
+// Keys are counted by their top 14 bits (64 bins per octave) over the 108 octaves from 2^-76 to 2^32, by their top 11 bits
+// below and above, in 16-bit counters: 16 KB that eight blocks read from one another.  (All of the top 15 bits, 64 KB: the
+// sum over the blocks took 3 us, now 1.  With 128 octaves from 2^-96 on and nothing below, buckets around 1e-30 at 0.01
+// had no lower bound, so that all of them were listed: 16M float32 elements 3120 us instead of 46.)
+constexpr int kSampleShift = 17, kSampleCoarse = 3;  // a fine bin is 2^17 keys, a coarse one 2^20
+constexpr unsigned int kSampleBins = 8192;
+constexpr unsigned int kSampleFine = 51u << 6, kSampleAbove = 159u << 6;  // key >> 17 of the first fine one, and behind the last
+constexpr unsigned int kSampleFineBin = kSampleFine >> kSampleCoarse;     // their bins
+constexpr unsigned int kSampleAboveBin = kSampleFineBin + kSampleAbove - kSampleFine;
+static_assert(kSampleAboveBin + ((1u << 14) - kSampleAbove >> kSampleCoarse) <= kSampleBins, "every key has a bin");
 __device__ __forceinline__ unsigned int sample_bin(uint32_t key) {  // 0: not counted
-  return min(max(key >> kSampleShift, kSampleBase) - kSampleBase, kSampleBins - 1);
+  const int at = (int)(key >> kSampleShift), fine = min(max(at, (int)kSampleFine), (int)kSampleAbove);
+  return ((at - fine) >> kSampleCoarse) + fine + (int)kSampleFineBin - (int)kSampleFine;  // (a select per range: 0.3 us more)
 }
-__device__ __forceinline__ uint32_t sample_bin_begin(unsigned int bin) { return (bin + kSampleBase) << kSampleShift; }
-__device__ __forceinline__ uint32_t sample_bin_end(unsigned int bin) { return bin + 1 < kSampleBins ? sample_bin_begin(bin + 1) : 0x80000000u; }
+__device__ __forceinline__ uint32_t sample_bin_begin(unsigned int bin) {  // (behind the last bin: 0x80000000)
+  if (bin < kSampleFineBin) return bin << (kSampleShift + kSampleCoarse);
+  if (bin < kSampleAboveBin) return (bin - kSampleFineBin + kSampleFine) << kSampleShift;
+  return (((bin - kSampleAboveBin) << kSampleCoarse) + kSampleAbove) << kSampleShift;
+}
+__device__ __forceinline__ uint32_t sample_bin_end(unsigned int bin) { return sample_bin_begin(bin + 1); }
 
 // Clears the per-call control region and sets ctl->lo and ctl->hi from a stratified sample of the bucket (of
 // bucket + addend when an addend is given).  rank_lo, rank_hi: ranks from the top among the sampled keys.  A rank
