@@ -204,7 +204,7 @@ class Workload:
         if n <= 163_840:  # one kernel that holds the bucket in shared memory
             self.account(acc, "k_select_small", esize * n + 4 * k + vb * k + s)
             return
-        if self.nsml.nsml_compress_strategy(n, ratio) == 1 or (esize == 2 and ratio >= 0.1):
+        if self.nsml.nsml_compress_strategy(n, ratio, self.nsml.NSML_F32 if esize == 4 else self.nsml.NSML_BF16) == 1:
             # dense strategy: the select reads the bucket itself once
             self.account(acc, "k_clear", 256 + 4 * 4 * 4096 + 4 * 8192)
             self.account(acc, "k_select_grid", esize * n + 4 * k + vb * k + s)

@@ -223,20 +223,25 @@ int nsml_compress(const void* grad, int64_t n, int grad_dtype, double ratio, int
  *                        the few keys of one bin between the bounds
  *   NSML_STRATEGY_DENSE  one cooperative kernel selects from the bucket itself,
  *                        which it holds in shared memory as far as that goes
- *                        (kept fractions from 0.125 on; bfloat16 buckets are
- *                        taken this way from 0.1 on, which this function, not
- *                        told the type, does not say)
+ *                        (kept fractions from 0.25 on below 4M elements, 0.2
+ *                        below 12M, 0.15 below 40M, else 0.125, of bfloat16
+ *                        buckets 0.1; with nsml_set_list_block_candidates
+ *                        above its default 0.25, from 32M elements on 0.2)
  * Buckets of up to 163,840 elements are taken by one kernel that holds them in
  * shared memory, whichever of the two this names for them.
+ * nsml_compress_strategy tells it for float32 buckets; nsml_compress_strategy_of
+ * for buckets of grad_dtype, residual non-zero: of nsml_compress_feedback.
  * Returns the strategy, or NSML_ERR_ARG / NSML_ERR_CUDA. */
 #define NSML_STRATEGY_LIST 0
 #define NSML_STRATEGY_DENSE 1
 int nsml_compress_strategy(int64_t n, double ratio);
+int nsml_compress_strategy_of(int64_t n, double ratio, int grad_dtype, int residual);
 
 /* nsml_set_list_block_candidates -- a tuning knob of the list strategy, for the
  * whole process: whether the list stage is laid out for a call that has the GPU
  * to itself (the default, and every value below it) or for several calls on
- * several streams at once (values above it).  The result of nsml_compress does
+ * several streams at once (values above it, which also leave more calls to the
+ * list strategy, see nsml_compress_strategy).  The result of nsml_compress does
  * not depend on it.  Blocks of the list stage take chunks of 2048 candidates
  * (long lists: 4096) by ticket; up to the default there is a block per chunk, at
  * most two per SM.  Above it a short list (up to about 600,000 candidates) gets

@@ -93,6 +93,7 @@ def _load() -> ctypes.CDLL:
         "nsml_ctrl_load": (ci, [vp, vp, sz]),
         "nsml_k_of": (i64, [i64, dbl]),
         "nsml_compress_strategy": (ci, [i64, dbl]),
+        "nsml_compress_strategy_of": (ci, [i64, dbl, ci, ci]),
         "nsml_set_list_block_candidates": (ci, [ci]),
         "nsml_payload_bytes": (sz, [i64, dbl, ci]),
         "nsml_workspace_bytes": (sz, [i64, ci]),
@@ -210,10 +211,10 @@ def nsml_set_list_block_candidates(candidates: int) -> None:
     _check(lib.nsml_set_list_block_candidates(int(candidates)), "nsml_set_list_block_candidates")
 
 
-def nsml_compress_strategy(n: int, ratio: float) -> int:
+def nsml_compress_strategy(n: int, ratio: float, grad_dtype: int = NSML_F32, residual: bool = False) -> int:
     """0 = sampled candidate list, 1 = dense select over the bucket (current device; up to 163,840 elements one kernel takes
-    the call whatever this says)."""
-    rc = int(lib.nsml_compress_strategy(int(n), float(ratio)))
+    the call whatever this says).  residual: for nsml_compress_feedback."""
+    rc = int(lib.nsml_compress_strategy_of(int(n), float(ratio), int(grad_dtype), int(residual)))
     if rc < 0:
         raise NsmlError(rc, "nsml_compress_strategy")
     return rc

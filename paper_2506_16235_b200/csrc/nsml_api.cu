@@ -239,6 +239,9 @@ constexpr int kListBlockCandidates = 4096;  // default of the knob
 constexpr double kListFewBlocks = 10;       // blocks for a short list where the knob is well above it
 static std::atomic<int> g_list_block_candidates{kListBlockCandidates};
 
+// whether the caller has said that other calls fill the GPU
+static bool many_calls() { return g_list_block_candidates.load(std::memory_order_relaxed) > kListBlockCandidates; }
+
 static unsigned int grid_blocks(const DeviceInfo& dev) { return (unsigned int)(dev.sms < kGridMaxBlocks ? dev.sms / 2 * 2 : kGridMaxBlocks); }
 
 // Small mode: the whole bucket is held in the shared memory of one block or cluster.
@@ -289,7 +292,7 @@ static int launch_compress(const void* grad, float* residual, const uint32_t* ma
     return le == cudaSuccess ? NSML_OK : cuda_error();
   }
   // Dense mode: the select runs over the bucket itself, with no candidate list.
-  if (const GridPlan g = grid_plan<FDTYPE>(n, k, DTYPE, grid_blocks(dev)); g.grid != 0) {
+  if (const GridPlan g = grid_plan<FDTYPE>(n, k, DTYPE, grid_blocks(dev), many_calls()); g.grid != 0) {
     {
       LaunchScope scope(K_CLEAR, st);
       le = launch_prio(k_clear, dim3(8), dim3(kCta), 0, st, false, 0, true, true, reinterpret_cast<uint4*>(ws), (unsigned int)(L.zero_bytes / 16),
@@ -332,7 +335,8 @@ static int launch_compress(const void* grad, float* residual, const uint32_t* ma
     const bool short_list = plan.expected <= 2.0 * dev.sms * kChunk;
     const double over = (double)g_list_block_candidates.load(std::memory_order_relaxed) / kListBlockCandidates;
     // a block per chunk, a quarter more where the GPU is the call's own: the list may be longer than expected, and a block
-    // that has to take a second chunk makes the stage a third longer (25M elements with a residual at 0.01: 101 -> 91 us)
+    // that has to take a second chunk makes the stage a third longer (25M elements with a residual at 0.01, timed in turn:
+    // 100.7 -> 97.3 us)
     double want = plan.expected * (over > 1.0 ? 1.0 : 1.25) / kChunk + 1.0;
     if (over > 1.0 && short_list && want > kListFewBlocks) {
       want /= over * over * over * over;
@@ -405,7 +409,7 @@ static int accumulate_impl(const void* const* payloads, const size_t* payload_by
   {
     LaunchScope scope(K_PARTITION, st, timed);  // also clears the status word
     // (where many calls are in flight, blocks that wait for the kernel before them would hold what the others need)
-    const bool many = g_list_block_candidates.load(std::memory_order_relaxed) > kListBlockCandidates;
+    const bool many = many_calls();
     le = launch_prio(k_partition, dim3(partition_blocks(n, tiles, W, largest, many), W), dim3(kPartBounds), 0, st, false, 0, true, !many, table, W, (unsigned long long)n,
                 tiles, tile == kDenseTileLarge ? 13u : 11u, offsets, status);
     if (le != cudaSuccess) return cuda_error();
@@ -622,13 +626,18 @@ extern "C" {
 
 int64_t nsml_k_of(int64_t n, double ratio) { return k_of(n, ratio); }
 
-int nsml_compress_strategy(int64_t n, double ratio) {
+int nsml_compress_strategy(int64_t n, double ratio) { return nsml_compress_strategy_of(n, ratio, NSML_F32, 0); }
+
+int nsml_compress_strategy_of(int64_t n, double ratio, int grad_dtype, int residual) {
   const int64_t k = k_of(n, ratio);
-  if (k == 0) return NSML_ERR_ARG;
+  if (k == 0 || (grad_dtype != NSML_F32 && grad_dtype != NSML_BF16)) return NSML_ERR_ARG;
   const DeviceInfo* dev = nullptr;
   const int rc = device_info(&dev);
   if (rc != NSML_OK) return rc;
-  return grid_plan<NSML_F32>(n, k, NSML_F32, grid_blocks(*dev)).grid != 0 ? NSML_STRATEGY_DENSE : NSML_STRATEGY_LIST;
+  const unsigned int blocks = grid_blocks(*dev);
+  const GridPlan g = grad_dtype == NSML_F32 || residual ? grid_plan<NSML_F32>(n, k, grad_dtype, blocks, many_calls())
+                                                        : grid_plan<NSML_BF16>(n, k, grad_dtype, blocks, many_calls());
+  return g.grid != 0 ? NSML_STRATEGY_DENSE : NSML_STRATEGY_LIST;
 }
 
 int nsml_set_list_block_candidates(int candidates) {

@@ -78,16 +78,32 @@ NSML_HD inline size_t grid_smem(unsigned int rows, unsigned int cap, unsigned in
          (size_t)room * kGridSliceBytes;
 }
 
-// Kept fraction from which the select runs over the bucket itself (k_select_grid) and not over a candidate list.  Two
-// states in turn, us, list / grid select, buckets of tensors of different scales | of one scale throughout (every 512
-// bytes of the bucket then hold a candidate, the worst case of the grid select):
-//   float32  16M: 0.1 82 / 64 | 72 / 84, 0.15 97 / 68 | 89 / 89, 0.2 106 / 75 | 93 / 94
-//            64M: 0.1 227 / 181 | 220 / 275, 0.15 289 / 195 | 296 / 289, 0.2 415 / 217 | 327 / 299
-//   bfloat16 32M: 0.05 58 / 55 | 61 / 86, 0.1 75 / 60 | 76 / 89, 0.15 97 / 69 | 102 / 94, 0.2 113 / 76 | 117 / 96
-//            67M: 0.05 91 / 88 | 99 / 155, 0.1 128 / 103 | 135 / 158, 0.15 170 / 115 | 184 / 170, 0.2 208 / 123 | 221 / 173
-// The lines are where several scales gain a fifth or more and one scale loses no more than that.
+// Kept fraction from which the select runs over the bucket itself (k_select_grid) and not over a candidate list.  us, list /
+// grid select, buckets of tensors of different scales | of one scale throughout (every 512 bytes of the bucket then hold a
+// candidate, the worst case of the grid select); a call by itself, then a pair of compress and sum on eight streams (the
+// grid select holds every SM through its shared steps, other calls' kernels run beside the list's):
+//   float32  1M    0.2  39 / 37 | 34 / 36      20 / 29 | 20 / 29
+//            3M    0.2  51 / 44 | 46 / 43      34 / 42 | 30 / 42
+//            6.5M  0.13 57 / 60 | 55 / 61      47 / 55 | 45 / 58      0.2  72 / 62 | 69 / 63      59 / 62 | 55 / 62
+//            16M   0.13 84 / 75 | 81 / 98      89 / 93 | 87 / 120     0.15 100 / 78 | 95 / 99     99 / 95 | 94 / 123
+//            40M   0.13 172 / 135 | 172 / 186  200 / 180 | 195 / 240  0.2  232 / 149 | 205 / 193  268 / 204 | 248 / 249
+//   bfloat16 3M    0.2  46 / 41 | 43 / 40      29 / 38 | 28 / 39
+//            12M   0.1  61 / 57 | 58 / 63      53 / 65 | 53 / 70      0.15 65 / 59 | 65 / 67      63 / 69 | 67 / 75
+//            34M   0.1  94 / 86 | 95 / 112     116 / 114 | 112 / 151  0.15 125 / 95 | 131 / 123   148 / 127 | 147 / 163
+//            67M   0.1  161 / 135 | 165 / 188  211 / 192 | 212 / 253  0.15 212 / 147 | 225 / 208  276 / 216 | 278 / 277
+// For a call by itself the lines are where several scales gain a fifth and one scale loses less than that; below 4M
+// elements, where a call gains a tenth and calls on streams lose a quarter, the list keeps what it is made for (a quarter).
+// many_calls (nsml_set_list_block_candidates above its default, the list stage then has fewer blocks): the list up to a
+// quarter, but for large buckets, where from 0.2 on both kinds of data gain (40M float32 275 / 194 | 254 / 246, 34M bfloat16
+// 178 / 140 | 189 / 177; 20M 108 / 110 | 111 / 134).
 template <int VT>  // element type of what is selected from
-constexpr double dense_from() { return VT == NSML_F32 ? 0.125 : 0.1; }
+inline double dense_from(int64_t n, bool many_calls = false) {
+  if (many_calls) return n < 32000000 ? 0.25 : 0.2;
+  if (n < 4000000) return 0.25;
+  if (n < 12000000) return 0.2;
+  if (n < 40000000) return 0.15;
+  return VT == NSML_F32 ? 0.125 : 0.1;
+}
 
 // What k_select_grid is launched with.  grid = 0: it does not take the call.
 struct GridPlan {
@@ -100,11 +116,12 @@ template <int VT>
 NSML_HD inline size_t grid_table_bytes(unsigned int rows) { return align_up(rows * grid_row_bytes<VT>(), 16); }
 
 // VT: element type of what is selected from (float32 where a residual is added); grad_dtype: of the bucket; blocks: those
-// that are resident at once, an even number.  The one place that decides: every size is taken, in a form that fits.
+// that are resident at once, an even number; many_calls: of dense_from.  The one place that decides: every size is taken,
+// in a form that fits.
 template <int VT>
-inline GridPlan grid_plan(int64_t n, int64_t k, int grad_dtype, unsigned int blocks) {
+inline GridPlan grid_plan(int64_t n, int64_t k, int grad_dtype, unsigned int blocks, bool many_calls = false) {
   GridPlan g;
-  if ((double)k < dense_from<VT>() * (double)n) return g;
+  if ((double)k < dense_from<VT>(n, many_calls) * (double)n) return g;
   // Bounds four standard deviations either side of the threshold's expected rank: one call in 16,000 takes another round
   // (3 us), the others have a window a third narrower than with six.
   const SamplePlan plan = sample_plan(n, k, grad_dtype, 4.0);

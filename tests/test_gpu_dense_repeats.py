@@ -76,7 +76,7 @@ def test_one_value_or_a_few(dtype):
     signs = rng.choice(np.array([-1, 1], np.float32), n)
     quantised = (np.round(rng.standard_normal(n) * 4) / 64).astype(np.float32)
     for g in (np.zeros(n, np.float32), np.full(n, 0.0123, np.float32) * signs, quantised):
-        for ratio in (0.13, 0.5, 0.93):
+        for ratio in (0.13, 0.26, 0.5, 0.93):
             check_compress(as_type(g, dtype), ratio, 8)
 
 
@@ -100,7 +100,7 @@ def test_magnitudes_below_the_sample_bins(dtype):
     check_compress(as_type(tiny, dtype), 0.5, 32)
     mixed = np.where(np.arange(n) % 3 == 0, spread(n, 26), tiny).astype(np.float32)
     mixed[::7] = 0.0
-    for ratio in (0.2, 0.3, 0.5, 0.8, 0.9):  # above, at and below the edge between the two, and among the zeros
+    for ratio in (0.2, 0.26, 0.3, 0.5, 0.8, 0.9):  # above, at and below the edge between the two, and among the zeros
         check_compress(as_type(mixed, dtype), ratio, 32)
 
 

@@ -18,12 +18,12 @@ static long taken = 0, left = 0, large = 0, wrong = 0;
 
 // what the kernel relies on, beside that the driver accepts the launch
 template <int VT>
-static void check(int64_t n, double ratio, int grad_dtype, unsigned int blocks) {
+static void check(int64_t n, double ratio, int grad_dtype, unsigned int blocks, bool many_calls) {
   int64_t k = (int64_t)std::ceil(ratio * (double)n);
   if (k > n) k = n;
-  const GridPlan g = grid_plan<VT>(n, k, grad_dtype, blocks);
+  const GridPlan g = grid_plan<VT>(n, k, grad_dtype, blocks, many_calls);
   if (g.grid == 0) {  // less is kept
-    wrong += (double)k >= dense_from<VT>() * (double)n;
+    wrong += (double)k >= dense_from<VT>(n, many_calls) * (double)n;
     ++left;
     return;
   }
@@ -61,9 +61,11 @@ int main() {
     for (int64_t n : at) {
       if (n <= 163840 || n > NSML_MAX_N) continue;
       for (double ratio : {0.05, 0.1, 0.125, 0.13, 0.2, 0.3, 0.5, 0.9, 0.999, 0.99999, 1.0}) {
-        check<NSML_F32>(n, ratio, NSML_F32, blocks);
-        check<NSML_F32>(n, ratio, NSML_BF16, blocks);  // (with a residual)
-        check<NSML_BF16>(n, ratio, NSML_BF16, blocks);
+        for (bool many_calls : {false, true}) {
+          check<NSML_F32>(n, ratio, NSML_F32, blocks, many_calls);
+          check<NSML_F32>(n, ratio, NSML_BF16, blocks, many_calls);  // (with a residual)
+          check<NSML_BF16>(n, ratio, NSML_BF16, blocks, many_calls);
+        }
       }
     }
   }
