@@ -225,7 +225,7 @@ int nsml_compress(const void* grad, int64_t n, int grad_dtype, double ratio, int
  *                        which it holds in shared memory as far as that goes
  *                        (kept fractions from 0.25 on below 4M elements, 0.2
  *                        below 12M, 0.15 below 40M, else 0.125, of bfloat16
- *                        buckets 0.1; with nsml_set_list_block_candidates
+ *                        buckets 0.1; with a residual 0.125 from 12M on; with nsml_set_list_block_candidates
  *                        above its default 0.25, from 32M elements on 0.2)
  * Buckets of up to 163,840 elements are taken by one kernel that holds them in
  * shared memory, whichever of the two this names for them.

@@ -292,7 +292,7 @@ static int launch_compress(const void* grad, float* residual, const uint32_t* ma
     return le == cudaSuccess ? NSML_OK : cuda_error();
   }
   // Dense mode: the select runs over the bucket itself, with no candidate list.
-  if (const GridPlan g = grid_plan<FDTYPE>(n, k, DTYPE, grid_blocks(dev), many_calls()); g.grid != 0) {
+  if (const GridPlan g = grid_plan<FDTYPE>(n, k, DTYPE, grid_blocks(dev), many_calls(), residual != nullptr); g.grid != 0) {
     {
       LaunchScope scope(K_CLEAR, st);
       le = launch_prio(k_clear, dim3(8), dim3(kCta), 0, st, false, 0, true, true, reinterpret_cast<uint4*>(ws), (unsigned int)(L.zero_bytes / 16),
@@ -635,7 +635,7 @@ int nsml_compress_strategy_of(int64_t n, double ratio, int grad_dtype, int resid
   const int rc = device_info(&dev);
   if (rc != NSML_OK) return rc;
   const unsigned int blocks = grid_blocks(*dev);
-  const GridPlan g = grad_dtype == NSML_F32 || residual ? grid_plan<NSML_F32>(n, k, grad_dtype, blocks, many_calls())
+  const GridPlan g = grad_dtype == NSML_F32 || residual ? grid_plan<NSML_F32>(n, k, grad_dtype, blocks, many_calls(), residual != 0)
                                                         : grid_plan<NSML_BF16>(n, k, grad_dtype, blocks, many_calls());
   return g.grid != 0 ? NSML_STRATEGY_DENSE : NSML_STRATEGY_LIST;
 }

@@ -91,17 +91,21 @@ NSML_HD inline size_t grid_smem(unsigned int rows, unsigned int cap, unsigned in
 //            12M   0.1  61 / 57 | 58 / 63      53 / 65 | 53 / 70      0.15 65 / 59 | 65 / 67      63 / 69 | 67 / 75
 //            34M   0.1  94 / 86 | 95 / 112     116 / 114 | 112 / 151  0.15 125 / 95 | 131 / 123   148 / 127 | 147 / 163
 //            67M   0.1  161 / 135 | 165 / 188  211 / 192 | 212 / 253  0.15 212 / 147 | 225 / 208  276 / 216 | 278 / 277
+//   with a residual, which the list stage subtracts from by scattered reads and writes (one call by itself):
+//   float32  6.5M  0.125 63 / 67 | 61 / 68    0.15 64 / 67 | 61 / 67     0.2  81 / 68 | 79 / 67
+//            16M   0.125 115 / 101 | 117 / 104  25M 168 / 146 | 164 / 159  45M 275 / 240 | 274 / 256
+//   bfloat16 6.5M  0.125 63 / 63 | 60 / 63    16M 112 / 97 | 110 / 101   45M 249 / 223 | 253 / 241
 // For a call by itself the lines are where several scales gain a fifth and one scale loses less than that; below 4M
 // elements, where a call gains a tenth and calls on streams lose a quarter, the list keeps what it is made for (a quarter).
 // many_calls (nsml_set_list_block_candidates above its default, the list stage then has fewer blocks): the list up to a
 // quarter, but for large buckets, where from 0.2 on both kinds of data gain (40M float32 275 / 194 | 254 / 246, 34M bfloat16
 // 178 / 140 | 189 / 177; 20M 108 / 110 | 111 / 134).
 template <int VT>  // element type of what is selected from
-inline double dense_from(int64_t n, bool many_calls = false) {
+inline double dense_from(int64_t n, bool many_calls = false, bool residual = false) {
   if (many_calls) return n < 32000000 ? 0.25 : 0.2;
   if (n < 4000000) return 0.25;
   if (n < 12000000) return 0.2;
-  if (n < 40000000) return 0.15;
+  if (n < 40000000 && !residual) return 0.15;
   return VT == NSML_F32 ? 0.125 : 0.1;
 }
 
@@ -116,12 +120,13 @@ template <int VT>
 NSML_HD inline size_t grid_table_bytes(unsigned int rows) { return align_up(rows * grid_row_bytes<VT>(), 16); }
 
 // VT: element type of what is selected from (float32 where a residual is added); grad_dtype: of the bucket; blocks: those
-// that are resident at once, an even number; many_calls: of dense_from.  The one place that decides: every size is taken,
+// that are resident at once, an even number; many_calls, residual: of dense_from.  The one place that decides: every size is taken,
 // in a form that fits.
 template <int VT>
-inline GridPlan grid_plan(int64_t n, int64_t k, int grad_dtype, unsigned int blocks, bool many_calls = false) {
+inline GridPlan grid_plan(int64_t n, int64_t k, int grad_dtype, unsigned int blocks, bool many_calls = false,
+                          bool residual = false) {
   GridPlan g;
-  if ((double)k < dense_from<VT>(n, many_calls) * (double)n) return g;
+  if ((double)k < dense_from<VT>(n, many_calls, residual) * (double)n) return g;
   // Bounds four standard deviations either side of the threshold's expected rank: one call in 16,000 takes another round
   // (3 us), the others have a window a third narrower than with six.
   const SamplePlan plan = sample_plan(n, k, grad_dtype, 4.0);

@@ -44,7 +44,9 @@ def ran(g, ratio, residual):
 def lines(many_calls, dtype, residual):
     if many_calls:
         return MANY
-    return LONE + [(40_000_000, 0.1 if dtype == torch.bfloat16 and not residual else 0.125)]
+    if residual:
+        return LONE[:4] + [(12_000_000, 0.125), (40_000_000, 0.125)]
+    return LONE + [(40_000_000, 0.1 if dtype == torch.bfloat16 else 0.125)]
 
 
 @pytest.mark.parametrize("many_calls", [False, True])

@@ -18,12 +18,12 @@ static long taken = 0, left = 0, large = 0, wrong = 0;
 
 // what the kernel relies on, beside that the driver accepts the launch
 template <int VT>
-static void check(int64_t n, double ratio, int grad_dtype, unsigned int blocks, bool many_calls) {
+static void check(int64_t n, double ratio, int grad_dtype, unsigned int blocks, bool many_calls, bool residual = false) {
   int64_t k = (int64_t)std::ceil(ratio * (double)n);
   if (k > n) k = n;
-  const GridPlan g = grid_plan<VT>(n, k, grad_dtype, blocks, many_calls);
+  const GridPlan g = grid_plan<VT>(n, k, grad_dtype, blocks, many_calls, residual);
   if (g.grid == 0) {  // less is kept
-    wrong += (double)k >= dense_from<VT>(n, many_calls) * (double)n;
+    wrong += (double)k >= dense_from<VT>(n, many_calls, residual) * (double)n;
     ++left;
     return;
   }
@@ -63,7 +63,8 @@ int main() {
       for (double ratio : {0.05, 0.1, 0.125, 0.13, 0.2, 0.3, 0.5, 0.9, 0.999, 0.99999, 1.0}) {
         for (bool many_calls : {false, true}) {
           check<NSML_F32>(n, ratio, NSML_F32, blocks, many_calls);
-          check<NSML_F32>(n, ratio, NSML_BF16, blocks, many_calls);  // (with a residual)
+          check<NSML_F32>(n, ratio, NSML_F32, blocks, many_calls, true);
+          check<NSML_F32>(n, ratio, NSML_BF16, blocks, many_calls, true);
           check<NSML_BF16>(n, ratio, NSML_BF16, blocks, many_calls);
         }
       }
