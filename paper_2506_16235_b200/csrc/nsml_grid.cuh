@@ -6,9 +6,11 @@
 // segments b, b + G, ...; a round of all blocks is a row), so that all SMs read one
 // compact, moving window of it and a tensor whose gradients are larger than others' is
 // spread over all of them.  A warp owns a slice, a 32nd, of each of its block's segments.
-// Slices with a key >= lo stay in shared memory as they are while there is room (33 MB on
-// 148 SMs: 8M float32); the others are read from the bucket once more when the survivors
-// are written.  Phases, separated by grid barriers:
+// Slices with a key >= lo stay in shared memory as they are while there is room beside the
+// tables and lists, which grow with the bucket (148 SMs, at 0.5: 26.7 MB for 6.5M float32
+// elements, which is all of them, 22.7 for 20M, 11.6 for 64M; bfloat16 26.4 for 20M, 19.6 for
+// 64M; LARGE 30.7); the others are read from the bucket once more when the survivors are
+// written.  Phases, separated by grid barriers:
 //   sample  the bounds lo and hi of the threshold (nsml_select.cuh), by 16 of the blocks;
 //           meanwhile every block has its first loads in flight
 //   stream  per slice: kept or not, its largest key, its number of keys >= hi; the keys of
