@@ -79,7 +79,8 @@ __device__ __forceinline__ void find_digit_from_top(const unsigned int (&own)[PE
 // Keys are counted by their top 14 bits (64 bins per octave) over the 108 octaves from 2^-76 to 2^32, by their top 11 bits
 // below and above, in 16-bit counters: 16 KB that eight blocks read from one another.  (All of the top 15 bits, 64 KB: the
 // sum over the blocks took 3 us, now 1.  With 128 octaves from 2^-96 on and nothing below, buckets around 1e-30 at 0.01
-// had no lower bound, so that all of them were listed: 16M float32 elements 3120 us instead of 46.)
+// had no lower bound, so that all of them were listed: 16M float32 elements 3120 us, now 53,
+// where an ordinary call takes 47.)
 constexpr int kSampleShift = 17, kSampleCoarse = 3;  // a fine bin is 2^17 keys, a coarse one 2^20
 constexpr unsigned int kSampleBins = 8192;
 constexpr unsigned int kSampleFine = 51u << 6, kSampleAbove = 159u << 6;  // key >> 17 of the first fine one, and behind the last
